@@ -79,8 +79,10 @@ void local_energy_forcebias(const LocalEnergyArgs& a, cudaStream_t st);
 int thc_pivoted_cholesky(const double* Mk, int n, double rtol, double* work, double* U_out, int* rank,
                          cudaStream_t st);
 // Per walker w of a chunk: g[w][mu] = T_w[mu][mu] and ex[w] = sum_{mu nu} Mk[mu][nu] T_w[mu][nu]
-// T_w[nu][mu], for T [wc][Nmu][Nmu] complex (fixed summation order).
-void thc_exchange(const cplx* T, int wc, int Nmu, const double* Mk, cplx* g, cplx* ex, cudaStream_t st);
+// T_w[nu][mu], for T [wc][Nmu][Nmu] complex (fixed summation order).  part: scratch of
+// wc * thc_exchange_shares(wc, Nmu) entries.
+int thc_exchange_shares(int wc, int Nmu);
+void thc_exchange(const cplx* T, int wc, int Nmu, const double* Mk, cplx* g, cplx* ex, cplx* part, cudaStream_t st);
 // Force-bias-only densities: g[w][mu] = sum_a Yt[a][mu] Z[w][a][mu] (Yt [N][Nmu], Z [W][N][Nmu]).
 void thc_gdiag(const cplx* Yt, const cplx* Z, int W, int N, int Nmu, cplx* g, cudaStream_t st);
 // XD[w][i][mu] = X[i][mu] d[w][mu] for the walkers of a chunk (X real [M][Nmu]).

@@ -68,6 +68,7 @@ struct Fp64Buffers {
     cplx* Z[2] = {nullptr, nullptr};       // Theta_s^T X: [W][N_s][Nmu]
     cplx* gs[2] = {nullptr, nullptr};      // densities at the points, per spin: [W][Nmu]
     cplx* ex[2] = {nullptr, nullptr};      // exchange sums per spin: [W]
+    cplx* ex_part = nullptr;               // their partial sums for a chunk of walkers
     cplx* Tthc = nullptr;                  // T = Yt^T Z for a chunk of walkers: [thc_wc][Nmu][Nmu]
     cplx* dv = nullptr;                    // U c per walker: [W][Nmu]
     cplx* XD = nullptr;                    // X diag(U c) for a chunk of walkers: [thc_wc][M][Nmu]

@@ -84,6 +84,9 @@ int fp64_alloc(afqmc_walkers* wk) {
         f.thc_wc = (int)std::max<size_t>(1, std::min<size_t>((size_t)W, budget / per_w));
         AFQMC_TRY(dalloc(&f.Tthc, (size_t)f.thc_wc * Nmu * Nmu));
         AFQMC_TRY(dalloc(&f.XD, (size_t)f.thc_wc * M * Nmu));
+        size_t parts = 0;   // of any chunk of 1 .. thc_wc walkers
+        for (int wc = 1; wc <= f.thc_wc; ++wc) parts = std::max(parts, (size_t)wc * thc_exchange_shares(wc, Nmu));
+        AFQMC_TRY(dalloc(&f.ex_part, parts));
         AFQMC_TRY(dalloc(&f.dv, (size_t)W * Nmu));
     } else {
         const size_t per_n = nd * W * Nmax * Nmax * sizeof(cplx);
@@ -111,7 +114,7 @@ void fp64_free(afqmc_walkers* wk) {
         for (void* p : ps)
             if (p) cudaFree(p);
     }
-    void* more[] = {f.Bh, f.T, f.A, f.msd_cc, f.msd_ls, f.msd_E, f.msd_t, f.msd_flag, f.msd_Es, f.Tthc, f.dv, f.XD};
+    void* more[] = {f.ex_part, f.Bh, f.T, f.A, f.msd_cc, f.msd_ls, f.msd_E, f.msd_t, f.msd_flag, f.msd_Es, f.Tthc, f.dv, f.XD};
     for (void* p : more)
         if (p) cudaFree(p);
     f = Fp64Buffers{};
@@ -165,7 +168,8 @@ void measure_det(afqmc_walkers* wk, int I, bool measure, int W, cplx* logS_out, 
                     g.B.ptr = f.Z[s] + (int64_t)w0 * N * Nmu; g.B.ld = Nmu; g.B.s1 = (int64_t)N * Nmu;
                     g.C = f.Tthc; g.ldc = Nmu; g.sc1 = (int64_t)Nmu * Nmu;
                     zgemm(g, st);
-                    thc_exchange(f.Tthc, wc, Nmu, wk->ham->Mk, f.gs[s] + (int64_t)w0 * Nmu, f.ex[s] + w0, st);
+                    thc_exchange(f.Tthc, wc, Nmu, wk->ham->Mk, f.gs[s] + (int64_t)w0 * Nmu, f.ex[s] + w0,
+                                 f.ex_part, st);
                 }
             } else {
                 thc_gdiag(f.Yt[s], f.Z[s], W, N, Nmu, f.gs[s], st);
