@@ -1770,7 +1770,13 @@ namespace {
 // sum_n L_n L_n^+ for symmetric (real) or Hermitian (complex) L_n, in `parts` partial sums:
 // for such L_n it equals X^+ X with X[(n, k)][i] = L[n][k][i], a contiguous [Nchol*M][M]
 // matrix.  The K = Nchol*M reduction is split into `parts` GEMMs (fixed split, reduced in a
-// fixed order by the caller's kernel) to fill the GPU.  Returns the workspace, or NULL.
+// fixed order by the caller's kernel) to fill the GPU.  gram_parts: two CTAs a SM over the
+// output's tiles, at least 4 vectors a part beyond 16.  Returns the workspace, or NULL.
+int gram_parts(int M, int Nchol) {
+    const int tiles = ((M + 63) / 64) * ((M + 63) / 64);
+    return std::max(1, std::min({Nchol, (304 + tiles - 1) / tiles, std::max(16, Nchol / 4)}));
+}
+
 cplx* gram_of_cholesky(const void* L, bool real, int M, int Nchol, int parts, cudaStream_t st) {
     const int per = (Nchol + parts - 1) / parts;  // Cholesky vectors per part
     cplx* buf = nullptr;
@@ -1779,26 +1785,32 @@ cplx* gram_of_cholesky(const void* L, bool real, int M, int Nchol, int parts, cu
         return nullptr;
     }
     fill_cplx(buf, (int64_t)parts * M * M, cplx{0.0, 0.0}, st);
-    for (int p = 0; p < parts; ++p) {
-        const int n0 = p * per, n1 = std::min(Nchol, n0 + per);
-        if (n1 <= n0) continue;
+    // every full part in one launch (64 x 64 tiles of one part alone would leave most SMs idle),
+    // then the rest
+    const int whole = Nchol / per, rest = Nchol - whole * per;
+    auto run = [&](int first, int count, int vectors) {
+        if (count < 1 || vectors < 1) return;
         GemmArgs g;
         g.m = g.n = M;
-        g.k = (n1 - n0) * M;
-        const void* X = real ? (const void*)(static_cast<const double*>(L) + (int64_t)n0 * M * M)
-                             : (const void*)(static_cast<const cplx*>(L) + (int64_t)n0 * M * M);
-        g.A.ptr = X; g.A.real = real; g.A.op = real ? OP_T : OP_C; g.A.ld = M;
-        g.B.ptr = X; g.B.real = real; g.B.op = OP_N; g.B.ld = M;
-        g.C = buf + (int64_t)p * M * M; g.ldc = M;
+        g.k = vectors * M;
+        g.nb1 = count;
+        const int64_t off = (int64_t)first * per * M * M;
+        const void* X = real ? (const void*)(static_cast<const double*>(L) + off)
+                             : (const void*)(static_cast<const cplx*>(L) + off);
+        g.A.ptr = X; g.A.real = real; g.A.op = real ? OP_T : OP_C; g.A.ld = M; g.A.s1 = (int64_t)per * M * M;
+        g.B.ptr = X; g.B.real = real; g.B.op = OP_N; g.B.ld = M; g.B.s1 = (int64_t)per * M * M;
+        g.C = buf + (int64_t)first * M * M; g.ldc = M; g.sc1 = (int64_t)M * M;
         zgemm(g, st);
-    }
+    };
+    run(0, whole, per);
+    run(whole, 1, rest);
     return buf;
 }
 
 }  // namespace
 
 void build_hprime(const double* h, const double* L, int M, int Nchol, double* hp, cudaStream_t st) {
-    const int parts = std::min(Nchol, 16);
+    const int parts = gram_parts(M, Nchol);
     cplx* buf = gram_of_cholesky(L, true, M, Nchol, parts, st);
     if (!buf) return;
     count_launch();
@@ -1807,7 +1819,7 @@ void build_hprime(const double* h, const double* L, int M, int Nchol, double* hp
 }
 
 void build_hprime_hermitian(const double* h, const cplx* V, int M, int Nv, cplx* hp, cudaStream_t st) {
-    const int parts = std::min(Nv, 16);
+    const int parts = gram_parts(M, Nv);
     cplx* buf = gram_of_cholesky(V, false, M, Nv, parts, st);
     if (!buf) return;
     count_launch();
