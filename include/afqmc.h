@@ -51,7 +51,10 @@ extern "C" {
 #define AFQMC_ERR_UNSUPPORTED -8  /* valid request the library does not handle  */
 
 /* ---- options ----------------------------------------------------------- */
-#define AFQMC_PREC_FP64    0  /* every contraction in FP64 (DFMA)                       */
+#define AFQMC_PREC_FP64    0  /* every contraction in FP64: the multiply-add pipe, or for
+                                 large products the tensor cores on operands cut into exact
+                                 fp16 digits (58 bits and more below each row's largest
+                                 entry, one rounding per result)                        */
 #define AFQMC_PREC_BF16X3  1  /* contractions on tcgen05 tensor cores (kind::f16, FP32
                                  accumulation) on operands split into row-scaled fp16
                                  slices whose leading products sum exactly: two slices

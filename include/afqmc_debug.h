@@ -69,6 +69,19 @@ int afqmc_debug_set_launch_policy(int grid_cap, int bn_max, int energy_bk);
 int afqmc_debug_inverse(const double* S, int N, int count, int variant, int with_inverse, double* Sout,
                         double* logdet, float* ms);
 
+/* One batched FP64 product of the walker step, C = alpha op(A) op(B) + beta C (and D += C), on host
+ * data.  d holds, as 64-bit integers: m, n, k, the three batch counts, then real (1: doubles, 0:
+ * complex), op (0 N, 1 T, 2 C), leading dimension and the three batch strides of A, the same of B,
+ * the leading dimension and batch strides of C and of D (elements), 28 values; sizes their element
+ * counts (A, B, C, D; D 0: none); ab = Re and Im of alpha, then of beta.  C and D are complex, read
+ * and written.  form: 0 the tiled multiply-add kernel, 1 the tensor-core form (sliced operands) in
+ * a workspace of ws_bytes, 2 what the step would choose, 3 one output per thread (*chose, may be
+ * NULL, receives the step's choice: 0, 1, or 2 for one output per thread).  *ms
+ * (may be NULL) receives the device time of a second run when reps > 0 (C and D then hold the result
+ * of reps + 1 runs). */
+int afqmc_debug_gemm(const long long* d, const long long* sizes, const double* ab, const double* A, const double* B,
+                     double* C, double* D, int form, long long ws_bytes, int reps, int* chose, float* ms);
+
 /* The adaptive choice of energy products (afqmc_opts.energy_terms = 1) on host data: for the
  * Frobenius norms norms[n] >= 0 of the nch rotated Cholesky vectors Ltilde_n, flags[g] = 1
  * (the lo*lo product is formed) for every group g of G consecutive vectors except the groups

@@ -552,6 +552,7 @@ static int init_walkers_impl(afqmc_ham_t ham, int ND, const double* Psi_up, cons
         for (int I = 0; I < ND; ++I) {
             const cplx* Psi = f.Psi[s] + I * mn;
             GemmArgs g;   // tmp[n] = Psi^+ L_n   [N][M]
+            g.ws = &f.ws;
             g.m = N; g.n = M; g.k = M; g.nb1 = nch;
             g.A.ptr = Psi; g.A.op = OP_C; g.A.ld = N;
             g.B.ptr = ham->L; g.B.real = !ham->cplx_L; g.B.ld = M; g.B.s1 = (int64_t)M * M;

@@ -135,6 +135,7 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
                 g.A.ld = M; g.A.s1 = (int64_t)N * M;
                 g.B.ptr = f.Theta[s]; g.B.ld = N; g.B.s2 = MN;
                 g.C = f.T; g.ldc = N; g.sc1 = (int64_t)W * N * N; g.sc2 = (int64_t)N * N;
+                g.ws = &f.ws;
                 zgemm(g, st);
             }
             {   // U[w][c] = -Theta_w T[c][w]  (+ c_n Theta_w below)
@@ -144,6 +145,7 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
                 g.B.ptr = f.T; g.B.ld = N; g.B.s1 = (int64_t)N * N; g.B.s2 = (int64_t)W * N * N;
                 g.alpha = cplx{-1.0, 0.0};
                 g.C = U; g.ldc = N; g.sc1 = (int64_t)nc * MN; g.sc2 = MN;
+                g.ws = &f.ws;
                 zgemm(g, st);
             }
             count_launch();
@@ -156,6 +158,7 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
                 g.B.ptr = U; g.B.ld = N; g.B.s1 = (int64_t)nc * MN;
                 g.beta = cplx{1.0, 0.0};
                 g.C = G; g.ldc = N; g.sc1 = MN;
+                g.ws = &f.ws;
                 zgemm(g, st);
             }
             if (want_L) {
@@ -166,6 +169,7 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
                 g.A.ptr = V; g.A.ld = N; g.A.s1 = MN;
                 g.B.ptr = f.Psi[s]; g.B.op = OP_C; g.B.ld = N;
                 g.C = F; g.ldc = M; g.sc1 = (int64_t)M * M;
+                g.ws = &f.ws;
                 zgemm(g, st);
                 count_launch();
                 add_re_transpose_kernel<<<nb((int64_t)nc * M * M), kT, 0, st>>>(F, nc, M, dLd + (int64_t)n0 * M * M);
@@ -178,6 +182,7 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
             g.B.ptr = f.Theta[s]; g.B.ld = N; g.B.s1 = MN;
             g.beta = cplx{1.0, 0.0};
             g.C = G; g.ldc = N; g.sc1 = MN;
+            g.ws = &f.ws;
             zgemm(g, st);   // G <- h Theta + G  (this is Y)
         }
         {   // Z = Psi^+ Y
@@ -186,6 +191,7 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
             g.A.ptr = f.Psi[s]; g.A.op = OP_C; g.A.ld = N;
             g.B.ptr = G; g.B.ld = N; g.B.s1 = MN;
             g.C = Z; g.ldc = N; g.sc1 = (int64_t)N * N;
+            g.ws = &f.ws;
             zgemm(g, st);
         }
         {   // F_w = Y - Theta Z   (in place in G)
@@ -196,6 +202,7 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
             g.alpha = cplx{-1.0, 0.0};
             g.beta = cplx{1.0, 0.0};
             g.C = G; g.ldc = N; g.sc1 = MN;
+            g.ws = &f.ws;
             zgemm(g, st);
         }
         count_launch();

@@ -1,5 +1,6 @@
 // Diagnostic entry points (include/afqmc_debug.h): one tensor-core building block per
 // call, host arrays in and out, for isolated parity tests.
+#include <algorithm>
 #include <cmath>
 #include <string>
 #include <vector>
@@ -275,5 +276,73 @@ extern "C" int afqmc_debug_wait_probe(long long limit_cycles, int release, unsig
     if (e != cudaSuccess) return fail(AFQMC_ERR_CUDA, std::string("debug_wait_probe: ") + cudaGetErrorString(e));
     AFQMC_CUDA_TRY(cudaMemcpy(status, flags.p, sizeof(unsigned), cudaMemcpyDeviceToHost));
     if (ms) *ms = t;
+    return AFQMC_OK;
+}
+
+extern "C" int afqmc_debug_gemm(const long long* d, const long long* sizes, const double* ab, const double* A,
+                                const double* B, double* C, double* D, int form, long long ws_bytes, int reps,
+                                int* chose, float* ms) {
+    if (!d || !sizes || !ab || !A || !B || !C || form < 0 || form > 3 || ws_bytes < 0 || reps < 0)
+        return fail(AFQMC_ERR_BADARG, "debug_gemm: bad arguments");
+    GemmArgs g;
+    g.m = (int)d[0]; g.n = (int)d[1]; g.k = (int)d[2];
+    g.nb0 = (int)d[3]; g.nb1 = (int)d[4]; g.nb2 = (int)d[5];
+    auto operand = [&](GemmOperand& X, const long long* q) {
+        X.real = q[0] != 0; X.op = (int)q[1]; X.ld = q[2]; X.s0 = q[3]; X.s1 = q[4]; X.s2 = q[5];
+    };
+    operand(g.A, d + 6);
+    operand(g.B, d + 12);
+    g.ldc = d[18]; g.sc0 = d[19]; g.sc1 = d[20]; g.sc2 = d[21];
+    g.ldd = d[22]; g.sd0 = d[23]; g.sd1 = d[24]; g.sd2 = d[25];
+    g.alpha = cplx{ab[0], ab[1]};
+    g.beta = cplx{ab[2], ab[3]};
+    DevBuf da, db, dc, dd, dw, flags;
+    const size_t ba = (size_t)sizes[0] * (g.A.real ? 8 : 16), bb = (size_t)sizes[1] * (g.B.real ? 8 : 16),
+                 bc = (size_t)sizes[2] * 16, bd = (size_t)sizes[3] * 16;
+    if (cudaMalloc(&da.p, ba) != cudaSuccess || cudaMalloc(&db.p, bb) != cudaSuccess || cudaMalloc(&dc.p, bc) != cudaSuccess ||
+        cudaMalloc(&dd.p, std::max<size_t>(bd, 16)) != cudaSuccess || cudaMalloc(&flags.p, 4) != cudaSuccess ||
+        cudaMalloc(&dw.p, std::max<size_t>((size_t)ws_bytes, 16)) != cudaSuccess)
+        return fail(AFQMC_ERR_OOM, "debug: allocation");
+    AFQMC_CUDA_TRY(cudaMemcpy(da.p, A, ba, cudaMemcpyHostToDevice));
+    AFQMC_CUDA_TRY(cudaMemcpy(db.p, B, bb, cudaMemcpyHostToDevice));
+    AFQMC_CUDA_TRY(cudaMemcpy(dc.p, C, bc, cudaMemcpyHostToDevice));
+    if (D) AFQMC_CUDA_TRY(cudaMemcpy(dd.p, D, bd, cudaMemcpyHostToDevice));
+    AFQMC_CUDA_TRY(cudaMemset(flags.p, 0, 4));
+    g.A.ptr = da.p;
+    g.B.ptr = db.p;
+    g.C = static_cast<cplx*>(dc.p);
+    g.D = D ? static_cast<cplx*>(dd.p) : nullptr;
+    SliceScratch ws;
+    ws.buf = dw.p;
+    ws.bytes = (size_t)ws_bytes;
+    ws.flags = static_cast<unsigned*>(flags.p);
+    if (chose) *chose = zgemm_form(g, &ws);
+    cudaEvent_t e0, e1;
+    AFQMC_CUDA_TRY(cudaEventCreate(&e0));
+    AFQMC_CUDA_TRY(cudaEventCreate(&e1));
+    int rc = AFQMC_OK;
+    for (int r = 0; r <= reps && rc == AFQMC_OK; ++r) {
+        if (r == reps) cudaEventRecord(e0);
+        if (form == 1) {
+            rc = slice_gemm(g, &ws, 0);
+        } else {
+            if (form == 2) g.ws = &ws;
+            zgemm_as(g, form == 2 ? zgemm_form(g, &ws) : form == 3 ? 2 : 0, 0);
+        }
+        if (r == reps) cudaEventRecord(e1);
+    }
+    float t = 0.f;
+    const cudaError_t e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) cudaEventElapsedTime(&t, e0, e1);
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    AFQMC_TRY(rc);
+    AFQMC_CUDA_TRY(e);
+    if (ms) *ms = t;
+    unsigned fl = 0;
+    AFQMC_CUDA_TRY(cudaMemcpy(&fl, flags.p, 4, cudaMemcpyDeviceToHost));
+    if (fl & FLAG_TIMEOUT) return fail(AFQMC_ERR_TIMEOUT, "debug_gemm: device wait timed out");
+    AFQMC_CUDA_TRY(cudaMemcpy(C, dc.p, bc, cudaMemcpyDeviceToHost));
+    if (D) AFQMC_CUDA_TRY(cudaMemcpy(D, dd.p, bd, cudaMemcpyDeviceToHost));
     return AFQMC_OK;
 }

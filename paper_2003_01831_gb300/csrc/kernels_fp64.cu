@@ -176,6 +176,58 @@ __global__ void __launch_bounds__(kThreads) zgemm_kernel(GemmArgs g) {
     }
 }
 
+// One output per thread, for products too small to fill tiles (few electrons, few walkers): a 64 x 64
+// or 32 x 32 tile does its padding's multiply-adds too, on one SM (25 us for a 24 x 5 output and
+// K = 24), where this spreads the outputs alone over all SMs.  Neighbouring threads run along a row
+// of the output, so A is a broadcast and B coalesced for op N.
+constexpr int kSmallT = 64;
+template <bool AR, bool BR>
+__global__ void __launch_bounds__(kSmallT) zgemm_small_kernel(GemmArgs g) {
+    using TA = typename Elem<AR>::T;
+    using TB = typename Elem<BR>::T;
+    const int64_t id = (int64_t)blockIdx.x * kSmallT + threadIdx.x;
+    const int c = (int)(id % g.n), r = (int)(id / g.n % g.m);
+    const int64_t b = id / ((int64_t)g.m * g.n);
+    const int64_t b2 = b % g.nb2, b1 = b / g.nb2 % g.nb1, b0 = b / g.nb2 / g.nb1;
+    if (b0 >= g.nb0) return;
+    const int64_t sa = g.A.op == OP_N ? 1 : g.A.ld, sb = g.B.op == OP_N ? g.B.ld : 1;
+    int64_t ia = b0 * g.A.s0 + b1 * g.A.s1 + b2 * g.A.s2 + (int64_t)r * (g.A.op == OP_N ? g.A.ld : 1);
+    int64_t ib = b0 * g.B.s0 + b1 * g.B.s1 + b2 * g.B.s2 + (int64_t)c * (g.B.op == OP_N ? 1 : g.B.ld);
+    cplx acc{0.0, 0.0};
+    const bool ca = g.A.op == OP_C, cb = g.B.op == OP_C;
+    int k = 0;
+    for (; k + 8 <= g.k; k += 8) {   // eight loads of each operand in flight
+        TA a[8];
+        TB v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            load_elem(a[q], g.A.ptr, ia + q * sa, ca);
+            load_elem(v[q], g.B.ptr, ib + q * sb, cb);
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) mac(acc, a[q], v[q]);
+        ia += 8 * sa;
+        ib += 8 * sb;
+    }
+    for (; k < g.k; ++k) {
+        TA a;
+        TB v;
+        load_elem(a, g.A.ptr, ia, ca);
+        load_elem(v, g.B.ptr, ib, cb);
+        mac(acc, a, v);
+        ia += sa;
+        ib += sb;
+    }
+    cplx v = g.alpha * acc;
+    cplx* cp = g.C + b0 * g.sc0 + b1 * g.sc1 + b2 * g.sc2 + (int64_t)r * g.ldc + c;
+    if (g.beta.re != 0.0 || g.beta.im != 0.0) v = v + g.beta * (*cp);
+    *cp = v;
+    if (g.D) {
+        cplx* dp = g.D + b0 * g.sd0 + b1 * g.sd1 + b2 * g.sd2 + (int64_t)r * g.ldd + c;
+        *dp = *dp + v;
+    }
+}
+
 // ------------------------------------------------------------------ Gauss-Jordan
 constexpr int kGJU = 8;   // element updates in flight per thread
 __global__ void __launch_bounds__(kThreads)
@@ -1502,25 +1554,63 @@ inline unsigned blocks_for(int64_t n, int t = kThreads) { return (unsigned)((n +
 }  // namespace
 
 // ================================================================== launchers
-// 32 x 32 tiles when they cover the output with at most 60% of the 64 x 64 tiles' area
-// (small blocks of few-electron systems), 64 x 64 otherwise.
-void zgemm(const GemmArgs& g, cudaStream_t st) {
-    if (g.m <= 0 || g.n <= 0) return;
-    const int64_t nbatch = (int64_t)g.nb0 * g.nb1 * g.nb2;
+// 32 x 32 tiles when they cover the output with at most 60% of the 64 x 64 tiles' area (small
+// blocks of few-electron systems), 64 x 64 otherwise.
+static int zgemm_tile(const GemmArgs& g) {
     const int64_t a64 = (int64_t)((g.m + 63) / 64) * ((g.n + 63) / 64) * 4096;
     const int64_t a32 = (int64_t)((g.m + 31) / 32) * ((g.n + 31) / 32) * 1024;
-    const bool small = 10 * a32 <= 6 * a64;
-    const int ts = small ? 32 : 64;
-    dim3 grid((g.n + ts - 1) / ts, (g.m + ts - 1) / ts, (unsigned)std::min<int64_t>(nbatch, 65535));
+    return 10 * a32 <= 6 * a64 ? 32 : 64;
+}
+
+// The form of a product, by estimated time (microseconds; constants fitted to products of M = 24 to
+// 128, N = 5 to 32, W = 2 to 512):
+//   * 0, tiles: the padded multiply-adds at 85% of the FP64 pipe (5.2e5 a microsecond over all SMs), no less than one
+//     tile's on its SM;
+//   * 2, one output per thread: the multiply-adds alone, at 3.0e5 a microsecond, and the latency of
+//     its loads along K;
+//   * 1, the tensor cores (where the caller gives a workspace): slice_gemm_us, gemm_slices.cu.
+int zgemm_form(const GemmArgs& g, const SliceScratch* ws) {
+    const double nbatch = (double)g.nb0 * g.nb1 * g.nb2;
+    const double per = (g.A.real ? 1.0 : 2.0) * (g.B.real ? 1.0 : 2.0) * g.k;   // multiply-adds an output
+    const int ts = zgemm_tile(g);
+    const double tiles = nbatch * ((g.m + ts - 1) / ts) * ((g.n + ts - 1) / ts);
+    const double tiled_us = 3.0 + ceil(tiles / 152.0) * ts * ts * per / 3.4e3;
+    const double outputs = nbatch * g.m * g.n;
+    const double thread_us = outputs < 1e11 ? 3.0 + std::max(outputs * per / 3.0e5, 0.05 * g.k) + 0.01 * g.k : 1e30;
+    const double slice_us = ws && ws->buf && g.k > 0 ? slice_gemm_us(g) : 1e30;
+    if (slice_us < std::min(tiled_us, thread_us)) return 1;
+    return thread_us < tiled_us ? 2 : 0;
+}
+
+void zgemm_as(const GemmArgs& g, int form, cudaStream_t st) {
+    if (g.m <= 0 || g.n <= 0) return;
+    if (form == 1 && slice_gemm(g, g.ws, st) == AFQMC_OK) return;
+    if (g.ws) g.ws->a = g.ws->b = SliceScratch::Packed{};   // no slices for the next product to keep
+    const int64_t nbatch = (int64_t)g.nb0 * g.nb1 * g.nb2;
     count_launch();
+    if (form == 2) {
+        const unsigned blocks = (unsigned)((nbatch * g.m * g.n + kSmallT - 1) / kSmallT);
+        if (g.A.real && g.B.real) zgemm_small_kernel<true, true><<<blocks, kSmallT, 0, st>>>(g);
+        else if (g.A.real) zgemm_small_kernel<true, false><<<blocks, kSmallT, 0, st>>>(g);
+        else if (g.B.real) zgemm_small_kernel<false, true><<<blocks, kSmallT, 0, st>>>(g);
+        else zgemm_small_kernel<false, false><<<blocks, kSmallT, 0, st>>>(g);
+        return;
+    }
+    const int ts = zgemm_tile(g);
+    dim3 grid((g.n + ts - 1) / ts, (g.m + ts - 1) / ts, (unsigned)std::min<int64_t>(nbatch, 65535));
     auto go = [&](auto k32, auto k64) {
-        if (small) k32<<<grid, kThreads, 0, st>>>(g);
+        if (ts == 32) k32<<<grid, kThreads, 0, st>>>(g);
         else k64<<<grid, kThreads, 0, st>>>(g);
     };
     if (g.A.real && g.B.real) go(zgemm_kernel<true, true, 32>, zgemm_kernel<true, true, 64>);
     else if (g.A.real) go(zgemm_kernel<true, false, 32>, zgemm_kernel<true, false, 64>);
     else if (g.B.real) go(zgemm_kernel<false, true, 32>, zgemm_kernel<false, true, 64>);
     else go(zgemm_kernel<false, false, 32>, zgemm_kernel<false, false, 64>);
+}
+
+void zgemm(const GemmArgs& g, cudaStream_t st) {
+    if (g.m <= 0 || g.n <= 0) return;
+    zgemm_as(g, zgemm_form(g, g.ws), st);
 }
 
 void batched_inverse_logdet(cplx* S, int64_t stride, int N, int count, cplx* logdet, bool with_inverse,

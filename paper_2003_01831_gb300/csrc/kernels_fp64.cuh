@@ -18,6 +18,18 @@ struct GemmOperand {
     int64_t s0 = 0;
 };
 
+// Workspace of the products that run on the tensor cores (gemm_slices.cu): device memory for the
+// operands' slices and the status word their bounded waits report to; a, b: the shapes of the
+// operands whose slices it holds (of the last product).
+struct SliceScratch {
+    void* buf = nullptr;
+    size_t bytes = 0;
+    unsigned* flags = nullptr;
+    struct Packed {
+        int64_t rows = -1, pitch = 0, batches = 0;
+    } a, b;
+};
+
 // C[b] = alpha op(A[b]) op(B[b]) + beta C[b];  if D != null also D[b] += (that result).
 // batch index b = (b0 * nb1 + b1) * nb2 + b2, nbatch = nb0 * nb1 * nb2.
 struct GemmArgs {
@@ -31,8 +43,22 @@ struct GemmArgs {
     int64_t ldd = 0, sd1 = 0, sd2 = 0;
     int nb0 = 1;
     int64_t sc0 = 0, sd0 = 0;
+    SliceScratch* ws = nullptr;   // allows the tensor-core form, in this workspace
+    // the operand (with alpha, for the one it multiplies) is that of the previous product in this
+    // workspace: its slices are taken as they are
+    bool keep_a = false, keep_b = false;
 };
 
+// The FP64 products' tensor-core form (gemm_slices.cu): its expected time in microseconds (huge where
+// it does not apply), the workspace it wants (a smaller one is used in pieces) and the product.
+double slice_gemm_us(const GemmArgs& g);
+size_t slice_gemm_bytes(const GemmArgs& g);
+int slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st);
+
+// The product in the form expected to be fastest: zgemm_form's 0 (tiles), 1 (tensor cores, where
+// there is a workspace) or 2 (one output per thread).  zgemm_as: in the form given.
+int zgemm_form(const GemmArgs& g, const SliceScratch* ws);
+void zgemm_as(const GemmArgs& g, int form, cudaStream_t st);
 void zgemm(const GemmArgs& g, cudaStream_t st);
 
 // In-place Gauss-Jordan inverse (with_inverse) or LU elimination (log-det only) of `count`

@@ -82,13 +82,6 @@ struct SharedCtl {
     double red[8][4];   // energy epilogue: per-warp (t.re, t.im, X.re, X.im)
 };
 
-__device__ __forceinline__ bool wait_drain(uint64_t* bar, uint32_t parity) {
-    const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity))
-        if (clock64() - t0 > kTimeoutCycles) return false;
-    return true;
-}
-
 // --------------------------------------------------------------------------- epilogues
 __device__ __forceinline__ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
@@ -1909,6 +1902,25 @@ int launch_energy_pair(const CUtensorMap* m, const EnergyShape& es, unsigned* fl
     cudaError_t e = cudaLaunchKernelEx(&cfg, kern, m[0], m[1], m[2], m[3], m[4], m[5], es, flags);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return fail(AFQMC_ERR_CUDA, std::string("tc_energy (CTA pairs) launch: ") + cudaGetErrorString(e));
+    return AFQMC_OK;
+}
+
+int make_map4(CUtensorMap* m, const void* base, const uint64_t* dims, const uint64_t* strides, const uint32_t* box,
+              int swizzle) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return fail(AFQMC_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
+    cuuint64_t d[4], st[3];
+    cuuint32_t b[4], es[4] = {1, 1, 1, 1};
+    for (int i = 0; i < 4; ++i) {
+        d[i] = dims[i];
+        b[i] = box[i];
+        if (i < 3) st[i] = strides[i];
+    }
+    const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void*>(base), d, st, b, es,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE,
+                          swizzle == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(AFQMC_ERR_CUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
     return AFQMC_OK;
 }
 

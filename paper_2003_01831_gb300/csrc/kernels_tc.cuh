@@ -216,5 +216,9 @@ void split_rows(const float* src, int64_t src_stride, int64_t rows, int64_t K, b
                 cudaStream_t st, bf16* rounded = nullptr);   // rounded (optional): r = fp16(x / scale)
 
 int tc_num_sms();
+// 4-D fp16 tensor map (innermost dimension first; strides of dimensions 1 .. 3 in bytes; swizzle 64
+// or 128 bytes = the innermost box).
+int make_map4(CUtensorMap* m, const void* base, const uint64_t* dims, const uint64_t* strides, const uint32_t* box,
+              int swizzle);
 
 }  // namespace afqmc

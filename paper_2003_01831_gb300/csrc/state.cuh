@@ -51,6 +51,7 @@ struct Fp64Buffers {
     cplx* Theta[2] = {nullptr, nullptr};   // [W][M][N_s]
     cplx* t[2] = {nullptr, nullptr};       // [W][Nchol]
     cplx* X[2] = {nullptr, nullptr};       // [W][Nchol]
+    SliceScratch ws;                       // operand slices of the products on the tensor cores
     cplx* T = nullptr;                     // trace chunk [nc][W][N][N]
     int nc = 0;
     cplx* A = nullptr;                     // [W][M][M] HS potential

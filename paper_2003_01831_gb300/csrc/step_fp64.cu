@@ -31,8 +31,9 @@ void add_logdet(const cplx* a, const cplx* b, cplx* out, int n, cudaStream_t st)
 
 // Y[w] = op(X) Phi[w]-style helpers --------------------------------------------------------
 // S_w = Psi^+ Phi_w   (N x N)
-void overlap(const cplx* Psi, const cplx* Phi, cplx* S, int M, int N, int W, cudaStream_t st) {
+void overlap(const cplx* Psi, const cplx* Phi, cplx* S, int M, int N, int W, SliceScratch* ws, cudaStream_t st) {
     GemmArgs g;
+    g.ws = ws;
     g.m = N; g.n = N; g.k = M; g.nb1 = W;
     g.A.ptr = Psi; g.A.op = OP_C; g.A.ld = N;
     g.B.ptr = Phi; g.B.op = OP_N; g.B.ld = N; g.B.s1 = (int64_t)M * N;
@@ -95,6 +96,31 @@ int fp64_alloc(afqmc_walkers* wk) {
         AFQMC_TRY(dalloc(&f.T, (size_t)f.nc * nd * W * Nmax * Nmax));
     }
     AFQMC_TRY(dalloc(&f.A, (size_t)W * M * M));
+    if (wk->opts.precision == AFQMC_PREC_FP64) {
+        // slices of the step's largest products, up to a bound beyond which they run in pieces
+        auto shape = [&](int64_t m, int64_t n, int64_t k, int64_t nba, int64_t nbb, int64_t nbs, bool ar, bool br) {
+            GemmArgs g;   // nba batches of A's own, nbb of B's own, nbs shared
+            g.m = (int)m; g.n = (int)n; g.k = (int)k;
+            g.nb0 = (int)nba; g.nb1 = (int)nbb; g.nb2 = (int)nbs;
+            g.A.real = ar; g.B.real = br;
+            g.A.s0 = 1; g.B.s1 = 1; g.A.s2 = g.B.s2 = 1;
+            return slice_gemm_bytes(g);
+        };
+        const bool rl = !wk->ham->cplx_L;
+        size_t need = 0;
+        for (int s = 0; s < 2; ++s) {
+            const int N = wk->N[s];
+            need = std::max({need, shape(N, N, M, 1, W, nd, false, false), shape(M, N, N, 1, 1, nd * W, false, false),
+                             shape(M, N, M, 1, 1, W, false, false), shape(M, N, M, 1, W, 1, rl, false)});
+            if (Nmu > 0) need = std::max({need, shape(N, Nmu, M, W, 1, 1, false, true), shape(Nmu, Nmu, N, 1, f.thc_wc, 1, false, false)});
+            else need = std::max(need, shape(N, N, M, f.nc, W, nd, false, false));
+        }
+        if (Nmu > 0) need = std::max(need, shape(M, M, Nmu, f.thc_wc, 1, 1, false, true));
+        else need = std::max(need, shape(W, (int64_t)M * M, nch, 1, 1, 1, false, rl));
+        f.ws.bytes = std::min(need, (size_t)768 << 20);
+        AFQMC_TRY(dalloc(reinterpret_cast<char**>(&f.ws.buf), f.ws.bytes));
+        f.ws.flags = wk->flags;
+    }
     if (ND > 1) {
         AFQMC_TRY(dalloc(&f.msd_cc, (size_t)ND));
         AFQMC_TRY(dalloc(&f.msd_ls, (size_t)ND * W));
@@ -114,7 +140,7 @@ void fp64_free(afqmc_walkers* wk) {
         for (void* p : ps)
             if (p) cudaFree(p);
     }
-    void* more[] = {f.ex_part, f.Bh, f.T, f.A, f.msd_cc, f.msd_ls, f.msd_E, f.msd_t, f.msd_flag, f.msd_Es, f.Tthc, f.dv, f.XD};
+    void* more[] = {f.ws.buf, f.ex_part, f.Bh, f.T, f.A, f.msd_cc, f.msd_ls, f.msd_E, f.msd_t, f.msd_flag, f.msd_Es, f.Tthc, f.dv, f.XD};
     for (void* p : more)
         if (p) cudaFree(p);
     f = Fp64Buffers{};
@@ -138,7 +164,7 @@ void measure_det(afqmc_walkers* wk, int I, bool measure, int W, cplx* logS_out, 
                                      : (const void*)(static_cast<const cplx*>(f.Lt[s]) + lt);
         const void* LtT = wk->Lt_real ? (const void*)(static_cast<const double*>(f.LtT[s]) + lt)
                                       : (const void*)(static_cast<const cplx*>(f.LtT[s]) + lt);
-        overlap(Psi, f.Phi[s], f.S[s], M, N, W, st);
+        overlap(Psi, f.Phi[s], f.S[s], M, N, W, &f.ws, st);
         batched_inverse_logdet(f.S[s], (int64_t)N * N, N, W, f.ld[s], true, inv_flags, st);
         {   // Theta_w = Phi_w S_w^-1
             GemmArgs g;
@@ -146,6 +172,7 @@ void measure_det(afqmc_walkers* wk, int I, bool measure, int W, cplx* logS_out, 
             g.A.ptr = f.Phi[s]; g.A.ld = N; g.A.s1 = (int64_t)M * N;
             g.B.ptr = f.S[s]; g.B.ld = N; g.B.s1 = (int64_t)N * N;
             g.C = f.Theta[s]; g.ldc = N; g.sc1 = (int64_t)M * N;
+            g.ws = &f.ws;
             zgemm(g, st);
         }
         if (s == 0 && wk->ev0 && timed) cudaEventRecord(wk->ev0, st);
@@ -158,6 +185,7 @@ void measure_det(afqmc_walkers* wk, int I, bool measure, int W, cplx* logS_out, 
             z.A.ptr = f.Theta[s]; z.A.op = OP_T; z.A.ld = N; z.A.s1 = (int64_t)M * N;
             z.B.ptr = wk->ham->X; z.B.real = true; z.B.ld = Nmu;
             z.C = f.Z[s]; z.ldc = Nmu; z.sc1 = (int64_t)N * Nmu;
+            z.ws = &f.ws;
             zgemm(z, st);
             if (measure) {
                 for (int w0 = 0; w0 < W; w0 += f.thc_wc) {
@@ -167,6 +195,7 @@ void measure_det(afqmc_walkers* wk, int I, bool measure, int W, cplx* logS_out, 
                     g.A.ptr = f.Yt[s]; g.A.op = OP_T; g.A.ld = Nmu;
                     g.B.ptr = f.Z[s] + (int64_t)w0 * N * Nmu; g.B.ld = Nmu; g.B.s1 = (int64_t)N * Nmu;
                     g.C = f.Tthc; g.ldc = Nmu; g.sc1 = (int64_t)Nmu * Nmu;
+                    g.ws = &f.ws;
                     zgemm(g, st);
                     thc_exchange(f.Tthc, wc, Nmu, wk->ham->Mk, f.gs[s] + (int64_t)w0 * Nmu, f.ex[s] + w0,
                                  f.ex_part, st);
@@ -179,6 +208,7 @@ void measure_det(afqmc_walkers* wk, int I, bool measure, int W, cplx* logS_out, 
             t.A.ptr = f.gs[s]; t.A.ld = Nmu;
             t.B.ptr = wk->ham->U; t.B.real = true; t.B.ld = nch;
             t.C = f.t[s]; t.ldc = nch;
+            t.ws = &f.ws;
             zgemm(t, st);
         } else if (measure) {
             for (int n0 = 0; n0 < nch; n0 += f.nc) {
@@ -192,6 +222,8 @@ void measure_det(afqmc_walkers* wk, int I, bool measure, int W, cplx* logS_out, 
                 g.A.ld = M; g.A.s1 = (int64_t)N * M; g.A.s2 = 0;
                 g.B.ptr = f.Theta[s]; g.B.ld = N; g.B.s1 = 0; g.B.s2 = (int64_t)M * N;
                 g.C = f.T; g.ldc = N; g.sc1 = (int64_t)W * N * N; g.sc2 = (int64_t)N * N;
+                g.keep_b = n0 > 0;   // Theta's slices stay from chunk to chunk
+                g.ws = &f.ws;
                 zgemm(g, st);
                 trace_terms(f.T, nc, W, N, n0, f.t[s], f.X[s], nch, st);
             }
@@ -202,6 +234,7 @@ void measure_det(afqmc_walkers* wk, int I, bool measure, int W, cplx* logS_out, 
             g.A.ptr = f.Theta[s]; g.A.op = OP_N; g.A.ld = (int64_t)M * N;
             g.B.real = wk->Lt_real; g.B.ptr = LtT; g.B.op = OP_T; g.B.ld = (int64_t)M * N;
             g.C = f.t[s]; g.ldc = nch;
+            g.ws = &f.ws;
             zgemm(g, st);
         }
         if (s == 1 && wk->ev1 && timed) { cudaEventRecord(wk->ev1, st); wk->ev_valid = true; }
@@ -242,6 +275,7 @@ void measure_msd(afqmc_walkers* wk, bool measure, int W, cudaStream_t st) {
             g.A.ptr = f.Psi[s] + I0 * mn; g.A.op = OP_C; g.A.ld = N; g.A.s1 = mn;
             g.B.ptr = f.Phi[s]; g.B.ld = N; g.B.s2 = mn;
             g.C = f.S[s]; g.ldc = N; g.sc1 = (int64_t)W * nn; g.sc2 = nn;
+            g.ws = &f.ws;
             zgemm(g, st);
             batched_inverse_logdet(f.S[s], nn, N, nd * W, f.ld[s], true, f.msd_flag, st);
             GemmArgs t;   // Theta[I][w] = Phi_w S[I][w]^-1
@@ -249,6 +283,7 @@ void measure_msd(afqmc_walkers* wk, bool measure, int W, cudaStream_t st) {
             t.A.ptr = f.Phi[s]; t.A.ld = N; t.A.s2 = mn;
             t.B.ptr = f.S[s]; t.B.ld = N; t.B.s1 = (int64_t)W * nn; t.B.s2 = nn;
             t.C = f.Theta[s]; t.ldc = N; t.sc1 = (int64_t)W * mn; t.sc2 = mn;
+            t.ws = &f.ws;
             zgemm(t, st);
             const size_t esz = wk->Lt_real ? sizeof(double) : sizeof(cplx);
             const char* Lt = static_cast<const char*>(f.Lt[s]) + esz * (size_t)(I0 * ltI);
@@ -262,7 +297,9 @@ void measure_msd(afqmc_walkers* wk, bool measure, int W, cudaStream_t st) {
                     e.A.ptr = Lt + esz * (size_t)((int64_t)n0 * N * M);
                     e.A.ld = M; e.A.s0 = (int64_t)N * M; e.A.s1 = ltI;
                     e.B.ptr = f.Theta[s]; e.B.ld = N; e.B.s1 = (int64_t)W * mn; e.B.s2 = mn;
+                    e.keep_b = n0 > 0;
                     e.C = f.T; e.ldc = N; e.sc0 = (int64_t)nd * W * nn; e.sc1 = (int64_t)W * nn; e.sc2 = nn;
+                    e.ws = &f.ws;
                     zgemm(e, st);
                     trace_terms(f.T, nc, nd * W, N, n0, f.t[s], f.X[s], nch, st);
                 }
@@ -272,6 +309,7 @@ void measure_msd(afqmc_walkers* wk, bool measure, int W, cudaStream_t st) {
                 b.A.ptr = f.Theta[s]; b.A.ld = mn; b.A.s1 = (int64_t)W * mn;
                 b.B.real = wk->Lt_real; b.B.ptr = LtT; b.B.op = OP_T; b.B.ld = mn; b.B.s1 = ltI;
                 b.C = f.t[s]; b.ldc = nch; b.sc1 = (int64_t)W * nch;
+                b.ws = &f.ws;
                 zgemm(b, st);
             }
         }
@@ -343,6 +381,7 @@ int fp64_propagate_and_weight(afqmc_walkers* wk, const double* x, cudaStream_t s
         d.A.ptr = wk->coef; d.A.ld = nch;
         d.B.ptr = wk->ham->U; d.B.real = true; d.B.op = OP_T; d.B.ld = nch;
         d.C = f.dv; d.ldc = Nmu;
+        d.ws = &f.ws;
         zgemm(d, st);
         for (int w0 = 0; w0 < W; w0 += f.thc_wc) {
             const int wc = std::min(f.thc_wc, W - w0);
@@ -352,6 +391,7 @@ int fp64_propagate_and_weight(afqmc_walkers* wk, const double* x, cudaStream_t s
             g.A.ptr = f.XD; g.A.ld = Nmu; g.A.s1 = (int64_t)M * Nmu;
             g.B.ptr = wk->ham->X; g.B.real = true; g.B.op = OP_T; g.B.ld = Nmu;
             g.C = f.A + (int64_t)w0 * M * M; g.ldc = M; g.sc1 = (int64_t)M * M;
+            g.ws = &f.ws;
             zgemm(g, st);
         }
     } else {   // A_w = sum_n c[w][n] L_n
@@ -360,40 +400,54 @@ int fp64_propagate_and_weight(afqmc_walkers* wk, const double* x, cudaStream_t s
         g.A.ptr = wk->coef; g.A.ld = nch;
         g.B.ptr = wk->ham->L; g.B.real = !wk->ham->cplx_L; g.B.ld = (int64_t)M * M;
         g.C = f.A; g.ldc = (int64_t)M * M;
+        g.ws = &f.ws;
         zgemm(g, st);
     }
     const double sq = sqrt(wk->tau);
+    // both spins go through each stage together, so that the slices of A_w serve every Taylor term
+    cplx *P0[2], *P1[2];
     for (int s = 0; s < 2; ++s) {
         const int N = wk->N[s];
         const int64_t mn = (int64_t)M * N;
-        cplx* P0 = f.Pa[s];
-        cplx* P1 = f.Pb[s];
+        P0[s] = f.Pa[s];
+        P1[s] = f.Pb[s];
         GemmArgs g;   // P0 = B Phi
         g.m = M; g.n = N; g.k = M; g.nb1 = W;
         g.A.ptr = f.Bh; g.A.real = !wk->ham->cplx_L; g.A.ld = M;
         g.B.ptr = f.Phi[s]; g.B.ld = N; g.B.s1 = mn;
-        g.C = P0; g.ldc = N; g.sc1 = mn;
+        g.C = P0[s]; g.ldc = N; g.sc1 = mn;
+        g.ws = &f.ws;
         zgemm(g, st);
-        cudaMemcpyAsync(f.Pnew[s], P0, sizeof(cplx) * W * mn, cudaMemcpyDeviceToDevice, st);
-        for (int k = 1; k <= wk->opts.k_taylor; ++k) {
+        cudaMemcpyAsync(f.Pnew[s], P0[s], sizeof(cplx) * W * mn, cudaMemcpyDeviceToDevice, st);
+    }
+    for (int k = 1; k <= wk->opts.k_taylor; ++k)
+        for (int s = 0; s < 2; ++s) {
+            const int N = wk->N[s];
+            const int64_t mn = (int64_t)M * N;
             GemmArgs t;   // P1 = (i sqrt(tau) / k) A_w P0 ;  Pnew += P1
             t.m = M; t.n = N; t.k = M; t.nb1 = W;
             t.A.ptr = f.A; t.A.ld = M; t.A.s1 = (int64_t)M * M;
-            t.B.ptr = P0; t.B.ld = N; t.B.s1 = mn;
+            t.B.ptr = P0[s]; t.B.ld = N; t.B.s1 = mn;
             t.alpha = cplx{0.0, sq / k};
-            t.C = P1; t.ldc = N; t.sc1 = mn;
+            t.C = P1[s]; t.ldc = N; t.sc1 = mn;
             t.D = f.Pnew[s]; t.ldd = N; t.sd1 = mn;
+            t.ws = &f.ws;
+            t.keep_a = k > 1 || s > 0;
             zgemm(t, st);
-            std::swap(P0, P1);
+            std::swap(P0[s], P1[s]);
         }
+    for (int s = 0; s < 2; ++s) {
+        const int N = wk->N[s];
+        const int64_t mn = (int64_t)M * N;
         GemmArgs b2;  // Phi' = B Pnew  -> Pa
         b2.m = M; b2.n = N; b2.k = M; b2.nb1 = W;
         b2.A.ptr = f.Bh; b2.A.real = !wk->ham->cplx_L; b2.A.ld = M;
         b2.B.ptr = f.Pnew[s]; b2.B.ld = N; b2.B.s1 = mn;
         b2.C = f.Pa[s]; b2.ldc = N; b2.sc1 = mn;
+        b2.ws = &f.ws;
         zgemm(b2, st);
         if (wk->ND == 1) {
-            overlap(f.Psi[s], f.Pa[s], f.S[s], M, N, W, st);
+            overlap(f.Psi[s], f.Pa[s], f.S[s], M, N, W, &f.ws, st);
             batched_inverse_logdet(f.S[s], (int64_t)N * N, N, W, f.ld[s], false, wk->flags, st);
         }
     }
@@ -411,6 +465,7 @@ int fp64_propagate_and_weight(afqmc_walkers* wk, const double* x, cudaStream_t s
                 g.A.ptr = f.Psi[s] + I0 * mn; g.A.op = OP_C; g.A.ld = N; g.A.s1 = mn;
                 g.B.ptr = f.Pa[s]; g.B.ld = N; g.B.s2 = mn;
                 g.C = f.S[s]; g.ldc = N; g.sc1 = (int64_t)W * nn; g.sc2 = nn;
+                g.ws = &f.ws;
                 zgemm(g, st);
                 batched_inverse_logdet(f.S[s], nn, N, nd * W, f.ld[s], false, f.msd_flag, st);
             }
