@@ -64,16 +64,44 @@ struct Digits {
     static constexpr int kStageBytes = S * (kRows + kCols) * kChunk * 2;
 };
 
+// Division of 0 <= x < 2^31 by a fixed divisor d: x / d = (x mul) >> (32 + shift) with mul =
+// ceil(2^(32 + shift) / d), shift = ceil(log2 d) - 1 (d > 1), which is exact for such x
+// (Granlund and Montgomery, PLDI 1994).
+struct Div {
+    uint32_t mul = 0, d = 1;
+    int shift = 0;
+    Div() = default;
+    explicit Div(int64_t n) : d((uint32_t)n) {
+        if (d <= 1) return;
+        while ((1u << (shift + 1)) < d) ++shift;
+        mul = (uint32_t)(((1ull << (32 + shift)) + d - 1) / d);
+    }
+    __device__ __forceinline__ uint32_t div(uint32_t x) const { return d <= 1 ? x : __umulhi(x, mul) >> shift; }
+    __device__ __forceinline__ void divmod(uint32_t x, uint32_t& q, uint32_t& r) const {
+        q = div(x);
+        r = x - q * d;
+    }
+};
+
 // Index spaces: up to three batch dimensions, each with its count and stride.
 struct Dims {
     int64_t cnt[3], str[3];
 };
-
-__device__ __host__ __forceinline__ int64_t dims_offset(const Dims& d, int64_t i) {
-    const int64_t i2 = i % d.cnt[2], q = i / d.cnt[2];
-    const int64_t i1 = q % d.cnt[1], i0 = q / d.cnt[1];
-    return i0 * d.str[0] + i1 * d.str[1] + i2 * d.str[2];
-}
+// The same for the device: index i -> sum of digit times stride.
+struct Strides {
+    Div c1, c2;
+    int64_t str[3] = {0, 0, 0};
+    Strides() = default;
+    explicit Strides(const Dims& d) : c1(d.cnt[1]), c2(d.cnt[2]) {
+        for (int i = 0; i < 3; ++i) str[i] = d.str[i];
+    }
+    __device__ __forceinline__ int64_t at(uint32_t i) const {
+        uint32_t q, i0, i1, i2;
+        c2.divmod(i, q, i2);
+        c1.divmod(q, i0, i1);
+        return (int64_t)i0 * str[0] + (int64_t)i1 * str[1] + (int64_t)i2 * str[2];
+    }
+};
 
 struct PackArgs {
     const void* ptr;
@@ -82,7 +110,8 @@ struct PackArgs {
     int n, k, koff;            // row index count, contracted length, padded length of one part
     int klen, pieces;          // the contracted index in `pieces` pieces of klen (<= koff)
     int64_t Kp;                // row pitch of the slices (parts x koff)
-    Dims own, shared;          // batch dimensions folded into the rows / kept as batches
+    Strides own, shared;       // batch dimensions folded into the rows / kept as batches
+    Div dn, dbatch;            // by n, by nbatch
     int64_t own_rows;          // rows before expansion
     int64_t nbatch;
     __half* out;               // [S][pieces][nbatch][own_rows (x 2)][Kp]
@@ -147,12 +176,14 @@ __global__ void __launch_bounds__(256) pack_slices_kernel(PackArgs a) {
     __shared__ int rowexp[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t r0 = (int64_t)blockIdx.x * 32, bt = blockIdx.y;   // bt = (piece, shared batch)
-    const int piece = (int)(bt / a.nbatch), kn = min(a.klen, a.k - piece * a.klen);
+    uint32_t piece, sb;
+    a.dbatch.divmod(blockIdx.y, piece, sb);
+    const int kn = min(a.klen, a.k - (int)piece * a.klen);
     if (threadIdx.x < 32) {
         const int64_t r = r0 + threadIdx.x;
-        off[threadIdx.x] = r < a.own_rows ? dims_offset(a.shared, bt % a.nbatch) + dims_offset(a.own, r / a.n) +
-                                                (r % a.n) * a.si + (int64_t)piece * a.klen * a.sk
-                                          : -1;
+        uint32_t ob, i;
+        a.dn.divmod((uint32_t)r, ob, i);
+        off[threadIdx.x] = r < a.own_rows ? a.shared.at(sb) + a.own.at(ob) + i * a.si + (int64_t)piece * a.klen * a.sk : -1;
     }
     __syncthreads();
     if (a.idx_contig) {
@@ -244,15 +275,16 @@ __global__ void __launch_bounds__(256) pack_slices_kernel(PackArgs a) {
 struct OutArgs {
     int64_t rows, cols;        // per batch, after expansion
     int rexp, cexp;            // which side is expanded (at most one)
-    int rn, cn;                // row / column index counts within one own batch
+    Div rn, cn;                // row / column index counts within one own batch
     int64_t rs, cs;            // output strides of the row / column index (complex elements)
-    Dims rown, cown, shared;   // output strides of the batch dimensions
-    Dims drown, dcown, dshared;
+    Strides rown, cown, shared;    // output strides of the batch dimensions
+    Strides drown, dcown, dshared;
     int64_t drs, dcs;
-    const int *er, *ec;        // exponents [nbatch][rows before expansion]
+    const int *er, *ec;        // exponents [pieces][nbatch][rows before expansion]
     cplx *C, *D;
     double beta;
-    int64_t rt, ct, tiles;     // row tiles, column tiles, all tiles
+    int64_t tiles;             // row tiles x column tiles x batches
+    Div drt, dper, dtiles;     // by row tiles, tiles of a batch, all tiles
     int nk;                    // stages of one piece
     int pieces;                // pieces of the contracted index
     int64_t nbatch;            // shared batches
@@ -260,6 +292,11 @@ struct OutArgs {
     // their sums to C + group * gstride
     int groups, pg;
     int64_t gstride;
+    __device__ __forceinline__ void tile(uint32_t t, uint32_t& b, uint32_t& ct, uint32_t& rt) const {
+        uint32_t q;
+        dper.divmod(t, b, q);
+        drt.divmod(q, ct, rt);
+    }
 };
 
 struct Ctl {
@@ -268,23 +305,30 @@ struct Ctl {
     int abort;
 };
 
-// FP64 value of I 2^x, rounded to nearest.  x beyond the exponent range gives 0, infinity or (from
-// a row marked kNanExp) NaN.
-__device__ __forceinline__ double round64(long long I, int x) {
-    const unsigned sign = (unsigned)(I >> 32) & 0x80000000u;
-    const unsigned long long X0 = I < 0 ? 0ull - (unsigned long long)I : (unsigned long long)I;
+// FP64 value of I 2^x, rounded to nearest.  The common case, a result well inside the exponent range
+// with |I| >= 2^32, takes one count of leading zeros and two funnel shifts; the other (small and zero
+// I; x beyond the range: 0, infinity or, from a row marked kNanExp, NaN) is out of line.
+__device__ __noinline__ double round64_rare(unsigned hi0, unsigned lo0, unsigned sign, int x) {
+    const unsigned long long X0 = ((unsigned long long)hi0 << 32) | lo0;
+    if (x > kNanExp / 2) return __longlong_as_double(0x7ff8000000000000ll);
+    if (X0 == 0) return 0.0;
     const int lz = __clzll((long long)X0);
-    const unsigned long long X = X0 << (lz & 63);
-    const unsigned long long m = (X >> 11) + ((X >> 10) & 1ull);   // 2^52 .. 2^53
-    const int eb = 1023 + 63 - lz + x;                             // biased exponent
-    unsigned hi = (unsigned)(m >> 32) + ((unsigned)(eb - 1) << 20);
-    unsigned lo = (unsigned)m;
-    if ((unsigned)(eb - 1) > 2045u || lz == 64) {
-        const bool nan = x > kNanExp / 2, inf = !nan && lz < 64 && eb > 2046;
-        hi = nan ? 0x7ff80000u : (inf ? 0x7ff00000u : 0u);
-        lo = 0u;
-    }
-    return __hiloint2double((int)(hi | sign), (int)lo);
+    const unsigned long long X = X0 << lz, m = (X >> 11) + ((X >> 10) & 1ull);   // 2^52 .. 2^53
+    const int eb = 1023 + 63 - lz + x;
+    const unsigned long long r = eb < 1 ? 0ull : (eb > 2046 ? 0x7ff0000000000000ull : ((unsigned long long)(eb - 1) << 52) + m);
+    return __longlong_as_double((long long)(r | ((unsigned long long)sign << 32)));
+}
+__device__ __forceinline__ double round64(long long I, int x) {
+    const int s = (int)(I >> 63);
+    const unsigned long long X = (unsigned long long)((I ^ s) - s);
+    const unsigned hi0 = (unsigned)(X >> 32), lo0 = (unsigned)X, sign = (unsigned)s & 0x80000000u;
+    const int lz = __clz((int)hi0);
+    const int eb1 = 1023 + 63 - 1 + x - lz;   // biased exponent - 1
+    if (hi0 == 0u || (unsigned)eb1 > 2045u) return round64_rare(hi0, lo0, sign, x);
+    const unsigned hi = __funnelshift_l(lo0, hi0, lz), lo = lo0 << lz;
+    // bits 63 .. 11 plus the rounding bit; the leading one carries into the exponent field
+    const unsigned long long m = (((unsigned long long)(hi >> 11) << 32) | __funnelshift_r(lo, hi, 11)) + ((lo >> 10) & 1u);
+    return __hiloint2double((int)(((unsigned)(m >> 32) + ((unsigned)eb1 << 20)) | sign), (int)(unsigned)m);
 }
 
 // Barrier of the epilogue warps with the conjunction of `pred`.
@@ -380,7 +424,9 @@ __device__ __forceinline__ void store_pair(const OutArgs& o, const RowOut& r, co
 // tensor memory, and rounds and stores while the next tile's products run.  MULTI: the contracted
 // index in several pieces, whose rounded results are added in registers.
 // Measured (T_n = Ltilde_n Theta of M = 128, N = 32, 64 vectors x 512 walkers): 14.3 ms by
-// the multiply-add tiles, 0.66 ms here (26 TFLOP/s; about 80 cycles an MMA).
+// the multiply-add tiles, 0.56 ms here (31 TFLOP/s): about 65 cycles an MMA, 32 of them its
+// products (80 before A stayed in the collector and one elected lane issued from uniform registers),
+// and 3400 cycles a tile to empty tensor memory.
 template <int S, bool MULTI>
 __global__ void __launch_bounds__(kThreadsG, 1)
     slice_gemm_kernel(const __grid_constant__ CUtensorMap tR, const __grid_constant__ CUtensorMap tQ, OutArgs o,
@@ -416,25 +462,25 @@ __global__ void __launch_bounds__(kThreadsG, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const int64_t per = o.rt * o.ct;
-    const int64_t work = MULTI ? o.tiles * o.groups : o.tiles;
+    const uint32_t work = (uint32_t)(MULTI ? o.tiles * o.groups : o.tiles);
     if (warp == 0) {
         if (lane == 0) {
             int64_t g = 0;
             bool ok = true;
-            for (int64_t w = blockIdx.x; w < work && ok; w += gridDim.x) {
-                const int64_t t = w % o.tiles;
-                const int b = (int)(t / per), ct = (int)(t % per / o.rt), rt = (int)(t % per % o.rt);
-                const int p0 = MULTI ? (int)(w / o.tiles) * o.pg : 0, p1 = MULTI ? min(o.pieces, p0 + o.pg) : 1;
+            for (uint32_t w = blockIdx.x; w < work && ok; w += gridDim.x) {
+                uint32_t grp, t, b, ct, rt;
+                o.dtiles.divmod(w, grp, t);
+                o.tile(t, b, ct, rt);
+                const int p0 = MULTI ? (int)grp * o.pg : 0, p1 = MULTI ? min(o.pieces, p0 + o.pg) : 1;
                 for (int pc = p0; pc < p1 && ok; ++pc)
                     for (int kb = 0; kb < o.nk; ++kb, ++g) {
                         const int st = (int)(g % kStages);
                         if (!mbar_wait(&ctl->empty[st], (uint32_t)((g / kStages) & 1) ^ 1u, &ctl->abort)) { ok = false; break; }
                         uint8_t* s = sbase + (size_t)st * P::kStageBytes;
                         mbar_arrive_expect_tx(&ctl->full[st], P::kStageBytes);
-                        const int z = (int)(pc * o.nbatch) + b;
-                        tma_load_4d(s, &tR, &ctl->full[st], kb * kChunk, rt * kRows, z, 0);
-                        tma_load_4d(s + S * kRows * kChunk * 2, &tQ, &ctl->full[st], kb * kChunk, ct * kCols, z, 0);
+                        const int z = (int)(pc * o.nbatch + b);
+                        tma_load_4d(s, &tR, &ctl->full[st], kb * kChunk, (int)rt * kRows, z, 0);
+                        tma_load_4d(s + S * kRows * kChunk * 2, &tQ, &ctl->full[st], kb * kChunk, (int)ct * kCols, z, 0);
                     }
             }
             if (!ok)
@@ -442,59 +488,76 @@ __global__ void __launch_bounds__(kThreadsG, 1)
                     wait_drain(&ctl->full[j % kStages], (uint32_t)((j / kStages) & 1));
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(kRows, kCols, true);
-            const uint32_t tmem = ctl->tmem_base;
-            int64_t g = 0;
-            int it = 0;
-            bool ok = true;
-            for (int64_t w = blockIdx.x; w < work && ok; w += gridDim.x) {
-                const int p0 = MULTI ? (int)(w / o.tiles) * o.pg : 0, p1 = MULTI ? min(o.pieces, p0 + o.pg) : 1;
-                for (int pc = p0; pc < p1 && ok; ++pc, ++it) {
-                    if (!mbar_wait(&ctl->tempty, ((uint32_t)it & 1u) ^ 1u, &ctl->abort)) { ok = false; break; }
+        // the whole warp runs the loop, one elected lane issues: the MMAs follow each other as fast as
+        // the tensor core takes them only while their descriptors stay in uniform registers
+        constexpr uint32_t idesc = idesc_bf16(kRows, kCols, true);
+        const uint32_t tmem = ctl->tmem_base;
+        const uint64_t d0 = desc_sw64(smem_u32(sbase));
+        const uint32_t lo0 = (uint32_t)d0, hi0 = (uint32_t)(d0 >> 32);
+        int64_t g = 0;
+        int it = 0;
+        bool ok = true;
+        for (uint32_t w = blockIdx.x; w < work && ok; w += gridDim.x) {
+            const int p0 = MULTI ? (int)o.dtiles.div(w) * o.pg : 0, p1 = MULTI ? min(o.pieces, p0 + o.pg) : 1;
+            for (int pc = p0; pc < p1 && ok; ++pc, ++it) {
+                if (!warp_wait(&ctl->tempty, ((uint32_t)it & 1u) ^ 1u, &ctl->abort)) { ok = false; break; }
+                tc_fence_after();
+                for (int kb = 0; kb < o.nk; ++kb, ++g) {
+                    const int st = (int)(g % kStages);
+                    if (!warp_wait(&ctl->full[st], (uint32_t)((g / kStages) & 1), &ctl->abort)) { ok = false; break; }
                     tc_fence_after();
-                    for (int kb = 0; kb < o.nk; ++kb, ++g) {
-                        const int st = (int)(g % kStages);
-                        if (!mbar_wait(&ctl->full[st], (uint32_t)((g / kStages) & 1), &ctl->abort)) { ok = false; break; }
-                        tc_fence_after();
-                        const uint32_t sr = smem_u32(sbase + (size_t)st * P::kStageBytes);
-                        const uint32_t sq = sr + S * kRows * kChunk * 2;
+                    if (elect_one()) {
+                        const uint32_t sr = lo0 + st * (P::kStageBytes >> 4);
+                        const uint32_t sq = sr + (S * kRows * kChunk * 2 >> 4);
 #pragma unroll
                         for (int kk = 0; kk < kChunk / 16; ++kk)
 #pragma unroll
-                            for (int p = 0; p < S; ++p)
+                            for (int p = 0; p < S; ++p)   // slice p of R stays in the collector
 #pragma unroll
-                                for (int d = p; d < P::D; ++d)
-                                    mma_bf16(tmem + d * kCols, desc_sw64(sr + p * kRows * kChunk * 2 + kk * 32),
-                                             desc_sw64(sq + (d - p) * kCols * kChunk * 2 + kk * 32), idesc,
-                                             (kb | kk | p) != 0 ? 1u : 0u);
+                                for (int d = p; d < P::D; ++d) {
+                                    const uint32_t D = tmem + d * kCols, a = sr + ((p * kRows * kChunk * 2 + kk * 32) >> 4),
+                                                   b = sq + (((d - p) * kCols * kChunk * 2 + kk * 32) >> 4),
+                                                   acc = (kk | p) != 0 ? 1u : (kb != 0 ? 1u : 0u);
+                                    if (p == S - 1) mma_f16_lo<kKeepNone>(D, a, b, hi0, idesc, acc);
+                                    else if (d == p) mma_f16_lo<kKeepFirst>(D, a, b, hi0, idesc, acc);
+                                    else if (d < P::D - 1) mma_f16_lo<kKeepMore>(D, a, b, hi0, idesc, acc);
+                                    else mma_f16_lo<kKeepLast>(D, a, b, hi0, idesc, acc);
+                                }
                         mma_commit(&ctl->empty[st]);
                     }
-                    if (!ok) break;
-                    mma_commit(&ctl->tfull);
+                    __syncwarp();
                 }
+                if (!ok) break;
+                if (elect_one()) mma_commit(&ctl->tfull);
+                __syncwarp();
             }
+        }
+        if (elect_one()) {
             mma_commit(&ctl->done);
             wait_drain(&ctl->done, 0);
         }
+        __syncwarp();
     } else {
         const int q = warp & 3, h = (warp - 2) >> 2;   // lane quadrant, columns [16 h, 16 h + 16)
         const int et = threadIdx.x - 64;
         const uint32_t tq = ctl->tmem_base + ((uint32_t)(q * 32) << 16) + 16 * h;
-        const int rx = o.rexp ? 2 : 1, cx = o.cexp ? 2 : 1;
+        const int rx = o.rexp ? 1 : 0, cx = o.cexp ? 1 : 0;
         constexpr int kShift = -2 * (P::BETA - 1) - Gather<S>::kPoint;
         int it = 0;
         bool ok = true;
-        for (int64_t w = blockIdx.x; w < work && ok; w += gridDim.x) {
-            const int64_t t = w % o.tiles;
-            const int p0 = MULTI ? (int)(w / o.tiles) * o.pg : 0, p1 = MULTI ? min(o.pieces, p0 + o.pg) : 1;
-            const int64_t b = t / per, ct = t % per / o.rt, rt = t % per % o.rt;
-            const int64_t r = rt * kRows + q * 32 + lane, ri = r / rx;
+        for (uint32_t w = blockIdx.x; w < work && ok; w += gridDim.x) {
+            uint32_t grp, t, b, ct, rt, ob, i;
+            o.dtiles.divmod(w, grp, t);
+            o.tile(t, b, ct, rt);
+            const int p0 = MULTI ? (int)grp * o.pg : 0, p1 = MULTI ? min(o.pieces, p0 + o.pg) : 1;
+            const int64_t r = (int64_t)rt * kRows + q * 32 + lane;
+            const uint32_t ri = (uint32_t)r >> rx;
             RowOut ro;
             ro.ok = r < o.rows;
-            ro.roff = ro.ok ? dims_offset(o.shared, b) + dims_offset(o.rown, ri / o.rn) + ri % o.rn * o.rs : 0;
-            ro.rdof = ro.ok && o.D ? dims_offset(o.dshared, b) + dims_offset(o.drown, ri / o.rn) + ri % o.rn * o.drs : 0;
-            if (MULTI && ro.ok) ro.roff += w / o.tiles * o.gstride;
+            o.rn.divmod(ri, ob, i);
+            ro.roff = ro.ok ? o.shared.at(b) + o.rown.at(ob) + i * o.rs : 0;
+            ro.rdof = ro.ok && o.D ? o.dshared.at(b) + o.drown.at(ob) + i * o.drs : 0;
+            if (MULTI && ro.ok) ro.roff += grp * o.gstride;
             ro.comp = o.rexp ? (int)(r & 1) : 0;
             double acc[MULTI ? 16 : 1];
             if (MULTI) {
@@ -508,13 +571,16 @@ __global__ void __launch_bounds__(kThreadsG, 1)
                 int* cexp = cexp2 + (it & 1) * kCols;
                 const int64_t z = pc * o.nbatch + b;
                 if (et < kCols) {
-                    const int64_t c = ct * kCols + et, ci = c / cx;
+                    const int64_t c = (int64_t)ct * kCols + et;
+                    const uint32_t ci = (uint32_t)c >> cx;
                     const bool in = c < o.cols;
-                    coff[et] = in ? dims_offset(o.cown, ci / o.cn) + ci % o.cn * o.cs : -1;
-                    cdof[et] = in && o.D ? dims_offset(o.dcown, ci / o.cn) + ci % o.cn * o.dcs : 0;
-                    cexp[et] = in ? o.ec[z * (o.cols / cx) + ci] : 0;
+                    uint32_t cob, cj;
+                    o.cn.divmod(ci, cob, cj);
+                    coff[et] = in ? o.cown.at(cob) + cj * o.cs : -1;
+                    cdof[et] = in && o.D ? o.dcown.at(cob) + cj * o.dcs : 0;
+                    cexp[et] = in ? o.ec[z * (o.cols >> cx) + ci] : 0;
                 }
-                const int er = ro.ok ? o.er[z * (o.rows / rx) + ri] : 0;
+                const int er = ro.ok ? o.er[z * (o.rows >> rx) + ri] : 0;
                 int got = 1;
                 if (lane == 0) got = mbar_wait(&ctl->tfull, (uint32_t)it & 1u, &ctl->abort) ? 1 : 0;
                 got = __shfl_sync(0xffffffffu, got, 0);
@@ -676,8 +742,10 @@ PackArgs pack_args(const GemmOperand& X, bool is_a, int n, int k, const Plan& p,
     a.klen = p.klen;
     a.pieces = p.pieces;
     a.Kp = (int64_t)p.parts * p.koff;
-    a.own = is_a ? p.aown : p.bown;
-    a.shared = is_a ? p.shared_a : p.shared_b;
+    a.own = Strides(is_a ? p.aown : p.bown);
+    a.shared = Strides(is_a ? p.shared_a : p.shared_b);
+    a.dn = Div(n);
+    a.dbatch = Div(p.ns);
     a.own_rows = (is_a ? p.na : p.nb) * n;
     a.nbatch = p.ns;
     const int64_t rows = is_a ? p.rows_a : p.rows_b;
@@ -754,31 +822,36 @@ int run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st
     o.cols = rc;
     o.rexp = p.swap ? p.exp_a : p.exp_b;
     o.cexp = p.swap ? p.exp_b : p.exp_a;
-    o.rn = p.swap ? g.m : g.n;
-    o.cn = p.swap ? g.n : g.m;
+    o.rn = Div(p.swap ? g.m : g.n);
+    o.cn = Div(p.swap ? g.n : g.m);
     o.rs = p.swap ? g.ldc : 1;
     o.cs = p.swap ? 1 : g.ldc;
     o.drs = p.swap ? g.ldd : 1;
     o.dcs = p.swap ? 1 : g.ldd;
-    o.rown = p.swap ? p.aown_c : p.bown_c;
-    o.cown = p.swap ? p.bown_c : p.aown_c;
-    o.drown = p.swap ? p.aown_d : p.bown_d;
-    o.dcown = p.swap ? p.bown_d : p.aown_d;
-    o.shared = p.shared_c;
-    o.dshared = p.shared_d;
+    Dims rown = p.swap ? p.aown_c : p.bown_c, cown = p.swap ? p.bown_c : p.aown_c, shared = p.shared_c;
+    o.drown = Strides(p.swap ? p.aown_d : p.bown_d);
+    o.dcown = Strides(p.swap ? p.bown_d : p.aown_d);
+    o.dshared = Strides(p.shared_d);
     o.er = R.exps;
     o.ec = Q.exps;
     o.C = g.C;
     o.D = g.D;
     o.beta = g.beta.re;
-    o.rt = up(rr, kRows) / kRows;
-    o.ct = up(rc, kCols) / kCols;
     o.tiles = p.tiles;
+    o.drt = Div(up(rr, kRows) / kRows);
+    o.dper = Div(p.tiles / p.ns);
+    o.dtiles = Div(p.tiles);
     o.nk = (int)(up((int64_t)p.parts * p.koff, kChunk) / kChunk);
     o.pieces = p.pieces;
     o.nbatch = p.ns;
     o.groups = p.groups;
     o.pg = p.pg;
+    auto place = [&] {
+        o.rown = Strides(rown);
+        o.cown = Strides(cown);
+        o.shared = Strides(shared);
+    };
+    place();
     const int64_t mn = (int64_t)g.m * g.n, total = (int64_t)g.nb0 * g.nb1 * g.nb2 * mn;
     if (p.groups > 1) {   // the groups' sums side by side, dense, then added in order
         o.C = reinterpret_cast<cplx*>(buf + p.bytes_b);
@@ -788,8 +861,9 @@ int run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st
         const int64_t dense[3] = {(int64_t)g.nb1 * g.nb2 * mn, (int64_t)g.nb2 * mn, mn};
         (p.swap ? o.rs : o.cs) = g.n;
         for (int i = 0; i < 3; ++i)
-            for (Dims* d : {&o.rown, &o.cown, &o.shared})
+            for (Dims* d : {&rown, &cown, &shared})
                 if (d->cnt[i] > 1) d->str[i] = dense[i];
+        place();
         AFQMC_TRY(p.S == 7 ? launch_gemm<7>(mr, mq, o, ws->flags, st) : launch_gemm<8>(mr, mq, o, ws->flags, st));
         count_launch();
         sum_groups_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(o.C, p.groups, total, g);
@@ -802,13 +876,14 @@ int run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st
 
 size_t slice_gemm_bytes(const GemmArgs& g) { return make_plan(g).bytes + 1024; }
 
-// Expected time in microseconds: three launches with little in each, the persistent tiles at 80 cycles an MMA and 6000
+// Expected time in microseconds: three launches with little in each, the persistent tiles at 65 cycles an MMA and 6000
 // for the epilogue, and the operands' packing.
 double slice_gemm_us(const GemmArgs& g) {
     if (g.beta.im != 0.0 || (g.A.real && g.B.real && g.alpha.im != 0.0)) return 1e30;
     const Plan p = make_plan(g);
-    if (p.ns * p.pieces > 65535) return 1e30;   // the pack kernel's grid
-    const double cyc = p.S * (p.S + 1) / 2 * (up((int64_t)p.parts * p.koff, 16) / 16) * 80.0 + 6000.0;
+    // the pack kernel's grid, 31-bit indices
+    if (p.ns * p.pieces > 65535 || std::max(p.rows_a, p.rows_b) >= 1ll << 31 || p.tiles * p.groups >= 1ll << 31) return 1e30;
+    const double cyc = p.S * (p.S + 1) / 2 * (up((int64_t)p.parts * p.koff, 16) / 16) * 65.0 + 6000.0;
     const double waves = (double)((p.tiles * p.groups + tc_num_sms() - 1) / tc_num_sms());
     return 26.0 + p.pg * waves * cyc / 1.9e3 + (double)p.bytes / 2.0e6 + (p.groups > 1 ? 4.0 : 0.0);
 }

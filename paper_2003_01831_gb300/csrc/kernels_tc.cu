@@ -283,14 +283,6 @@ __device__ void mma_loop(uint8_t* sbase, SharedCtl* ctl, int64_t ntiles, int nk)
     wait_drain(&ctl->done, 0);
 }
 
-// Epilogue-warp wait: lane 0 polls, the warp follows.
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-    int ok = 1;
-    if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, abort_flag) ? 1 : 0;
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    return ok != 0;
-}
-
 // 32 columns of an accumulator pair: v = acc1 (+ acc2); both loads issued before one wait.
 template <bool EXACT>
 __device__ __forceinline__ void load_acc32(uint32_t taddr1, uint32_t taddr2, float (&v)[32]) {
