@@ -79,7 +79,6 @@ struct SharedCtl {
     uint64_t done;
     uint32_t tmem_base;
     int abort;
-    double red[8][4];   // energy epilogue: per-warp (t.re, t.im, X.re, X.im)
 };
 
 // --------------------------------------------------------------------------- epilogues
@@ -438,13 +437,10 @@ __device__ __forceinline__ void zero_regs(uint32_t (&u)[n]) {
 }
 
 // Energy kernel pipeline: K chunks of BK = 16 (32-byte swizzle, six 24 KB stages) or 32
-// (64-byte swizzle, three 48 KB stages) in 144 KB of shared memory, one TMEM buffer
-// (accumulator 1 in columns 0..255, accumulator 2 in 256..511).  The operands come from L2
-// (~1-2 us under load), so the ring holds as many stages as the shared memory left by the
-// epilogue allows: the epilogue keeps the real part of its rows of T in registers and stages
-// only one plane (128 x 128 fp32, 66 KB) in shared memory (see the epilogue).  With the
-// walker-spin window below, the wider chunks (half the barrier round trips per flop) are
-// faster.
+// (64-byte swizzle, three 48 KB stages) in 144 KB of shared memory, two accumulators of 256
+// TMEM columns (see Turns).  The operands come from L2 (~1-2 us under load), so the ring holds as
+// many stages as the 66 KB of the epilogue's exchange allow.  With the walker-spin window below,
+// the wider chunks (half the barrier round trips per flop) are faster.
 constexpr int kEStageRing = 144 * 1024;
 // One stage: AP planes of the Ltilde rows (hi, lo and, for the rounded products, r) of 128
 // rows each, then the hi and lo planes of BR Theta rows (256 for one CTA per tile, 128 per CTA
@@ -463,8 +459,10 @@ constexpr int kEBKDefault = 32;
 // in L2 while the L~ pairs stream through it once per window; the 152 CTAs then share ~19 L~
 // n-groups and 8 Theta groups at a time.
 constexpr int kEWsSuperDefault = 8;
-constexpr int kEPitch = 129;                     // plane tile row pitch (floats): conflict-free
-constexpr int kETileFloats = 128 * kEPitch;      // rows and columns
+constexpr int kEPitch = 129;                     // plane row pitch (floats) of the generic epilogue: conflict-free
+constexpr int kEBlock = 32 * 33;                 // one 32 x 32 block of the fixed epilogue at pitch 33
+constexpr int kETileFloats = 16 * kEBlock;       // 16 blocks; the generic epilogue's 128 x 129 plane fits too
+static_assert(kETileFloats >= 128 * kEPitch, "epilogue exchange space");
 
 template <int BK>
 __device__ __forceinline__ uint64_t edesc(uint32_t saddr) {
@@ -551,29 +549,31 @@ __device__ __forceinline__ void energy_stage_load_pair(uint8_t* s, SharedCtl* ct
     tma_load_2d_pair(s + C::kBOff + C::kBBytes, mp[4], fb, x, yb);
 }
 
-// The MMAs of one such stage (rank 0 of the pair), accumulating from the tile's first stage.
+// The MMAs of one such stage (rank 0 of the pair), accumulating from the tile's first stage.  sa: low
+// word of the descriptor of the stage's first plane, hi: the high word of all of them.
 template <int BK, int AP>
-__device__ __forceinline__ void energy_stage_mma_pair(uint32_t sa, uint32_t d1, uint32_t d2, int kb, bool single,
-                                                      bool lolo) {
+__device__ __forceinline__ void energy_stage_mma_pair(uint32_t sa, uint32_t hi, uint32_t d1, uint32_t d2, int kb,
+                                                      bool single, bool lolo) {
     using C = EStage<BK, AP, 128>;
     constexpr uint32_t idesc = idesc_bf16(256, 256, true);   // fp16 planes, M = 256 over the pair, N = 256
-    const uint32_t sb = sa + C::kBOff;
+    constexpr uint32_t A = C::kABytes >> 4, B = C::kBBytes >> 4;
+    const uint32_t sb = sa + (C::kBOff >> 4);
+    const uint32_t more = kb != 0 ? 1u : 0u;
     if (AP == 3 && single) {
 #pragma unroll
         for (int c = 0; c < 2; ++c)
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk)
-                mma_f16_pair(d1, edesc<BK>(sa + c * C::kABytes + kk * 32), edesc<BK>(sb + c * C::kBBytes + kk * 32),
-                             idesc, (kb | c | kk) != 0 ? 1u : 0u);
+                mma_f16_pair_lo(d1, sa + c * A + kk * 2, sb + c * B + kk * 2, hi, idesc, (c | kk) != 0 ? 1u : more);
         return;
     }
-    const uint32_t sal = sa + C::kABytes, sar = sa + 2 * C::kABytes, sbl = sb + C::kBBytes;
 #pragma unroll
     for (int kk = 0; kk < BK / 16; ++kk) {
-        const uint32_t off = kk * 32;
-        energy_products<AP>([&](uint32_t d, uint64_t a, uint64_t b, uint32_t c) { mma_f16_pair(d, a, b, idesc, c); },
-                            d1, d2, edesc<BK>(sa + off), edesc<BK>(sal + off), edesc<BK>(sar + off),
-                            edesc<BK>(sb + off), edesc<BK>(sbl + off), (kb | kk) != 0 ? 1u : 0u, lolo);
+        const uint32_t acc = kk != 0 ? 1u : more, al = sa + A + kk * 2, bl = sb + B + kk * 2;
+        mma_f16_pair_lo(d1, sa + kk * 2, sb + kk * 2, hi, idesc, acc);                              // hi hi
+        mma_f16_pair_lo(d2, AP == 3 ? sa + 2 * A + kk * 2 : sa + kk * 2, bl, hi, idesc, acc);      // r lo (hi lo)
+        mma_f16_pair_lo(d2, al, sb + kk * 2, hi, idesc, 1u);                                        // lo hi
+        if (AP == 2 && lolo) mma_f16_pair_lo(d2, al, bl, hi, idesc, 1u);
     }
 }
 
@@ -634,148 +634,224 @@ __device__ __forceinline__ int ebar_and(int pred) {
     return r;
 }
 
+// Which accumulators a tile uses.  Tensor memory holds two of 256 columns.  A three- or two-product
+// tile fills both (hi*hi in the first, the rest in the second); a single-product tile fills one,
+// the two in turn, so that its MMAs run while the tile before it is drained.  The MMA issuer and
+// the epilogue warps each keep one of these and take the same turns: part is the accumulator of a
+// single-product tile (0 otherwise), the counts give the barriers' phases.
+struct Turns {
+    uint32_t full[2] = {0, 0}, empty[2] = {0, 0};
+    int next = 0;
+    __device__ __forceinline__ int part(bool single) {
+        if (!single) return 0;
+        const int p = next;
+        next ^= 1;
+        return p;
+    }
+    // parity of the next wait on tfull[p] / tempty[p]
+    __device__ __forceinline__ uint32_t full_parity(int p) { return full[p]++ & 1u; }
+    __device__ __forceinline__ uint32_t empty_parity(int p) { return (empty[p]++ & 1u) ^ 1u; }
+};
+__device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void pair_arrive(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
+
 // Epilogue of one tile of the energy kernels (warps 2..17 of a CTA): n-group ng of this CTA's
-// accumulator rows, walker-spin group wg, the CTA's it-th tile (accumulator barrier phase).
+// accumulator rows, walker-spin group wg; part and d2 (second accumulator used): see Turns.
 // release() is called by lane 0 of each warp once the warp's tensor-memory reads are complete.
 // Returns false when a wait gave up (all sixteen warps then leave together).
+//
+// The tile's accumulator columns are, per walker-spin j of the tile, Np real columns then Np
+// imaginary ones.  A warp owns one 32 x 32 block of the tile: rows 32 q .. + 31 (its tensor-memory
+// quadrant) and the compact columns 32 h .. + 31, i.e. rows 32 r .. and columns 32 c .. of one
+// (n-block, walker-spin) block of Np / 32 by Np / 32 such.  With T = Tr + i Ti,
+//   t = sum_a T_aa,  X = sum_ab T_ab T_ba = sum over r = c blocks + 2 sum over pairs of (r, c), (c, r).
+// Of such a pair one warp (the writer) puts its T in shared memory and the other (the reader) forms
+// both orders' products with its own T from registers; a warp on the diagonal exchanges within
+// itself.  That halves the shared-memory traffic of exchanging every block, and a pair waits for
+// each other alone: a tile has one barrier of all sixteen warps (with the wait for the accumulators),
+// which also separates this tile's exchange space and sums from the last one's.  Block rows lie at
+// pitch 33: writes (lanes over rows) and reads (lanes over columns) are free of bank conflicts.
+//
+// What bounds a single-product tile is shared memory: at 128 bytes a cycle the MMAs' operands and
+// the copies that bring them take all of it by themselves, and the exchange comes on top.  Kernel
+// times against a 128 x 128 plane exchanged by all, one accumulator pair and 64-bit descriptors
+// (ms; M, N, walkers): 512, 128, 128: 33.6 -> 27.9; 256, 64, 256: 5.25 -> 4.36 (all tiles three
+// products: 7.06 -> 6.74); 256, 128, 64: 5.30 -> 4.20; 128, 32, 512: 1.27 -> 1.14.  Barriers in
+// shared memory per pair and per tile instead of the sixteen-warp one, with scales fetched ahead
+// through shared memory, took longer (31.4, 5.03, 6.95, 5.11, 1.18).
 template <int Np, typename Release>
-__device__ __forceinline__ bool energy_epilogue_tile(const EnergyShape& es, SharedCtl* ctl, float* plane,
-                                                     float* colscale, double* ered, int ng, int wg, int it, bool d2,
+__device__ __forceinline__ bool energy_epilogue_tile(const EnergyShape& es, SharedCtl* ctl, float* xbuf, double* ered,
+                                                     int ng, int wg, int part, uint32_t parity, bool d2,
                                                      Release release) {
-    constexpr int Q = Np / 32;     // TMEM quadrants per n-block
+    constexpr int Q = Np / 32;     // blocks along an n-block
     constexpr int G = 128 / Np;    // n-blocks (rows) and walker-spins (columns) per tile
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // Epilogue.  The tile's accumulator columns are, per walker-spin j of the tile, Np real
-    // columns then Np imaginary ones.  Compact column cc = j Np + b (b < Np) names element b
-    // of walker-spin j; this thread owns row `row` and the 32 compact columns
-    // [32 h, 32 h + 32), all in one walker-spin j.  Per (n-block, walker-spin) block, with
-    // T = Tr + i Ti:
-    //   t = Tr_aa + i Ti_aa,
-    //   X = sum_ab T_ab T_ba = sum Tr_ab Tr_ba - sum Ti_ab Ti_ba + 2 i sum Tr_ab Ti_ba
-    // (sum Ti_ab Tr_ba = sum Tr_ab Ti_ba by relabelling).  The drain writes Ti to the plane
-    // tile and keeps the thread's Tr in registers; the TiTi and TrTi sums read the plane;
-    // then Tr replaces it for the TrTr sum.  Partner reads T_ba run along a row of the plane
-    // (lanes = consecutive a), own-row reads down a column (pitch 129): both conflict-free.
-    const int q = warp & 3;                // TMEM lane quadrant: rows 32 q .. 32 q + 31
-    const int h = (warp - 2) >> 2;         // compact columns [32 h, 32 h + 32)
-    const int row = q * 32 + lane;         // tile row = (n-block i_blk, a)
-    const int i_blk = row / Np, a = row % Np;
-    const int et = threadIdx.x - 64;       // 0..511
-    const uint32_t tq = ctl->tmem_base + ((uint32_t)(q * 32) << 16);
-    const int cc0 = h * 32;                      // first compact column of this thread
-    const int j = cc0 / Np, b0 = cc0 % Np;       // its walker-spin and first element
-    const int col_re = j * 2 * Np + b0, col_im = col_re + Np;
-    float* own = plane + row * kEPitch;                      // this row of the plane
-    const float* pbase = plane + (i_blk * Np + b0) * kEPitch + j * Np + a;   // T_(b0+k) a
-    const int cd = j * Np + a;                               // compact column of T_aa
-    const bool diag = cd >= cc0 && cd < cc0 + 32;
-    if (et < 256) {
-        const int64_t brow = (int64_t)wg * 256 + et;
-        colscale[et] = brow < (int64_t)es.nws * 2 * Np ? es.b_scale[brow] : 0.0f;
+    const int q = warp & 3, h = (warp - 2) >> 2;
+    const int ib = q / Q, r = q % Q, j = h / Q, c = h % Q;
+    // pairs of blocks, readers spread over the quadrants (and so over the schedulers)
+    bool reader = false;
+    int pair = 0;
+    if (Q == 4) {
+        const int d = (c - r) & 3;
+        reader = d == 1 || (d == 2 && r < 2);
+        const int rr = reader ? r : c;           // the reader's r
+        pair = (d == 2) ? 4 + rr : rr;
+    } else if (Q == 2) {
+        reader = r != c && (r == (j & 1));
+        pair = ib * 2 + j;
     }
+    const bool diag = r == c;
+    const int wq = reader ? ib * Q + c : q, wh = reader ? j * Q + r : h;   // the writer's block of the pair
+    float* own = xbuf + (wq + 4 * wh) * kEBlock;                            // re (or the diagonal's one block)
+    float* own2 = xbuf + (ib * Q + (wh % Q) + 4 * (j * Q + (wq % Q))) * kEBlock;   // im: the reader's place
+    const int row = q * 32 + lane;               // tile row (n-block ib, element 32 r + lane)
     const int64_t arow = (int64_t)ng * 128 + row;
     const float sa = arow < (int64_t)es.Nchol * Np ? es.a_scale[arow] : 0.0f;
-    ebar();
-    // Drain.  Each warp waits for the tile, moves its Im columns of both accumulators
-    // (scaled to true units) into the plane, loads its Re columns and releases tensor
-    // memory at once (one arrival per warp), so the next tile's MMAs overlap the Re
-    // scaling and everything after it.  If any warp's wait gave up, all sixteen leave
-    // together after the release.
-    const bool got = warp_wait(&ctl->tfull[0], (uint32_t)it & 1u, &ctl->abort);
+    const int col_re = j * 2 * Np + 32 * c, col_im = col_re + Np;
+    const int ws = wg * G + j;
+    const float4* sre = reinterpret_cast<const float4*>(es.b_scale + (int64_t)wg * 256 + col_re);
+    const float4* sim = reinterpret_cast<const float4*>(es.b_scale + (int64_t)wg * 256 + col_im);
+    const bool live = ws < es.nws;               // columns beyond the last walker-spin have no scales
+    const uint32_t tq = ctl->tmem_base + 256u * part + ((uint32_t)(q * 32) << 16);
+
+    const bool got = warp_wait(&ctl->tfull[part], parity, &ctl->abort);
+    if (!ebar_and(got ? 1 : 0)) return false;    // all sixteen warps leave together
     tc_fence_after();
-    float tr[32];
-    {
-        uint32_t u1[32], u2[32];
-        tmem_ld32_nw(tq + col_im, u1);
-        if (d2) tmem_ld32_nw(tq + 256 + col_im, u2);
-        else zero_regs(u2);   // a single-product tile leaves accumulator 2 unwritten
-        tmem_ld_wait();
+    // T without the row scale, in registers; tensor memory is released as soon as the last load is in
+    float tr[32], ti[32];
+    auto scaled = [&](float (&t)[32], const float4* sc) {
 #pragma unroll
         for (int g = 0; g < 8; ++g) {
-            const float4 cs = *reinterpret_cast<const float4*>(colscale + col_im + 4 * g);
-            own[cc0 + 4 * g + 0] = (__uint_as_float(u1[4 * g + 0]) + __uint_as_float(u2[4 * g + 0])) * (sa * cs.x);
-            own[cc0 + 4 * g + 1] = (__uint_as_float(u1[4 * g + 1]) + __uint_as_float(u2[4 * g + 1])) * (sa * cs.y);
-            own[cc0 + 4 * g + 2] = (__uint_as_float(u1[4 * g + 2]) + __uint_as_float(u2[4 * g + 2])) * (sa * cs.z);
-            own[cc0 + 4 * g + 3] = (__uint_as_float(u1[4 * g + 3]) + __uint_as_float(u2[4 * g + 3])) * (sa * cs.w);
+            const float4 f = live ? __ldg(sc + g) : make_float4(0.f, 0.f, 0.f, 0.f);
+            t[4 * g] *= f.x;
+            t[4 * g + 1] *= f.y;
+            t[4 * g + 2] *= f.z;
+            t[4 * g + 3] *= f.w;
         }
-    }
-    {
+    };
+    if (d2) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            uint32_t u1[16], u2[16];
+            tmem_ld16_nw(tq + col_im + 16 * k, u1);
+            tmem_ld16_nw(tq + 256 + col_im + 16 * k, u2);
+            tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 16; ++e) ti[16 * k + e] = __uint_as_float(u1[e]) + __uint_as_float(u2[e]);
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            uint32_t u1[16], u2[16];
+            tmem_ld16_nw(tq + col_re + 16 * k, u1);
+            tmem_ld16_nw(tq + 256 + col_re + 16 * k, u2);
+            tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 16; ++e) tr[16 * k + e] = __uint_as_float(u1[e]) + __uint_as_float(u2[e]);
+        }
+    } else {
         uint32_t u1[32], u2[32];
         tmem_ld32_nw(tq + col_re, u1);
-        if (d2) tmem_ld32_nw(tq + 256 + col_re, u2);
-        else zero_regs(u2);
+        tmem_ld32_nw(tq + col_im, u2);
         tmem_ld_wait();
-        tc_fence_before();
+#pragma unroll
+        for (int e = 0; e < 32; ++e) {
+            tr[e] = __uint_as_float(u1[e]);
+            ti[e] = __uint_as_float(u2[e]);
+        }
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) release();
+    scaled(tr, sre);
+    scaled(ti, sim);
+
+    float v0 = 0.f, v1 = 0.f, v2 = 0.f, v3 = 0.f;   // Re t, Im t, Re X, Im X of this lane
+    if (diag) {
+        float* mine = own + lane * 33;
+        float sii = 0.f, sri = 0.f, srr = 0.f;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) mine[k] = ti[k] * sa;
         __syncwarp();
-        if (lane == 0 && got) release();   // tensor memory free
 #pragma unroll
-        for (int g = 0; g < 8; ++g) {
-            const float4 cs = *reinterpret_cast<const float4*>(colscale + col_re + 4 * g);
-            tr[4 * g + 0] = (__uint_as_float(u1[4 * g + 0]) + __uint_as_float(u2[4 * g + 0])) * (sa * cs.x);
-            tr[4 * g + 1] = (__uint_as_float(u1[4 * g + 1]) + __uint_as_float(u2[4 * g + 1])) * (sa * cs.y);
-            tr[4 * g + 2] = (__uint_as_float(u1[4 * g + 2]) + __uint_as_float(u2[4 * g + 2])) * (sa * cs.z);
-            tr[4 * g + 3] = (__uint_as_float(u1[4 * g + 3]) + __uint_as_float(u2[4 * g + 3])) * (sa * cs.w);
+        for (int k = 0; k < 32; ++k) {
+            const float p = own[k * 33 + lane];   // Ti[k][lane]
+            sii = fmaf(ti[k], p, sii);
+            sri = fmaf(tr[k], p, sri);
+        }
+        v1 = mine[lane];
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 32; ++k) mine[k] = tr[k] * sa;
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 32; ++k) srr = fmaf(tr[k], own[k * 33 + lane], srr);
+        v0 = mine[lane];
+        v2 = (srr - sii) * sa;
+        v3 = 2.0f * sri * sa;
+    } else if (reader) {
+        pair_sync(3 + pair);
+        float srr = 0.f, sii = 0.f, sri = 0.f, sir = 0.f;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+            const float pr = own[k * 33 + lane], pi = own2[k * 33 + lane];   // T[k][lane] of the writer
+            srr = fmaf(tr[k], pr, srr);
+            sii = fmaf(ti[k], pi, sii);
+            sri = fmaf(tr[k], pi, sri);
+            sir = fmaf(ti[k], pr, sir);
+        }
+        v2 = 2.0f * (srr - sii) * sa;
+        v3 = 2.0f * (sri + sir) * sa;
+    } else {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+            own[lane * 33 + k] = tr[k] * sa;
+            own2[lane * 33 + k] = ti[k] * sa;
+        }
+        pair_arrive(3 + pair);
+    }
+    // four sums over the lanes: two exchanges halve the values a lane carries, three more add
+    {
+        const bool up = (lane & 16) != 0;
+        const float s0 = up ? v0 : v2, s1 = up ? v1 : v3;
+        v0 = (up ? v2 : v0) + __shfl_xor_sync(0xffffffffu, s0, 16);
+        v1 = (up ? v3 : v1) + __shfl_xor_sync(0xffffffffu, s1, 16);
+        const bool odd = (lane & 8) != 0;
+        const float s2 = odd ? v0 : v1;
+        v0 = (odd ? v1 : v0) + __shfl_xor_sync(0xffffffffu, s2, 8);
+    }
+    v0 += __shfl_xor_sync(0xffffffffu, v0, 4);
+    v0 += __shfl_xor_sync(0xffffffffu, v0, 2);
+    v0 += __shfl_xor_sync(0xffffffffu, v0, 1);      // lane 0: t.re, 8: t.im, 16: X.re, 24: X.im
+    const int n = ng * G + ib;
+    if (Q == 1) {   // the block is the whole output
+        if ((lane & 7) == 0 && n < es.Nchol && ws < es.nws) {
+            cplx* o = ((lane & 16) ? es.X_out : es.t_out) + (int64_t)ws * es.Nchol + n;
+            reinterpret_cast<double*>(o)[(lane >> 3) & 1] = (double)v0;
+        }
+        return true;
+    }
+    // the blocks' sums meet in shared memory; warp 2 adds them in a fixed order (fp32: GB300's FP64
+    // pipe is 1/64 of the fp32 one), one lane per value of each output
+    float* red = reinterpret_cast<float*>(ered);
+    if ((lane & 7) == 0) red[(q + 4 * h) * 4 + (lane >> 3)] = v0;
+    if (warp != 2) {
+        asm volatile("bar.arrive 15, 512;" ::: "memory");
+        return true;
+    }
+    asm volatile("bar.sync 15, 512;" ::: "memory");
+    if (lane < 4 * G * G) {
+        const int o = lane >> 2, oi = o / G, oj = o % G;
+        float sum = 0.f;
+#pragma unroll
+        for (int cc = 0; cc < Q; ++cc)
+#pragma unroll
+            for (int rr = 0; rr < Q; ++rr) sum += red[((oi * Q + rr) + 4 * (oj * Q + cc)) * 4 + (lane & 3)];
+        const int nn = ng * G + oi, ww = wg * G + oj;
+        if (nn < es.Nchol && ww < es.nws) {
+            cplx* out = ((lane & 2) ? es.X_out : es.t_out) + (int64_t)ww * es.Nchol + nn;
+            reinterpret_cast<double*>(out)[lane & 1] = (double)sum;
         }
     }
-    if (!ebar_and(got ? 1 : 0)) return false;   // all sixteen warps leave together
-    ebar();                                    // Ti plane complete
-    // TiTi and TrTi sums over this thread's b, and the diagonal Ti_aa
-    float sii = 0.f, sri = 0.f;
-#pragma unroll
-    for (int k = 0; k < 32; ++k) {
-        const float p = pbase[k * kEPitch];    // Ti[b0 + k][a] of walker-spin j
-        sii = fmaf(own[cc0 + k], p, sii);
-        sri = fmaf(tr[k], p, sri);
-    }
-    const float dim_ = diag ? own[cd] : 0.f;
-    ebar();                                    // every read of the Ti plane done
-#pragma unroll
-    for (int k = 0; k < 32; ++k) own[cc0 + k] = tr[k];
-    ebar();                                    // Tr plane complete
-    // TrTr sum continues the -TiTi one, so Re X is accumulated in one register
-    float srr = -sii;
-#pragma unroll
-    for (int k = 0; k < 32; ++k) srr = fmaf(tr[k], pbase[k * kEPitch], srr);
-    const float dre = diag ? own[cd] : 0.f;
-    float v0 = dre, v1 = dim_, v2 = srr, v3 = 2.0f * sri;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        v0 += __shfl_xor_sync(0xffffffffu, v0, o);
-        v1 += __shfl_xor_sync(0xffffffffu, v1, o);
-        v2 += __shfl_xor_sync(0xffffffffu, v2, o);
-        v3 += __shfl_xor_sync(0xffffffffu, v3, o);
-    }
-    // partial sums in fp32: the final reduction runs on one thread per output, and a chain of
-    // FP64 adds there (GB300's FP64 pipe is 1/64 of the fp32 one) cost a third of a
-    // single-product tile's epilogue
-    float* eredf = reinterpret_cast<float*>(ered);
-    if (lane < 16) {   // eredf[h][q][jj][v] for every walker-spin slot (zeros but j)
-        const int jj = lane >> 2, v = lane & 3;
-        const float val = jj != j ? 0.f : (v == 0 ? v0 : (v == 1 ? v1 : (v == 2 ? v2 : v3)));
-        eredf[((h * 4 + q) * 4 + jj) * 4 + v] = val;
-    }
-    ebar();
-    // one thread per (n-block, walker-spin) output: sum over the n-block's quadrants and
-    // the four column quarters, in a fixed order
-    if (et < G * G) {
-        const int ib = et / G, jo = et % G;
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-        for (int hh = 0; hh < 4; ++hh)
-            for (int qq = ib * Q; qq < (ib + 1) * Q; ++qq) {
-                const float4 e = *reinterpret_cast<const float4*>(eredf + ((hh * 4 + qq) * 4 + jo) * 4);
-                s0 += e.x;
-                s1 += e.y;
-                s2 += e.z;
-                s3 += e.w;
-            }
-        const int n = ng * G + ib;
-        const int ws = wg * G + jo;
-        if (n < es.Nchol && ws < es.nws) {
-            es.t_out[(int64_t)ws * es.Nchol + n] = cplx{(double)s0, (double)s1};
-            es.X_out[(int64_t)ws * es.Nchol + n] = cplx{(double)s2, (double)s3};
-        }
-    }
-    ebar();   // ered, colscale and the plane are read before the next tile rewrites them
     return true;
 }
 
@@ -791,8 +867,8 @@ __device__ __forceinline__ bool energy_epilogue_tile(const EnergyShape& es, Shar
 // in a fixed order.
 template <typename Release>
 __device__ __forceinline__ bool energy_epilogue_tile_gen(const EnergyShape& es, SharedCtl* ctl, float* plane,
-                                                         float* colscale, int ng, int wg, int it, bool d2,
-                                                         Release release) {
+                                                         float* colscale, int ng, int wg, int acc, uint32_t parity,
+                                                         bool d2, Release release) {
     const int Np = es.Np, G = es.G, GN = G * Np;
     // x / Np and x / G by multiply and shift (exact for the x < 256 used here)
     const uint32_t np_inv = es.np_inv, g_inv = es.g_inv;
@@ -805,7 +881,7 @@ __device__ __forceinline__ bool energy_epilogue_tile_gen(const EnergyShape& es, 
     const bool rok = row < GN;
     const int i_blk = divn(row), a = row - i_blk * Np;
     const int et = threadIdx.x - 64;       // 0..511
-    const uint32_t tq = ctl->tmem_base + ((uint32_t)(q * 32) << 16);
+    const uint32_t tq = ctl->tmem_base + 256u * acc + ((uint32_t)(q * 32) << 16);
     float* own = plane + row * kEPitch;
     if (et < 256) {
         const int64_t brow = (int64_t)wg * 2 * GN + et;
@@ -820,7 +896,7 @@ __device__ __forceinline__ bool energy_epilogue_tile_gen(const EnergyShape& es, 
     auto tcol = [&](int k) { return ccol(k) < GN ? ccol(k) + divn(ccol(k)) * Np : 0; };   // j 2 Np + b0
     auto icol = [&](int k) { return ccol(k) < GN ? tcol(k) + Np : 0; };
     ebar();
-    const bool got = warp_wait(&ctl->tfull[0], (uint32_t)it & 1u, &ctl->abort);
+    const bool got = warp_wait(&ctl->tfull[acc], parity, &ctl->abort);
     tc_fence_after();
     // Im of both accumulators, scaled to true units, into the plane: the loads of all four
     // chunks in flight at once, one wait
@@ -961,21 +1037,16 @@ __device__ __forceinline__ bool energy_epilogue_tile_gen(const EnergyShape& es, 
     return true;
 }
 
-// Epilogue of the single-system energy kernels: tile_of(t, ng, wg, d2) names the tile of persistent
-// iteration t and whether its second accumulator was written (false for a single-product tile).
-template <int Np, typename TileOf, typename Release>
-__device__ void energy_epilogue(const EnergyShape& es, SharedCtl* ctl, float* plane, float* colscale, double* ered,
-                                int64_t t_first, int64_t t_end, int64_t t_step, TileOf tile_of, Release release) {
-    int it = 0;
-    for (int64_t t = t_first; t < t_end; t += t_step, ++it) {
-        int ng, wg;
-        bool d2;
-        tile_of(t, ng, wg, d2);
-        bool ok;
-        if constexpr (Np == 0) ok = energy_epilogue_tile_gen(es, ctl, plane, colscale, ng, wg, it, d2, release);
-        else ok = energy_epilogue_tile<Np>(es, ctl, plane, colscale, ered, ng, wg, it, d2, release);
-        if (!ok) break;
-    }
+// One tile by the epilogue its Np takes (0: es.Np at run time).
+template <int Np, typename Release>
+__device__ __forceinline__ bool energy_epilogue_any(const EnergyShape& es, SharedCtl* ctl, float* xbuf, float* colscale,
+                                                    double* ered, int ng, int wg, bool single, Turns& turns,
+                                                    Release release) {
+    const int part = turns.part(single);
+    const uint32_t parity = turns.full_parity(part);
+    auto done = [&] { release(single, part); };
+    if constexpr (Np == 0) return energy_epilogue_tile_gen(es, ctl, xbuf, colscale, ng, wg, part, parity, !single, done);
+    else return energy_epilogue_tile<Np>(es, ctl, xbuf, ered, ng, wg, part, parity, !single, done);
 }
 
 template <int Np, int BK, int AP>
@@ -1023,13 +1094,14 @@ __global__ void __launch_bounds__(kEThreads, 1)
     } else if (warp == 1) {
         if (lane == 0) energy_mma<BK, AP>(sbase, ctl, es);
     } else {
-        energy_epilogue<Np>(
-            es, ctl, plane, colscale, ered, blockIdx.x, es.tiles, gridDim.x,
-            [&](int64_t t, int& ng, int& wg, bool& d2) {
-                energy_tile(es, t, ng, wg);
-                d2 = true;
-            },
-            [&]() { mbar_arrive(&ctl->tempty[0]); });
+        Turns turns;
+        for (int64_t t = blockIdx.x; t < es.tiles; t += gridDim.x) {
+            int ng, wg;
+            energy_tile(es, t, ng, wg);
+            if (!energy_epilogue_any<Np>(es, ctl, plane, colscale, ered, ng, wg, false, turns,
+                                         [&](bool, int) { mbar_arrive(&ctl->tempty[0]); }))
+                break;
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -1051,21 +1123,27 @@ __global__ void __launch_bounds__(kEThreads, 1)
 // Synchronisation: rank 0's full[] barriers count both CTAs' TMA bytes (rank 0 posts the
 // expected total); rank 0's MMA commits arrive on both CTAs' empty[] and tfull barriers
 // (multicast); every epilogue warp of both CTAs arrives on rank 0's tempty.
-template <int BK, int AP>
-__device__ void energy_producer2(uint8_t* sbase, SharedCtl* ctl, const CUtensorMap* tAh, const CUtensorMap* tAl,
-                                 const CUtensorMap* tAr, const CUtensorMap* tBh, const CUtensorMap* tBl,
-                                 const CUtensorMap* tBr, const EnergyShape& es, uint32_t rank) {
+//
+// The pair kernels' tiles: tile t of cluster_id_x(), + ncluster_x(), ... < ntiles; at(t) describes it.
+struct PairTile {
+    const EnergyShape* es;
+    const CUtensorMap* map;    // Ltilde hi, lo, r and Theta hi, lo, r' (six in a row)
+    int ngp, wg;
+};
+
+template <int BK, int AP, typename At>
+__device__ void energy_producer_pair(uint8_t* sbase, SharedCtl* ctl, int64_t ntiles, uint32_t rank, At at) {
     using C = EStage<BK, AP, 128>;
-    const CUtensorMap* const mp[6] = {tAh, tAl, tAr, tBh, tBl, tBr};
     int64_t g = 0;
     bool ok = true;
-    for (int64_t t = cluster_id_x(); t < es.tiles2 && ok; t += ncluster_x()) {
-        int ngp, wg;
-        energy_tile_rows(es, t, es.n_pairs, ngp, wg);
-        const int ng = 2 * ngp + (int)rank;
-        const bool single = energy_pair_single(es, ngp);
+    for (int64_t t = cluster_id_x(); t < ntiles && ok; t += ncluster_x()) {
+        const PairTile pt = at(t);
+        const EnergyShape& es = *pt.es;
+        const int ng = 2 * pt.ngp + (int)rank;
+        const bool single = energy_pair_single(es, pt.ngp);
         const int nst = single ? es.nk / 2 : es.nk;   // es.nk is even (M % 64 == 0)
-        const int ya = ng * es.G * es.Np, yb = wg * 2 * es.G * es.Np + (int)rank * 128;
+        const int ya = ng * es.G * es.Np, yb = pt.wg * 2 * es.G * es.Np + (int)rank * 128;
+        const CUtensorMap* const mp[6] = {pt.map, pt.map + 1, pt.map + 2, pt.map + 3, pt.map + 4, pt.map + 5};
         for (int kb = 0; kb < nst; ++kb, ++g) {
             const int st = (int)(g % C::kStages);
             const uint32_t ph = (uint32_t)((g / C::kStages) & 1);
@@ -1087,46 +1165,103 @@ __device__ void energy_producer2(uint8_t* sbase, SharedCtl* ctl, const CUtensorM
     }
 }
 
-template <int BK, int AP>
-__device__ void energy_mma2(uint8_t* sbase, SharedCtl* ctl, const EnergyShape& es) {
+// One thread.  (The whole warp waiting, with a lane elected for each stage's MMAs, took 1.75 times as
+// long: the wait, shuffle and election stand between every two stages.)
+template <int BK, int AP, typename At>
+__device__ void energy_mma_pair(uint8_t* sbase, SharedCtl* ctl, int64_t ntiles, At at) {
     using C = EStage<BK, AP, 128>;
-    const uint32_t d1 = ctl->tmem_base, d2 = d1 + 256;
+    const uint32_t base = ctl->tmem_base;
+    const uint64_t d0 = edesc<BK>(smem_u32(sbase));
+    const uint32_t lo0 = (uint32_t)d0, hi0 = (uint32_t)(d0 >> 32);
+    Turns turns;
     int64_t g = 0;
-    int it = 0;
     bool ok = true;
-    for (int64_t t = cluster_id_x(); t < es.tiles2 && ok; t += ncluster_x(), ++it) {
-        int ngp, wg;
-        energy_tile_rows(es, t, es.n_pairs, ngp, wg);
+    for (int64_t t = cluster_id_x(); t < ntiles && ok; t += ncluster_x()) {
+        const PairTile pt = at(t);
+        const EnergyShape& es = *pt.es;
         bool lolo = es.lolo != 0;
         if (es.lolo_group) {
-            lolo = es.lolo_group[2 * ngp] != 0;
-            if (2 * ngp + 1 < es.n_groups) lolo = lolo || es.lolo_group[2 * ngp + 1] != 0;
+            lolo = es.lolo_group[2 * pt.ngp] != 0;
+            if (2 * pt.ngp + 1 < es.n_groups) lolo = lolo || es.lolo_group[2 * pt.ngp + 1] != 0;
         }
-        const bool single = energy_pair_single(es, ngp);
+        const bool single = energy_pair_single(es, pt.ngp);
         const int nst = single ? es.nk / 2 : es.nk;
-        if (!mbar_wait(&ctl->tempty[0], ((uint32_t)it & 1u) ^ 1u, &ctl->abort)) break;
+        const int part = turns.part(single);
+        if (!mbar_wait(&ctl->tempty[part], turns.empty_parity(part), &ctl->abort)) break;
+        if (!single && !mbar_wait(&ctl->tempty[1], turns.empty_parity(1), &ctl->abort)) break;
         tc_fence_after();
+        const uint32_t d1 = base + 256u * part, d2 = base + 256u;
         for (int kb = 0; kb < nst; ++kb, ++g) {
             const int st = (int)(g % C::kStages);
             const uint32_t ph = (uint32_t)((g / C::kStages) & 1);
             if (!mbar_wait(&ctl->full[st], ph, &ctl->abort)) { ok = false; break; }
             tc_fence_after();
-            energy_stage_mma_pair<BK, AP>(smem_u32(sbase + (size_t)st * C::kStageBytes), d1, d2, kb, single, lolo);
+            energy_stage_mma_pair<BK, AP>(lo0 + st * (C::kStageBytes >> 4), hi0, d1, d2, kb, single, lolo);
             mma_commit_pair(&ctl->empty[st], 3);   // the stage is free in both CTAs
         }
         if (!ok) break;
-        mma_commit_pair(&ctl->tfull[0], 3);        // both CTAs' accumulators are complete
+        mma_commit_pair(&ctl->tfull[part], 3);   // both CTAs' accumulators are complete
     }
     mma_commit_pair(&ctl->done, 1);
     wait_drain(&ctl->done, 0);
 }
 
+// Barriers and tensor memory of a CTA pair, set up and given back.
+template <int kStages>
+__device__ __forceinline__ void energy_pair_begin(SharedCtl* ctl) {
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kStages; ++i) {
+            mbar_init(&ctl->full[i], 1);
+            mbar_init(&ctl->empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&ctl->tfull[i], 1);
+            mbar_init(&ctl->tempty[i], 2 * (kEEpi / 32));   // one arrival per epilogue warp of both CTAs
+        }
+        mbar_init(&ctl->done, 1);
+        ctl->abort = 0;
+        fence_mbar_init();
+    }
+    __syncthreads();
+    cluster_sync();   // both CTAs' barriers exist before any copy or arrival reaches them
+    if (threadIdx.x >> 5 == 1) {
+        tmem_alloc_pair(&ctl->tmem_base, 512);
+        tmem_relinquish_pair();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    cluster_sync();   // tensor memory allocated in both CTAs before the first MMA
+}
+__device__ __forceinline__ void energy_pair_end(SharedCtl* ctl, unsigned* flags) {
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();   // both CTAs are done with tensor memory and each other's shared memory
+    if (threadIdx.x >> 5 == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(ctl->tmem_base, 512);
+    }
+    if (threadIdx.x == 0 && ctl->abort) atomicOr(flags, FLAG_TIMEOUT);
+}
+// An epilogue warp is done with a tile's accumulators: rank 0's tempty barriers (both for a tile that
+// used both).
+struct PairRelease {
+    uint32_t e0, e1;
+    __device__ __forceinline__ explicit PairRelease(SharedCtl* ctl)
+        : e0(mapa_shared(&ctl->tempty[0], 0)), e1(mapa_shared(&ctl->tempty[1], 0)) {}
+    __device__ __forceinline__ void operator()(bool single, int part) const {
+        mbar_arrive_cluster(part == 0 ? e0 : e1);
+        if (!single) mbar_arrive_cluster(e1);
+    }
+};
+
+struct EnergyMaps {
+    CUtensorMap m[6];   // Ltilde hi, lo, r and Theta hi, lo, r'
+};
+
 template <int Np, int BK, int AP>
 __global__ void __launch_bounds__(kEThreads, 1)
-    tc_energy_pair_kernel(const __grid_constant__ CUtensorMap tAh, const __grid_constant__ CUtensorMap tAl,
-                          const __grid_constant__ CUtensorMap tAr, const __grid_constant__ CUtensorMap tBh,
-                          const __grid_constant__ CUtensorMap tBl, const __grid_constant__ CUtensorMap tBr,
-                          EnergyShape es, unsigned* flags) {
+    tc_energy_pair_kernel(const __grid_constant__ EnergyMaps maps, const __grid_constant__ EnergyShape es, unsigned* flags) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sbase = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     using C = EStage<BK, AP, 128>;
@@ -1136,60 +1271,32 @@ __global__ void __launch_bounds__(kEThreads, 1)
     SharedCtl* ctl = reinterpret_cast<SharedCtl*>(ered + 256);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
-    if (warp == 0 && lane == 0) {
-        tma_prefetch_desc(&tAh);
-        tma_prefetch_desc(&tAl);
-        if (AP == 3) tma_prefetch_desc(&tAr);
-        tma_prefetch_desc(&tBh);
-        tma_prefetch_desc(&tBl);
-        if (AP == 3 && es.single_group) tma_prefetch_desc(&tBr);
-    }
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < C::kStages; ++i) {
-            mbar_init(&ctl->full[i], 1);
-            mbar_init(&ctl->empty[i], 1);
-        }
-        mbar_init(&ctl->tfull[0], 1);
-        mbar_init(&ctl->tempty[0], 2 * (kEEpi / 32));   // one arrival per epilogue warp of both CTAs
-        mbar_init(&ctl->done, 1);
-        ctl->abort = 0;
-        fence_mbar_init();
-    }
-    __syncthreads();
-    cluster_sync();   // both CTAs' barriers exist before any copy or arrival reaches them
-    if (warp == 1) {
-        tmem_alloc_pair(&ctl->tmem_base, 512);
-        tmem_relinquish_pair();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    cluster_sync();   // tensor memory allocated in both CTAs before the first MMA
-
+    if (warp == 0 && lane == 0)
+        for (int i = 0; i < 6; ++i)
+            if ((AP == 3 || i != 2) && (i != 5 || es.single_group)) tma_prefetch_desc(&maps.m[i]);
+    energy_pair_begin<C::kStages>(ctl);
+    auto at = [&](int64_t t) {
+        PairTile p;
+        p.es = &es;
+        p.map = maps.m;
+        energy_tile_rows(es, t, es.n_pairs, p.ngp, p.wg);
+        return p;
+    };
     if (warp == 0) {
-        if (lane == 0) energy_producer2<BK, AP>(sbase, ctl, &tAh, &tAl, &tAr, &tBh, &tBl, &tBr, es, rank);
+        if (lane == 0) energy_producer_pair<BK, AP>(sbase, ctl, es.tiles2, rank, at);
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) energy_mma2<BK, AP>(sbase, ctl, es);
+        if (lane == 0 && rank == 0) energy_mma_pair<BK, AP>(sbase, ctl, es.tiles2, at);
     } else {
-        const uint32_t tempty0 = mapa_shared(&ctl->tempty[0], 0);
-        energy_epilogue<Np>(
-            es, ctl, plane, colscale, ered, cluster_id_x(), es.tiles2, ncluster_x(),
-            [&](int64_t t, int& ng, int& wg, bool& d2) {
-                int ngp;
-                energy_tile_rows(es, t, es.n_pairs, ngp, wg);
-                ng = 2 * ngp + (int)rank;
-                d2 = !energy_pair_single(es, ngp);
-            },
-            [&]() { mbar_arrive_cluster(tempty0); });
+        const PairRelease release(ctl);
+        Turns turns;
+        for (int64_t t = cluster_id_x(); t < es.tiles2; t += ncluster_x()) {
+            const PairTile p = at(t);
+            if (!energy_epilogue_any<Np>(es, ctl, plane, colscale, ered, 2 * p.ngp + (int)rank, p.wg,
+                                         energy_pair_single(es, p.ngp), turns, release))
+                break;
+        }
     }
-    tc_fence_before();
-    __syncthreads();
-    cluster_sync();   // both CTAs are done with tensor memory and each other's shared memory
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc_pair(ctl->tmem_base, 512);
-    }
-    if (threadIdx.x == 0 && ctl->abort) atomicOr(flags, FLAG_TIMEOUT);
+    energy_pair_end(ctl, flags);
 }
 
 // ---------------------------------------------------------------- energy kernel, many systems
@@ -1198,75 +1305,6 @@ __global__ void __launch_bounds__(kEThreads, 1)
 // every system, each system with its own operands (tensor maps kept in global memory), K,
 // Np and outputs.  Per tile the arithmetic, and its order, are the single-system CTA-pair
 // kernel's; only the tile's source changes.
-template <int BK, int AP>
-__device__ void energy_producer_multi(uint8_t* sbase, SharedCtl* ctl, const EnergySys* sys, const EnergyWork* work,
-                                      int64_t nwork, uint32_t rank) {
-    using C = EStage<BK, AP, 128>;
-    int64_t g = 0;
-    bool ok = true;
-    for (int64_t t = cluster_id_x(); t < nwork && ok; t += ncluster_x()) {
-        const EnergyWork w = work[t];
-        const EnergySys* S = sys + w.sys;
-        const bool single = energy_pair_single(S->es, w.ngp);
-        const int nst = single ? S->es.nk / 2 : S->es.nk;
-        const int ng = 2 * w.ngp + (int)rank;
-        const CUtensorMap* const mp[6] = {&S->map[0], &S->map[1], &S->map[2], &S->map[3], &S->map[4], &S->map[5]};
-        const int ya = ng * S->es.G * S->es.Np, yb = w.wg * 2 * S->es.G * S->es.Np + (int)rank * 128;
-        for (int kb = 0; kb < nst; ++kb, ++g) {
-            const int st = (int)(g % C::kStages);
-            const uint32_t ph = (uint32_t)((g / C::kStages) & 1);
-            if (!mbar_wait(&ctl->empty[st], ph ^ 1u, &ctl->abort)) { ok = false; break; }
-            energy_stage_load_pair<BK, AP>(sbase + (size_t)st * C::kStageBytes, ctl, st, mp, kb, ya, yb, single, rank);
-        }
-    }
-    if (!ok) {
-        if (rank == 0) {
-            const int64_t first = g > C::kStages ? g - C::kStages : 0;
-            for (int64_t j = first; j < g; ++j)
-                wait_drain(&ctl->full[j % C::kStages], (uint32_t)((j / C::kStages) & 1));
-        } else {
-            const long long t0 = clock64();
-            while (clock64() - t0 < (1LL << 22)) {
-            }
-        }
-    }
-}
-
-template <int BK, int AP>
-__device__ void energy_mma_multi(uint8_t* sbase, SharedCtl* ctl, const EnergySys* sys, const EnergyWork* work,
-                                 int64_t nwork) {
-    using C = EStage<BK, AP, 128>;
-    const uint32_t d1 = ctl->tmem_base, d2 = d1 + 256;
-    int64_t g = 0;
-    int it = 0;
-    bool ok = true;
-    for (int64_t t = cluster_id_x(); t < nwork && ok; t += ncluster_x(), ++it) {
-        const EnergyWork w = work[t];
-        const EnergyShape& es = sys[w.sys].es;
-        bool lolo = es.lolo != 0;
-        if (es.lolo_group) {
-            lolo = es.lolo_group[2 * w.ngp] != 0;
-            if (2 * w.ngp + 1 < es.n_groups) lolo = lolo || es.lolo_group[2 * w.ngp + 1] != 0;
-        }
-        const bool single = energy_pair_single(es, w.ngp);
-        const int nst = single ? es.nk / 2 : es.nk;
-        if (!mbar_wait(&ctl->tempty[0], ((uint32_t)it & 1u) ^ 1u, &ctl->abort)) break;
-        tc_fence_after();
-        for (int kb = 0; kb < nst; ++kb, ++g) {
-            const int st = (int)(g % C::kStages);
-            const uint32_t ph = (uint32_t)((g / C::kStages) & 1);
-            if (!mbar_wait(&ctl->full[st], ph, &ctl->abort)) { ok = false; break; }
-            tc_fence_after();
-            energy_stage_mma_pair<BK, AP>(smem_u32(sbase + (size_t)st * C::kStageBytes), d1, d2, kb, single, lolo);
-            mma_commit_pair(&ctl->empty[st], 3);
-        }
-        if (!ok) break;
-        mma_commit_pair(&ctl->tfull[0], 3);
-    }
-    mma_commit_pair(&ctl->done, 1);
-    wait_drain(&ctl->done, 0);
-}
-
 template <int BK, int AP>
 __global__ void __launch_bounds__(kEThreads, 1)
     tc_energy_multi_kernel(const EnergySys* __restrict__ sys, const EnergyWork* __restrict__ work, int64_t nwork,
@@ -1280,61 +1318,39 @@ __global__ void __launch_bounds__(kEThreads, 1)
     SharedCtl* ctl = reinterpret_cast<SharedCtl*>(ered + 256);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < C::kStages; ++i) {
-            mbar_init(&ctl->full[i], 1);
-            mbar_init(&ctl->empty[i], 1);
-        }
-        mbar_init(&ctl->tfull[0], 1);
-        mbar_init(&ctl->tempty[0], 2 * (kEEpi / 32));
-        mbar_init(&ctl->done, 1);
-        ctl->abort = 0;
-        fence_mbar_init();
-    }
-    __syncthreads();
-    cluster_sync();
-    if (warp == 1) {
-        tmem_alloc_pair(&ctl->tmem_base, 512);
-        tmem_relinquish_pair();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    cluster_sync();
-
+    energy_pair_begin<C::kStages>(ctl);
+    auto at = [&](int64_t t) {
+        const EnergyWork w = work[t];
+        PairTile p;
+        p.es = &sys[w.sys].es;
+        p.map = sys[w.sys].map;
+        p.ngp = w.ngp;
+        p.wg = w.wg;
+        return p;
+    };
     if (warp == 0) {
-        if (lane == 0) energy_producer_multi<BK, AP>(sbase, ctl, sys, work, nwork, rank);
+        if (lane == 0) energy_producer_pair<BK, AP>(sbase, ctl, nwork, rank, at);
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) energy_mma_multi<BK, AP>(sbase, ctl, sys, work, nwork);
+        if (lane == 0 && rank == 0) energy_mma_pair<BK, AP>(sbase, ctl, nwork, at);
     } else {
-        const uint32_t tempty0 = mapa_shared(&ctl->tempty[0], 0);
-        auto release = [&]() { mbar_arrive_cluster(tempty0); };
-        int it = 0;
-        for (int64_t t = cluster_id_x(); t < nwork; t += ncluster_x(), ++it) {
-            const EnergyWork w = work[t];
-            const EnergyShape& es = sys[w.sys].es;
-            const int ng = 2 * w.ngp + (int)rank;
-            const bool d2 = !energy_pair_single(es, w.ngp);
+        const PairRelease release(ctl);
+        Turns turns;
+        for (int64_t t = cluster_id_x(); t < nwork; t += ncluster_x()) {
+            const PairTile p = at(t);
+            const EnergyShape& es = *p.es;
+            const int ng = 2 * p.ngp + (int)rank;
+            const bool single = energy_pair_single(es, p.ngp);
             bool ok;
             switch (es.Np) {
-                case 32: ok = energy_epilogue_tile<32>(es, ctl, plane, colscale, ered, ng, w.wg, it, d2, release); break;
-                case 64: ok = energy_epilogue_tile<64>(es, ctl, plane, colscale, ered, ng, w.wg, it, d2, release); break;
-                case 128:
-                    ok = energy_epilogue_tile<128>(es, ctl, plane, colscale, ered, ng, w.wg, it, d2, release);
-                    break;
-                default: ok = energy_epilogue_tile_gen(es, ctl, plane, colscale, ng, w.wg, it, d2, release); break;
+                case 32: ok = energy_epilogue_any<32>(es, ctl, plane, colscale, ered, ng, p.wg, single, turns, release); break;
+                case 64: ok = energy_epilogue_any<64>(es, ctl, plane, colscale, ered, ng, p.wg, single, turns, release); break;
+                case 128: ok = energy_epilogue_any<128>(es, ctl, plane, colscale, ered, ng, p.wg, single, turns, release); break;
+                default: ok = energy_epilogue_any<0>(es, ctl, plane, colscale, ered, ng, p.wg, single, turns, release); break;
             }
             if (!ok) break;
         }
     }
-    tc_fence_before();
-    __syncthreads();
-    cluster_sync();
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc_pair(ctl->tmem_base, 512);
-    }
-    if (threadIdx.x == 0 && ctl->abort) atomicOr(flags, FLAG_TIMEOUT);
+    energy_pair_end(ctl, flags);
 }
 
 // --------------------------------------------------------------------------- row split
@@ -1891,7 +1907,9 @@ int launch_energy_pair(const CUtensorMap* m, const EnergyShape& es, unsigned* fl
     if (launch_policy().grid_cap > 0) pairs = std::max(1, std::min(pairs, launch_policy().grid_cap / 2));
     cfg.gridDim = dim3((unsigned)(2 * std::min<int64_t>(es.tiles2, pairs)));
     count_launch();
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, m[0], m[1], m[2], m[3], m[4], m[5], es, flags);
+    EnergyMaps maps;
+    std::copy(m, m + 6, maps.m);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, maps, es, flags);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return fail(AFQMC_ERR_CUDA, std::string("tc_energy (CTA pairs) launch: ") + cudaGetErrorString(e));
     return AFQMC_OK;
