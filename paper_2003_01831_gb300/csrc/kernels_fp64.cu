@@ -616,26 +616,34 @@ __global__ void __launch_bounds__(kGJT)
 // The inverse and log-determinant of an N x N complex matrix, 32 < N <= 128, held entirely in
 // registers: one CTA for N <= 64, else a cluster of two CTAs (the two halves of a 128 x 128
 // complex matrix fill two register files).  CTA r owns the 64 consecutive columns
-// [64 r, 64 r + 64); warp w of it owns four of them, and lane l holds rows l, l + 32, ... (RQ of
-// them), so the thread's block is a[RQ][4].  Pivoting is implicit: step k picks, among the rows
+// [64 r, 64 r + 64); warp w of it owns CW of them, and lane l holds rows l, l + 32, ... (RQ of
+// them), so the thread's block is RQ x CW.  Pivoting is implicit: step k picks, among the rows
 // not pivoted yet, the one with the largest |re| + |im| in column k (lowest row on ties), scales
 // it and eliminates column k from every other row, in place, so that after N steps the stored
 // array X satisfies X[p_k][j] = inverse[k][p_j] for the pivot rows p_k.  det = sign(p) prod(pivot).
-// The warp owning column k+1 updates that column first, searches its pivot and publishes the
-// column and the pivot row (to both CTAs' shared memory) before finishing its own update, so one
-// cluster barrier per step orders the steps and the search is off the critical path.  The
-// pivot row reaches the other lanes of each warp by shuffles; the column k multipliers are
-// read from shared memory.  The chain from one pivot to the next (search, reciprocal, publication)
-// bounds a step; with the search by integer warp reductions and the float-pair reciprocal by
-// Newton steps, 2048 inverses of N = 128 went from 25.5 to 20.1 ms (NumFF) and 45.7 to 41.3 ms
-// (NumD, near its FP64 pipe's 28 ms).
+// Four columns are a panel.  Its four steps are taken first, on the panel alone, by RQ neighbouring
+// warps, the owner among them (one row a lane, so the chain from one pivot to the next is short:
+// search, reciprocal, one row's update), which publish each step's column, pivot row and pivot (to both CTAs'
+// shared memory); then all other warps take the same steps, in the same order, on their columns, each
+// warp by itself (the pivot row reaches its lanes by shuffles, the multipliers come from shared
+// memory), and the next panel's warps go on to that panel.  One barrier per panel orders them.
+// Steps that each had a barrier, with the next column updated and searched by its one owner warp,
+// left the fp32 pipe idle for two thirds of the time.  32 < N <= 64 runs two matrices an SM
+// (CW = 8, 256 threads; a panel of eight columns would spill).  Float pairs are packed two columns to a 64-bit register, which halves the
+// instructions; conversions from and to FP64 are by integer operations where they can be (the FP64
+// pipe takes 64 cycles for a warp's instruction).
+// Measured, a barrier per step -> this: 2048 inverses of N = 128 25.5 -> 13.2 ms in float pairs (the
+// fp32 pipe's 6.6 ms for the updates, the panels' chains the rest) and 45.7 -> 37.4 ms in FP64 (the
+// FP64 pipe's 28 ms); 512 of N = 64 1.38 -> 0.54 and 2.13 -> 1.74 ms.
 constexpr int kGJRegCols = 64;      // columns per CTA
-constexpr int kGJRegThreads = 512;  // 16 warps x 4 columns
+constexpr int kGJPanel = 4;         // columns per panel
+template <int CW>
+constexpr int kGJRegThreads = 32 * (kGJRegCols / CW);   // a warp per CW columns
 
 // Element arithmetic of the register Gauss-Jordan kernel.  NumD: FP64 complex.  NumFF: each of
 // re, im a float pair hi + lo (~2^-44 relative, the TwoProduct / TwoSum error-free transforms on
-// the fp32 pipe, which is ~64x GB300's FP64 pipe); pivot reciprocals, the read-out and the
-// log-determinant are FP64 either way.
+// the fp32 pipe, which is ~64x GB300's FP64 pipe), pivot reciprocals as exact as FP64 rounded to
+// such a pair; the read-out and the log-determinant are FP64 either way.
 struct NumD {
     using T = cplx;
     __device__ static T from(cplx v) { return v; }
@@ -650,7 +658,17 @@ struct NumD {
     static constexpr unsigned kInf = 0x7ff00000u;   // high word of infinity
     __device__ static T recip(const T& v);
     __device__ static T mul(const T& a, const T& b) { return a * b; }
-    __device__ static void upd(T& a, const T& m, const T& p) { cfma(a, cplx{-m.re, -m.im}, p); }   // a -= m p
+    template <int RQ, int CW>
+    struct Tile {   // a thread's RQ x CW block
+        T a[RQ][CW];
+        __device__ T get(int q, int u) const { return a[q][u]; }
+        __device__ void set(int q, int u, const T& v) { a[q][u] = v; }
+    };
+    template <int RQ, int CW>   // row q: a -= m p
+    __device__ static void upd(Tile<RQ, CW>& t, int q, const T& m, const Tile<1, CW>& p) {
+#pragma unroll
+        for (int u = 0; u < CW; ++u) cfma(t.a[q][u], cplx{-m.re, -m.im}, p.a[0][u]);
+    }
     __device__ static T negmul(const T& m, const T& b) { const cplx w = m * b; return cplx{-w.re, -w.im}; }
     __device__ static T shfl(const T& v, int src) {
         return cplx{__shfl_sync(0xffffffffu, v.re, src), __shfl_sync(0xffffffffu, v.im, src)};
@@ -663,10 +681,12 @@ struct NumD {
 struct NumFF {
     using T = ffc;
     __device__ static T from(cplx v) {
-        const float rh = (float)v.re, ih = (float)v.im;
-        return ffc{rh, (float)(v.re - (double)rh), ih, (float)(v.im - (double)ih)};
+        ffc r;
+        ff_split(v.re, r.rh, r.rl);
+        ff_split(v.im, r.ih, r.il);
+        return r;
     }
-    __device__ static cplx to(const T& v) { return cplx{(double)v.rh + (double)v.rl, (double)v.ih + (double)v.il}; }
+    __device__ static cplx to(const T& v) { return cplx{widen(v.rh) + widen(v.rl), widen(v.ih) + widen(v.il)}; }
     __device__ static void key(const T& v, unsigned& hi, unsigned& lo) {
         hi = __float_as_uint(fabsf(v.rh) + fabsf(v.ih));
         lo = 0u;
@@ -682,11 +702,32 @@ struct NumFF {
         ff_fma(r.ih, r.il, a.ih, a.il, b.rh, b.rl);
         return r;
     }
-    __device__ static void upd(T& a, const T& m, const T& p) {   // a -= m p
-        ff_fma(a.rh, a.rl, -m.rh, -m.rl, p.rh, p.rl);
-        ff_fma(a.rh, a.rl, m.ih, m.il, p.ih, p.il);
-        ff_fma(a.ih, a.il, -m.rh, -m.rl, p.ih, p.il);
-        ff_fma(a.ih, a.il, -m.ih, -m.il, p.rh, p.rl);
+    template <int RQ, int CW>
+    struct Tile {   // a thread's RQ x CW block, columns 2 j and 2 j + 1 packed
+        f32x2 rh[RQ][CW / 2], rl[RQ][CW / 2], ih[RQ][CW / 2], il[RQ][CW / 2];
+        __device__ T get(int q, int u) const {
+            return ffc{part(rh[q][u / 2], u), part(rl[q][u / 2], u), part(ih[q][u / 2], u), part(il[q][u / 2], u)};
+        }
+        __device__ void set(int q, int u, const T& v) {
+            put(rh[q][u / 2], u, v.rh);
+            put(rl[q][u / 2], u, v.rl);
+            put(ih[q][u / 2], u, v.ih);
+            put(il[q][u / 2], u, v.il);
+        }
+        __device__ static float part(f32x2 x, int u) { return u & 1 ? f2_hi(x) : f2_lo(x); }
+        __device__ static void put(f32x2& x, int u, float v) { x = u & 1 ? f2(f2_lo(x), v) : f2(v, f2_hi(x)); }
+    };
+    template <int RQ, int CW>   // row q: a -= m p
+    __device__ static void upd(Tile<RQ, CW>& t, int q, const T& m, const Tile<1, CW>& p) {
+        const f32x2 rh = f2(m.rh, m.rh), nrh = f2(-m.rh, -m.rh), nrl = f2(-m.rl, -m.rl);
+        const f32x2 ih = f2(m.ih, m.ih), nih = f2(-m.ih, -m.ih), il = f2(m.il, m.il), nil = f2(-m.il, -m.il);
+#pragma unroll
+        for (int j = 0; j < CW / 2; ++j) {
+            ff_fma2(t.rh[q][j], t.rl[q][j], nrh, rh, nrl, p.rh[0][j], p.rl[0][j]);
+            ff_fma2(t.rh[q][j], t.rl[q][j], ih, nih, il, p.ih[0][j], p.il[0][j]);
+            ff_fma2(t.ih[q][j], t.il[q][j], nrh, rh, nrl, p.ih[0][j], p.il[0][j]);
+            ff_fma2(t.ih[q][j], t.il[q][j], nih, ih, nil, p.rh[0][j], p.rl[0][j]);
+        }
     }
     __device__ static T negmul(const T& m, const T& b) {
         const T w = mul(m, b);
@@ -713,184 +754,276 @@ __device__ __forceinline__ cplx crecip(cplx z) {
     return cplx{ldexp(xr * r, 1 - e), ldexp(-xi * r, 1 - e)};
 }
 
-template <class T, int RQ>
-__device__ __forceinline__ T sel_q(const T (&v)[RQ][4], int q, int u) {
-    T r = v[0][u];
+// entry (q, u) of a tile with q (sel_q) or u (sel_u) known at run time only
+template <class Num, int RQ, int CW>
+__device__ __forceinline__ typename Num::T sel_q(const typename Num::template Tile<RQ, CW>& t, int q, int u) {
+    typename Num::T r = t.get(0, u);
 #pragma unroll
     for (int i = 1; i < RQ; ++i)
-        if (q == i) r = v[i][u];
+        if (q == i) r = t.get(i, u);
     return r;
 }
-template <class T, int RQ>
-__device__ __forceinline__ T sel_u(const T (&v)[RQ][4], int q, int u) {
-    T r = v[q][0];
+template <class Num, int RQ, int CW>
+__device__ __forceinline__ typename Num::T sel_u(const typename Num::template Tile<RQ, CW>& t, int q, int u) {
+    typename Num::T r = t.get(q, 0);
 #pragma unroll
-    for (int i = 1; i < 4; ++i)
-        if (u == i) r = v[q][i];
+    for (int i = 1; i < CW; ++i)
+        if (u == i) r = t.get(q, i);
     return r;
 }
 
 __device__ __forceinline__ cplx NumD::recip(const cplx& v) { return crecip(v); }
-// 1 / z for a float pair: z scaled by a power of two as in crecip, then 1 / |z|^2 by two FP64 Newton
-// steps from the float reciprocal (2^-23 -> 2^-46 -> rounding), a dozen FP64 operations in place of
-// the FP64 division, frexp and ldexp that were most of the chain from one pivot to the next.  (The
-// same in float pairs throughout is as fast and 5% less exact at N = 128.)
+// 1 / z for a float pair, on the fp32 pipe: z scaled by a power of two as in crecip, q = conj(z) / |z|^2
+// in single precision, then one Newton step q (1 + e + e^2), e = 1 - z q, with e and the product as
+// float pairs (2^-22 -> 2^-50, as FP64 rounded to a pair).  In FP64 (an instruction of its pipe takes 200 cycles of a chain) this
+// was two thirds of the way from one pivot to the next.
 __device__ __forceinline__ ffc NumFF::recip(const ffc& z) {
     const float mx = fmaxf(fabsf(z.rh), fabsf(z.ih));
     const int ex = (int)((__float_as_uint(mx) >> 23) & 0xffu);          // biased exponent
     const int es = min(max(254 - ex, 1), 253);                          // 2^(es - 127) mx in [1, 2)
     const float s = __uint_as_float((unsigned)es << 23);
-    const double xr = (double)(z.rh * s) + (double)(z.rl * s), xi = (double)(z.ih * s) + (double)(z.il * s);
-    const double d = fma(xr, xr, xi * xi);
-    double r = (double)__frcp_rn((float)d);
-    r = fma(r, fma(-d, r, 1.0), r);
-    r = fma(r, fma(-d, r, 1.0), r);
-    const ffc q = from(cplx{xr * r, -xi * r});
-    return ffc{q.rh * s, q.rl * s, q.ih * s, q.il * s};
+    const float ah = z.rh * s, al = z.rl * s, bh = z.ih * s, bl = z.il * s;
+    const float r = __frcp_rn(fmaf(ah, ah, bh * bh));
+    const float qr = ah * r, qi = -(bh * r);
+    // e = 1 - (ah + al + i (bh + bl)) (qr + i qi): the leading products' and sums' errors and the low
+    // products gathered with their own errors (without those, four times the error of FP64)
+    auto low = [](float a, float b, float ga, float gb, float ha, float hb, float c, float& lead) {
+        // lead + (a + b + ga gb + ha hb + c) as a float pair; returns the low half
+        const float g = ga * gb, ge = fmaf(ga, gb, -g), h = ha * hb, he = fmaf(ha, hb, -h);
+        float l1, c1, l2, c2, l3, c3, l4, c4, c5;
+        two_sum(a, b, l1, c1);
+        two_sum(g, h, l2, c2);
+        two_sum(l1, l2, l3, c3);
+        two_sum(l3, c, l4, c4);
+        two_sum(lead, l4, lead, c5);
+        return c5 + ((c1 + c2) + (c3 + c4) + (ge + he));
+    };
+    const float p1 = ah * qr, e1 = fmaf(ah, qr, -p1), p2 = bh * qi, e2 = fmaf(bh, qi, -p2);
+    float s1, t1, xh, t2, s3, t3;
+    two_sum(1.0f, -p1, s1, t1);
+    two_sum(s1, p2, xh, t2);
+    const float xl = low(e2, -e1, -al, qr, bl, qi, t1 + t2, xh);
+    const float p3 = ah * qi, e3 = fmaf(ah, qi, -p3), p4 = bh * qr, e4 = fmaf(bh, qr, -p4);
+    two_sum(p3, p4, s3, t3);
+    const float nl = low(e3, e4, al, qi, bl, qr, t3, s3);
+    const float yh = -s3, yl = -nl;
+    // f = e + e^2, q (1 + f)
+    const float fl = fmaf(xh, xh, fmaf(-yh, yh, xl)), gl = fmaf(2.0f * xh, yh, yl);
+    auto add = [&](float q, float a, float b, float c, float d, float bl2, float dl) {   // q + a (b + bl2) + c (d + dl)
+        const float m1 = a * b, h1 = fmaf(a, b, -m1), m2 = c * d, h2 = fmaf(c, d, -m2);
+        float u, v, h, l;
+        two_sum(m1, m2, u, v);
+        v = fmaf(a, bl2, fmaf(c, dl, v + (h1 + h2)));
+        two_sum(q, u, h, l);
+        l += v;
+        const float hi = h + l;
+        return make_float2(hi * s, (l - (hi - h)) * s);
+    };
+    const float2 re = add(qr, qr, xh, -qi, yh, fl, gl), im = add(qi, qr, yh, qi, xh, gl, fl);
+    return ffc{re.x, re.y, im.x, im.y};
 }
 
-// Pivot search over column k (local sub-column uk of the calling warp) and publication of the
-// column (pre-elimination values), the pivot row (or -1 singular / -2 non-finite), the pivot and
-// its reciprocal (once here instead of in every thread).
-template <class Num, int C, int RQ>
-__device__ __forceinline__ void gj_reg_publish(const typename Num::T (&a)[RQ][4], int uk, unsigned used, int N,
-                                               int lane, int owner_rank, typename Num::T* colbuf, int* pbuf,
-                                               typename Num::T* invbuf, typename Num::T* pivbuf) {
+// barrier of the RQ warps that work on a panel (a group at a time, ordered by the CTA's barriers)
+template <int RQ>
+__device__ __forceinline__ void gj_panel_sync() {
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * RQ) : "memory");
+}
+// v scaled by a power of two so that its larger component lies in [1, 2); returns the exponent taken
+// out.  v finite and not zero.
+__device__ __forceinline__ int gj_normalise(cplx& v) {
+    int e = 0;
+    frexp(fmax(fabs(v.re), fabs(v.im)), &e);
+    v = cplx{ldexp(v.re, 1 - e), ldexp(v.im, 1 - e)};
+    return e - 1;
+}
+
+// Shared memory of a CTA: the panel being applied and the next one being published (buffers b and
+// b ^ 1), the panel's columns on their way between its owner and the warps that work on it, and for
+// each of these the best pivot and its row (two steps in turn).
+template <class Num, int RQ>
+struct GJShared {
     using T = typename Num::T;
-    unsigned bh = 0u, bl = 0u, bi = 0xffffffffu;   // the lane's largest unused entry, first row on ties
-    T col[RQ];
+    T col[2][kGJPanel][32 * RQ];            // columns before their elimination: the multipliers
+    T inv[2][kGJPanel], piv[2][kGJPanel];   // pivots and their reciprocals
+    int p[2][kGJPanel];                     // pivot rows (or -1 singular, -2 non-finite)
+    T x[2][kGJPanel][32 * RQ];
+    T row[2][RQ][kGJPanel];
+    unsigned key[2][RQ][3];
+    T pivs[32 * RQ];
+    int perm[32 * RQ], pinv[32 * RQ];
+    cplx det[RQ];
+    int dexp[RQ];
+};
+// The steps of one panel (columns c0 ...), by RQ warps: warp q has the rows 32 q ... + 31.  used:
+// bit q, row lane + 32 q is a pivot row already.
+template <class Num, int C, int RQ>
+__device__ __forceinline__ void gj_panel(GJShared<Num, RQ>& sh, int b, int c0, int N, int q, int lane, int rank,
+                                         unsigned& used) {
+    constexpr int CW = kGJPanel;
+    using T = typename Num::T;
+    const int i = lane + 32 * q;
+    typename Num::template Tile<1, CW> x;
 #pragma unroll
-    for (int q = 0; q < RQ; ++q) {
-        col[q] = sel_u<T, RQ>(a, q, uk);
-        const int i = lane + 32 * q;
-        if (i < N && !((used >> q) & 1u)) {
-            unsigned kh, kl;
-            Num::key(col[q], kh, kl);
-            if (bi == 0xffffffffu || kh > bh || (kh == bh && kl > bl)) { bh = kh; bl = kl; bi = (unsigned)i; }
+    for (int u = 0; u < CW; ++u) x.set(0, u, sh.x[b][u][i]);
+#pragma unroll 1
+    for (int s = 0; s < CW && c0 + s < N; ++s) {
+        const int e = s & 1;
+        const T m = sel_u<Num, 1, CW>(x, 0, s);
+        sh.col[b][s][i] = m;
+        if (C > 1) Num::st_peer(peer_addr(&sh.col[b][s][i], (uint32_t)(rank ^ 1)), m);
+        // the warp's largest unused entry, lowest row on ties
+        const bool open = i < N && !((used >> q) & 1u);
+        unsigned kh = 0u, kl = 0u;
+        if (open) Num::key(m, kh, kl);
+        const unsigned mh = __reduce_max_sync(0xffffffffu, kh);
+        const unsigned ml = Num::kTwoWords ? __reduce_max_sync(0xffffffffu, kh == mh ? kl : 0u) : 0u;
+        const unsigned hit = __ballot_sync(0xffffffffu, open && kh == mh && kl == ml);
+        const int wl = hit ? __ffs(hit) - 1 : 0;
+        if (lane == wl) {
+            sh.key[e][q][0] = hit ? mh : 0u;
+            sh.key[e][q][1] = hit ? ml : 0u;
+            sh.key[e][q][2] = hit ? (unsigned)i : 0xffffffffu;
+#pragma unroll
+            for (int u = 0; u < CW; ++u) sh.row[e][q][u] = x.get(0, u);
         }
-    }
-    const unsigned mh = __reduce_max_sync(0xffffffffu, bh);
-    const unsigned ml = Num::kTwoWords ? __reduce_max_sync(0xffffffffu, bh == mh ? bl : 0u) : 0u;
-    const unsigned mi = __reduce_min_sync(0xffffffffu, bh == mh && bl == ml ? bi : 0xffffffffu);
-    // a zero column is singular; a NaN or infinite pivot magnitude is non-finite
-    const int code = mh >= Num::kInf ? -2 : ((mh | ml) == 0u ? -1 : (int)mi);
+        gj_panel_sync<RQ>();
+        unsigned bh = sh.key[e][0][0], bl = sh.key[e][0][1], bi = sh.key[e][0][2];
 #pragma unroll
-    for (int q = 0; q < RQ; ++q) {
-        const int i = lane + 32 * q;
-        colbuf[i] = col[q];
-        if (C > 1) Num::st_peer(peer_addr(&colbuf[i], (uint32_t)(owner_rank ^ 1)), col[q]);
-    }
-    // the pivot value from the lane that holds row mi
-    const int bl2 = code >= 0 ? (code & 31) : 0, bq = code >= 0 ? (code >> 5) : 0;
-    T pv = col[0];
-#pragma unroll
-    for (int q = 1; q < RQ; ++q)
-        if (bq == q) pv = col[q];
-    pv = Num::shfl(pv, bl2);
-    const T inv = Num::recip(pv);   // every lane: no divergence on the chain
-    if (lane == 0) {
-        *pbuf = code;
-        *invbuf = inv;
-        *pivbuf = pv;
-        if (C > 1) {
-            st_peer_s32(peer_addr(pbuf, (uint32_t)(owner_rank ^ 1)), code);
-            Num::st_peer(peer_addr(invbuf, (uint32_t)(owner_rank ^ 1)), inv);
-            Num::st_peer(peer_addr(pivbuf, (uint32_t)(owner_rank ^ 1)), pv);
+        for (int w = 1; w < RQ; ++w) {
+            const unsigned h = sh.key[e][w][0], l = sh.key[e][w][1], r = sh.key[e][w][2];
+            if (r != 0xffffffffu && (bi == 0xffffffffu || h > bh || (h == bh && l > bl))) { bh = h; bl = l; bi = r; }
         }
+        // a zero column is singular; a NaN or infinite pivot magnitude is non-finite
+        const int p = bh >= Num::kInf ? -2 : ((bh | bl) == 0u ? -1 : (int)bi);
+        if (p < 0) {   // the same in all RQ warps
+            if (q == 0 && lane == 0) {
+                sh.p[b][s] = p;
+                if (C > 1) st_peer_s32(peer_addr(&sh.p[b][s], (uint32_t)(rank ^ 1)), p);
+            }
+            break;
+        }
+        const int pl = p & 31, pq = p >> 5;
+        const T pv = sh.row[e][pq][s];
+        const T inv = Num::recip(pv);
+        if (q == 0 && lane == 0) {
+            sh.p[b][s] = p;
+            sh.inv[b][s] = inv;
+            sh.piv[b][s] = pv;
+            if (C > 1) {
+                st_peer_s32(peer_addr(&sh.p[b][s], (uint32_t)(rank ^ 1)), p);
+                Num::st_peer(peer_addr(&sh.inv[b][s], (uint32_t)(rank ^ 1)), inv);
+                Num::st_peer(peer_addr(&sh.piv[b][s], (uint32_t)(rank ^ 1)), pv);
+            }
+        }
+        const T mine = Num::mul(sh.row[e][pq][lane & (CW - 1)], inv);   // lane u scales entry u
+        typename Num::template Tile<1, CW> prow;
+#pragma unroll
+        for (int u = 0; u < CW; ++u) prow.set(0, u, Num::shfl(mine, u));
+        Num::upd(x, 0, m, prow);
+        const T val = i == p ? inv : Num::negmul(m, inv);   // column c0 + s of the inverse
+#pragma unroll
+        for (int u = 0; u < CW; ++u) {
+            const T w = i == p ? prow.get(0, u) : x.get(0, u);
+            x.set(0, u, u == s ? val : w);
+        }
+        if (lane == pl) used |= 1u << pq;
     }
+#pragma unroll
+    for (int u = 0; u < CW; ++u) sh.x[b][u][i] = x.get(0, u);
 }
 
-template <class Num, int C, int RQ>
-__global__ void __launch_bounds__(kGJRegThreads, 1)
+template <class Num, int C, int RQ, int CW>
+__global__ void __launch_bounds__(kGJRegThreads<CW>, CW / 4)
     gj_reg_kernel(cplx* Sbase, int64_t stride, int N, cplx* logdet, unsigned* flags) {
     using T = typename Num::T;
-    constexpr int NR = 32 * RQ;
-    __shared__ T colbuf[2][NR];
-    __shared__ int pbuf[2];
-    __shared__ T invbuf[2];
-    __shared__ T pivbuf[2];
-    __shared__ int perm[NR];
-    __shared__ int pinv[NR];
-    __shared__ T pivs[NR];
+    __shared__ GJShared<Num, RQ> sh;
     const int rank = C == 1 ? 0 : (int)cluster_rank();
     const int64_t mat = C == 1 ? blockIdx.x : blockIdx.x / C;
     cplx* G = Sbase + mat * stride;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int c0 = rank * kGJRegCols + warp * 4;   // first global column of this thread
-    T a[RQ][4];
+    const int c0 = rank * kGJRegCols + warp * CW;                                  // first global column of this warp
+    const int g0 = rank * kGJRegCols + warp / RQ * RQ * CW, g1 = g0 + RQ * CW;     // columns of its group of RQ warps
+    typename Num::template Tile<RQ, CW> a;
 #pragma unroll
     for (int q = 0; q < RQ; ++q) {
         const int i = lane + 32 * q;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < CW; ++u) {
             const int j = c0 + u;
-            a[q][u] = Num::from((i < N && j < N) ? G[(int64_t)i * N + j] : cplx{0.0, 0.0});
+            a.set(q, u, Num::from((i < N && j < N) ? G[(int64_t)i * N + j] : cplx{0.0, 0.0}));
         }
     }
     unsigned used = 0;   // bit q: row lane + 32 q is a pivot row already
-    auto owns = [&](int k) { return k < N && (k >> 6) == rank && ((k & 63) >> 2) == warp; };
-    if (owns(0)) gj_reg_publish<Num, C, RQ>(a, 0, used, N, lane, rank, colbuf[0], &pbuf[0], &invbuf[0], &pivbuf[0]);
-    gj_sync<C>();
-    int singular = 0;
-    for (int k = 0; k < N; ++k) {
-        const int b = k & 1;
-        const int p = pbuf[b];
-        if (p < 0) { singular = p; break; }
-        const T inv = invbuf[b];
-        if (threadIdx.x == 0) { perm[k] = p; pivs[k] = pivbuf[b]; }
+    // step s of the panel published in buffer b, on this warp's columns: a -= m prow, prow in the
+    // pivot row
+    auto step = [&](int b, int s) {
+        const int p = sh.p[b][s];
+        const T inv = sh.inv[b][s];
         const int pl = p & 31, pq = p >> 5;
-        // the warp's four pivot-row entries: gathered from lane pl, each scaled by one lane
-        // (lane u % 4 scales entry u), then shared again
-        T rp[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) rp[u] = Num::shfl(sel_q<T, RQ>(a, pq, u), pl);
-        T mine = rp[0];
-#pragma unroll
-        for (int u = 1; u < 4; ++u)
-            if ((lane & 3) == u) mine = rp[u];
-        mine = Num::mul(mine, inv);
-        T prow[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) prow[u] = Num::shfl(mine, u);
         if (lane == pl) used |= 1u << pq;
-        const bool ownk = owns(k);
-        const int uk = k & 3;
-        const bool own1 = owns(k + 1);
-        const int u1 = (k + 1) & 3;
-        // one element: a -= m prow, or prow in the pivot row; column k of the inverse (-m / piv,
-        // 1 / piv in the pivot row) is written afterwards by its owner warp alone
-        auto upd = [&](int q, int u, const T& m) {
-            T v = a[q][u];
-            Num::upd(v, m, prow[u]);
-            a[q][u] = lane + 32 * q == p ? prow[u] : v;
-        };
-        if (own1) {   // look-ahead: column k+1 first, then its pivot search and publication
+        // the warp's pivot-row entries: gathered from lane pl, each scaled by one lane (lane
+        // u % CW scales entry u), then shared again
+        T mine = Num::shfl(sel_q<Num, RQ, CW>(a, pq, 0), pl);
 #pragma unroll
-            for (int q = 0; q < RQ; ++q) {
-                const T m = colbuf[b][lane + 32 * q];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (u == u1) upd(q, u, m);
-            }
-            gj_reg_publish<Num, C, RQ>(a, u1, used, N, lane, rank, colbuf[b ^ 1], &pbuf[b ^ 1], &invbuf[b ^ 1],
-                                       &pivbuf[b ^ 1]);
+        for (int u = 1; u < CW; ++u) {
+            const T e = Num::shfl(sel_q<Num, RQ, CW>(a, pq, u), pl);
+            if ((lane & (CW - 1)) == u) mine = e;
         }
+        mine = Num::mul(mine, inv);
+        typename Num::template Tile<1, CW> prow;
+#pragma unroll
+        for (int u = 0; u < CW; ++u) prow.set(0, u, Num::shfl(mine, u));
 #pragma unroll
         for (int q = 0; q < RQ; ++q) {
-            const T m = colbuf[b][lane + 32 * q];
+            if (32 * q >= N) break;
+            Num::upd(a, q, sh.col[b][s][lane + 32 * q], prow);
+            if (q == pq) {   // the same in every thread
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (!(own1 && u == u1)) upd(q, u, m);
-        }
-        if (ownk) {   // warp-uniform: column k of the inverse
-#pragma unroll
-            for (int q = 0; q < RQ; ++q) {
-                const T val = lane + 32 * q == p ? inv : Num::negmul(colbuf[b][lane + 32 * q], inv);
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (u == uk) a[q][u] = val;
+                for (int u = 0; u < CW; ++u) a.set(q, u, lane == pl ? prow.get(0, u) : a.get(q, u));
             }
         }
+    };
+    // panel t, published in buffer b: by the owner's group of RQ warps.  The owner's columns wait in
+    // sh.x until it has taken the panel's steps on its others.
+    auto panel = [&](int t, int b) {
+        const int pc = t * kGJPanel;
+        if (pc < g0 || pc >= g1 || pc >= N) return;
+#pragma unroll
+        for (int o = 0; o < CW; o += kGJPanel)
+            if (pc == c0 + o) {
+#pragma unroll
+                for (int q = 0; q < RQ; ++q)
+#pragma unroll
+                    for (int u = 0; u < kGJPanel; ++u) sh.x[b][u][lane + 32 * q] = a.get(q, o + u);
+            }
+        gj_panel_sync<RQ>();
+        gj_panel<Num, C, RQ>(sh, b, pc, N, warp % RQ, lane, rank, used);
+    };
+    if (C > 1) gj_sync<C>();   // the peer runs before anything is written to its shared memory
+    panel(0, 0);
+    gj_sync<C>();
+    int singular = 0;
+    for (int t = 0; t * kGJPanel < N; ++t) {
+        const int b = t & 1, pc = t * kGJPanel, ns = min(kGJPanel, N - pc);
+        for (int s = 0; s < ns && !singular; ++s) {
+            const int p = sh.p[b][s];
+            if (p < 0) singular = p;
+            else if (threadIdx.x == 0) { sh.perm[pc + s] = p; sh.pivs[pc + s] = sh.piv[b][s]; }
+        }
+        if (singular) break;
+        if (g0 < N && (CW > kGJPanel || pc != c0)) {
+#pragma unroll 1
+            for (int s = 0; s < ns; ++s) step(b, s);
+        }
+#pragma unroll
+        for (int o = 0; o < CW; o += kGJPanel)
+            if (pc == c0 + o) {
+#pragma unroll
+                for (int q = 0; q < RQ; ++q)
+#pragma unroll
+                    for (int u = 0; u < kGJPanel; ++u) a.set(q, o + u, sh.x[b][u][lane + 32 * q]);
+            }
+        panel(t + 1, b ^ 1);
         gj_sync<C>();
     }
     if (singular) {
@@ -902,31 +1035,31 @@ __global__ void __launch_bounds__(kGJRegThreads, 1)
         return;
     }
     __syncthreads();
-    if (threadIdx.x < N) pinv[perm[threadIdx.x]] = threadIdx.x;
-    if (rank == 0 && warp == 0) {
-        // log|det| and arg det: sums over the pivots in a fixed order, plus pi for an odd
-        // pivot permutation (N - number of cycles transpositions)
-        double la = 0.0, ph = 0.0;
-        for (int k = lane; k < N; k += 32) {
-            const cplx pv = Num::to(pivs[k]);
-            la += log(hypot(pv.re, pv.im));
-            ph += atan2(pv.im, pv.re);
+    if (threadIdx.x < N) sh.pinv[sh.perm[threadIdx.x]] = threadIdx.x;
+    // log|det| and arg det from the product of the pivots (fixed order: a lane each, a tree over the
+    // warp, the RQ warps in turn), the exponents apart, times -1 for an odd pivot permutation, whose
+    // sign is that of its inversions (pairs of steps whose pivot rows are out of order)
+    int odd = 0;
+    if (rank == 0 && warp < RQ) {
+        const int k = (int)threadIdx.x;
+        cplx v{1.0, 0.0};
+        int ex = 0;
+        if (k < N) {
+            v = Num::to(sh.pivs[k]);
+            ex = gj_normalise(v);
+            const int pk = sh.perm[k];
+            for (int j = 0; j < k; ++j) odd ^= sh.perm[j] > pk ? 1 : 0;
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            la += __shfl_xor_sync(0xffffffffu, la, o);
-            ph += __shfl_xor_sync(0xffffffffu, ph, o);
+            v = v * cplx{__shfl_xor_sync(0xffffffffu, v.re, o), __shfl_xor_sync(0xffffffffu, v.im, o)};
+            ex += __shfl_xor_sync(0xffffffffu, ex, o);
         }
+        ex += gj_normalise(v);
+        odd = __popc(__ballot_sync(0xffffffffu, odd)) & 1;
         if (lane == 0) {
-            unsigned seen[4] = {0u, 0u, 0u, 0u};
-            int cycles = 0;
-            for (int s0 = 0; s0 < N; ++s0) {
-                if ((seen[s0 >> 5] >> (s0 & 31)) & 1u) continue;
-                ++cycles;
-                for (int x = s0; !((seen[x >> 5] >> (x & 31)) & 1u); x = perm[x]) seen[x >> 5] |= 1u << (x & 31);
-            }
-            if ((N - cycles) & 1) ph += M_PI;
-            logdet[mat] = cplx{la, atan2(sin(ph), cos(ph))};
+            sh.det[warp] = v;
+            sh.dexp[warp] = 2 * ex + odd;
         }
     }
     __syncthreads();
@@ -934,12 +1067,24 @@ __global__ void __launch_bounds__(kGJRegThreads, 1)
     for (int q = 0; q < RQ; ++q) {
         const int i = lane + 32 * q;
         if (i >= N) continue;
-        const int64_t orow = (int64_t)pinv[i] * N;
+        const int64_t orow = (int64_t)sh.pinv[i] * N;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < CW; ++u) {
             const int j = c0 + u;
-            if (j < N) G[orow + perm[j]] = Num::to(a[q][u]);
+            if (j < N) G[orow + sh.perm[j]] = Num::to(a.get(q, u));
         }
+    }
+    if (rank == 0 && warp == 0) {
+        cplx v = sh.det[0];
+        int ex = sh.dexp[0] >> 1, sign = sh.dexp[0];
+#pragma unroll
+        for (int w = 1; w < RQ; ++w) {
+            v = v * sh.det[w];
+            ex += sh.dexp[w] >> 1;
+            sign += sh.dexp[w];
+        }
+        if (sign & 1) v = cplx{-v.re, -v.im};
+        if (lane == 0) logdet[mat] = cplx{log(hypot(v.re, v.im)) + ex * M_LN2, atan2(v.im, v.re)};
     }
     if (C > 1) cluster_sync_all();
 }
@@ -1621,13 +1766,13 @@ void batched_inverse_logdet(cplx* S, int64_t stride, int N, int count, cplx* log
         const bool ff = variant == 3 || (variant == 0 && float_float);
         count_launch();
         if (N <= kGJRegCols) {
-            if (ff) gj_reg_kernel<NumFF, 1, 2><<<count, kGJRegThreads, 0, st>>>(S, stride, N, logdet, flags);
-            else gj_reg_kernel<NumD, 1, 2><<<count, kGJRegThreads, 0, st>>>(S, stride, N, logdet, flags);
+            if (ff) gj_reg_kernel<NumFF, 1, 2, 8><<<count, kGJRegThreads<8>, 0, st>>>(S, stride, N, logdet, flags);
+            else gj_reg_kernel<NumD, 1, 2, 4><<<count, kGJRegThreads<4>, 0, st>>>(S, stride, N, logdet, flags);
             return;
         }
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)count * 2);
-        cfg.blockDim = dim3(kGJRegThreads);
+        cfg.blockDim = dim3(kGJRegThreads<4>);
         cfg.dynamicSmemBytes = 0;
         cfg.stream = st;
         cudaLaunchAttribute at[1];
@@ -1637,8 +1782,8 @@ void batched_inverse_logdet(cplx* S, int64_t stride, int N, int count, cplx* log
         at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        if (ff) cudaLaunchKernelEx(&cfg, gj_reg_kernel<NumFF, 2, 4>, S, stride, N, logdet, flags);
-        else cudaLaunchKernelEx(&cfg, gj_reg_kernel<NumD, 2, 4>, S, stride, N, logdet, flags);
+        if (ff) cudaLaunchKernelEx(&cfg, gj_reg_kernel<NumFF, 2, 4, 4>, S, stride, N, logdet, flags);
+        else cudaLaunchKernelEx(&cfg, gj_reg_kernel<NumD, 2, 4, 4>, S, stride, N, logdet, flags);
         return;
     }
     // one warp per matrix up to 32 rows (variant 1 keeps the shared-memory kernel reachable for
