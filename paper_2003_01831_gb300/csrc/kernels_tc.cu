@@ -112,7 +112,14 @@ __device__ void epilogue_row(const EpiParams& e, int b, int64_t r, int64_t c0, c
 // Epilogue of the three-slice GEMM: 32 consecutive columns [c0, c0+32) of row r, each value a
 // float-float pair vh + vl.
 __device__ __forceinline__ void st32f(float* o, const float (&v)[32]) {
-    if (aligned16(o)) {
+    if ((reinterpret_cast<uintptr_t>(o) & 31) == 0) {   // whole sectors: a lane's rows are far apart
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o + 8 * g), "f"(v[8 * g]),
+                         "f"(v[8 * g + 1]), "f"(v[8 * g + 2]), "f"(v[8 * g + 3]), "f"(v[8 * g + 4]),
+                         "f"(v[8 * g + 5]), "f"(v[8 * g + 6]), "f"(v[8 * g + 7])
+                         : "memory");
+    } else if (aligned16(o)) {
 #pragma unroll
         for (int g = 0; g < 8; ++g)
             reinterpret_cast<float4*>(o)[g] = make_float4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
@@ -129,7 +136,16 @@ __device__ void epilogue_row3(const EpiParams& e, int b, int64_t r, int64_t c0, 
     switch (e.kind) {
         case EPI3_F64: {
             double* o = e.out_f64 + b * e.ob + r * e.ld + c0;
-            if (full && aligned16(o)) {
+            if (full && (reinterpret_cast<uintptr_t>(o) & 31) == 0) {
+#pragma unroll
+                for (int g = 0; g < 8; ++g)
+                    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(o + 4 * g),
+                                 "d"((double)vh[4 * g] + (double)vl[4 * g]),
+                                 "d"((double)vh[4 * g + 1] + (double)vl[4 * g + 1]),
+                                 "d"((double)vh[4 * g + 2] + (double)vl[4 * g + 2]),
+                                 "d"((double)vh[4 * g + 3] + (double)vl[4 * g + 3])
+                                 : "memory");
+            } else if (full && aligned16(o)) {
 #pragma unroll
                 for (int g = 0; g < 16; ++g)
                     reinterpret_cast<double2*>(o)[g] =
@@ -1490,12 +1506,20 @@ __global__ void __launch_bounds__(256) split_rows_f32_kernel(const float* src, i
 // ~1e-9 of |x_a||x_b|.
 constexpr double kS3 = 1.0 / 128.0;
 
-constexpr int kG3ABytes = kBM * kBK * 2;          // one plane, 128 rows x 64
-constexpr int kG3BBytes = 128 * kBK * 2;          // B tile: 128 rows
-constexpr int kG3StageBytes = 3 * (kG3ABytes + kG3BBytes);   // 96 KB
-constexpr int kG3Stages = 2;
+// Two stages of 64 K (96 KB each; four of 32 are as fast).  Sixteen warps drain a tile: they fold the
+// four accumulators into registers, release tensor memory, and scale and store while the next tile's
+// MMAs run; four warps that released it after their stores took half of a tile's time at K = 256.
+// Measured at M = 256, 256 walkers (us): the Taylor terms' products 149 -> 108 (their operands and
+// result take 79 at the copy rate), the potential 442 -> 352 (200 at the MMA rate, 4 GB through L2).
+constexpr int kG3BK = 64;
+constexpr int kG3ABytes = kBM * kG3BK * 2;        // one plane, 128 rows
+constexpr int kG3BBytes = 128 * kG3BK * 2;        // B tile: 128 rows
+constexpr int kG3StageBytes = 3 * (kG3ABytes + kG3BBytes);
+constexpr int kG3Stages = 192 * 1024 / kG3StageBytes;
+constexpr int kG3Epi = 512;                       // 16 warps: 4 quadrants of rows x 4 groups of 32 columns
+constexpr int kG3Threads = 64 + kG3Epi;
 
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(kG3Threads, 1)
     tc_gemm3_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUtensorMap tA1,
                     const __grid_constant__ CUtensorMap tA2, const __grid_constant__ CUtensorMap tB0,
                     const __grid_constant__ CUtensorMap tB1, const __grid_constant__ CUtensorMap tB2, TileShape sh,
@@ -1511,7 +1535,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             mbar_init(&ctl->empty[i], 1);
         }
         mbar_init(&ctl->tfull[0], 1);
-        mbar_init(&ctl->tempty[0], 128);
+        mbar_init(&ctl->tempty[0], kG3Epi / 32);
         mbar_init(&ctl->done, 1);
         ctl->abort = 0;
         fence_mbar_init();
@@ -1540,7 +1564,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                     if (!mbar_wait(&ctl->empty[st], ph ^ 1u, &ctl->abort)) { ok = false; break; }
                     uint8_t* sp = sbase + (size_t)st * kG3StageBytes;
                     mbar_arrive_expect_tx(&ctl->full[st], kG3StageBytes);
-                    const int x = kb * kBK;
+                    const int x = kb * kG3BK;
                     for (int q = 0; q < 3; ++q) {
                         if (three_d) {
                             tma_load_3d(sp + q * kG3ABytes, A[q], &ctl->full[st], x, rt * kBM, az);
@@ -1561,7 +1585,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     } else if (warp == 1) {
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_bf16(kBM, 128, true);
+            constexpr uint32_t A = kG3ABytes >> 4, B = kG3BBytes >> 4;
             const uint32_t d1 = ctl->tmem_base, d2 = d1 + 128, d3 = d1 + 256, d4 = d1 + 384;
+            const uint64_t d0 = kG3BK == 64 ? desc_sw128(smem_u32(sbase)) : desc_sw64(smem_u32(sbase));
+            const uint32_t lo0 = (uint32_t)d0, hi = (uint32_t)(d0 >> 32);
             int64_t g = 0;
             int it = 0;
             bool ok = true;
@@ -1573,22 +1600,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                     const uint32_t ph = (uint32_t)((g / kG3Stages) & 1);
                     if (!mbar_wait(&ctl->full[st], ph, &ctl->abort)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(sbase + (size_t)st * kG3StageBytes);
-                    const uint32_t sb = sa + 3 * kG3ABytes;
 #pragma unroll
-                    for (int kk = 0; kk < kBK / 16; ++kk) {
-                        const uint32_t off = kk * 32;
-                        const uint64_t ah = desc_sw128(sa + off), am = desc_sw128(sa + kG3ABytes + off),
-                                       al = desc_sw128(sa + 2 * kG3ABytes + off);
-                        const uint64_t bh = desc_sw128(sb + off), bm = desc_sw128(sb + kG3BBytes + off),
-                                       bl = desc_sw128(sb + 2 * kG3BBytes + off);
+                    for (int kk = 0; kk < kG3BK / 16; ++kk) {
+                        const uint32_t ah = lo0 + st * (kG3StageBytes >> 4) + 2 * kk, am = ah + A, al = am + A;
+                        const uint32_t bh = al + A, bm = bh + B, bl = bm + B;
                         const uint32_t acc = (kb | kk) != 0 ? 1u : 0u;
-                        mma_bf16(d1, ah, bh, idesc, acc);
-                        mma_bf16(d2, ah, bm, idesc, acc);
-                        mma_bf16(d2, am, bh, idesc, 1u);
-                        mma_bf16(d3, ah, bl, idesc, acc);
-                        mma_bf16(d3, al, bh, idesc, 1u);
-                        mma_bf16(d4, am, bm, idesc, acc);
+                        mma_f16_lo<kKeepNone>(d1, ah, bh, hi, idesc, acc);
+                        mma_f16_lo<kKeepNone>(d2, ah, bm, hi, idesc, acc);
+                        mma_f16_lo<kKeepNone>(d3, ah, bl, hi, idesc, acc);
+                        mma_f16_lo<kKeepNone>(d2, am, bh, hi, idesc, 1u);
+                        mma_f16_lo<kKeepNone>(d4, am, bm, hi, idesc, acc);
+                        mma_f16_lo<kKeepNone>(d3, al, bh, hi, idesc, 1u);
                     }
                     mma_commit(&ctl->empty[st]);
                 }
@@ -1599,45 +1621,49 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             wait_drain(&ctl->done, 0);
         }
     } else {
-        const int g4 = warp & 3;
-        const uint32_t tb = ctl->tmem_base + ((uint32_t)(g4 * 32) << 16);
+        const int g4 = warp & 3, c = (warp - 2) >> 2;
+        const uint32_t tb = ctl->tmem_base + ((uint32_t)(g4 * 32) << 16) + c * 32;
         int it = 0;
         for (int64_t t = blockIdx.x; t < sh.tiles; t += gridDim.x, ++it) {
-            if (!warp_wait(&ctl->tfull[0], (uint32_t)it & 1u, &ctl->abort)) break;
-            tc_fence_after();
             int b, rt, ct;
             tile_coords(sh, t, b, rt, ct);
             const int az = three_d ? (b / sh.am.div) % sh.am.mod : 0;
             const int bz = three_d ? (b / sh.bm.div) % sh.bm.mod : 0;
-            const int64_t r = (int64_t)rt * kBM + g4 * 32 + lane;
+            const int64_t r = (int64_t)rt * kBM + g4 * 32 + lane, c0 = (int64_t)ct * 128 + c * 32;
             const float sa = r < sh.a_rows ? sh.a_scale[(int64_t)az * sh.a_rows + r] : 0.0f;
+            const float sb = c0 + lane < sh.b_rows ? sh.b_scale[(int64_t)bz * sh.b_rows + c0 + lane] : 0.0f;
+            if (!warp_wait(&ctl->tfull[0], (uint32_t)it & 1u, &ctl->abort)) break;
+            tc_fence_after();
             // value = sa sb (acc1 + 2^-7 (acc2 + acc3) + 2^-14 acc4) as the float-float pair
             // hi = sa sb acc1 (an integer times powers of two: exact), lo = sa sb (the rest);
             // the row and column scales are powers of two, so both products are exact
-#pragma unroll 1
-            for (int c = 0; c < 4; ++c) {
+            float vh[32], vl[32];
+            {
                 uint32_t a1[32], a2[32];
-                float vh[32], vl[32];
-                tmem_ld32_nw(tb + 128 + c * 32, a1);   // acc2
-                tmem_ld32_nw(tb + 256 + c * 32, a2);   // acc3
+                tmem_ld32_nw(tb + 128, a1);   // acc2
+                tmem_ld32_nw(tb + 256, a2);   // acc3
                 tmem_ld_wait();
 #pragma unroll
                 for (int q = 0; q < 32; ++q) vl[q] = __uint_as_float(a1[q]) + __uint_as_float(a2[q]);
-                tmem_ld32_nw(tb + c * 32, a1);         // acc1
-                tmem_ld32_nw(tb + 384 + c * 32, a2);   // acc4
+                tmem_ld32_nw(tb, a1);         // acc1
+                tmem_ld32_nw(tb + 384, a2);   // acc4
                 tmem_ld_wait();
-                const int64_t c0 = (int64_t)ct * 128 + c * 32;
 #pragma unroll
                 for (int q = 0; q < 32; ++q) {
-                    const int64_t col = c0 + q;
-                    const float sc = col < sh.b_rows ? sa * sh.b_scale[(int64_t)bz * sh.b_rows + col] : 0.0f;
-                    vl[q] = fmaf((float)kS3, vl[q], (float)(kS3 * kS3) * __uint_as_float(a2[q])) * sc;
-                    vh[q] = __uint_as_float(a1[q]) * sc;
+                    vl[q] = fmaf((float)kS3, vl[q], (float)(kS3 * kS3) * __uint_as_float(a2[q]));
+                    vh[q] = __uint_as_float(a1[q]);
                 }
-                epilogue_row3(epi, b, r, c0, vh, vl);
             }
             tc_fence_before();
-            mbar_arrive(&ctl->tempty[0]);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->tempty[0]);   // the next tile's MMAs run meanwhile
+#pragma unroll
+            for (int q = 0; q < 32; ++q) {
+                const float sc = sa * __shfl_sync(0xffffffffu, sb, q);
+                vl[q] *= sc;
+                vh[q] *= sc;
+            }
+            epilogue_row3(epi, b, r, c0, vh, vl);
         }
     }
     tc_fence_before();
@@ -2169,8 +2195,8 @@ int tc_gemm3(const Split3& A, BatchMap amap, const Split3& B, BatchMap bmap, int
     const bool three_d = nbatch > 1 || amap.mod != (1 << 30);
     CUtensorMap m[6];
     for (int q = 0; q < 3; ++q) {
-        AFQMC_TRY(make_map(&m[q], A.p[q], A.K, A.rows, A.batch, A.K, A.batch_stride, kBM, three_d, true));
-        AFQMC_TRY(make_map(&m[3 + q], B.p[q], B.K, B.rows, B.batch, B.K, B.batch_stride, 128, three_d, true));
+        AFQMC_TRY(make_map(&m[q], A.p[q], A.K, A.rows, A.batch, A.K, A.batch_stride, kBM, three_d, true, 2 * kG3BK));
+        AFQMC_TRY(make_map(&m[3 + q], B.p[q], B.K, B.rows, B.batch, B.K, B.batch_stride, 128, three_d, true, 2 * kG3BK));
     }
     TileShape sh;
     sh.rows = rows;
@@ -2179,7 +2205,7 @@ int tc_gemm3(const Split3& A, BatchMap amap, const Split3& B, BatchMap bmap, int
     sh.nbatch = nbatch;
     sh.rt = (int)((rows + kBM - 1) / kBM);
     sh.ct = (int)((cols + 127) / 128);
-    sh.nk = (int)((K + kBK - 1) / kBK);
+    sh.nk = (int)((K + kG3BK - 1) / kG3BK);
     sh.tiles = (int64_t)sh.rt * sh.ct * nbatch;
     // unbatched: 2-D maps and batch coordinate 0 (the kernel tests the same condition)
     sh.am = three_d ? amap : BatchMap{1, 1 << 30};
@@ -2193,7 +2219,7 @@ int tc_gemm3(const Split3& A, BatchMap amap, const Split3& B, BatchMap bmap, int
     const int cap = launch_policy().grid_cap > 0 ? std::min(launch_policy().grid_cap, tc_num_sms()) : tc_num_sms();
     const int grid = (int)std::min<int64_t>(sh.tiles, cap);
     count_launch();
-    tc_gemm3_kernel<<<grid, kGemmThreads, smem, st>>>(m[0], m[1], m[2], m[3], m[4], m[5], sh, epi, flags);
+    tc_gemm3_kernel<<<grid, kG3Threads, smem, st>>>(m[0], m[1], m[2], m[3], m[4], m[5], sh, epi, flags);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(AFQMC_ERR_CUDA, std::string("tc_gemm3 launch: ") + cudaGetErrorString(e));
     return AFQMC_OK;
