@@ -164,82 +164,100 @@ __device__ __forceinline__ void digits_of(double x, int e, unsigned short (&d)[S
     d[0] = __half_as_ushort(__float2half_rn((float)(int)v));
 }
 
-// 32 rows per block.  Pass 1 finds each row's exponent, pass 2 stages 64 contracted entries at a
-// time in shared memory (coalesced along whichever index is contiguous) and writes the digits,
-// two neighbours per store.  Bound by the integer work of the digits; at 8 bytes in and 2 S out
-// per entry it costs a few percent of the products it feeds.
-template <int S>
-__global__ void __launch_bounds__(256) pack_slices_kernel(PackArgs a) {
-    __shared__ cplx tile[32][65];
-    __shared__ int64_t off[32];
-    __shared__ int emax[8][32];
-    __shared__ int rowexp[32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t r0 = (int64_t)blockIdx.x * 32, bt = blockIdx.y;   // bt = (piece, shared batch)
+// RB rows per block (8, or 32 of at most 64 entries).  Pass 1 finds each row's exponent, pass 2 takes
+// 2048 entries at a time from shared memory (filled coalesced along whichever index is contiguous,
+// by pass 1 already if the rows fit) and writes the digits, two neighbours per store.  Most calls
+// have a few hundred rows, so a block's chain of loads and digits is the time, not the bytes
+// (8 in and 2 S out per entry): 32 rows a block of any length took 83 us for 1024 complex rows of
+// 3072 (55 now), 25 for 64 x 32 rows of 128 (9), 13 for 90 real rows of 90 (4).
+constexpr int kPackT = 256;
+template <int S, int RB>
+__global__ void __launch_bounds__(kPackT) pack_slices_kernel(PackArgs a) {
+    constexpr int KB = 2048 / RB, KS = kPackT / RB;
+    __shared__ cplx tile[RB][KB + 1];
+    __shared__ int64_t off[RB];
+    __shared__ int rowexp[RB];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t r0 = (int64_t)blockIdx.x * RB, bt = blockIdx.y;   // bt = (piece, shared batch)
     uint32_t piece, sb;
     a.dbatch.divmod(blockIdx.y, piece, sb);
     const int kn = min(a.klen, a.k - (int)piece * a.klen);
-    if (threadIdx.x < 32) {
-        const int64_t r = r0 + threadIdx.x;
+    if (tid < RB) {
+        const int64_t r = r0 + tid;
         uint32_t ob, i;
         a.dn.divmod((uint32_t)r, ob, i);
-        off[threadIdx.x] = r < a.own_rows ? a.shared.at(sb) + a.own.at(ob) + i * a.si + (int64_t)piece * a.klen * a.sk : -1;
+        off[tid] = r < a.own_rows ? a.shared.at(sb) + a.own.at(ob) + i * a.si + (int64_t)piece * a.klen * a.sk : -1;
+        rowexp[tid] = 0;
     }
     __syncthreads();
+    const bool once = a.koff <= KB;
     if (a.idx_contig) {
+        const int i = tid % RB;
         int m = 0;
-        if (off[lane] >= 0)
-            for (int kk = warp; kk < kn; kk += 8) {
-                const cplx v = pack_load(a, off[lane] + kk * a.sk);
+        if (off[i] >= 0) {
+#pragma unroll 4
+            for (int kk = tid / RB; kk < kn; kk += KS) {
+                const cplx v = pack_load(a, off[i] + kk * a.sk);
                 m = max(m, max(exp_field(v.re), exp_field(v.im)));
+                if (once) tile[i][kk] = v;
             }
-        emax[warp][lane] = m;
-        __syncthreads();
-        if (warp == 0) {
-            for (int q = 1; q < 8; ++q) m = max(m, emax[q][lane]);
-            rowexp[lane] = m;
+            atomicMax(&rowexp[i], m);
         }
     } else {
-        for (int i = warp * 4; i < warp * 4 + 4; ++i) {
+        for (int i = warp; i < RB; i += kPackT / 32) {
             int m = 0;
-            if (off[i] >= 0)
+            if (off[i] >= 0) {
+#pragma unroll 4
                 for (int kk = lane; kk < kn; kk += 32) {
                     const cplx v = pack_load(a, off[i] + kk * a.sk);
                     m = max(m, max(exp_field(v.re), exp_field(v.im)));
+                    if (once) tile[i][kk] = v;
                 }
+            }
             m = __reduce_max_sync(0xffffffffu, m);
             if (lane == 0) rowexp[i] = m;
         }
     }
+    if (once) {
+        const int pad = a.koff - kn;   // a few entries
+        for (int q = tid; q < RB * pad; q += kPackT) tile[q % RB][kn + q / RB] = cplx{0.0, 0.0};
+    }
     __syncthreads();
-    if (threadIdx.x < 32) {
-        const int m = rowexp[threadIdx.x];
+    if (tid < RB) {
+        const int m = rowexp[tid];
         const int e = m == 0x7ff ? kNanExp : (m == 0 ? 0 : m - 1022);   // largest entry < 2^e
-        rowexp[threadIdx.x] = e;
-        if (off[threadIdx.x] >= 0) a.exps[bt * a.own_rows + r0 + threadIdx.x] = e;
+        rowexp[tid] = e;
+        if (off[tid] >= 0) a.exps[bt * a.own_rows + r0 + tid] = e;
     }
     const int64_t rows = a.own_rows * (a.expand ? 2 : 1);
-    for (int k0 = 0; k0 < a.koff; k0 += 64) {
+    for (int k0 = 0; k0 < a.koff; k0 += KB) {
+        const int kc = min(KB, a.koff - k0);   // even, as koff is
         __syncthreads();
-        if (a.idx_contig) {
-            for (int kk = warp; kk < 64; kk += 8) {
-                cplx v{0.0, 0.0};
-                if (off[lane] >= 0 && k0 + kk < kn) v = pack_load(a, off[lane] + (k0 + kk) * a.sk);
-                tile[lane][kk] = v;
+        if (!once) {
+            if (a.idx_contig) {
+                const int i = tid % RB;
+#pragma unroll 4
+                for (int kk = tid / RB; kk < kc; kk += KS) {
+                    cplx v{0.0, 0.0};
+                    if (off[i] >= 0 && k0 + kk < kn) v = pack_load(a, off[i] + (k0 + kk) * a.sk);
+                    tile[i][kk] = v;
+                }
+            } else {
+                for (int i = warp; i < RB; i += kPackT / 32) {
+#pragma unroll 4
+                    for (int kk = lane; kk < kc; kk += 32) {
+                        cplx v{0.0, 0.0};
+                        if (off[i] >= 0 && k0 + kk < kn) v = pack_load(a, off[i] + (k0 + kk) * a.sk);
+                        tile[i][kk] = v;
+                    }
+                }
             }
-        } else {
-            for (int q = threadIdx.x; q < 32 * 64; q += 256) {
-                const int i = q >> 6, kk = q & 63;
-                cplx v{0.0, 0.0};
-                if (off[i] >= 0 && k0 + kk < kn) v = pack_load(a, off[i] + (k0 + kk) * a.sk);
-                tile[i][kk] = v;
-            }
+            __syncthreads();
         }
-        __syncthreads();
-        const int kk = 2 * lane;
-        if (k0 + kk >= a.koff) continue;   // koff is even
+        const int half = kc / 2;
 #pragma unroll 1
-        for (int i = warp * 4; i < warp * 4 + 4; ++i) {
+        for (int q = tid; q < RB * half; q += kPackT) {
+            const int i = q / half, kk = 2 * (q - i * half);
             if (off[i] < 0) break;
             const int e = rowexp[i];
             const cplx v0 = tile[i][kk], v1 = tile[i][kk + 1];
@@ -721,7 +739,10 @@ Plan make_plan(const GemmArgs& g) {
 template <int S>
 void launch_pack(const PackArgs& a, cudaStream_t st) {
     count_launch();
-    pack_slices_kernel<S><<<dim3((unsigned)((a.own_rows + 31) / 32), (unsigned)(a.nbatch * a.pieces)), 256, 0, st>>>(a);
+    const int rb = a.koff <= 64 ? 32 : 8;
+    const dim3 grid((unsigned)((a.own_rows + rb - 1) / rb), (unsigned)(a.nbatch * a.pieces));
+    if (rb == 32) pack_slices_kernel<S, 32><<<grid, kPackT, 0, st>>>(a);
+    else pack_slices_kernel<S, 8><<<grid, kPackT, 0, st>>>(a);
 }
 
 PackArgs pack_args(const GemmOperand& X, bool is_a, int n, int k, const Plan& p, void* buf, cplx alpha) {
