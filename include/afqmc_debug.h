@@ -75,9 +75,9 @@ int afqmc_debug_inverse(const double* S, int N, int count, int variant, int with
  * the leading dimension and batch strides of C and of D (elements), 28 values; sizes their element
  * counts (A, B, C, D; D 0: none); ab = Re and Im of alpha, then of beta.  C and D are complex, read
  * and written.  form: 0 the tiled multiply-add kernel, 1 the tensor-core form (sliced operands) in
- * a workspace of ws_bytes, 2 what the step would choose, 3 one output per thread (*chose, may be
- * NULL, receives the step's choice: 0, 1, or 2 for one output per thread).  *ms
- * (may be NULL) receives the device time of a second run when reps > 0 (C and D then hold the result
+ * a workspace of ws_bytes, 2 what the step would choose, 3, 4, 5 one output by one, four or
+ * eight threads (*chose, may be NULL, receives the step's choice: 0, 1, or 2, 3, 4 for the last
+ * three).  *ms (may be NULL) receives the device time of a second run when reps > 0 (C and D then hold the result
  * of reps + 1 runs). */
 int afqmc_debug_gemm(const long long* d, const long long* sizes, const double* ab, const double* A, const double* B,
                      double* C, double* D, int form, long long ws_bytes, int reps, int* chose, float* ms);

@@ -282,7 +282,7 @@ extern "C" int afqmc_debug_wait_probe(long long limit_cycles, int release, unsig
 extern "C" int afqmc_debug_gemm(const long long* d, const long long* sizes, const double* ab, const double* A,
                                 const double* B, double* C, double* D, int form, long long ws_bytes, int reps,
                                 int* chose, float* ms) {
-    if (!d || !sizes || !ab || !A || !B || !C || form < 0 || form > 3 || ws_bytes < 0 || reps < 0)
+    if (!d || !sizes || !ab || !A || !B || !C || form < 0 || form > 5 || ws_bytes < 0 || reps < 0)
         return fail(AFQMC_ERR_BADARG, "debug_gemm: bad arguments");
     GemmArgs g;
     g.m = (int)d[0]; g.n = (int)d[1]; g.k = (int)d[2];
@@ -327,7 +327,7 @@ extern "C" int afqmc_debug_gemm(const long long* d, const long long* sizes, cons
             rc = slice_gemm(g, &ws, 0);
         } else {
             if (form == 2) g.ws = &ws;
-            zgemm_as(g, form == 2 ? zgemm_form(g, &ws) : form == 3 ? 2 : 0, 0);
+            zgemm_as(g, form == 2 ? zgemm_form(g, &ws) : form >= 3 ? form - 1 : 0, 0);
         }
         if (r == reps) cudaEventRecord(e1);
     }

@@ -16,6 +16,7 @@
 
 #include "ffc.cuh"
 #include "kernels_fp64.cuh"
+#include "kernels_tc.cuh"
 
 namespace afqmc {
 
@@ -176,49 +177,79 @@ __global__ void __launch_bounds__(kThreads) zgemm_kernel(GemmArgs g) {
     }
 }
 
-// One output per thread, for products too small to fill tiles (few electrons, few walkers): a 64 x 64
-// or 32 x 32 tile does its padding's multiply-adds too, on one SM (25 us for a 24 x 5 output and
-// K = 24), where this spreads the outputs alone over all SMs.  Neighbouring threads run along a row
-// of the output, so A is a broadcast and B coalesced for op N.
+// One output per thread, or by P neighbouring threads that share its contraction, for products too
+// small to fill tiles (few electrons, few walkers): a 64 x 64 or 32 x 32 tile does its padding's
+// multiply-adds too, on one SM (25 us for a 24 x 5 output and K = 24), where this spreads the outputs
+// alone over all SMs.  Neighbouring outputs run along a row, so A is a broadcast and B coalesced for
+// op N.  An FP64 instruction holds its scheduler's pipe for 64 cycles and its result takes 200, so
+// P > 1 takes fewer steps of the chain as long as it finds idle schedulers (zgemm_form): 9.2 us
+// with one thread for 16 x 24 x 5 outputs and K = 24, 4.0 with eight.
 constexpr int kSmallT = 64;
-template <bool AR, bool BR>
-__global__ void __launch_bounds__(kSmallT) zgemm_small_kernel(GemmArgs g) {
+template <int P>
+struct SmallSum {   // P = 1: zgemm_kernel's order of sums; P > 1: the products of a complex one apart
+    cplx a{0.0, 0.0}, b{0.0, 0.0};
+    template <class X, class Y>
+    __device__ __forceinline__ void add(const X& x, const Y& y) {
+        if constexpr (P > 1 && std::is_same<X, cplx>::value && std::is_same<Y, cplx>::value) {
+            a.re = fma(x.re, y.re, a.re);
+            b.re = fma(x.im, y.im, b.re);
+            a.im = fma(x.re, y.im, a.im);
+            b.im = fma(x.im, y.re, b.im);
+        } else {
+            mac(a, x, y);
+        }
+    }
+    __device__ __forceinline__ cplx total() const { return P > 1 ? cplx{a.re - b.re, a.im + b.im} : a; }
+};
+template <bool AR, bool BR, int P>
+__global__ void __launch_bounds__(kSmallT) zgemm_small_kernel(GemmArgs g, uint32_t outputs) {
     using TA = typename Elem<AR>::T;
     using TB = typename Elem<BR>::T;
-    const int64_t id = (int64_t)blockIdx.x * kSmallT + threadIdx.x;
-    const int c = (int)(id % g.n), r = (int)(id / g.n % g.m);
-    const int64_t b = id / ((int64_t)g.m * g.n);
-    const int64_t b2 = b % g.nb2, b1 = b / g.nb2 % g.nb1, b0 = b / g.nb2 / g.nb1;
-    if (b0 >= g.nb0) return;
-    const int64_t sa = g.A.op == OP_N ? 1 : g.A.ld, sb = g.B.op == OP_N ? g.B.ld : 1;
-    int64_t ia = b0 * g.A.s0 + b1 * g.A.s1 + b2 * g.A.s2 + (int64_t)r * (g.A.op == OP_N ? g.A.ld : 1);
-    int64_t ib = b0 * g.B.s0 + b1 * g.B.s1 + b2 * g.B.s2 + (int64_t)c * (g.B.op == OP_N ? 1 : g.B.ld);
-    cplx acc{0.0, 0.0};
+    const uint32_t id = (blockIdx.x * kSmallT + threadIdx.x) / P;
+    const int part = threadIdx.x % P;
+    const unsigned all = __ballot_sync(0xffffffffu, id < outputs);   // whole groups of P
+    if (id >= outputs) return;
+    const uint32_t n = (uint32_t)g.n, m = (uint32_t)g.m, nb1 = (uint32_t)g.nb1, nb2 = (uint32_t)g.nb2;
+    const uint32_t rc = id / n, b = rc / m, b01 = b / nb2;
+    const int c = (int)(id - rc * n), r = (int)(rc - b * m);
+    const int64_t b2 = b - b01 * nb2, b0 = b01 / nb1, b1 = b01 - b0 * nb1;
+    const int64_t sa = (g.A.op == OP_N ? 1 : g.A.ld) * (int64_t)P, sb = (g.B.op == OP_N ? g.B.ld : 1) * (int64_t)P;
+    int64_t ia = b0 * g.A.s0 + b1 * g.A.s1 + b2 * g.A.s2 + (int64_t)r * (g.A.op == OP_N ? g.A.ld : 1) + part * (sa / P);
+    int64_t ib = b0 * g.B.s0 + b1 * g.B.s1 + b2 * g.B.s2 + (int64_t)c * (g.B.op == OP_N ? 1 : g.B.ld) + part * (sb / P);
+    SmallSum<P> acc;
     const bool ca = g.A.op == OP_C, cb = g.B.op == OP_C;
-    int k = 0;
-    for (; k + 8 <= g.k; k += 8) {   // eight loads of each operand in flight
-        TA a[8];
-        TB v[8];
+    constexpr int U = P == 1 ? 8 : 4;   // loads of each operand in flight
+    int k = part;
+    for (; k + (U - 1) * P < g.k; k += U * P) {
+        TA a[U];
+        TB v[U];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < U; ++q) {
             load_elem(a[q], g.A.ptr, ia + q * sa, ca);
             load_elem(v[q], g.B.ptr, ib + q * sb, cb);
         }
 #pragma unroll
-        for (int q = 0; q < 8; ++q) mac(acc, a[q], v[q]);
-        ia += 8 * sa;
-        ib += 8 * sb;
+        for (int q = 0; q < U; ++q) acc.add(a[q], v[q]);
+        ia += U * sa;
+        ib += U * sb;
     }
-    for (; k < g.k; ++k) {
+#pragma unroll
+    for (int q = 0; q < U - 1; ++q) {   // the rest, loads in flight too
+        if (k + q * P >= g.k) break;
         TA a;
         TB v;
-        load_elem(a, g.A.ptr, ia, ca);
-        load_elem(v, g.B.ptr, ib, cb);
-        mac(acc, a, v);
-        ia += sa;
-        ib += sb;
+        load_elem(a, g.A.ptr, ia + q * sa, ca);
+        load_elem(v, g.B.ptr, ib + q * sb, cb);
+        acc.add(a, v);
     }
-    cplx v = g.alpha * acc;
+    cplx sum = acc.total();
+#pragma unroll
+    for (int o = P / 2; o > 0; o >>= 1) {
+        sum.re += __shfl_xor_sync(all, sum.re, o);
+        if (!AR || !BR) sum.im += __shfl_xor_sync(all, sum.im, o);
+    }
+    if (part != 0) return;
+    cplx v = g.alpha * sum;
     cplx* cp = g.C + b0 * g.sc0 + b1 * g.sc1 + b2 * g.sc2 + (int64_t)r * g.ldc + c;
     if (g.beta.re != 0.0 || g.beta.im != 0.0) v = v + g.beta * (*cp);
     *cp = v;
@@ -744,14 +775,40 @@ struct NumFF {
     }
 };
 
-// 1 / z with one FP64 division: z is first scaled by an exact power of two so that its larger
-// component lies in [1, 2), which keeps |z|^2 away from overflow and underflow.
+// v 2^n, by the exponent field where v and the result are normal.
+__device__ __forceinline__ double scale2(double v, int n) {
+    const int hi = __double2hiint(v), lo = __double2loint(v), e = (hi >> 20) & 0x7ff;
+    if (((hi << 1) | lo) == 0) return v;
+    if (e == 0 || e == 0x7ff || (unsigned)(e + n - 1) >= 2046u) return ldexp(v, n);
+    return __hiloint2double(hi + (n << 20), lo);
+}
+// z scaled by a power of two so that its larger component lies in [1, 2); returns the exponent taken
+// out.  z finite and not zero.
+__device__ __forceinline__ int cnormalise(cplx& z) {
+    int e = max((__double2hiint(z.re) >> 20) & 0x7ff, (__double2hiint(z.im) >> 20) & 0x7ff) - 1023;
+    if (e == -1023) {   // both subnormal
+        frexp(fmax(fabs(z.re), fabs(z.im)), &e);
+        --e;
+    }
+    z = cplx{scale2(z.re, -e), scale2(z.im, -e)};
+    return e;
+}
+// 1 / z: |z|^2 of z scaled as above, which keeps it away from overflow and underflow, and 1 / |z|^2
+// as r (1 + e + e^2), e = 1 - |z|^2 r, from the float reciprocal r (e^3 < 2^-66, so the last rounding
+// is all the error).  Six dependent FP64 operations, at 200 cycles each, where frexp, ldexp and the
+// division took some twenty.
 __device__ __forceinline__ cplx crecip(cplx z) {
-    int e = 0;
-    frexp(fmax(fabs(z.re), fabs(z.im)), &e);
-    const double xr = ldexp(z.re, 1 - e), xi = ldexp(z.im, 1 - e);
-    const double r = 1.0 / fma(xr, xr, xi * xi);
-    return cplx{ldexp(xr * r, 1 - e), ldexp(-xi * r, 1 - e)};
+    const int n = -cnormalise(z);
+    const double d = fma(z.re, z.re, z.im * z.im);   // in [1, 8)
+    const float df = __uint_as_float((unsigned)((unsigned long long)__double_as_longlong(d) >> 29) - (896u << 23));
+    const double r0 = widen(__frcp_rn(df));
+    const double e = fma(-d, r0, 1.0);
+    const double r = fma(r0, fma(e, e, e), r0);
+    return cplx{scale2(z.re * r, n), scale2(-z.im * r, n)};
+}
+// log det from the product of the pivots v (scaled, exponent ex apart)
+__device__ __forceinline__ cplx log_of_product(cplx v, int ex) {
+    return cplx{0.5 * log(fma(v.re, v.re, v.im * v.im)) + ex * M_LN2, atan2(v.im, v.re)};
 }
 
 // entry (q, u) of a tile with q (sel_q) or u (sel_u) known at run time only
@@ -828,15 +885,6 @@ template <int RQ>
 __device__ __forceinline__ void gj_panel_sync() {
     asm volatile("bar.sync 1, %0;" ::"n"(32 * RQ) : "memory");
 }
-// v scaled by a power of two so that its larger component lies in [1, 2); returns the exponent taken
-// out.  v finite and not zero.
-__device__ __forceinline__ int gj_normalise(cplx& v) {
-    int e = 0;
-    frexp(fmax(fabs(v.re), fabs(v.im)), &e);
-    v = cplx{ldexp(v.re, 1 - e), ldexp(v.im, 1 - e)};
-    return e - 1;
-}
-
 // Shared memory of a CTA: the panel being applied and the next one being published (buffers b and
 // b ^ 1), the panel's columns on their way between its owner and the warps that work on it, and for
 // each of these the best pivot and its row (two steps in turn).
@@ -1046,7 +1094,7 @@ __global__ void __launch_bounds__(kGJRegThreads<CW>, CW / 4)
         int ex = 0;
         if (k < N) {
             v = Num::to(sh.pivs[k]);
-            ex = gj_normalise(v);
+            ex = cnormalise(v);
             const int pk = sh.perm[k];
             for (int j = 0; j < k; ++j) odd ^= sh.perm[j] > pk ? 1 : 0;
         }
@@ -1055,7 +1103,7 @@ __global__ void __launch_bounds__(kGJRegThreads<CW>, CW / 4)
             v = v * cplx{__shfl_xor_sync(0xffffffffu, v.re, o), __shfl_xor_sync(0xffffffffu, v.im, o)};
             ex += __shfl_xor_sync(0xffffffffu, ex, o);
         }
-        ex += gj_normalise(v);
+        ex += cnormalise(v);
         odd = __popc(__ballot_sync(0xffffffffu, odd)) & 1;
         if (lane == 0) {
             sh.det[warp] = v;
@@ -1083,8 +1131,10 @@ __global__ void __launch_bounds__(kGJRegThreads<CW>, CW / 4)
             ex += sh.dexp[w] >> 1;
             sign += sh.dexp[w];
         }
+        ex += cnormalise(v);
         if (sign & 1) v = cplx{-v.re, -v.im};
-        if (lane == 0) logdet[mat] = cplx{log(hypot(v.re, v.im)) + ex * M_LN2, atan2(v.im, v.re)};
+        const cplx ld = log_of_product(v, ex);
+        if (lane == 0) logdet[mat] = ld;
     }
     if (C > 1) cluster_sync_all();
 }
@@ -1097,13 +1147,12 @@ __global__ void __launch_bounds__(kGJRegThreads<CW>, CW / 4)
 // not used yet, lowest row on ties); the pivot row passes through shared memory, where lane j
 // scales entry j, and every lane reads it back as broadcasts.  Each step's pivot column is always
 // register column 0: the update writes column j to j - 1 and the new column of the inverse
-// to NC - 1, which after NC steps restores the order, so the step is one loop body with static
-// register indices.  INV = false stops at the log-determinant and updates the trailing columns
+// to NC - 1, so the step is one loop body with static register indices.  INV = false stops at the log-determinant and updates the trailing columns
 // only (in groups of 8).
 // Bound by the FP64 pipe (2 multiply-adds per SM and clock: 0.22 ms for the inverses of 1024
 // matrices of N = 32), which the 512-thread shared-memory kernel missed by its four barriers
 // a step on blocks of one matrix each.  Measured, the shared-memory kernel -> this one: 1024
-// inverses of N = 32 3.79 -> 0.37 ms, N = 16 1.79 -> 0.13 ms; log-determinants alone 3.28 -> 0.26 ms.
+// inverses of N = 32 3.79 -> 0.33 ms, N = 16 1.79 -> 0.10 ms; log-determinants alone 3.28 -> 0.22 ms.
 constexpr int kGJWarpMax = 32;
 constexpr int kGJWarps = 2;   // matrices per CTA
 
@@ -1122,12 +1171,12 @@ __global__ void __launch_bounds__(32 * kGJWarps)
         a[j] = cplx{lane == j ? 1.0 : 0.0, 0.0};
         if (lane < N && j < N) a[j] = G[(int64_t)lane * N + j];
     }
-    bool used = lane >= NC;
+    bool used = lane >= N;
     int mystep = 0, myperm = 0;         // lane i: step that used row i; lane k: pivot row of step k
     cplx mypiv{1.0, 0.0};               // lane k: pivot of step k
     int bad = 0;
 #pragma unroll 1
-    for (int k = 0; k < NC; ++k) {
+    for (int k = 0; k < N; ++k) {
         // largest |re| + |im| by its bit pattern (ordered for non-negative doubles; infinities and
         // NaN come out on top)
         const unsigned long long key = used ? 0ull : (unsigned long long)__double_as_longlong(abs1(a[0]));
@@ -1182,31 +1231,32 @@ __global__ void __launch_bounds__(32 * kGJWarps)
         }
         return;
     }
-    // log|det| and arg det: sums over the pivots, plus pi for an odd pivot permutation, whose
-    // sign is that of its inversions (pairs of steps whose pivot rows are out of order)
-    double la = lane < NC ? log(hypot(mypiv.re, mypiv.im)) : 0.0;
-    double ph = lane < NC ? atan2(mypiv.im, mypiv.re) : 0.0;
+    // log|det| and arg det from the product of the pivots, times -1 for an odd pivot permutation,
+    // whose sign is that of its inversions (pairs of steps whose pivot rows are out of order)
+    cplx v = mypiv;
+    int ex = cnormalise(v);
     int odd = 0;
 #pragma unroll
     for (int j = 0; j < NC; ++j) {
         const int pj = __shfl_sync(0xffffffffu, myperm, j);
-        if (lane < NC && j < lane && pj > myperm) odd ^= 1;
+        if (lane < N && j < lane && pj > myperm) odd ^= 1;
     }
     odd = __popc(__ballot_sync(0xffffffffu, odd)) & 1;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        la += __shfl_xor_sync(0xffffffffu, la, o);
-        ph += __shfl_xor_sync(0xffffffffu, ph, o);
+    for (int o = NC > 16 ? 16 : NC / 2; o > 0; o >>= 1) {   // the first NC lanes' pivots; the others' are 1
+        v = v * cplx{__shfl_xor_sync(0xffffffffu, v.re, o), __shfl_xor_sync(0xffffffffu, v.im, o)};
+        ex += __shfl_xor_sync(0xffffffffu, ex, o);
     }
-    if (lane == 0) {
-        if (odd) ph += M_PI;
-        logdet[mat] = cplx{la, atan2(sin(ph), cos(ph))};
-    }
+    ex += cnormalise(v);
+    if (odd) v = cplx{-v.re, -v.im};
+    const cplx ld = log_of_product(v, ex);
+    if (lane == 0) logdet[mat] = ld;
     if (INV) {   // row i of the array is row mystep of the inverse; column j is its column perm[j]
 #pragma unroll
-        for (int j = 0; j < NC; ++j) {
+        for (int u = 0; u < NC; ++u) {
+            const int j = u + N < NC ? u + N : u + N - NC;   // N steps moved column j to register u
             const int c = __shfl_sync(0xffffffffu, myperm, j);
-            if (lane < N && j < N) G[(int64_t)mystep * N + c] = a[j];
+            if (lane < N && j < N) G[(int64_t)mystep * N + c] = a[u];
         }
     }
 }
@@ -1711,7 +1761,7 @@ static int zgemm_tile(const GemmArgs& g) {
 // 128, N = 5 to 32, W = 2 to 512):
 //   * 0, tiles: the padded multiply-adds at 85% of the FP64 pipe (5.2e5 a microsecond over all SMs), no less than one
 //     tile's on its SM;
-//   * 2, one output per thread: the multiply-adds alone, at 3.0e5 a microsecond, and the latency of
+//   * 2, one output per thread (3, 4: by four or eight): the multiply-adds alone, at 3.0e5 a microsecond, and the latency of
 //     its loads along K;
 //   * 1, the tensor cores (where the caller gives a workspace): slice_gemm_us, gemm_slices.cu.
 int zgemm_form(const GemmArgs& g, const SliceScratch* ws) {
@@ -1721,10 +1771,14 @@ int zgemm_form(const GemmArgs& g, const SliceScratch* ws) {
     const double tiles = nbatch * ((g.m + ts - 1) / ts) * ((g.n + ts - 1) / ts);
     const double tiled_us = 3.0 + ceil(tiles / 152.0) * ts * ts * per / 3.4e3;
     const double outputs = nbatch * g.m * g.n;
-    const double thread_us = outputs < 1e11 ? 3.0 + std::max(outputs * per / 3.0e5, 0.05 * g.k) + 0.01 * g.k : 1e30;
+    const double thread_us = outputs < 2e9 ? 3.0 + std::max(outputs * per / 3.0e5, 0.05 * g.k) + 0.01 * g.k : 1e30;
     const double slice_us = ws && ws->buf && g.k > 0 ? slice_gemm_us(g) : 1e30;
     if (slice_us < std::min(tiled_us, thread_us)) return 1;
-    return thread_us < tiled_us ? 2 : 0;
+    if (thread_us >= tiled_us) return 0;
+    // threads to an output while one each would leave schedulers without a warp: their pipes' work is
+    // the same, in more and shorter chains
+    const double room = 128.0 * tc_num_sms();
+    return outputs * 4 <= room && g.k >= 16 ? 4 : (outputs <= room && g.k >= 8 ? 3 : 2);
 }
 
 void zgemm_as(const GemmArgs& g, int form, cudaStream_t st) {
@@ -1733,12 +1787,17 @@ void zgemm_as(const GemmArgs& g, int form, cudaStream_t st) {
     if (g.ws) g.ws->a = g.ws->b = SliceScratch::Packed{};   // no slices for the next product to keep
     const int64_t nbatch = (int64_t)g.nb0 * g.nb1 * g.nb2;
     count_launch();
-    if (form == 2) {
-        const unsigned blocks = (unsigned)((nbatch * g.m * g.n + kSmallT - 1) / kSmallT);
-        if (g.A.real && g.B.real) zgemm_small_kernel<true, true><<<blocks, kSmallT, 0, st>>>(g);
-        else if (g.A.real) zgemm_small_kernel<true, false><<<blocks, kSmallT, 0, st>>>(g);
-        else if (g.B.real) zgemm_small_kernel<false, true><<<blocks, kSmallT, 0, st>>>(g);
-        else zgemm_small_kernel<false, false><<<blocks, kSmallT, 0, st>>>(g);
+    if (form >= 2) {
+        const int64_t outputs = nbatch * g.m * g.n;
+        auto go = [&](auto p1, auto p4, auto p8) {
+            const int p = form == 4 ? 8 : form == 3 ? 4 : 1;
+            const unsigned blocks = (unsigned)((outputs * p + kSmallT - 1) / kSmallT);
+            (p == 8 ? p8 : p == 4 ? p4 : p1)<<<blocks, kSmallT, 0, st>>>(g, (uint32_t)outputs);
+        };
+        if (g.A.real && g.B.real) go(zgemm_small_kernel<true, true, 1>, zgemm_small_kernel<true, true, 4>, zgemm_small_kernel<true, true, 8>);
+        else if (g.A.real) go(zgemm_small_kernel<true, false, 1>, zgemm_small_kernel<true, false, 4>, zgemm_small_kernel<true, false, 8>);
+        else if (g.B.real) go(zgemm_small_kernel<false, true, 1>, zgemm_small_kernel<false, true, 4>, zgemm_small_kernel<false, true, 8>);
+        else go(zgemm_small_kernel<false, false, 1>, zgemm_small_kernel<false, false, 4>, zgemm_small_kernel<false, false, 8>);
         return;
     }
     const int ts = zgemm_tile(g);

@@ -56,7 +56,7 @@ size_t slice_gemm_bytes(const GemmArgs& g);
 int slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st);
 
 // The product in the form expected to be fastest: zgemm_form's 0 (tiles), 1 (tensor cores, where
-// there is a workspace) or 2 (one output per thread).  zgemm_as: in the form given.
+// there is a workspace), 2 (one output per thread), 3 or 4 (by four or eight threads).  zgemm_as: in the form given.
 int zgemm_form(const GemmArgs& g, const SliceScratch* ws);
 void zgemm_as(const GemmArgs& g, int form, cudaStream_t st);
 void zgemm(const GemmArgs& g, cudaStream_t st);
