@@ -912,8 +912,9 @@ double slice_gemm_us(const GemmArgs& g) {
 int slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st) {
     const Plan p = make_plan(g);
     if (p.bytes + 1024 <= ws->bytes) return run_plan(g, p, ws, st);
-    // too large for the workspace: halve a long contraction (the output is then added up in two
-    // rounds), else the largest of the batch dimensions, n and m
+    // too large for the workspace: cut a long contraction (the output is then added up in rounds) after
+    // as many pieces as fit, in equal shares for the CTAs of a tile where that is possible; else
+    // halve the largest of the batch dimensions, n and m
     GemmArgs lo = g, hi = g;
     lo.keep_a = lo.keep_b = hi.keep_a = hi.keep_b = false;
     const int64_t big = std::max<int64_t>({g.nb0, g.nb1, g.nb2});
@@ -925,7 +926,10 @@ int slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st) {
         hi.D = g.D ? g.D + dd : nullptr;
     };
     if (p.pieces >= 8) {
-        lo.k = p.pieces / 2 * p.klen;
+        const int64_t fit = (int64_t)(ws->bytes / ((p.bytes + 1024) / p.pieces + 1));
+        const int64_t share = std::max<int64_t>(1, tc_num_sms() / std::max<int64_t>(p.tiles, 1));
+        const int64_t n = fit > share ? fit / share * share : std::max<int64_t>(1, fit);
+        lo.k = (int)std::min<int64_t>(n, p.pieces - 1) * p.klen;
         hi.k = g.k - lo.k;
         shift(lo.k * (g.A.op == OP_N ? 1 : g.A.ld), lo.k * (g.B.op == OP_N ? g.B.ld : 1), 0, 0);
         lo.D = nullptr;
