@@ -104,7 +104,7 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
     const int Nmax = std::max(wk->N[0], wk->N[1]);
     const int64_t per_u = (int64_t)W * M * Nmax;                 // complex elements per Cholesky vector
     const int nu = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)f.nc, (int64_t)nch,
-                                                                 ((int64_t)768 << 20) / (per_u * 16)}));
+                                                                 ((int64_t)256 << 20) / (per_u * 16)}));
     cplx *U = nullptr, *V = nullptr, *F = nullptr, *G = nullptr, *Z = nullptr, *gP = nullptr;
     double* dLd = nullptr;
     AFQMC_CUDA_TRY(cudaMallocAsync(&U, sizeof(cplx) * nu * per_u, st));

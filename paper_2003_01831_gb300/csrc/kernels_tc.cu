@@ -476,7 +476,7 @@ constexpr int kEBKDefault = 32;
 // n-groups and 8 Theta groups at a time.
 constexpr int kEWsSuperDefault = 8;
 constexpr int kEPitch = 129;                     // plane row pitch (floats) of the generic epilogue: conflict-free
-constexpr int kEBlock = 32 * 33;                 // one 32 x 32 block of the fixed epilogue at pitch 33
+constexpr int kEBlock = 32 * 36;                 // one 32 x 32 block of the fixed epilogue (pitch 33, or 36 for 16-byte stores)
 constexpr int kETileFloats = 16 * kEBlock;       // 16 blocks; the generic epilogue's 128 x 129 plane fits too
 static_assert(kETileFloats >= 128 * kEPitch, "epilogue exchange space");
 
@@ -685,22 +685,25 @@ __device__ __forceinline__ void pair_arrive(int id) { asm volatile("bar.arrive %
 // both orders' products with its own T from registers; a warp on the diagonal exchanges within
 // itself.  That halves the shared-memory traffic of exchanging every block, and a pair waits for
 // each other alone: a tile has one barrier of all sixteen warps (with the wait for the accumulators),
-// which also separates this tile's exchange space and sums from the last one's.  Block rows lie at
-// pitch 33: writes (lanes over rows) and reads (lanes over columns) are free of bank conflicts.
+// which also separates this tile's exchange space and sums from the last one's (none for Np = 32,
+// where no warp needs another).  Block rows lie at pitch 33: writes (lanes over rows) and reads
+// (lanes over columns) are free of bank conflicts; so are 16-byte writes at pitch 36, faster for
+// Np = 32 (0.87 -> 0.81 ms below) and slower else (3.63 -> 4.16).
 //
 // What bounds a single-product tile is shared memory: at 128 bytes a cycle the MMAs' operands and
 // the copies that bring them take all of it by themselves, and the exchange comes on top.  Kernel
 // times against a 128 x 128 plane exchanged by all, one accumulator pair and 64-bit descriptors
-// (ms; M, N, walkers): 512, 128, 128: 33.6 -> 27.9; 256, 64, 256: 5.25 -> 4.36 (all tiles three
-// products: 7.06 -> 6.74); 256, 128, 64: 5.30 -> 4.20; 128, 32, 512: 1.27 -> 1.14.  Barriers in
+// (ms; M, N, walkers): 512, 128, 128: 33.6 -> 26.2; 256, 64, 256: 5.25 -> 3.63 (all tiles three
+// products: 7.06 -> 5.79); 256, 128, 64: 5.30 -> 3.52; 128, 32, 512: 1.27 -> 0.81.  Barriers in
 // shared memory per pair and per tile instead of the sixteen-warp one, with scales fetched ahead
-// through shared memory, took longer (31.4, 5.03, 6.95, 5.11, 1.18).
+// through shared memory, took 12 to 22% longer.
 template <int Np, typename Release>
 __device__ __forceinline__ bool energy_epilogue_tile(const EnergyShape& es, SharedCtl* ctl, float* xbuf, double* ered,
                                                      int ng, int wg, int part, uint32_t parity, bool d2,
                                                      Release release) {
     constexpr int Q = Np / 32;     // blocks along an n-block
     constexpr int G = 128 / Np;    // n-blocks (rows) and walker-spins (columns) per tile
+    constexpr int P = Q == 1 ? 36 : 33;   // row pitch of a block
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int q = warp & 3, h = (warp - 2) >> 2;
     const int ib = q / Q, r = q % Q, j = h / Q, c = h % Q;
@@ -731,7 +734,11 @@ __device__ __forceinline__ bool energy_epilogue_tile(const EnergyShape& es, Shar
     const uint32_t tq = ctl->tmem_base + 256u * part + ((uint32_t)(q * 32) << 16);
 
     const bool got = warp_wait(&ctl->tfull[part], parity, &ctl->abort);
-    if (!ebar_and(got ? 1 : 0)) return false;    // all sixteen warps leave together
+    if (Q == 1) {   // no warp waits for another
+        if (!got) return false;
+    } else if (!ebar_and(got ? 1 : 0)) {
+        return false;                            // all sixteen warps leave together
+    }
     tc_fence_after();
     // T without the row scale, in registers; tensor memory is released as soon as the last load is in
     float tr[32], ti[32];
@@ -783,24 +790,32 @@ __device__ __forceinline__ bool energy_epilogue_tile(const EnergyShape& es, Shar
 
     float v0 = 0.f, v1 = 0.f, v2 = 0.f, v3 = 0.f;   // Re t, Im t, Re X, Im X of this lane
     if (diag) {
-        float* mine = own + lane * 33;
-        float sii = 0.f, sri = 0.f, srr = 0.f;
+        float* mine = own + lane * P;
+        auto put = [&](const float (&t)[32]) {
+            if (P % 4 == 0) {
 #pragma unroll
-        for (int k = 0; k < 32; ++k) mine[k] = ti[k] * sa;
+                for (int k = 0; k < 32; k += 4)
+                    *reinterpret_cast<float4*>(mine + k) = make_float4(t[k] * sa, t[k + 1] * sa, t[k + 2] * sa, t[k + 3] * sa);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 32; ++k) mine[k] = t[k] * sa;
+            }
+        };
+        float sii = 0.f, sri = 0.f, srr = 0.f;
+        put(ti);
         __syncwarp();
 #pragma unroll
         for (int k = 0; k < 32; ++k) {
-            const float p = own[k * 33 + lane];   // Ti[k][lane]
+            const float p = own[k * P + lane];   // Ti[k][lane]
             sii = fmaf(ti[k], p, sii);
             sri = fmaf(tr[k], p, sri);
         }
         v1 = mine[lane];
         __syncwarp();
-#pragma unroll
-        for (int k = 0; k < 32; ++k) mine[k] = tr[k] * sa;
+        put(tr);
         __syncwarp();
 #pragma unroll
-        for (int k = 0; k < 32; ++k) srr = fmaf(tr[k], own[k * 33 + lane], srr);
+        for (int k = 0; k < 32; ++k) srr = fmaf(tr[k], own[k * P + lane], srr);
         v0 = mine[lane];
         v2 = (srr - sii) * sa;
         v3 = 2.0f * sri * sa;
@@ -809,7 +824,7 @@ __device__ __forceinline__ bool energy_epilogue_tile(const EnergyShape& es, Shar
         float srr = 0.f, sii = 0.f, sri = 0.f, sir = 0.f;
 #pragma unroll
         for (int k = 0; k < 32; ++k) {
-            const float pr = own[k * 33 + lane], pi = own2[k * 33 + lane];   // T[k][lane] of the writer
+            const float pr = own[k * P + lane], pi = own2[k * P + lane];   // T[k][lane] of the writer
             srr = fmaf(tr[k], pr, srr);
             sii = fmaf(ti[k], pi, sii);
             sri = fmaf(tr[k], pi, sri);
@@ -820,8 +835,8 @@ __device__ __forceinline__ bool energy_epilogue_tile(const EnergyShape& es, Shar
     } else {
 #pragma unroll
         for (int k = 0; k < 32; ++k) {
-            own[lane * 33 + k] = tr[k] * sa;
-            own2[lane * 33 + k] = ti[k] * sa;
+            own[lane * P + k] = tr[k] * sa;
+            own2[lane * P + k] = ti[k] * sa;
         }
         pair_arrive(3 + pair);
     }
@@ -1266,8 +1281,8 @@ struct PairRelease {
     __device__ __forceinline__ explicit PairRelease(SharedCtl* ctl)
         : e0(mapa_shared(&ctl->tempty[0], 0)), e1(mapa_shared(&ctl->tempty[1], 0)) {}
     __device__ __forceinline__ void operator()(bool single, int part) const {
-        mbar_arrive_cluster(part == 0 ? e0 : e1);
-        if (!single) mbar_arrive_cluster(e1);
+        mbar_arrive_cluster_relaxed(part == 0 ? e0 : e1);
+        if (!single) mbar_arrive_cluster_relaxed(e1);
     }
 };
 
