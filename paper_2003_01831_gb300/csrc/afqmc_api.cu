@@ -117,6 +117,23 @@ int copy_out(void* dst, const void* src, size_t bytes, cudaStream_t st, bool* ne
     return AFQMC_OK;
 }
 
+cudaError_t call_alloc(afqmc_ham* ham, void** p, size_t bytes, cudaStream_t st) {
+    std::call_once(ham->call_pool_once, [ham] {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = ham->device;
+        uint64_t keep = kCallPoolKeep;
+        if (cudaMemPoolCreate(&ham->call_pool, &props) != cudaSuccess ||
+            cudaMemPoolSetAttribute(ham->call_pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            cudaGetLastError();
+            if (ham->call_pool) cudaMemPoolDestroy(ham->call_pool);
+            ham->call_pool = nullptr;
+        }
+    });
+    return ham->call_pool ? cudaMallocFromPoolAsync(p, bytes, ham->call_pool, st) : cudaMallocAsync(p, bytes, st);
+}
+
 int read_flags(unsigned* dflags, cudaStream_t st, unsigned* out) {
     unsigned h = 0;
     AFQMC_CUDA_TRY(cudaMemcpyAsync(&h, dflags, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
@@ -373,6 +390,7 @@ int afqmc_destroy_hamiltonian(afqmc_ham_t H) {
     cudaFree(H->Mk);
     cudaFree(H->U);
     cudaFree(H->flags);
+    if (H->call_pool) cudaMemPoolDestroy(H->call_pool);
     delete H;
     return AFQMC_OK;
 }

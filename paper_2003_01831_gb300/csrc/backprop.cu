@@ -144,12 +144,13 @@ int walker_chunks(int W, int M) {
 
 struct Scratch {
     std::vector<void*> p;
+    afqmc_ham* ham;
     cudaStream_t st;
-    explicit Scratch(cudaStream_t s) : st(s) {}
+    Scratch(afqmc_walkers* wk, cudaStream_t s) : ham(wk->ham), st(s) {}
     template <typename T>
     T* get(size_t count) {
         void* q = nullptr;
-        if (cudaMallocAsync(&q, sizeof(T) * std::max<size_t>(count, 1), st) != cudaSuccess) {
+        if (call_alloc(ham, &q, sizeof(T) * std::max<size_t>(count, 1), st) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;
         }
@@ -236,7 +237,7 @@ int bp_walker_sum_tc(afqmc_walkers* wk, const cplx* Th, const cplx* Q, int N, co
     const int64_t kc = std::min<int64_t>(8192, (K2 + 7) / 8 * 8);
     const int nbk = (int)((K2 + kc - 1) / kc);
     const int64_t na = (int64_t)nbk * 2 * M * kc, nbb = (int64_t)nbk * M * kc;
-    Scratch ts(st);
+    Scratch ts(wk, st);
     double* A64 = ts.get<double>(na);
     double* B64 = ts.get<double>(nbb);
     bf16* a3[3] = {ts.get<bf16>(na), ts.get<bf16>(na), ts.get<bf16>(na)};
@@ -281,7 +282,7 @@ int bp_rdm1(afqmc_walkers* wk, cplx* G[2], unsigned* flag, cudaStream_t st) {
     const int64_t MM = (int64_t)M * M, big = (int64_t)W * M * Nmax;
     const bool rB = !wk->ham->cplx_L;   // B and L are real unless the Hamiltonian is complex
     const double sq = sqrt(wk->tau);
-    Scratch sc(st);
+    Scratch sc(wk, st);
     cplx* Qs[2] = {sc.get<cplx>(big), sc.get<cplx>(big)};
     cplx* P0 = sc.get<cplx>(big);
     cplx* P1 = sc.get<cplx>(big);
@@ -441,7 +442,7 @@ int afqmc_bp_rdm1(afqmc_wk_t wk, double* rdm_up, double* rdm_dn, void* stream) {
                                           std::to_string(wk->bp_n) + " steps");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int64_t MM = (int64_t)wk->M * wk->M;
-    Scratch sc(st);
+    Scratch sc(wk, st);
     cplx* G = sc.get<cplx>(2 * MM);
     unsigned* flag = sc.get<unsigned>(1);
     if (!G || !flag) return fail(AFQMC_ERR_OOM, "bp_rdm1: output buffers");

@@ -936,12 +936,13 @@ namespace {
 // stream-ordered scratch of one call, freed when it goes out of scope
 struct CallScratch {
     std::vector<void*> p;
+    afqmc_ham* ham;
     cudaStream_t st;
-    explicit CallScratch(cudaStream_t s) : st(s) {}
+    CallScratch(afqmc_walkers* wk, cudaStream_t s) : ham(wk->ham), st(s) {}
     template <typename T>
     T* get(int64_t count) {
         void* q = nullptr;
-        if (cudaMallocAsync(&q, sizeof(T) * (size_t)std::max<int64_t>(count, 1), st) != cudaSuccess) {
+        if (call_alloc(ham, &q, sizeof(T) * (size_t)std::max<int64_t>(count, 1), st) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;
         }
@@ -958,7 +959,7 @@ int tc_bp_green(afqmc_walkers* wk, const double* QT, cplx* const* Phi0, cplx* co
     TcState* s = wk->tc;
     const int N = s->N, M = s->M, W = s->W, WS = 2 * W;
     const int64_t rows = (int64_t)WS * 2 * N, nT = rows * M, NN = (int64_t)N * N;
-    CallScratch sc(st);
+    CallScratch sc(wk, st);
     double* P0T = sc.get<double>(nT);
     bf16* q3[3] = {sc.get<bf16>(nT), sc.get<bf16>(nT), sc.get<bf16>(nT)};
     bf16* p3[3] = {sc.get<bf16>(nT), sc.get<bf16>(nT), sc.get<bf16>(nT)};
