@@ -77,32 +77,38 @@ __global__ void to_orbital_major_kernel(const cplx* src, int W, int M, int N, co
 // v_w[i][a], B[j][(w,a,0|1)] = (Re, Im) Q_w[j][a]; then Hr = A_re B^T and Hi = A_im B^T.  K' is
 // cut into nb chunks of kc (the three-slice GEMM's batches; the tail of the last is zero), so
 // A is [nb][2M][kc] and B [nb][M][kc], FP64 before the row split.
-__global__ void bp_pack_kernel(const cplx* Th, const cplx* Q, const cplx* weight, const cplx* tot, int W, int M,
-                               int N, int64_t kc, int nb, double* A, double* B) {
-    const int64_t total = (int64_t)nb * M * kc;
-    const int64_t K2 = 2LL * W * N;
+// (a thread forms the product of one w, a and i and writes the two contracted entries it gives; the
+// walkers' relative weights come from bp_weights_kernel: a division for every entry, twice, took 441 us
+// on the FP64 pipe for 128 walkers of 256 x 64; now 31)
+__global__ void bp_pack_kernel(const cplx* Th, const cplx* Q, const cplx* rel, int W, int M, int N, int64_t kc, int nb,
+                               double* A, double* B) {
+    const int64_t hc = kc / 2, total = (int64_t)nb * M * hc;
     for (int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; id < total; id += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t kk = id % kc;
-        const int64_t r = id / kc;
+        const int64_t hk = id % hc;
+        const int64_t r = id / hc;
         const int i = (int)(r % M);
         const int64_t b = r / M;
-        const int64_t kp = b * kc + kk;
-        double are = 0.0, aim = 0.0, bv = 0.0;
-        if (kp < K2) {
-            const int64_t K = kp >> 1;
-            const int c = (int)(kp & 1);
+        const int64_t K = b * hc + hk;
+        double2 re = make_double2(0.0, 0.0), im = re, q = re;
+        if (K < (int64_t)W * N) {
             const int w = (int)(K / N), a = (int)(K % N);
             const int64_t e = ((int64_t)w * M + i) * N + a;
-            const cplx ww = weight[w];
-            const cplx v = (ww.re == 0.0 && ww.im == 0.0) ? cplx{0.0, 0.0} : cdiv(ww, *tot) * Th[e];
-            are = c == 0 ? v.re : v.im;
-            aim = c == 0 ? v.im : -v.re;
-            bv = c == 0 ? Q[e].re : Q[e].im;
+            const cplx ww = rel[w];
+            const cplx v = (ww.re == 0.0 && ww.im == 0.0) ? cplx{0.0, 0.0} : ww * Th[e];
+            re = make_double2(v.re, v.im);
+            im = make_double2(v.im, -v.re);
+            q = make_double2(Q[e].re, Q[e].im);
         }
-        A[(b * 2 * M + i) * kc + kk] = are;
-        A[(b * 2 * M + M + i) * kc + kk] = aim;
-        B[(b * M + i) * kc + kk] = bv;
+        *reinterpret_cast<double2*>(A + (b * 2 * M + i) * kc + 2 * hk) = re;
+        *reinterpret_cast<double2*>(A + (b * 2 * M + M + i) * kc + 2 * hk) = im;
+        *reinterpret_cast<double2*>(B + (b * M + i) * kc + 2 * hk) = q;
     }
+}
+__global__ void bp_weights_kernel(const cplx* weight, const cplx* tot, int W, cplx* rel) {
+    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    if (w >= W) return;
+    const cplx ww = weight[w];
+    rel[w] = (ww.re == 0.0 && ww.im == 0.0) ? cplx{0.0, 0.0} : cdiv(ww, *tot);
 }
 
 // G[j][i] = sum_b (P_b[i][j] + i P_b[M + i][j]) over the chunk products P_b [2M][M], in chunk order
@@ -245,11 +251,14 @@ int bp_walker_sum_tc(afqmc_walkers* wk, const cplx* Th, const cplx* Q, int N, co
     float* as = ts.get<float>((int64_t)nbk * 2 * M);
     float* bs = ts.get<float>((int64_t)nbk * M);
     double* Pp = ts.get<double>((int64_t)nbk * 2 * MM);
-    if (!A64 || !B64 || !a3[0] || !a3[1] || !a3[2] || !b3[0] || !b3[1] || !b3[2] || !as || !bs || !Pp)
+    cplx* rel = ts.get<cplx>(W);
+    if (!rel || !A64 || !B64 || !a3[0] || !a3[1] || !a3[2] || !b3[0] || !b3[1] || !b3[2] || !as || !bs || !Pp)
         return fail(AFQMC_ERR_OOM, "bp_rdm1: tensor-core walker sum workspace");
     count_launch();
-    bp_pack_kernel<<<(unsigned)std::min<int64_t>(nb((int64_t)nbk * M * kc), 1 << 20), kT, 0, st>>>(
-        Th, Q, wk->weight, tot, W, M, N, kc, nbk, A64, B64);
+    bp_weights_kernel<<<nb(W), kT, 0, st>>>(wk->weight, tot, W, rel);
+    count_launch();
+    bp_pack_kernel<<<(unsigned)std::min<int64_t>(nb((int64_t)nbk * M * kc / 2), 1 << 20), kT, 0, st>>>(
+        Th, Q, rel, W, M, N, kc, nbk, A64, B64);
     split3_rows(A64, (int64_t)nbk * 2 * M, kc, a3[0], a3[1], a3[2], as, st);
     split3_rows(B64, (int64_t)nbk * M, kc, b3[0], b3[1], b3[2], bs, st);
     Split3 sa, sb;

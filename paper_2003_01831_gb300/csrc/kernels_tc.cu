@@ -1699,49 +1699,109 @@ __device__ __forceinline__ void row_scale(float ss, float& inv, float& sc) {
     sc = nrm > 0.f ? ldexpf(1.0f, e - 11) : 1.0f;
 }
 
-// Three slices of FP64 rows (same slicing as split3_rows_ff_kernel).  One warp per row: pass 1
-// finds the row's largest exponent and its sum of squares relative to it (fp32, rescaled as
-// the maximum grows, then merged across lanes), which fixes the row scale 2^(e-11) with
-// ||x||_2 < 2^e; pass 2 forms y = x 2^(11-e) as a float pair and slices it.
-__global__ void __launch_bounds__(256) split3_rows_kernel(const double* src, int64_t rows, int64_t K, __half* h,
-                                                          __half* m, __half* l, float* scale) {
-    const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (r >= rows) return;
-    const double* x = src + r * K;
-    int emax = 0;          // largest biased exponent met (0: none)
-    float ss = 0.f;        // sum of squares in units of 2^(2 (emax - 1023))
-    bool bad = false;
-    for (int64_t k = lane; k < K; k += 32) {
-        const uint32_t bh = (uint32_t)((unsigned long long)__double_as_longlong(x[k]) >> 32);
-        const int E = (int)((bh >> 20) & 0x7ffu);
-        if (E == 0x7ff) bad = true;
-        if (E == 0 || E == 0x7ff) continue;
-        if (E > emax) {
-            const int d = 2 * (emax - E);   // rescale the sum to the new maximum
-            ss = (emax == 0 || d < -126) ? 0.f : ss * __uint_as_float((uint32_t)(d + 127) << 23);
-            emax = E;
-        }
-        const int d = E - emax;             // <= 0
-        const float v = d < -60 ? 0.f : __uint_as_float(0x3f800000u | ((bh & 0xfffffu) << 3)) *
-                                            __uint_as_float((uint32_t)(d + 127) << 23);
-        ss = fmaf(v, v, ss);
-    }
-    int wmax = emax;
+// Three slices of FP64 rows (FF = false; x[0]) or of float pairs (FF; high parts x[0], low x[1]): a
+// row's sum of squares, in fp32, fixes its scale 2^(e-11) with ||x||_2 < 2^e; then y = x 2^(11-e) as a
+// float pair is sliced.  FP64 rows are squared relative to the row's largest exponent, truncated to 24 bits
+// (the 2^-10 margin of the scale covers that and the fp32 sum).  WPR warps take a row, four neighbouring
+// entries a lane at a time; the first 16 stay in registers from the sum to the slices (rows of 512
+// are then read once), so the kernel is bound by its bytes.  Against one warp for any row, an entry a
+// lane and both passes from memory: 65536 FP64 rows of 256 65 -> 54 us (34 at the copy rate), 1024 of
+// 8192 260 -> 32.
+template <bool FF, int WPR>
+__global__ void __launch_bounds__(256) split3_rows_kernel(const void* x0, const void* x1, int64_t rows, int64_t K,
+                                                          __half* h, __half* m, __half* l, float* scale) {
+    using T = typename std::conditional<FF, float, double>::type;
+    constexpr int R = 4, TR = 32 * WPR;
+    __shared__ int smax[8];
+    __shared__ float ssum[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = threadIdx.x % TR;
+    const int64_t r = (int64_t)blockIdx.x * (8 / WPR) + threadIdx.x / TR;
+    if (r >= rows) return;   // a whole row's threads (WPR = 8: the block)
+    const T* a = static_cast<const T*>(x0) + r * K;
+    const T* b = FF ? static_cast<const T*>(x1) + r * K : nullptr;
+    const bool vec = (K & 3) == 0 && ((reinterpret_cast<uintptr_t>(x0) | reinterpret_cast<uintptr_t>(x1)) & 15) == 0 &&
+                     ((reinterpret_cast<uintptr_t>(h) | reinterpret_cast<uintptr_t>(m) | reinterpret_cast<uintptr_t>(l)) & 7) == 0;
+    auto load = [&](const T* p, int64_t k, T (&v)[4]) {   // entries k .. k + 3, zeros past the row
+        if (vec && k < K) {
+            if constexpr (FF) {
+                const float4 q = *reinterpret_cast<const float4*>(p + k);
+                v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+            } else {
+                const double2 q0 = *reinterpret_cast<const double2*>(p + k), q1 = *reinterpret_cast<const double2*>(p + k + 2);
+                v[0] = q0.x; v[1] = q0.y; v[2] = q1.x; v[3] = q1.y;
+            }
+        } else {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) wmax = max(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
-    {
-        const int d = 2 * (emax - wmax);
-        ss = (emax == 0 || d < -126) ? 0.f : ss * __uint_as_float((uint32_t)(d + 127) << 23);
+            for (int q = 0; q < 4; ++q) v[q] = k + q < K ? p[k + q] : T(0);
+        }
+    };
+    const int64_t k0 = 4 * t, step = 4 * TR;
+    T va[R][4], vb[FF ? R : 1][4];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        load(a, k0 + i * step, va[i]);
+        if constexpr (FF) load(b, k0 + i * step, vb[i]);
     }
+    auto each = [&](auto f) {   // f(entries of a) over this thread's entries
+#pragma unroll
+        for (int i = 0; i < R; ++i) f(va[i]);
+        for (int64_t k = k0 + R * step; k < K; k += step) {
+            T v[4];
+            load(a, k, v);
+            f(v);
+        }
+    };
+    auto high = [](T x) { return (uint32_t)((unsigned long long)__double_as_longlong((double)x) >> 32); };
+    int wmax = 0;
+    bool bad = false;
+    if constexpr (!FF) {
+        each([&](const T (&v)[4]) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int E = (int)((high(v[q]) >> 20) & 0x7ffu);
+                wmax = max(wmax, E);
+            }
+        });
+        wmax = __reduce_max_sync(0xffffffffu, wmax);
+        if (WPR > 1) {
+            if (lane == 0) smax[warp] = wmax;
+            __syncthreads();
+#pragma unroll
+            for (int w = 0; w < WPR; ++w) wmax = max(wmax, smax[w]);
+        }
+        bad = wmax == 0x7ff;
+    }
+    float ss = 0.f;
+    each([&](const T (&v)[4]) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float y;
+            if constexpr (FF) {
+                y = v[q];
+            } else {
+                const uint32_t bh = high(v[q]);
+                const int E = (int)((bh >> 20) & 0x7ffu), d = E - wmax;   // <= 0
+                y = E == 0 || d < -60 ? 0.f : __uint_as_float(0x3f800000u | ((bh & 0xfffffu) << 3)) *
+                                                  __uint_as_float((uint32_t)(d + 127) << 23);
+            }
+            ss = fmaf(y, y, ss);
+        }
+    });
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    bad = __any_sync(0xffffffffu, bad);
-    // ||x|| < 2^(en) 2^(wmax - 1023); the 2^-10 margin covers the truncated mantissas and the
-    // fp32 sum
+    if (WPR > 1) {
+        if (lane == 0) ssum[warp] = ss;
+        __syncthreads();
+        ss = 0.f;
+#pragma unroll
+        for (int w = 0; w < WPR; ++w) ss += ssum[w];
+    }
+    // FP64: ||x|| < 2^(en) 2^(wmax - 1023)
     int kexp = 0;
-    float sc = 1.0f;
-    if (wmax > 0 && ss > 0.f) {
+    float inv = 1.0f, sc = 1.0f;
+    if constexpr (FF) {
+        row_scale(ss, inv, sc);
+    } else if (wmax > 0 && ss > 0.f) {
         int en = 0;
         frexpf(sqrtf(ss) * (1.0f + 0x1p-10f), &en);
         const int e = en + wmax - 1023;
@@ -1749,30 +1809,46 @@ __global__ void __launch_bounds__(256) split3_rows_kernel(const double* src, int
         sc = ldexpf(1.0f, e - 11);
     }
     if (bad) sc = __int_as_float(0x7fc00000);
-    if (lane == 0) scale[r] = sc;
-    const bool zero = !(wmax > 0 && ss > 0.f);
-    for (int64_t k = lane; k < K; k += 32) {
-        float yh = 0.f, yl = 0.f;
-        if (!zero) dbl_scaled_ff(x[k], kexp, yh, yl);
-        if (bad) yh = __int_as_float(0x7fc00000);
-        slice3(yh, yl, h[r * K + k], m[r * K + k], l[r * K + k]);
+    if (t == 0) scale[r] = sc;
+    const bool zero = !FF && !(wmax > 0 && ss > 0.f);
+    auto slice = [&](int64_t k, const T (&v)[4], const T (&w)[4]) {
+        if (k >= K) return;
+        __half hh[4], mm[4], ll[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float yh = 0.f, yl = 0.f;
+            if constexpr (FF) {
+                yh = v[q] * inv;
+                yl = w[q] * inv;
+            } else {
+                if (!zero) dbl_scaled_ff(v[q], kexp, yh, yl);
+                if (bad) yh = __int_as_float(0x7fc00000);
+            }
+            slice3(yh, yl, hh[q], mm[q], ll[q]);
+        }
+        const int64_t o = r * K + k;
+        if (vec) {
+            store4h(h + o, hh);
+            store4h(m + o, mm);
+            store4h(l + o, ll);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (k + q < K) {
+                    h[o + q] = hh[q];
+                    m[o + q] = mm[q];
+                    l[o + q] = ll[q];
+                }
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < R; ++i) slice(k0 + i * step, va[i], vb[FF ? i : 0]);
+    for (int64_t k = k0 + R * step; k < K; k += step) {
+        T v[4], w[4] = {};
+        load(a, k, v);
+        if constexpr (FF) load(b, k, w);
+        slice(k, v, w);
     }
-}
-
-__global__ void __launch_bounds__(256) split3_rows_ff_kernel(const float* xh, const float* xl, int64_t rows, int64_t K,
-                                                             __half* h, __half* m, __half* l, float* scale) {
-    const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (r >= rows) return;
-    const float* a = xh + r * K;
-    const float* b = xl + r * K;
-    float ss = 0.f;
-    for (int64_t k = lane; k < K; k += 32) ss = fmaf(a[k], a[k], ss);
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    float inv, sc;
-    row_scale(ss, inv, sc);
-    if (lane == 0) scale[r] = sc;
-    for (int64_t k = lane; k < K; k += 32) slice3(a[k] * inv, b[k] * inv, h[r * K + k], m[r * K + k], l[r * K + k]);
 }
 
 // Float-float helpers: exact product error and sum error (FMA-based).
@@ -2194,13 +2270,22 @@ void select_lolo_groups(const double* nrm, int nch, int G, double eta, uint8_t* 
     }
 }
 
+// A block per row where there are few of them (at most 32 an SM) and they are long.
+template <bool FF>
+static void launch_split3(const void* x0, const void* x1, int64_t rows, int64_t K, bf16* h, bf16* m, bf16* l, float* scale,
+                          cudaStream_t st) {
+    __half* p[3] = {reinterpret_cast<__half*>(h), reinterpret_cast<__half*>(m), reinterpret_cast<__half*>(l)};
+    if (K >= 512 && rows <= 32LL * tc_num_sms())
+        split3_rows_kernel<FF, 8><<<(unsigned)rows, 256, 0, st>>>(x0, x1, rows, K, p[0], p[1], p[2], scale);
+    else
+        split3_rows_kernel<FF, 1><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(x0, x1, rows, K, p[0], p[1], p[2], scale);
+}
+
 void split3_rows(const double* src, int64_t rows, int64_t K, bf16* h, bf16* m, bf16* l, float* scale,
                  cudaStream_t st) {
     if (rows <= 0) return;
     count_launch();
-    split3_rows_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(src, rows, K, reinterpret_cast<__half*>(h),
-                                                                   reinterpret_cast<__half*>(m),
-                                                                   reinterpret_cast<__half*>(l), scale);
+    launch_split3<false>(src, nullptr, rows, K, h, m, l, scale, st);
 }
 
 int tc_gemm3(const Split3& A, BatchMap amap, const Split3& B, BatchMap bmap, int64_t rows, int64_t cols, int64_t K,
@@ -2272,9 +2357,7 @@ void split3_rows_ff(const float* hi, const float* lo, int64_t rows, int64_t K, b
                     float* scale, cudaStream_t st) {
     if (rows <= 0) return;
     count_launch();
-    split3_rows_ff_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(
-        hi, lo, rows, K, reinterpret_cast<__half*>(h), reinterpret_cast<__half*>(m), reinterpret_cast<__half*>(l),
-        scale);
+    launch_split3<true>(hi, lo, rows, K, h, m, l, scale, st);
 }
 
 // The same Taylor step for M = 128 NG: lane t handles the four consecutive orbitals
