@@ -33,6 +33,8 @@
 #include <utility>
 #include <vector>
 
+#include <float.h>
+
 #include "ffc.cuh"
 #include "kernels_tc.cuh"
 #include "state.cuh"
@@ -490,110 +492,124 @@ __global__ void __launch_bounds__(kT) gram_planar_kernel(const double* PhiT, int
         }
 }
 
-// In place on G[ws]: upper Cholesky factor R (G = R^H R, real positive diagonal), then its
-// inverse, left in the upper triangle (the strict lower triangle is zeroed).  The upper
-// triangle is staged in shared memory, packed row by row, as float pairs (ffc.cuh: ~2^-44
-// relative on the fp32 pipe; the Gram matrix it factors is formed to ~1e-9), with the square
-// roots and reciprocals of the diagonal in FP64.  A non-positive or non-finite pivot sets
-// FLAG_NONFINITE and leaves the identity (the walker keeps its orbitals).
-__device__ __forceinline__ int upk(int i, int j, int N) { return i * N - (i * (i - 1)) / 2 + (j - i); }
-__device__ __forceinline__ ffc ff_from(cplx v) {
-    const float rh = (float)v.re, ih = (float)v.im;
-    return ffc{rh, (float)(v.re - (double)rh), ih, (float)(v.im - (double)ih)};
-}
-__device__ __forceinline__ cplx ff_to(const ffc& v) {
-    return cplx{(double)v.rh + (double)v.rl, (double)v.ih + (double)v.il};
-}
-__device__ __forceinline__ ffc ff_scaled(const ffc& a, float sh, float sl) {   // a s, s real
-    ffc r{0.f, 0.f, 0.f, 0.f};
-    ff_fma(r.rh, r.rl, a.rh, a.rl, sh, sl);
-    ff_fma(r.ih, r.il, a.ih, a.il, sh, sl);
-    return r;
-}
-__device__ __forceinline__ void ff_sub_conj_mul(ffc& a, const ffc& x, const ffc& y) {   // a -= conj(x) y
-    ff_fma(a.rh, a.rl, -x.rh, -x.rl, y.rh, y.rl);
-    ff_fma(a.rh, a.rl, -x.ih, -x.il, y.ih, y.il);
-    ff_fma(a.ih, a.il, -x.rh, -x.rl, y.ih, y.il);
-    ff_fma(a.ih, a.il, x.ih, x.il, y.rh, y.rl);
-}
-__device__ __forceinline__ void ff_add_mul(ffc& a, const ffc& x, const ffc& y) {   // a += x y
-    ff_fma(a.rh, a.rl, x.rh, x.rl, y.rh, y.rl);
-    ff_fma(a.rh, a.rl, -x.ih, -x.il, y.ih, y.il);
-    ff_fma(a.ih, a.il, x.rh, x.rl, y.ih, y.il);
-    ff_fma(a.ih, a.il, x.ih, x.il, y.rh, y.rl);
+// 1 / sqrt(d) for a float pair d > 0: one step y (1 + e / 2 + 3 e^2 / 8), e = 1 - d y^2, from the
+// single-precision value, e and the product as float pairs (2^-22 -> 2^-48).
+__device__ __forceinline__ void ff_rsqrt(float dh, float dl, float& rh, float& rl) {
+    const float y = rsqrtf(dh);
+    const float p = y * y, pe = fmaf(y, y, -p);
+    const float q = dh * p, qe = fmaf(dh, p, -q);
+    const float low = fmaf(dh, pe, fmaf(dl, p, qe));
+    const float eh = (1.0f - q) - low, el = ((1.0f - q) - eh) - low;
+    const float fh = 0.5f * eh, fl = fmaf(0.375f * eh, eh, 0.5f * el);
+    const float c = y * fh, ce = fmaf(y, fl, fmaf(y, fh, -c));
+    float s, t;
+    two_sum(y, c, s, t);
+    t += ce;
+    rh = s + t;
+    rl = t - (rh - s);
 }
 
-__global__ void __launch_bounds__(kT) chol_inv_kernel(cplx* G, int N, const cplx* weight, unsigned* flags) {
+// In place on G[ws]: the inverse X of the upper Cholesky factor R (G = R^H R, real positive
+// diagonal), in the upper triangle (the strict lower triangle is zeroed), for N <= 32 NQ.  The upper
+// triangle sits in shared memory, packed column by column, as float pairs (ffc.cuh: ~2^-44
+// relative on the fp32 pipe; the Gram matrix it factors is formed to ~1e-9).  Step k finishes row k of
+// R and column k of X and updates everything to the right of column k once: rows j > k are the
+// trailing triangle, G_ji -= conj(R_kj) R_ki; rows j <= k, whose rows of R are done with, hold the sums
+// X's columns come from, X_ji -= X_jk R_ki.  A warp takes every nwarp-th column, a lane the rows
+// lane + 32 q, whose factors (X_jk or conj(R_kj)) it keeps in registers over the step.
+// A non-positive or non-finite pivot sets FLAG_NONFINITE and leaves the identity (the walker keeps
+// its orbitals).  Bound by the fp32 pipe's N^3 / 3 complex updates and two barriers a step; the
+// factorisation followed by the inverse column by column, a dependent sum of up to N terms a thread,
+// and an FP64 square root and division a step, took 24.4 ms for 2048 matrices of N = 128 (6.1 now),
+// 0.83 for 512 of N = 64 (0.25) and 0.59 for 1024 of N = 32 (0.09).
+template <int NQ>
+constexpr int kCholT = NQ == 1 ? 128 : 128 * NQ;
+template <int NQ>
+__global__ void __launch_bounds__(kCholT<NQ>) chol_inv_kernel(cplx* G, int N, const cplx* weight, unsigned* flags) {
     extern __shared__ __align__(16) unsigned char qsm[];
-    ffc* U = reinterpret_cast<ffc*>(qsm);          // packed upper triangle, N (N+1) / 2
-    __shared__ int s_bad;
-    const int ws = blockIdx.x, t = threadIdx.x;
+    struct __align__(16) Pair {   // (re, im) high parts and low parts
+        f32x2 h, l;
+    };
+    Pair* U = reinterpret_cast<Pair*>(qsm);        // column i: rows 0 .. i from i (i + 1) / 2
+    __shared__ Pair rrow[32 * NQ];                 // R_ki, i > k
+    __shared__ float4 vec[32 * NQ];                // X_jk (j <= k), conj(R_kj) (j > k): rh, rl, ih, il
+    constexpr int T = kCholT<NQ>;
+    const int ws = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     cplx* Gw = G + (int64_t)ws * N * N;
     const bool dead = weight[ws / 2].re == 0.0 && weight[ws / 2].im == 0.0;
-    const int NP = N * (N + 1) / 2;
-    if (t == 0) s_bad = 0;
-    for (int i = 0; i < N; ++i)
-        for (int j = i + t; j < N; j += kT)
-            U[upk(i, j, N)] = ff_from(dead ? cplx{i == j ? 1.0 : 0.0, 0.0} : Gw[(int64_t)i * N + j]);
+    auto at = [](int j, int i) { return i * (i + 1) / 2 + j; };
+    for (int j = warp; j < N; j += T / 32)
+        for (int i = j + lane; i < N; i += 32) {
+            const cplx g = dead ? cplx{i == j ? 1.0 : 0.0, 0.0} : Gw[(int64_t)j * N + i];
+            ffc v;
+            ff_split(g.re, v.rh, v.rl);
+            ff_split(g.im, v.ih, v.il);
+            U[at(j, i)] = Pair{f2(v.rh, v.ih), f2(v.rl, v.il)};
+        }
     __syncthreads();
-    if (!dead) {
-        // right-looking Cholesky: row k of R, then the trailing upper triangle
-        for (int k = 0; k < N; ++k) {
-            const double d2 = (double)U[upk(k, k, N)].rh + (double)U[upk(k, k, N)].rl;
-            if (!(d2 > 0.0) || !isfinite(d2)) {
-                if (t == 0) s_bad = 1;
-                break;
+    bool bad = false;
+    for (int k = 0; k < N && !dead; ++k) {
+        const Pair d = U[at(k, k)];
+        const float dh = f2_lo(d.h), dl = f2_lo(d.l);
+        if (!(dh > 0.f) || !(dh <= FLT_MAX)) { bad = true; break; }   // the same in every thread
+        float ih, il;
+        ff_rsqrt(dh, dl, ih, il);
+        const f32x2 sh = f2(ih, ih), nsh = f2(-ih, -ih), sl = f2(il, il);
+        if (t < N) {
+            Pair x{0ull, 0ull};
+            const int e = t > k ? at(k, t) : at(t, k);
+            const Pair u = U[e];
+            if (t == k) x.h = f2(ih, 0.f), x.l = f2(il, 0.f);
+            else ff_fma2(x.h, x.l, sh, nsh, sl, u.h, u.l);
+            const float im = t > k ? -1.f : 1.f;
+            vec[t] = make_float4(f2_lo(x.h), f2_lo(x.l), im * f2_hi(x.h), im * f2_hi(x.l));
+            if (t > k) {
+                rrow[t] = x;
+                U[e] = Pair{0ull, 0ull};   // the sum of X_kt starts
+            } else if (t < k) {
+                U[e] = x;
             }
-            const double d = sqrt(d2), id = 1.0 / d;
-            const float idh = (float)id, idl = (float)(id - (double)idh);
-            __syncthreads();
-            for (int j = k + t; j < N; j += kT) {
-                const int e = upk(k, j, N);
-                U[e] = j == k ? ff_from(cplx{d, 0.0}) : ff_scaled(U[e], idh, idl);
-            }
-            __syncthreads();
-            const int nr = N - k - 1;
-            for (int e = t; e < nr * nr; e += kT) {   // trailing upper triangle k < i <= j
-                const int ii = k + 1 + e / nr, jj = k + 1 + e % nr;
-                if (jj < ii) continue;
-                ff_sub_conj_mul(U[upk(ii, jj, N)], U[upk(k, ii, N)], U[upk(k, jj, N)]);
-            }
-            __syncthreads();
         }
         __syncthreads();
-        if (!s_bad) {
-            // inverse of the upper triangular R, in place, column by column:
-            // X[j][j] = 1 / R[j][j]; X[i][j] = -(sum_{p=i..j-1} X[i][p] R[p][j]) / R[j][j]
-            // (N <= kT: thread i owns row i of column j)
-            for (int j = 0; j < N; ++j) {
-                const double ir = 1.0 / ((double)U[upk(j, j, N)].rh + (double)U[upk(j, j, N)].rl);
-                const float irh = (float)ir, irl = (float)(ir - (double)irh);
-                // row i < j reads X[i][p] (p < j, final) and R[p][j] (column j, still R): the new
-                // column is written only after every row has read it
-                ffc val{0.f, 0.f, 0.f, 0.f};
-                if (t < j) {
-                    ffc acc{0.f, 0.f, 0.f, 0.f};
-                    for (int p = t; p < j; ++p) ff_add_mul(acc, U[upk(t, p, N)], U[upk(p, j, N)]);
-                    val = ff_scaled(acc, -irh, -irl);
-                }
-                __syncthreads();
-                if (t < j) U[upk(t, j, N)] = val;
-                if (t == 0) U[upk(j, j, N)] = ff_from(cplx{ir, 0.0});
-                __syncthreads();
+        if (t == 0) U[at(k, k)] = Pair{f2(ih, 0.f), f2(il, 0.f)};   // not read in this step
+        f32x2 vr[NQ], nvr[NQ], vrl[NQ], vi[NQ], nvi[NQ], vil[NQ];     // -v.re, v.re; (v.im, -v.im), its negative
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const int j = lane + 32 * q;
+            const float4 v = j < N ? (j == k ? make_float4(ih, il, 0.f, 0.f) : vec[j]) : make_float4(0.f, 0.f, 0.f, 0.f);
+            vr[q] = f2(-v.x, -v.x);
+            nvr[q] = f2(v.x, v.x);
+            vrl[q] = f2(-v.y, -v.y);
+            vi[q] = f2(v.z, -v.z);
+            nvi[q] = f2(-v.z, v.z);
+            vil[q] = f2(v.w, -v.w);
+        }
+        for (int i = k + 1 + warp; i < N; i += T / 32) {
+            const Pair r = rrow[i];
+            const f32x2 sw_h = f2(f2_hi(r.h), f2_lo(r.h)), sw_l = f2(f2_hi(r.l), f2_lo(r.l));
+            Pair* col = U + at(0, i);
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                const int j = lane + 32 * q;
+                if (32 * q > i) break;
+                if (j > i) continue;
+                Pair u = col[j];
+                ff_fma2(u.h, u.l, vr[q], nvr[q], vrl[q], r.h, r.l);        // -v.re (r.re, r.im)
+                ff_fma2(u.h, u.l, vi[q], nvi[q], vil[q], sw_h, sw_l);      // (v.im r.im, -v.im r.re)
+                col[j] = u;
             }
         }
-    }
-    __syncthreads();
-    if (s_bad) {
-        if (t == 0) atomicOr(flags, FLAG_NONFINITE);
-        for (int e = t; e < NP; e += kT) U[e] = ffc{0.f, 0.f, 0.f, 0.f};
-        __syncthreads();
-        for (int i = t; i < N; i += kT) U[upk(i, i, N)] = ffc{1.f, 0.f, 0.f, 0.f};
         __syncthreads();
     }
-    for (int e = t; e < N * N; e += kT) {
-        const int i = e / N, j = e % N;
-        Gw[e] = i <= j ? ff_to(U[upk(i, j, N)]) : cplx{0.0, 0.0};
+    if (bad && t == 0) atomicOr(flags, FLAG_NONFINITE);
+    for (int e = t; e < N * N; e += T) {
+        const int j = e / N, i = e % N;
+        cplx g{i == j && bad ? 1.0 : 0.0, 0.0};
+        if (j <= i && !bad) {
+            const Pair u = U[at(j, i)];
+            g = cplx{widen(f2_lo(u.h)) + widen(f2_lo(u.l)), widen(f2_hi(u.h)) + widen(f2_hi(u.l))};
+        }
+        Gw[e] = g;
     }
 }
 
@@ -1292,7 +1308,7 @@ int tc_debug_terms(afqmc_walkers* wk, double* ST, double* Sinv, double* ThetaT, 
 int tc_qr(afqmc_walkers* wk, cudaStream_t st) {
     TcState* s = wk->tc;
     const int N = s->N, M = s->M, WS = 2 * s->W;
-    if (N > kT) return fail(AFQMC_ERR_UNSUPPORTED, "tc_qr: N above the Cholesky kernel's row limit");
+    if (N > 128) return fail(AFQMC_ERR_UNSUPPORTED, "tc_qr: N above the Cholesky kernel's row limit");
     const int nt = (N + kQT - 1) / kQT;
     const int nxt = s->cur ^ 1;
     const int64_t N2 = 2LL * N;
@@ -1318,9 +1334,14 @@ int tc_qr(afqmc_walkers* wk, cudaStream_t st) {
     }
     // Cholesky factor and its inverse X = R^-1 in place of the Gram matrices (dead walkers: X = I)
     const size_t sm = (size_t)N * (N + 1) / 2 * sizeof(cplx);
-    raise_dyn_smem(chol_inv_kernel, sm);
     count_launch();
-    chol_inv_kernel<<<WS, kT, sm, st>>>(s->S, N, wk->weight, wk->flags);
+    auto chol = [&](auto kernel, int threads) {
+        raise_dyn_smem(kernel, sm);
+        kernel<<<WS, threads, sm, st>>>(s->S, N, wk->weight, wk->flags);
+    };
+    if (N <= 32) chol(chol_inv_kernel<1>, kCholT<1>);
+    else if (N <= 64) chol(chol_inv_kernel<2>, kCholT<2>);
+    else chol(chol_inv_kernel<4>, kCholT<4>);
     // Q^T = (Phi X)^T into the proposal buffer, then back over the current walkers
     if (tc) {
         count_launch();
