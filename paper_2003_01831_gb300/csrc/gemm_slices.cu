@@ -46,7 +46,7 @@ namespace {
 constexpr int kRows = 128;      // tile rows (operand R)
 constexpr int kCols = 64;       // tile columns (operand Q): D accumulators of 64 fill tensor memory
 constexpr int kChunk = 32;      // contracted entries per stage (64-byte swizzle)
-constexpr int kStages = 2;
+constexpr int kMaxStages = 3;
 constexpr int kEpiWarps = 16;   // four per tensor-memory lane quadrant, 16 columns each
 constexpr int kThreadsG = 64 + 32 * kEpiWarps;
 constexpr int kNanExp = 1 << 20;   // exponent of a row with a NaN or an infinity
@@ -61,7 +61,26 @@ struct Digits {
     static constexpr int kFrac = kTail - BETA;         // fraction bits of the last digit
     // fixed-point value v = x 2^(kPoint - e): BETA - 1 bits above the first digit's unit
     static constexpr int kPoint = BETA - 1 + BETA * (S - 1) + kFrac;
-    static constexpr int kStageBytes = S * (kRows + kCols) * kChunk * 2;
+};
+// A stage of one CTA: the R rows of its tile and the Q rows, or half of them for a CTA pair.
+template <int S, bool PAIR>
+struct Stage {
+    static constexpr int kQRows = PAIR ? kCols / 2 : kCols;
+    static constexpr int kBytes = S * (kRows + kQRows) * kChunk * 2;
+    static constexpr int kCount = 216 * 1024 / kBytes < kMaxStages ? 216 * 1024 / kBytes : kMaxStages;
+    static_assert(kCount >= 2, "stage ring");
+};
+// Place in the ring of stages and the parity of its turn.
+template <int N>
+struct Ring {
+    int st = 0;
+    uint32_t phase = 0;
+    __device__ __forceinline__ void next() {
+        if (++st == N) {
+            st = 0;
+            phase ^= 1u;
+        }
+    }
 };
 
 // Division of 0 <= x < 2^31 by a fixed divisor d: x / d = (x mul) >> (32 + shift) with mul =
@@ -318,7 +337,7 @@ struct OutArgs {
 };
 
 struct Ctl {
-    uint64_t full[kStages], empty[kStages], tfull, tempty, done;
+    uint64_t full[kMaxStages], empty[kMaxStages], tfull, tempty, done;
     uint32_t tmem_base;
     int abort;
 };
@@ -434,98 +453,129 @@ __device__ __forceinline__ void store_pair(const OutArgs& o, const RowOut& r, co
 }
 
 // One persistent CTA per SM: warp 0 loads stages of all slices of both operands (one TMA copy
-// each), warp 1 issues the S (S + 1) / 2 MMAs (M = 128, N = 64) of every 16 contracted entries, the
+// each), warp 1 issues the S (S + 1) / 2 MMAs (N = 64) of every 16 contracted entries, the
 // other sixteen warps turn the accumulators into FP64.  An N of 64 leaves the tensor core waiting
-// for shared memory a third of the time (6 KB of operands per 32 cycles of products); a wider tile
-// has no room for its accumulators.  For the same reason the accumulators have one buffer: the
-// epilogue first folds each output's accumulators into a 64-bit integer in registers, releases
-// tensor memory, and rounds and stores while the next tile's products run.  MULTI: the contracted
-// index in several pieces, whose rounded results are added in registers.
+// for shared memory (47 cycles an MMA of 128 rows, 32 of them its products); a wider tile
+// has no room for its accumulators.  PAIR: two CTAs take two neighbouring row tiles with one MMA of
+// M = 256, each with half of the Q rows in its shared memory, which are then read and copied once
+// for both, in stages that leave room for a third.  For lack of tensor memory the accumulators
+// have one buffer: the epilogue first folds each output's accumulators into a 64-bit integer in
+// registers, releases tensor memory, and rounds and stores while the next tile's products run.
+// MULTI: the contracted index in several pieces, whose rounded results are added in registers.
 // Measured (T_n = Ltilde_n Theta of M = 128, N = 32, 64 vectors x 512 walkers): 14.3 ms by
-// the multiply-add tiles, 0.56 ms here (31 TFLOP/s): about 65 cycles an MMA, 32 of them its
-// products (80 before A stayed in the collector and one elected lane issued from uniform registers),
-// and 3400 cycles a tile to empty tensor memory.
-template <int S, bool MULTI>
+// the multiply-add tiles, 0.54 ms here without pairs (80 cycles an MMA before A stayed in the
+// collector and one elected lane issued from uniform registers), 0.48 ms with them; of a tile's
+// 17600 cycles without pairs 10500 issued MMAs, 2750 waited for copies and 3200 for the
+// accumulators to be read.  Copies of 128-byte rows (two slices side by side) and more, shorter stages
+// gained nothing (0.55, 0.68 ms).
+template <int S, bool MULTI, bool PAIR>
 __global__ void __launch_bounds__(kThreadsG, 1)
     slice_gemm_kernel(const __grid_constant__ CUtensorMap tR, const __grid_constant__ CUtensorMap tQ, OutArgs o,
                       unsigned* flags) {
     using P = Digits<S>;
+    using St = Stage<S, PAIR>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sbase = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    Ctl* ctl = reinterpret_cast<Ctl*>(sbase + kStages * P::kStageBytes);
+    Ctl* ctl = reinterpret_cast<Ctl*>(sbase + St::kCount * St::kBytes);
     // output offsets (C, D) and exponents of the tile's columns, for two pieces in turn
     int64_t* coff2 = reinterpret_cast<int64_t*>(ctl + 1);
     int64_t* cdof2 = coff2 + 2 * kCols;
     int* cexp2 = reinterpret_cast<int*>(cdof2 + 2 * kCols);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = PAIR ? cluster_ctarank() : 0;
+    const uint32_t first = PAIR ? cluster_id_x() : blockIdx.x, stride = PAIR ? ncluster_x() : gridDim.x;
     if (warp == 0 && lane == 0) {
         tma_prefetch_desc(&tR);
         tma_prefetch_desc(&tQ);
     }
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kStages; ++i) {
+        for (int i = 0; i < St::kCount; ++i) {
             mbar_init(&ctl->full[i], 1);
             mbar_init(&ctl->empty[i], 1);
         }
         mbar_init(&ctl->tfull, 1);
-        mbar_init(&ctl->tempty, kEpiWarps);
+        mbar_init(&ctl->tempty, (PAIR ? 2 : 1) * kEpiWarps);
         mbar_init(&ctl->done, 1);
         ctl->abort = 0;
         fence_mbar_init();
     }
+    if (PAIR) {
+        __syncthreads();
+        cluster_sync();   // both CTAs' barriers exist before any copy or arrival reaches them
+    }
     if (warp == 1) {
-        tmem_alloc(&ctl->tmem_base, 512);
-        tmem_relinquish();
+        if (PAIR) {
+            tmem_alloc_pair(&ctl->tmem_base, 512);
+            tmem_relinquish_pair();
+        } else {
+            tmem_alloc(&ctl->tmem_base, 512);
+            tmem_relinquish();
+        }
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (PAIR) cluster_sync();   // tensor memory allocated in both CTAs before the first MMA
     const uint32_t work = (uint32_t)(MULTI ? o.tiles * o.groups : o.tiles);
     if (warp == 0) {
         if (lane == 0) {
             int64_t g = 0;
+            Ring<St::kCount> ring;
             bool ok = true;
-            for (uint32_t w = blockIdx.x; w < work && ok; w += gridDim.x) {
+            for (uint32_t w = first; w < work && ok; w += stride) {
                 uint32_t grp, t, b, ct, rt;
                 o.dtiles.divmod(w, grp, t);
                 o.tile(t, b, ct, rt);
                 const int p0 = MULTI ? (int)grp * o.pg : 0, p1 = MULTI ? min(o.pieces, p0 + o.pg) : 1;
                 for (int pc = p0; pc < p1 && ok; ++pc)
-                    for (int kb = 0; kb < o.nk; ++kb, ++g) {
-                        const int st = (int)(g % kStages);
-                        if (!mbar_wait(&ctl->empty[st], (uint32_t)((g / kStages) & 1) ^ 1u, &ctl->abort)) { ok = false; break; }
-                        uint8_t* s = sbase + (size_t)st * P::kStageBytes;
-                        mbar_arrive_expect_tx(&ctl->full[st], P::kStageBytes);
-                        const int z = (int)(pc * o.nbatch + b);
-                        tma_load_4d(s, &tR, &ctl->full[st], kb * kChunk, (int)rt * kRows, z, 0);
-                        tma_load_4d(s + S * kRows * kChunk * 2, &tQ, &ctl->full[st], kb * kChunk, (int)ct * kCols, z, 0);
+                    for (int kb = 0; kb < o.nk; ++kb, ++g, ring.next()) {
+                        const int st = ring.st;
+                        if (!mbar_wait(&ctl->empty[st], ring.phase ^ 1u, &ctl->abort)) { ok = false; break; }
+                        uint8_t *s = sbase + (size_t)st * St::kBytes, *sq = s + S * kRows * kChunk * 2;
+                        const int z = (int)(pc * o.nbatch + b), x = kb * kChunk;
+                        if (PAIR) {   // rank 0's barrier counts both CTAs' bytes
+                            if (rank == 0) mbar_arrive_expect_tx(&ctl->full[st], 2 * St::kBytes);
+                            const uint32_t fb = mapa_shared(&ctl->full[st], 0);
+                            tma_load_4d_pair(s, &tR, fb, x, (int)(2 * rt + rank) * kRows, z, 0);
+                            tma_load_4d_pair(sq, &tQ, fb, x, (int)ct * kCols + (int)rank * St::kQRows, z, 0);
+                        } else {
+                            mbar_arrive_expect_tx(&ctl->full[st], St::kBytes);
+                            tma_load_4d(s, &tR, &ctl->full[st], x, (int)rt * kRows, z, 0);
+                            tma_load_4d(sq, &tQ, &ctl->full[st], x, (int)ct * kCols, z, 0);
+                        }
                     }
             }
-            if (!ok)
-                for (int64_t j = g > kStages ? g - kStages : 0; j < g; ++j)
-                    wait_drain(&ctl->full[j % kStages], (uint32_t)((j / kStages) & 1));
+            if (!ok && rank == 0)
+                for (int64_t j = g > St::kCount ? g - St::kCount : 0; j < g; ++j)
+                    wait_drain(&ctl->full[j % St::kCount], (uint32_t)((j / St::kCount) & 1));
+            if (!ok && rank != 0) {   // the peer cannot wait on rank 0's barriers: its copies get time to land
+                const long long t0 = clock64();
+                while (clock64() - t0 < (1LL << 22)) {
+                }
+            }
         }
     } else if (warp == 1) {
+      if (rank == 0) {
         // the whole warp runs the loop, one elected lane issues: the MMAs follow each other as fast as
         // the tensor core takes them only while their descriptors stay in uniform registers
-        constexpr uint32_t idesc = idesc_bf16(kRows, kCols, true);
+        constexpr uint32_t idesc = idesc_bf16(PAIR ? 2 * kRows : kRows, kCols, true);
         const uint32_t tmem = ctl->tmem_base;
         const uint64_t d0 = desc_sw64(smem_u32(sbase));
         const uint32_t lo0 = (uint32_t)d0, hi0 = (uint32_t)(d0 >> 32);
-        int64_t g = 0;
+        Ring<St::kCount> ring;
         int it = 0;
         bool ok = true;
-        for (uint32_t w = blockIdx.x; w < work && ok; w += gridDim.x) {
+        for (uint32_t w = first; w < work && ok; w += stride) {
             const int p0 = MULTI ? (int)o.dtiles.div(w) * o.pg : 0, p1 = MULTI ? min(o.pieces, p0 + o.pg) : 1;
             for (int pc = p0; pc < p1 && ok; ++pc, ++it) {
                 if (!warp_wait(&ctl->tempty, ((uint32_t)it & 1u) ^ 1u, &ctl->abort)) { ok = false; break; }
                 tc_fence_after();
-                for (int kb = 0; kb < o.nk; ++kb, ++g) {
-                    const int st = (int)(g % kStages);
-                    if (!warp_wait(&ctl->full[st], (uint32_t)((g / kStages) & 1), &ctl->abort)) { ok = false; break; }
+                for (int kb = 0; kb < o.nk; ++kb, ring.next()) {
+                    const int st = ring.st;
+                    if (!warp_wait(&ctl->full[st], ring.phase, &ctl->abort)) { ok = false; break; }
                     tc_fence_after();
                     if (elect_one()) {
-                        const uint32_t sr = lo0 + st * (P::kStageBytes >> 4);
+                        const uint32_t sr = lo0 + st * (St::kBytes >> 4);
                         const uint32_t sq = sr + (S * kRows * kChunk * 2 >> 4);
 #pragma unroll
                         for (int kk = 0; kk < kChunk / 16; ++kk)
@@ -534,27 +584,33 @@ __global__ void __launch_bounds__(kThreadsG, 1)
 #pragma unroll
                                 for (int d = p; d < P::D; ++d) {
                                     const uint32_t D = tmem + d * kCols, a = sr + ((p * kRows * kChunk * 2 + kk * 32) >> 4),
-                                                   b = sq + (((d - p) * kCols * kChunk * 2 + kk * 32) >> 4),
+                                                   b = sq + (((d - p) * St::kQRows * kChunk * 2 + kk * 32) >> 4),
                                                    acc = (kk | p) != 0 ? 1u : (kb != 0 ? 1u : 0u);
-                                    if (p == S - 1) mma_f16_lo<kKeepNone>(D, a, b, hi0, idesc, acc);
-                                    else if (d == p) mma_f16_lo<kKeepFirst>(D, a, b, hi0, idesc, acc);
-                                    else if (d < P::D - 1) mma_f16_lo<kKeepMore>(D, a, b, hi0, idesc, acc);
-                                    else mma_f16_lo<kKeepLast>(D, a, b, hi0, idesc, acc);
+                                    if (p == S - 1) mma_f16_lo<kKeepNone, PAIR>(D, a, b, hi0, idesc, acc);
+                                    else if (d == p) mma_f16_lo<kKeepFirst, PAIR>(D, a, b, hi0, idesc, acc);
+                                    else if (d < P::D - 1) mma_f16_lo<kKeepMore, PAIR>(D, a, b, hi0, idesc, acc);
+                                    else mma_f16_lo<kKeepLast, PAIR>(D, a, b, hi0, idesc, acc);
                                 }
-                        mma_commit(&ctl->empty[st]);
+                        if (PAIR) mma_commit_pair(&ctl->empty[st], 3);   // free in both CTAs
+                        else mma_commit(&ctl->empty[st]);
                     }
                     __syncwarp();
                 }
                 if (!ok) break;
-                if (elect_one()) mma_commit(&ctl->tfull);
+                if (elect_one()) {
+                    if (PAIR) mma_commit_pair(&ctl->tfull, 3);
+                    else mma_commit(&ctl->tfull);
+                }
                 __syncwarp();
             }
         }
         if (elect_one()) {
-            mma_commit(&ctl->done);
+            if (PAIR) mma_commit_pair(&ctl->done, 1);
+            else mma_commit(&ctl->done);
             wait_drain(&ctl->done, 0);
         }
         __syncwarp();
+      }
     } else {
         const int q = warp & 3, h = (warp - 2) >> 2;   // lane quadrant, columns [16 h, 16 h + 16)
         const int et = threadIdx.x - 64;
@@ -563,12 +619,12 @@ __global__ void __launch_bounds__(kThreadsG, 1)
         constexpr int kShift = -2 * (P::BETA - 1) - Gather<S>::kPoint;
         int it = 0;
         bool ok = true;
-        for (uint32_t w = blockIdx.x; w < work && ok; w += gridDim.x) {
+        for (uint32_t w = first; w < work && ok; w += stride) {
             uint32_t grp, t, b, ct, rt, ob, i;
             o.dtiles.divmod(w, grp, t);
             o.tile(t, b, ct, rt);
             const int p0 = MULTI ? (int)grp * o.pg : 0, p1 = MULTI ? min(o.pieces, p0 + o.pg) : 1;
-            const int64_t r = (int64_t)rt * kRows + q * 32 + lane;
+            const int64_t r = (int64_t)(PAIR ? 2 * rt + rank : rt) * kRows + q * 32 + lane;
             const uint32_t ri = (uint32_t)r >> rx;
             RowOut ro;
             ro.ok = r < o.rows;
@@ -611,7 +667,10 @@ __global__ void __launch_bounds__(kThreadsG, 1)
                 auto release = [&]() {   // every accumulator of this warp is in registers
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&ctl->tempty);
+                    if (lane == 0) {
+                        if (PAIR) mbar_arrive_cluster_relaxed(mapa_shared(&ctl->tempty, 0));
+                        else mbar_arrive(&ctl->tempty);
+                    }
                 };
                 if (MULTI) {
 #pragma unroll
@@ -651,9 +710,11 @@ __global__ void __launch_bounds__(kThreadsG, 1)
     }
     tc_fence_before();
     __syncthreads();
+    if (PAIR) cluster_sync();   // both CTAs are done with tensor memory and each other's shared memory
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(ctl->tmem_base, 512);
+        if (PAIR) tmem_dealloc_pair(ctl->tmem_base, 512);
+        else tmem_dealloc(ctl->tmem_base, 512);
     }
     if (threadIdx.x == 0 && ctl->abort) atomicOr(flags, FLAG_TIMEOUT);
 }
@@ -670,7 +731,8 @@ struct Plan {
     int parts = 1, koff = 0, klen = 0, pieces = 1, S = 7;
     bool exp_a = false, exp_b = false, swap = false;   // swap: A supplies the tile rows
     int64_t rows_a = 0, rows_b = 0;       // after expansion
-    int64_t tiles = 0;
+    int64_t tiles = 0;                    // pairs of row tiles with `pair`
+    bool pair = false;                    // a CTA pair to two neighbouring row tiles
     int groups = 1, pg = 1;               // CTAs that share a tile's pieces, pieces of each
     size_t bytes_p = 0;                   // their partial outputs
     size_t bytes_a = 0, bytes_b = 0, bytes = 0;
@@ -724,11 +786,16 @@ Plan make_plan(const GemmArgs& g) {
             }
         }
     p.tiles = best;
+    {   // pairs where they leave at most one row tile in ten empty
+        const int64_t rt = up(p.swap ? p.rows_a : p.rows_b, kRows) / kRows, pt = (rt + 1) / 2;
+        p.pair = rt >= 2 && (rt % 2 == 0 || rt >= 9);
+        if (p.pair) p.tiles = p.tiles / rt * pt;
+    }
     const int64_t Kp = (int64_t)p.parts * p.koff;
     const int64_t nz = p.ns * p.pieces;
     p.bytes_a = up((int64_t)p.S * nz * p.rows_a * Kp * 2, 1024) + up(4 * nz * p.na * g.m, 1024);
     p.bytes_b = up((int64_t)p.S * nz * p.rows_b * Kp * 2, 1024) + up(4 * nz * p.nb * g.n, 1024);
-    p.groups = (int)std::max<int64_t>(1, std::min<int64_t>(p.pieces, tc_num_sms() / std::max<int64_t>(p.tiles, 1)));
+    p.groups = (int)std::max<int64_t>(1, std::min<int64_t>(p.pieces, tc_num_sms() / (p.pair ? 2 : 1) / std::max<int64_t>(p.tiles, 1)));
     p.pg = (p.pieces + p.groups - 1) / p.groups;
     p.groups = (p.pieces + p.pg - 1) / p.pg;
     if (p.groups > 1) p.bytes_p = up((int64_t)p.groups * p.na * p.nb * p.ns * g.m * g.n * 16, 1024);
@@ -795,17 +862,34 @@ __global__ void __launch_bounds__(256) sum_groups_kernel(const cplx* part, int g
     }
 }
 
-template <int S>
+template <int S, bool PAIR>
 int launch_gemm(const CUtensorMap& r, const CUtensorMap& q, const OutArgs& o, unsigned* flags, cudaStream_t st) {
-    auto kern = o.pieces > 1 ? slice_gemm_kernel<S, true> : slice_gemm_kernel<S, false>;
-    const size_t sm = 1024 + (size_t)kStages * Digits<S>::kStageBytes + sizeof(Ctl) + 2 * kCols * (2 * sizeof(int64_t) + sizeof(int));
+    using St = Stage<S, PAIR>;
+    auto kern = o.pieces > 1 ? slice_gemm_kernel<S, true, PAIR> : slice_gemm_kernel<S, false, PAIR>;
+    const size_t sm = 1024 + (size_t)St::kCount * St::kBytes + sizeof(Ctl) + 2 * kCols * (2 * sizeof(int64_t) + sizeof(int));
     raise_dyn_smem(kern, sm);
-    const int grid = (int)std::min<int64_t>(o.tiles * o.groups, tc_num_sms());
+    constexpr int C = PAIR ? 2 : 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(C * std::min<int64_t>(o.tiles * o.groups, tc_num_sms() / C)));
+    cfg.blockDim = dim3(kThreadsG);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
     count_launch();
-    kern<<<grid, kThreadsG, sm, st>>>(r, q, o, flags);
+    cudaLaunchKernelEx(&cfg, kern, r, q, o, flags);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(AFQMC_ERR_CUDA, std::string("slice_gemm launch: ") + cudaGetErrorString(e));
     return AFQMC_OK;
+}
+int launch_gemm(const Plan& p, const CUtensorMap& r, const CUtensorMap& q, const OutArgs& o, unsigned* flags, cudaStream_t st) {
+    if (p.pair) return p.S == 7 ? launch_gemm<7, true>(r, q, o, flags, st) : launch_gemm<8, true>(r, q, o, flags, st);
+    return p.S == 7 ? launch_gemm<7, false>(r, q, o, flags, st) : launch_gemm<8, false>(r, q, o, flags, st);
 }
 
 // One product that fits the workspace: B's slices at its start, A's at its end,
@@ -837,7 +921,7 @@ int run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st
         return make_map4(m, x.out, dims, str, box, 64);
     };
     AFQMC_TRY(encode(&mr, R, rr, kRows));
-    AFQMC_TRY(encode(&mq, Q, rc, kCols));
+    AFQMC_TRY(encode(&mq, Q, rc, p.pair ? kCols / 2 : kCols));
     OutArgs o{};
     o.rows = rr;
     o.cols = rc;
@@ -859,7 +943,7 @@ int run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st
     o.D = g.D;
     o.beta = g.beta.re;
     o.tiles = p.tiles;
-    o.drt = Div(up(rr, kRows) / kRows);
+    o.drt = Div(up(rr, p.pair ? 2 * kRows : kRows) / (p.pair ? 2 * kRows : kRows));
     o.dper = Div(p.tiles / p.ns);
     o.dtiles = Div(p.tiles);
     o.nk = (int)(up((int64_t)p.parts * p.koff, kChunk) / kChunk);
@@ -885,27 +969,28 @@ int run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st
             for (Dims* d : {&rown, &cown, &shared})
                 if (d->cnt[i] > 1) d->str[i] = dense[i];
         place();
-        AFQMC_TRY(p.S == 7 ? launch_gemm<7>(mr, mq, o, ws->flags, st) : launch_gemm<8>(mr, mq, o, ws->flags, st));
+        AFQMC_TRY(launch_gemm(p, mr, mq, o, ws->flags, st));
         count_launch();
         sum_groups_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(o.C, p.groups, total, g);
         return AFQMC_OK;
     }
-    return p.S == 7 ? launch_gemm<7>(mr, mq, o, ws->flags, st) : launch_gemm<8>(mr, mq, o, ws->flags, st);
+    return launch_gemm(p, mr, mq, o, ws->flags, st);
 }
 
 }  // namespace
 
 size_t slice_gemm_bytes(const GemmArgs& g) { return make_plan(g).bytes + 1024; }
 
-// Expected time in microseconds: three launches with little in each, the persistent tiles at 65 cycles an MMA and 6000
+// Expected time in microseconds: three launches with little in each, the persistent tiles at 65 (pairs: 56) cycles an MMA and 6000
 // for the epilogue, and the operands' packing.
 double slice_gemm_us(const GemmArgs& g) {
     if (g.beta.im != 0.0 || (g.A.real && g.B.real && g.alpha.im != 0.0)) return 1e30;
     const Plan p = make_plan(g);
     // the pack kernel's grid, 31-bit indices
     if (p.ns * p.pieces > 65535 || std::max(p.rows_a, p.rows_b) >= 1ll << 31 || p.tiles * p.groups >= 1ll << 31) return 1e30;
-    const double cyc = p.S * (p.S + 1) / 2 * (up((int64_t)p.parts * p.koff, 16) / 16) * 65.0 + 6000.0;
-    const double waves = (double)((p.tiles * p.groups + tc_num_sms() - 1) / tc_num_sms());
+    const double cyc = p.S * (p.S + 1) / 2 * (up((int64_t)p.parts * p.koff, 16) / 16) * (p.pair ? 56.0 : 65.0) + 6000.0;
+    const int ctas = tc_num_sms() / (p.pair ? 2 : 1);
+    const double waves = (double)((p.tiles * p.groups + ctas - 1) / ctas);
     return 26.0 + p.pg * waves * cyc / 1.9e3 + (double)p.bytes / 2.0e6 + (p.groups > 1 ? 4.0 : 0.0);
 }
 
@@ -927,7 +1012,7 @@ int slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st) {
     };
     if (p.pieces >= 8) {
         const int64_t fit = (int64_t)(ws->bytes / ((p.bytes + 1024) / p.pieces + 1));
-        const int64_t share = std::max<int64_t>(1, tc_num_sms() / std::max<int64_t>(p.tiles, 1));
+        const int64_t share = std::max<int64_t>(1, tc_num_sms() / (p.pair ? 2 : 1) / std::max<int64_t>(p.tiles, 1));
         const int64_t n = fit > share ? fit / share * share : std::max<int64_t>(1, fit);
         lo.k = (int)std::min<int64_t>(n, p.pieces - 1) * p.klen;
         hi.k = g.k - lo.k;

@@ -130,47 +130,31 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64
 // descriptor.  KEEP: its place in a run of MMAs with the same A: the first of a run fills the tensor
 // core's collector buffer with A, the others take A from there instead of from shared memory.
 enum KeepA : int { kKeepNone, kKeepFirst, kKeepMore, kKeepLast };
-template <int KEEP>
+#define AFQMC_MMA_F16_LO(form)                                                                                  \
+    asm volatile(                                                                                              \
+        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"                                                            \
+        "mov.b64 a, {%1, %3};\n\t"                                                                             \
+        "mov.b64 b, {%2, %3};\n\t"                                                                             \
+        "setp.ne.b32 p, %5, 0;\n\t"                                                                            \
+        "tcgen05.mma." form " [%0], a, b, %4, p;\n\t}" ::"r"(tmem_d),                                          \
+        "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)                                             \
+        : "memory")
+template <int KEEP, bool PAIR = false>
 __device__ __forceinline__ void mma_f16_lo(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
                                            uint32_t accumulate) {
-    if (KEEP == kKeepNone) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
-            "mov.b64 a, {%1, %3};\n\t"
-            "mov.b64 b, {%2, %3};\n\t"
-            "setp.ne.b32 p, %5, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}" ::"r"(tmem_d),
-            "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
-            : "memory");
-    } else if (KEEP == kKeepFirst) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
-            "mov.b64 a, {%1, %3};\n\t"
-            "mov.b64 b, {%2, %3};\n\t"
-            "setp.ne.b32 p, %5, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], a, b, %4, p;\n\t}" ::"r"(tmem_d),
-            "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
-            : "memory");
-    } else if (KEEP == kKeepMore) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
-            "mov.b64 a, {%1, %3};\n\t"
-            "mov.b64 b, {%2, %3};\n\t"
-            "setp.ne.b32 p, %5, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%0], a, b, %4, p;\n\t}" ::"r"(tmem_d),
-            "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
-            : "memory");
+    if (PAIR) {
+        if (KEEP == kKeepNone) AFQMC_MMA_F16_LO("cta_group::2.kind::f16");
+        else if (KEEP == kKeepFirst) AFQMC_MMA_F16_LO("cta_group::2.kind::f16.collector::a::fill");
+        else if (KEEP == kKeepMore) AFQMC_MMA_F16_LO("cta_group::2.kind::f16.collector::a::use");
+        else AFQMC_MMA_F16_LO("cta_group::2.kind::f16.collector::a::lastuse");
     } else {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
-            "mov.b64 a, {%1, %3};\n\t"
-            "mov.b64 b, {%2, %3};\n\t"
-            "setp.ne.b32 p, %5, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%0], a, b, %4, p;\n\t}" ::"r"(tmem_d),
-            "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
-            : "memory");
+        if (KEEP == kKeepNone) AFQMC_MMA_F16_LO("cta_group::1.kind::f16");
+        else if (KEEP == kKeepFirst) AFQMC_MMA_F16_LO("cta_group::1.kind::f16.collector::a::fill");
+        else if (KEEP == kKeepMore) AFQMC_MMA_F16_LO("cta_group::1.kind::f16.collector::a::use");
+        else AFQMC_MMA_F16_LO("cta_group::1.kind::f16.collector::a::lastuse");
     }
 }
+#undef AFQMC_MMA_F16_LO
 // True in one lane of a converged warp, the same one every time.  Unlike a test of the lane number it
 // keeps the warp's values uniform, so that descriptors stay in uniform registers, where the MMA takes
 // them from.  To be asked for at each use: a stored answer loses that.
@@ -237,6 +221,14 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* m
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, "
         "%4}], [%2];" ::"r"(smem_u32(dst)),
         "l"(reinterpret_cast<uint64_t>(m)), "r"(bar_cluster_addr), "r"(x), "r"(y)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_4d_pair(void* dst, const CUtensorMap* m, uint32_t bar_cluster_addr, int x, int y,
+                                                 int z, int w) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, "
+        "%4, %5, %6}], [%2];" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(m)), "r"(bar_cluster_addr), "r"(x), "r"(y), "r"(z), "r"(w)
         : "memory");
 }
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst, uint32_t ncols) {
