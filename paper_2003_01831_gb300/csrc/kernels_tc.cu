@@ -1524,16 +1524,25 @@ constexpr double kS3 = 1.0 / 128.0;
 // Two stages of 64 K (96 KB each; four of 32 are as fast).  Sixteen warps drain a tile: they fold the
 // four accumulators into registers, release tensor memory, and scale and store while the next tile's
 // MMAs run; four warps that released it after their stores took half of a tile's time at K = 256.
-// Measured at M = 256, 256 walkers (us): the Taylor terms' products 149 -> 108 (their operands and
-// result take 79 at the copy rate), the potential 442 -> 352 (200 at the MMA rate, 4 GB through L2).
+// PAIR: two CTAs take two neighbouring row tiles with MMAs of M = 256, each with half of the B rows in
+// its shared memory, which L2 then delivers once for both (its 11 TB/s bound the long contractions), in three
+// stages of 72 KB; for which calls, see tc_gemm3.
+// Measured at M = 256, 256 walkers (us): the Taylor terms' products 149 -> 104 (their operands and
+// result take 79 at the copy rate), the potential 442 -> 352, in pairs 313 (200 at the MMA rate); at
+// M = 512, 1024 walkers the Taylor terms 2950 -> 2400, in pairs 2110.
 constexpr int kG3BK = 64;
 constexpr int kG3ABytes = kBM * kG3BK * 2;        // one plane, 128 rows
-constexpr int kG3BBytes = 128 * kG3BK * 2;        // B tile: 128 rows
-constexpr int kG3StageBytes = 3 * (kG3ABytes + kG3BBytes);
-constexpr int kG3Stages = 192 * 1024 / kG3StageBytes;
+template <bool PAIR>
+struct G3Stage {   // a CTA's 128 rows of A and 128 of B, or 64 of them in a pair
+    static constexpr int kBRows = PAIR ? 64 : 128;
+    static constexpr int kBBytes = kBRows * kG3BK * 2;
+    static constexpr int kBytes = 3 * (kG3ABytes + kBBytes);
+    static constexpr int kCount = 216 * 1024 / kBytes;
+};
 constexpr int kG3Epi = 512;                       // 16 warps: 4 quadrants of rows x 4 groups of 32 columns
 constexpr int kG3Threads = 64 + kG3Epi;
 
+template <bool PAIR>
 __global__ void __launch_bounds__(kG3Threads, 1)
     tc_gemm3_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUtensorMap tA1,
                     const __grid_constant__ CUtensorMap tA2, const __grid_constant__ CUtensorMap tB0,
@@ -1541,110 +1550,136 @@ __global__ void __launch_bounds__(kG3Threads, 1)
                     EpiParams epi, unsigned* flags) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sbase = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    SharedCtl* ctl = reinterpret_cast<SharedCtl*>(sbase + kG3Stages * kG3StageBytes);
+    using St = G3Stage<PAIR>;
+    SharedCtl* ctl = reinterpret_cast<SharedCtl*>(sbase + St::kCount * St::kBytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = PAIR ? cluster_ctarank() : 0;
+    const int64_t first = PAIR ? cluster_id_x() : blockIdx.x, stride = PAIR ? ncluster_x() : gridDim.x;
     const bool three_d = sh.am.mod != (1 << 30) || sh.nbatch > 1;
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kG3Stages; ++i) {
+        for (int i = 0; i < St::kCount; ++i) {
             mbar_init(&ctl->full[i], 1);
             mbar_init(&ctl->empty[i], 1);
         }
         mbar_init(&ctl->tfull[0], 1);
-        mbar_init(&ctl->tempty[0], kG3Epi / 32);
+        mbar_init(&ctl->tempty[0], (PAIR ? 2 : 1) * (kG3Epi / 32));
         mbar_init(&ctl->done, 1);
         ctl->abort = 0;
         fence_mbar_init();
     }
+    if (PAIR) {
+        __syncthreads();
+        cluster_sync();   // both CTAs' barriers exist before any copy or arrival reaches them
+    }
     if (warp == 1) {
-        tmem_alloc(&ctl->tmem_base, 512);
-        tmem_relinquish();
+        if (PAIR) {
+            tmem_alloc_pair(&ctl->tmem_base, 512);
+            tmem_relinquish_pair();
+        } else {
+            tmem_alloc(&ctl->tmem_base, 512);
+            tmem_relinquish();
+        }
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (PAIR) cluster_sync();   // tensor memory allocated in both CTAs before the first MMA
     if (warp == 0) {
         if (lane == 0) {
             const CUtensorMap* A[3] = {&tA0, &tA1, &tA2};
             const CUtensorMap* B[3] = {&tB0, &tB1, &tB2};
             int64_t g = 0;
             bool ok = true;
-            for (int64_t t = blockIdx.x; t < sh.tiles && ok; t += gridDim.x) {
+            for (int64_t t = first; t < sh.tiles && ok; t += stride) {
                 int b, rt, ct;
                 tile_coords(sh, t, b, rt, ct);
                 const int az = three_d ? (b / sh.am.div) % sh.am.mod : 0;
                 const int bz = three_d ? (b / sh.bm.div) % sh.bm.mod : 0;
+                const int ya = (PAIR ? 2 * rt + (int)rank : rt) * kBM, yb = ct * 128 + (int)rank * St::kBRows;
                 for (int kb = 0; kb < sh.nk; ++kb, ++g) {
-                    const int st = (int)(g % kG3Stages);
-                    const uint32_t ph = (uint32_t)((g / kG3Stages) & 1);
+                    const int st = (int)(g % St::kCount);
+                    const uint32_t ph = (uint32_t)((g / St::kCount) & 1);
                     if (!mbar_wait(&ctl->empty[st], ph ^ 1u, &ctl->abort)) { ok = false; break; }
-                    uint8_t* sp = sbase + (size_t)st * kG3StageBytes;
-                    mbar_arrive_expect_tx(&ctl->full[st], kG3StageBytes);
+                    uint8_t* sp = sbase + (size_t)st * St::kBytes;
                     const int x = kb * kG3BK;
-                    for (int q = 0; q < 3; ++q) {
-                        if (three_d) {
-                            tma_load_3d(sp + q * kG3ABytes, A[q], &ctl->full[st], x, rt * kBM, az);
-                            tma_load_3d(sp + 3 * kG3ABytes + q * kG3BBytes, B[q], &ctl->full[st], x, ct * 128, bz);
+                    if (!PAIR || rank == 0) mbar_arrive_expect_tx(&ctl->full[st], (PAIR ? 2 : 1) * St::kBytes);   // both CTAs' bytes
+                    const uint32_t fb = PAIR ? mapa_shared(&ctl->full[st], 0) : 0u;
+                    auto load = [&](uint8_t* d, const CUtensorMap* m, int y, int z) {
+                        if (PAIR) {
+                            if (three_d) tma_load_3d_pair(d, m, fb, x, y, z);
+                            else tma_load_2d_pair(d, m, fb, x, y);
                         } else {
-                            tma_load_2d(sp + q * kG3ABytes, A[q], &ctl->full[st], x, rt * kBM);
-                            tma_load_2d(sp + 3 * kG3ABytes + q * kG3BBytes, B[q], &ctl->full[st], x, ct * 128);
+                            if (three_d) tma_load_3d(d, m, &ctl->full[st], x, y, z);
+                            else tma_load_2d(d, m, &ctl->full[st], x, y);
                         }
+                    };
+                    for (int q = 0; q < 3; ++q) {
+                        load(sp + q * kG3ABytes, A[q], ya, az);
+                        load(sp + 3 * kG3ABytes + q * St::kBBytes, B[q], yb, bz);
                     }
                 }
             }
-            if (!ok) {
-                const int64_t first = g > kG3Stages ? g - kG3Stages : 0;
-                for (int64_t j = first; j < g; ++j)
-                    wait_drain(&ctl->full[j % kG3Stages], (uint32_t)((j / kG3Stages) & 1));
+            if (!ok && rank == 0) {
+                const int64_t j0 = g > St::kCount ? g - St::kCount : 0;
+                for (int64_t j = j0; j < g; ++j)
+                    wait_drain(&ctl->full[j % St::kCount], (uint32_t)((j / St::kCount) & 1));
+            } else if (!ok) {   // the peer cannot wait on rank 0's barriers: its copies get time to land
+                const long long t0 = clock64();
+                while (clock64() - t0 < (1LL << 22)) {
+                }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(kBM, 128, true);
-            constexpr uint32_t A = kG3ABytes >> 4, B = kG3BBytes >> 4;
+        if (lane == 0 && rank == 0) {
+            constexpr uint32_t idesc = idesc_bf16(PAIR ? 2 * kBM : kBM, 128, true);
+            constexpr uint32_t A = kG3ABytes >> 4, B = St::kBBytes >> 4;
             const uint32_t d1 = ctl->tmem_base, d2 = d1 + 128, d3 = d1 + 256, d4 = d1 + 384;
             const uint64_t d0 = kG3BK == 64 ? desc_sw128(smem_u32(sbase)) : desc_sw64(smem_u32(sbase));
             const uint32_t lo0 = (uint32_t)d0, hi = (uint32_t)(d0 >> 32);
             int64_t g = 0;
             int it = 0;
             bool ok = true;
-            for (int64_t t = blockIdx.x; t < sh.tiles && ok; t += gridDim.x, ++it) {
+            for (int64_t t = first; t < sh.tiles && ok; t += stride, ++it) {
                 if (!mbar_wait(&ctl->tempty[0], ((uint32_t)it & 1u) ^ 1u, &ctl->abort)) break;
                 tc_fence_after();
                 for (int kb = 0; kb < sh.nk; ++kb, ++g) {
-                    const int st = (int)(g % kG3Stages);
-                    const uint32_t ph = (uint32_t)((g / kG3Stages) & 1);
+                    const int st = (int)(g % St::kCount);
+                    const uint32_t ph = (uint32_t)((g / St::kCount) & 1);
                     if (!mbar_wait(&ctl->full[st], ph, &ctl->abort)) { ok = false; break; }
                     tc_fence_after();
 #pragma unroll
                     for (int kk = 0; kk < kG3BK / 16; ++kk) {
-                        const uint32_t ah = lo0 + st * (kG3StageBytes >> 4) + 2 * kk, am = ah + A, al = am + A;
+                        const uint32_t ah = lo0 + st * (St::kBytes >> 4) + 2 * kk, am = ah + A, al = am + A;
                         const uint32_t bh = al + A, bm = bh + B, bl = bm + B;
                         const uint32_t acc = (kb | kk) != 0 ? 1u : 0u;
-                        mma_f16_lo<kKeepNone>(d1, ah, bh, hi, idesc, acc);
-                        mma_f16_lo<kKeepNone>(d2, ah, bm, hi, idesc, acc);
-                        mma_f16_lo<kKeepNone>(d3, ah, bl, hi, idesc, acc);
-                        mma_f16_lo<kKeepNone>(d2, am, bh, hi, idesc, 1u);
-                        mma_f16_lo<kKeepNone>(d4, am, bm, hi, idesc, acc);
-                        mma_f16_lo<kKeepNone>(d3, al, bh, hi, idesc, 1u);
+                        mma_f16_lo<kKeepNone, PAIR>(d1, ah, bh, hi, idesc, acc);
+                        mma_f16_lo<kKeepNone, PAIR>(d2, ah, bm, hi, idesc, acc);
+                        mma_f16_lo<kKeepNone, PAIR>(d3, ah, bl, hi, idesc, acc);
+                        mma_f16_lo<kKeepNone, PAIR>(d2, am, bh, hi, idesc, 1u);
+                        mma_f16_lo<kKeepNone, PAIR>(d4, am, bm, hi, idesc, acc);
+                        mma_f16_lo<kKeepNone, PAIR>(d3, al, bh, hi, idesc, 1u);
                     }
-                    mma_commit(&ctl->empty[st]);
+                    if (PAIR) mma_commit_pair(&ctl->empty[st], 3);   // free in both CTAs
+                    else mma_commit(&ctl->empty[st]);
                 }
                 if (!ok) break;
-                mma_commit(&ctl->tfull[0]);
+                if (PAIR) mma_commit_pair(&ctl->tfull[0], 3);
+                else mma_commit(&ctl->tfull[0]);
             }
-            mma_commit(&ctl->done);
+            if (PAIR) mma_commit_pair(&ctl->done, 1);
+            else mma_commit(&ctl->done);
             wait_drain(&ctl->done, 0);
         }
     } else {
         const int g4 = warp & 3, c = (warp - 2) >> 2;
         const uint32_t tb = ctl->tmem_base + ((uint32_t)(g4 * 32) << 16) + c * 32;
         int it = 0;
-        for (int64_t t = blockIdx.x; t < sh.tiles; t += gridDim.x, ++it) {
+        for (int64_t t = first; t < sh.tiles; t += stride, ++it) {
             int b, rt, ct;
             tile_coords(sh, t, b, rt, ct);
             const int az = three_d ? (b / sh.am.div) % sh.am.mod : 0;
             const int bz = three_d ? (b / sh.bm.div) % sh.bm.mod : 0;
-            const int64_t r = (int64_t)rt * kBM + g4 * 32 + lane, c0 = (int64_t)ct * 128 + c * 32;
+            const int64_t r = (int64_t)(PAIR ? 2 * rt + (int)rank : rt) * kBM + g4 * 32 + lane, c0 = (int64_t)ct * 128 + c * 32;
             const float sa = r < sh.a_rows ? sh.a_scale[(int64_t)az * sh.a_rows + r] : 0.0f;
             const float sb = c0 + lane < sh.b_rows ? sh.b_scale[(int64_t)bz * sh.b_rows + c0 + lane] : 0.0f;
             if (!warp_wait(&ctl->tfull[0], (uint32_t)it & 1u, &ctl->abort)) break;
@@ -1671,7 +1706,10 @@ __global__ void __launch_bounds__(kG3Threads, 1)
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&ctl->tempty[0]);   // the next tile's MMAs run meanwhile
+            if (lane == 0) {   // the next tile's MMAs run meanwhile
+                if (PAIR) mbar_arrive_cluster_relaxed(mapa_shared(&ctl->tempty[0], 0));
+                else mbar_arrive(&ctl->tempty[0]);
+            }
 #pragma unroll
             for (int q = 0; q < 32; ++q) {
                 const float sc = sa * __shfl_sync(0xffffffffu, sb, q);
@@ -1683,9 +1721,11 @@ __global__ void __launch_bounds__(kG3Threads, 1)
     }
     tc_fence_before();
     __syncthreads();
+    if (PAIR) cluster_sync();   // both CTAs are done with tensor memory and each other's shared memory
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(ctl->tmem_base, 512);
+        if (PAIR) tmem_dealloc_pair(ctl->tmem_base, 512);
+        else tmem_dealloc(ctl->tmem_base, 512);
     }
     if (threadIdx.x == 0 && ctl->abort) atomicOr(flags, FLAG_TIMEOUT);
 }
@@ -2293,17 +2333,22 @@ int tc_gemm3(const Split3& A, BatchMap amap, const Split3& B, BatchMap bmap, int
     if (rows <= 0 || cols <= 0 || K <= 0 || nbatch <= 0) return AFQMC_OK;
     if (!A.scale || !B.scale) return fail(AFQMC_ERR_BADARG, "tc_gemm3: row scales required");
     const bool three_d = nbatch > 1 || amap.mod != (1 << 30);
+    // CTA pairs on neighbouring row tiles, where they leave at most one tile in ten empty and the contraction
+    // is long: up to K = 256 a tile is its epilogue, and two that wait for each other are slower (us,
+    // single -> pair: 1024 tiles of K = 256 70 -> 76; K = 512 106 -> 104; K = 640 105 -> 96)
+    const int64_t row_tiles = (rows + kBM - 1) / kBM;
+    const bool pair = K >= 512 && row_tiles >= 2 && (row_tiles % 2 == 0 || row_tiles >= 9) && launch_policy().grid_cap != 1;
     CUtensorMap m[6];
     for (int q = 0; q < 3; ++q) {
         AFQMC_TRY(make_map(&m[q], A.p[q], A.K, A.rows, A.batch, A.K, A.batch_stride, kBM, three_d, true, 2 * kG3BK));
-        AFQMC_TRY(make_map(&m[3 + q], B.p[q], B.K, B.rows, B.batch, B.K, B.batch_stride, 128, three_d, true, 2 * kG3BK));
+        AFQMC_TRY(make_map(&m[3 + q], B.p[q], B.K, B.rows, B.batch, B.K, B.batch_stride, pair ? 64 : 128, three_d, true, 2 * kG3BK));
     }
     TileShape sh;
     sh.rows = rows;
     sh.cols = cols;
     sh.K = K;
     sh.nbatch = nbatch;
-    sh.rt = (int)((rows + kBM - 1) / kBM);
+    sh.rt = (int)(pair ? (row_tiles + 1) / 2 : row_tiles);
     sh.ct = (int)((cols + 127) / 128);
     sh.nk = (int)((K + kG3BK - 1) / kG3BK);
     sh.tiles = (int64_t)sh.rt * sh.ct * nbatch;
@@ -2314,12 +2359,27 @@ int tc_gemm3(const Split3& A, BatchMap amap, const Split3& B, BatchMap bmap, int
     sh.b_scale = B.scale;
     sh.a_rows = A.rows;
     sh.b_rows = B.rows;
-    const size_t smem = 1024 + (size_t)kG3Stages * kG3StageBytes + sizeof(SharedCtl);
-    raise_dyn_smem(tc_gemm3_kernel, smem);
     const int cap = launch_policy().grid_cap > 0 ? std::min(launch_policy().grid_cap, tc_num_sms()) : tc_num_sms();
-    const int grid = (int)std::min<int64_t>(sh.tiles, cap);
+    auto launch = [&](auto kernel, int ctas, size_t stages) {
+        const size_t smem = 1024 + stages + sizeof(SharedCtl);
+        raise_dyn_smem(kernel, smem);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(ctas * std::min<int64_t>(sh.tiles, cap / ctas)));
+        cfg.blockDim = dim3(kG3Threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)ctas;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        cudaLaunchKernelEx(&cfg, kernel, m[0], m[1], m[2], m[3], m[4], m[5], sh, epi, flags);
+    };
     count_launch();
-    tc_gemm3_kernel<<<grid, kG3Threads, smem, st>>>(m[0], m[1], m[2], m[3], m[4], m[5], sh, epi, flags);
+    if (pair) launch(tc_gemm3_kernel<true>, 2, (size_t)G3Stage<true>::kCount * G3Stage<true>::kBytes);
+    else launch(tc_gemm3_kernel<false>, 1, (size_t)G3Stage<false>::kCount * G3Stage<false>::kBytes);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(AFQMC_ERR_CUDA, std::string("tc_gemm3 launch: ") + cudaGetErrorString(e));
     return AFQMC_OK;
