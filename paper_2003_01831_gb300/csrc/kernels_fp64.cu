@@ -1156,6 +1156,31 @@ __global__ void __launch_bounds__(kGJRegThreads<CW>, CW / 4)
 constexpr int kGJWarpMax = 32;
 constexpr int kGJWarps = 2;   // matrices per CTA
 
+// log det of one warp's matrix: lane k has the pivot of step k and its row (1 and 0 past N).
+template <int NC>
+__device__ __forceinline__ cplx gj_warp_logdet(cplx piv, int perm, int N) {
+    const int lane = threadIdx.x & 31;
+    // log|det| and arg det from the product of the pivots, times -1 for an odd pivot permutation,
+    // whose sign is that of its inversions (pairs of steps whose pivot rows are out of order)
+    cplx v = piv;
+    int ex = cnormalise(v);
+    int odd = 0;
+#pragma unroll
+    for (int j = 0; j < NC; ++j) {
+        const int pj = __shfl_sync(0xffffffffu, perm, j);
+        if (lane < N && j < lane && pj > perm) odd ^= 1;
+    }
+    odd = __popc(__ballot_sync(0xffffffffu, odd)) & 1;
+#pragma unroll
+    for (int o = NC > 16 ? 16 : NC / 2; o > 0; o >>= 1) {   // the first NC lanes' pivots; the others' are 1
+        v = v * cplx{__shfl_xor_sync(0xffffffffu, v.re, o), __shfl_xor_sync(0xffffffffu, v.im, o)};
+        ex += __shfl_xor_sync(0xffffffffu, ex, o);
+    }
+    ex += cnormalise(v);
+    if (odd) v = cplx{-v.re, -v.im};
+    return log_of_product(v, ex);
+}
+
 template <int NC, bool INV>
 __global__ void __launch_bounds__(32 * kGJWarps)
     gj_warp_kernel(cplx* Sbase, int64_t stride, int N, int count, cplx* logdet, unsigned* flags) {
@@ -1231,25 +1256,7 @@ __global__ void __launch_bounds__(32 * kGJWarps)
         }
         return;
     }
-    // log|det| and arg det from the product of the pivots, times -1 for an odd pivot permutation,
-    // whose sign is that of its inversions (pairs of steps whose pivot rows are out of order)
-    cplx v = mypiv;
-    int ex = cnormalise(v);
-    int odd = 0;
-#pragma unroll
-    for (int j = 0; j < NC; ++j) {
-        const int pj = __shfl_sync(0xffffffffu, myperm, j);
-        if (lane < N && j < lane && pj > myperm) odd ^= 1;
-    }
-    odd = __popc(__ballot_sync(0xffffffffu, odd)) & 1;
-#pragma unroll
-    for (int o = NC > 16 ? 16 : NC / 2; o > 0; o >>= 1) {   // the first NC lanes' pivots; the others' are 1
-        v = v * cplx{__shfl_xor_sync(0xffffffffu, v.re, o), __shfl_xor_sync(0xffffffffu, v.im, o)};
-        ex += __shfl_xor_sync(0xffffffffu, ex, o);
-    }
-    ex += cnormalise(v);
-    if (odd) v = cplx{-v.re, -v.im};
-    const cplx ld = log_of_product(v, ex);
+    const cplx ld = gj_warp_logdet<NC>(mypiv, myperm, N);
     if (lane == 0) logdet[mat] = ld;
     if (INV) {   // row i of the array is row mystep of the inverse; column j is its column perm[j]
 #pragma unroll
@@ -1258,6 +1265,123 @@ __global__ void __launch_bounds__(32 * kGJWarps)
             const int c = __shfl_sync(0xffffffffu, myperm, j);
             if (lane < N && j < N) G[(int64_t)mystep * N + c] = a[u];
         }
+    }
+}
+
+// The same by a team of four warps, for counts that leave schedulers without a matrix: warp w holds the
+// columns [w NC / 4, (w + 1) NC / 4), so a step's updates take a quarter of one pipe's time on four.  The
+// warp of column k + 1 updates that first, finds its pivot and publishes it with the column before the
+// rest of its update; one barrier a step.  The arithmetic is gj_warp_kernel's, bit for bit.
+// Measured, one warp -> team, inverses (ms): 128 of N = 32 0.240 -> 0.100, 122 of N = 23 0.135 -> 0.065,
+// 128 of N = 16 0.079 -> 0.043, 16 of N = 5 0.028 -> 0.021.
+constexpr int kGJTeam = 4;
+template <int NC, bool INV>
+__global__ void __launch_bounds__(32 * kGJTeam)
+    gj_team_kernel(cplx* Sbase, int64_t stride, int N, cplx* logdet, unsigned* flags) {
+    constexpr int CW = NC / kGJTeam;
+    __shared__ __align__(16) cplx col[2][32];       // the pivot column, before its elimination
+    __shared__ __align__(16) cplx row[kGJTeam][CW];
+    __shared__ cplx inv_s[2], piv_s[2], pivs[32];
+    __shared__ int p_s[2], perm[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c0 = warp * CW;
+    const int64_t mat = blockIdx.x;
+    cplx* G = Sbase + mat * stride;
+    cplx a[CW];
+#pragma unroll
+    for (int u = 0; u < CW; ++u) {
+        a[u] = cplx{lane == c0 + u ? 1.0 : 0.0, 0.0};
+        if (lane < N && c0 + u < N) a[u] = G[(int64_t)lane * N + c0 + u];
+    }
+    bool used = lane >= N;
+    int mystep = 0;
+    // pivot search in a column (entry v of this lane's row) and publication in buffer b
+    auto publish = [&](int b, const cplx& v) {
+        const unsigned long long key = used ? 0ull : (unsigned long long)__double_as_longlong(abs1(v));
+        const unsigned kh = (unsigned)(key >> 32);
+        const unsigned mh = __reduce_max_sync(0xffffffffu, kh);
+        const unsigned kl = kh == mh ? (unsigned)key : 0u;
+        const unsigned ml = __reduce_max_sync(0xffffffffu, kl);
+        const unsigned hit = __ballot_sync(0xffffffffu, !used && kh == mh && kl == ml);
+        const int p = mh >= 0x7ff00000u ? -2 : ((mh | ml) == 0u ? -1 : __ffs(hit) - 1);
+        col[b][lane] = v;
+        if (p >= 0) {   // the same in every lane
+            const cplx piv{__shfl_sync(0xffffffffu, v.re, p), __shfl_sync(0xffffffffu, v.im, p)};
+            const cplx inv = crecip(piv);
+            if (lane == 0) {
+                inv_s[b] = inv;
+                piv_s[b] = piv;
+            }
+        }
+        if (lane == 0) p_s[b] = p;
+    };
+    if (warp == 0) publish(0, a[0]);
+    __syncthreads();
+    int bad = 0;
+#pragma unroll 1
+    for (int k = 0; k < N; ++k) {
+        const int b = k & 1, p = p_s[b];
+        if (p < 0) { bad = p; break; }
+        const cplx inv = inv_s[b], m = col[b][lane], nm{-m.re, -m.im};
+        const bool isp = lane == p;
+        if (threadIdx.x == 0) {
+            perm[k] = p;
+            pivs[k] = piv_s[b];
+        }
+        if (isp) {
+            used = true;
+            mystep = k;
+#pragma unroll
+            for (int u = 0; u < CW; ++u) row[warp][u] = a[u];
+        }
+        __syncwarp();
+        cplx mine{0.0, 0.0};
+        if (lane < CW) mine = row[warp][lane] * inv;
+        __syncwarp();
+        if (lane < CW) row[warp][lane] = mine;
+        __syncwarp();
+        const int uk = k - c0, u1 = uk + 1;
+        auto update = [&](int u) {
+            const cplx pr = row[warp][u];
+            cplx v = a[u];
+            cfma(v, nm, pr);
+            a[u] = isp ? pr : v;
+        };
+        const bool next = u1 >= 0 && u1 < CW && k + 1 < N;
+        if (next) {
+#pragma unroll
+            for (int u = 0; u < CW; ++u)
+                if (u == u1) {
+                    update(u);
+                    publish(b ^ 1, a[u]);
+                }
+        }
+#pragma unroll
+        for (int u = 0; u < CW; ++u) {
+            if ((next && u == u1) || (!INV && u <= uk)) continue;
+            if (u == uk) {   // column k of the inverse: -m / piv, 1 / piv in the pivot row
+                const cplx last = nm * inv;
+                a[u] = isp ? inv : last;
+            } else {
+                update(u);
+            }
+        }
+        __syncthreads();
+    }
+    if (bad) {
+        if (threadIdx.x == 0) {
+            logdet[mat] = cplx{-INFINITY, 0.0};
+            atomicOr(flags, bad == -2 ? FLAG_NONFINITE : FLAG_SINGULAR);
+        }
+        return;
+    }
+    if (warp == 0) {
+        const cplx ld = gj_warp_logdet<NC>(lane < N ? pivs[lane] : cplx{1.0, 0.0}, lane < N ? perm[lane] : 0, N);
+        if (lane == 0) logdet[mat] = ld;
+    }
+    if (INV) {
+#pragma unroll
+        for (int u = 0; u < CW; ++u)
+            if (lane < N && c0 + u < N) G[(int64_t)mystep * N + perm[c0 + u]] = a[u];
     }
 }
 
@@ -1850,6 +1974,19 @@ void batched_inverse_logdet(cplx* S, int64_t stride, int N, int count, cplx* log
     if (N <= kGJWarpMax && variant != 1) {
         const unsigned grid = (unsigned)((count + kGJWarps - 1) / kGJWarps);
         count_launch();
+        // a team of warps to a matrix while the matrices leave schedulers idle (up to 4 an SM: 512
+        // of N = 32 0.25 -> 0.20 ms, 1024 0.33 -> 0.38)
+        if (variant != 4 && (variant == 5 || count <= 4 * tc_num_sms())) {
+            auto team = [&](auto inv, auto log_only) {
+                if (with_inverse) inv<<<(unsigned)count, 32 * kGJTeam, 0, st>>>(S, stride, N, logdet, flags);
+                else log_only<<<(unsigned)count, 32 * kGJTeam, 0, st>>>(S, stride, N, logdet, flags);
+            };
+            if (N <= 8) team(gj_team_kernel<8, true>, gj_team_kernel<8, false>);
+            else if (N <= 16) team(gj_team_kernel<16, true>, gj_team_kernel<16, false>);
+            else if (N <= 24) team(gj_team_kernel<24, true>, gj_team_kernel<24, false>);
+            else team(gj_team_kernel<32, true>, gj_team_kernel<32, false>);
+            return;
+        }
         auto go = [&](auto inv, auto log_only) {
             if (with_inverse) inv<<<grid, 32 * kGJWarps, 0, st>>>(S, stride, N, count, logdet, flags);
             else log_only<<<grid, 32 * kGJWarps, 0, st>>>(S, stride, N, count, logdet, flags);
