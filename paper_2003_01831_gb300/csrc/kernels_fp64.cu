@@ -1393,12 +1393,12 @@ __global__ void __launch_bounds__(32 * kGJTeam)
 // bank conflicts, and leave four sums.  Bound by the FP64 pipe (2 N^2 multiply-adds, 16 cycles a
 // warp instruction) beside the read of T; the old form, which read T_ba with a stride from global
 // memory and did every product twice, took 16.8 ms for the 655,360 matrices of a step at M = 128,
-// W = 512; this one 3.9 ms.
+// W = 512; this one 3.6 ms, with twelve matrices an SM in flight (3.9 with eight).
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
-template <int GROUP>
-__global__ void __launch_bounds__(kThreads)
+template <int GROUP, int T_>
+__global__ void __launch_bounds__(T_)
     trace_pairs_kernel(const cplx* T, int64_t count, int W, int N, int n0, cplx* t_out, cplx* X_out, int64_t ldo) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[kThreads / 32][4];
@@ -1409,7 +1409,7 @@ __global__ void __launch_bounds__(kThreads)
         if (GROUP == 32) __syncwarp();
         else __syncthreads();
     };
-    constexpr int kGroups = kThreads / GROUP;
+    constexpr int kGroups = T_ / GROUP;
     const int64_t NN = (int64_t)N * N;
     for (int64_t i0 = (int64_t)blockIdx.x * kGroups; i0 < count; i0 += (int64_t)gridDim.x * kGroups) {
         const int64_t i = i0 + grp;   // matrix (c, w)
@@ -2041,19 +2041,24 @@ void trace_terms(const cplx* T, int nc, int W, int N, int n0, cplx* t_out, cplx*
     if (count <= 0) return;
     const int P = N + (N & 1);
     const size_t one = (size_t)N * P * sizeof(cplx);
-    auto go = [&](auto kern, int groups, int ctas) {
+    auto go = [&](auto kern, int threads, int groups, int ctas) {
         raise_dyn_smem(kern, one * groups);
         const int64_t grid = std::min<int64_t>((count + groups - 1) / groups, ctas);
         count_launch();
-        kern<<<(unsigned)grid, kThreads, one * groups, st>>>(T, count, W, N, n0, t_out, X_out, ldo);
+        kern<<<(unsigned)grid, threads, one * groups, st>>>(T, count, W, N, n0, t_out, X_out, ldo);
     };
     // CTAs: as many as shared memory lets an SM hold, 152 SMs, a few rounds each
     if (N <= 32) {
-        go(trace_pairs_kernel<32>, kThreads / 32, 152 * std::max(1, std::min(8, (int)(220000 / (one * (kThreads / 32))))) * 4);
+        // one CTA of twelve matrices where two of eight do not fit an SM (N = 32: 3.9 -> 3.6 ms a step)
+        if (2 * 8 * one > 220000)
+            go(trace_pairs_kernel<32, 384>, 384, 12, 152 * 4);
+        else
+            go(trace_pairs_kernel<32, kThreads>, kThreads, kThreads / 32,
+               152 * std::max(1, std::min(8, (int)(220000 / (one * (kThreads / 32))))) * 4);
         return;
     }
     if (one <= 220000) {   // N <= 117
-        go(trace_pairs_kernel<kThreads>, 1, 152 * std::max(1, std::min(8, (int)(220000 / one))) * 4);
+        go(trace_pairs_kernel<kThreads, kThreads>, kThreads, 1, 152 * std::max(1, std::min(8, (int)(220000 / one))) * 4);
         return;
     }
     dim3 grid(W, nc);
