@@ -14,7 +14,8 @@
 // both factors laid out row-major over (walker, orbital).  The back-propagated trial is
 // re-orthonormalised every k_qr steps, which leaves the estimate unchanged.
 //
-// FP64 on the DFMA pipe (zgemm and the batched inverse) whatever the walker set's precision.
+// FP64 (zgemm and the batched inverse), but for the propagation, the Green's functions and the walker
+// sum of mixed-precision walker sets, which run on the tensor cores.
 #include <algorithm>
 
 #include "state.cuh"

@@ -1,4 +1,5 @@
-// FP64 (DFMA) kernels of the AFQMC walker step: batched complex GEMM, Gauss-Jordan
+// FP64 kernels of the AFQMC walker step: batched complex GEMM (its tensor-core form is in
+// gemm_slices.cu), Gauss-Jordan
 // inverse / log-det, trace epilogue, local energy and force bias, Philox fields,
 // phaseless weights, Gram-Schmidt re-orthonormalisation, estimator reduction.
 //

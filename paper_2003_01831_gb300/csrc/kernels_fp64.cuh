@@ -1,4 +1,4 @@
-// Launch interfaces of the FP64 (DFMA) kernels.  Internal to the library.
+// Launch interfaces of the FP64 kernels.  Internal to the library.
 #pragma once
 
 #include "common.cuh"

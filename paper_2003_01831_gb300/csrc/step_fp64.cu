@@ -1,6 +1,7 @@
 // FP64 walker-step driver: the phaseless AFQMC step (Sec. V; Zhang & Krakauer 2003,
-// Motta & Zhang 2018) as a sequence of DFMA kernels.  This is the precision reference
-// of the GPU path; the tensor-core path (step_tc.cu) replaces its contractions.
+// Motta & Zhang 2018) as a sequence of FP64 kernels, the large products on the tensor cores by exact
+// digit slices (gemm_slices.cu).  This is the precision reference of the GPU path; the mixed path
+// (step_tc.cu) replaces its contractions.
 #include <algorithm>
 
 #include "state.cuh"
