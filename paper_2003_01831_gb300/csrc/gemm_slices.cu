@@ -1014,7 +1014,8 @@ int slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st) {
         const int64_t fit = (int64_t)(ws->bytes / ((p.bytes + 1024) / p.pieces + 1));
         const int64_t share = std::max<int64_t>(1, tc_num_sms() / (p.pair ? 2 : 1) / std::max<int64_t>(p.tiles, 1));
         const int64_t n = fit > share ? fit / share * share : std::max<int64_t>(1, fit);
-        lo.k = (int)std::min<int64_t>(n, p.pieces - 1) * p.klen;
+        // (at least a 64th, which may be cut again: bounds the depth of the cuts)
+        lo.k = (int)std::min<int64_t>(std::max<int64_t>(n, p.pieces / 64), p.pieces - 1) * p.klen;
         hi.k = g.k - lo.k;
         shift(lo.k * (g.A.op == OP_N ? 1 : g.A.ld), lo.k * (g.B.op == OP_N ? g.B.ld : 1), 0, 0);
         lo.D = nullptr;
