@@ -685,8 +685,11 @@ __device__ __forceinline__ void pair_arrive(int id) { asm volatile("bar.arrive %
 // both orders' products with its own T from registers; a warp on the diagonal exchanges within
 // itself.  That halves the shared-memory traffic of exchanging every block, and a pair waits for
 // each other alone: a tile has one barrier of all sixteen warps (with the wait for the accumulators),
-// which also separates this tile's exchange space and sums from the last one's (none for Np = 32,
-// where no warp needs another).  Block rows lie at pitch 33: writes (lanes over rows) and reads
+// which also separates this tile's exchange space and sums from the last one's.  Np = 32 needs none
+// where every tile of the launch is one of Np = 32, since then no warp reads another's block; TOGETHER
+// asks for it where a tile of another size may come before (its readers may still be at the blocks
+// that this tile's warps write) or after (which waits for all sixteen warps, so none may leave
+// alone).  Block rows lie at pitch 33: writes (lanes over rows) and reads
 // (lanes over columns) are free of bank conflicts; so are 16-byte writes at pitch 36, faster for
 // Np = 32 (0.87 -> 0.81 ms below) and slower else (3.63 -> 4.16).
 //
@@ -697,7 +700,7 @@ __device__ __forceinline__ void pair_arrive(int id) { asm volatile("bar.arrive %
 // products: 7.06 -> 5.79); 256, 128, 64: 5.30 -> 3.52; 128, 32, 512: 1.27 -> 0.81.  Barriers in
 // shared memory per pair and per tile instead of the sixteen-warp one, with scales fetched ahead
 // through shared memory, took 12 to 22% longer.
-template <int Np, typename Release>
+template <int Np, bool TOGETHER, typename Release>
 __device__ __forceinline__ bool energy_epilogue_tile(const EnergyShape& es, SharedCtl* ctl, float* xbuf, double* ered,
                                                      int ng, int wg, int part, uint32_t parity, bool d2,
                                                      Release release) {
@@ -734,7 +737,7 @@ __device__ __forceinline__ bool energy_epilogue_tile(const EnergyShape& es, Shar
     const uint32_t tq = ctl->tmem_base + 256u * part + ((uint32_t)(q * 32) << 16);
 
     const bool got = warp_wait(&ctl->tfull[part], parity, &ctl->abort);
-    if (Q == 1) {   // no warp waits for another
+    if (Q == 1 && !TOGETHER) {   // no warp waits for another
         if (!got) return false;
     } else if (!ebar_and(got ? 1 : 0)) {
         return false;                            // all sixteen warps leave together
@@ -1068,8 +1071,8 @@ __device__ __forceinline__ bool energy_epilogue_tile_gen(const EnergyShape& es, 
     return true;
 }
 
-// One tile by the epilogue its Np takes (0: es.Np at run time).
-template <int Np, typename Release>
+// One tile by the epilogue its Np takes (0: es.Np at run time).  TOGETHER: a launch of several Np.
+template <int Np, bool TOGETHER = false, typename Release>
 __device__ __forceinline__ bool energy_epilogue_any(const EnergyShape& es, SharedCtl* ctl, float* xbuf, float* colscale,
                                                     double* ered, int ng, int wg, bool single, Turns& turns,
                                                     Release release) {
@@ -1077,7 +1080,7 @@ __device__ __forceinline__ bool energy_epilogue_any(const EnergyShape& es, Share
     const uint32_t parity = turns.full_parity(part);
     auto done = [&] { release(single, part); };
     if constexpr (Np == 0) return energy_epilogue_tile_gen(es, ctl, xbuf, colscale, ng, wg, part, parity, !single, done);
-    else return energy_epilogue_tile<Np>(es, ctl, xbuf, ered, ng, wg, part, parity, !single, done);
+    else return energy_epilogue_tile<Np, TOGETHER>(es, ctl, xbuf, ered, ng, wg, part, parity, !single, done);
 }
 
 template <int Np, int BK, int AP>
@@ -1373,9 +1376,9 @@ __global__ void __launch_bounds__(kEThreads, 1)
             const bool single = energy_pair_single(es, p.ngp);
             bool ok;
             switch (es.Np) {
-                case 32: ok = energy_epilogue_any<32>(es, ctl, plane, colscale, ered, ng, p.wg, single, turns, release); break;
-                case 64: ok = energy_epilogue_any<64>(es, ctl, plane, colscale, ered, ng, p.wg, single, turns, release); break;
-                case 128: ok = energy_epilogue_any<128>(es, ctl, plane, colscale, ered, ng, p.wg, single, turns, release); break;
+                case 32: ok = energy_epilogue_any<32, true>(es, ctl, plane, colscale, ered, ng, p.wg, single, turns, release); break;
+                case 64: ok = energy_epilogue_any<64, true>(es, ctl, plane, colscale, ered, ng, p.wg, single, turns, release); break;
+                case 128: ok = energy_epilogue_any<128, true>(es, ctl, plane, colscale, ered, ng, p.wg, single, turns, release); break;
                 default: ok = energy_epilogue_any<0>(es, ctl, plane, colscale, ered, ng, p.wg, single, turns, release); break;
             }
             if (!ok) break;
