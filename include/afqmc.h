@@ -53,8 +53,9 @@ extern "C" {
 /* ---- options ----------------------------------------------------------- */
 #define AFQMC_PREC_FP64    0  /* every contraction in FP64: the multiply-add pipe, or for
                                  large products the tensor cores on operands cut into exact
-                                 fp16 digits (58 bits and more below each row's largest
-                                 entry, one rounding per result)                        */
+                                 fp16 digits, each result of which is certified to lie within
+                                 the error bound of the multiply-add loop, (k + 1) 2^-53
+                                 sum |a_k b_k|, or formed by that loop                  */
 #define AFQMC_PREC_BF16X3  1  /* contractions on tcgen05 tensor cores (kind::f16, FP32
                                  accumulation) on operands split into row-scaled fp16
                                  slices whose leading products sum exactly: two slices

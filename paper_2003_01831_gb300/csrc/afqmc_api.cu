@@ -603,6 +603,7 @@ static int init_walkers_impl(afqmc_ham_t ham, int ND, const double* Psi_up, cons
                                     reinterpret_cast<cplx*>(f.Bh), st)
                      : expm_real(ham->hp, -0.5 * tau, M, f.Bh, st);
     if (rc) return bail(rc);
+    fp64_split_propagator(wk, st);
     // trial energy E_T: the trial's energy shift (its variational energy unless two determinants
     // of an expansion are exactly orthogonal; those pairs are left out).  One determinant: its local energy with
     // walker 0 placed at it.  ND determinants: with walker 0 at each D_J in turn, the local

@@ -23,18 +23,17 @@ namespace {
 constexpr int kT = 256;
 inline unsigned nb(int64_t n) { return (unsigned)((n + kT - 1) / kT); }
 
-// T[c][w] -= c_n 1   (c_n = t0[w][n] + t1[w][n]; N x N matrices): U = -Theta T then has its c_n Theta
-// term from the product itself.  Adding that to U, another read and write of all of U, took 0.44 ms
-// of 4 a chunk at M = 128, N = 32, 32 walkers and 384 vectors.
-__global__ void shift_diagonal_kernel(cplx* T, const cplx* t0, const cplx* t1, int W, int nc, int n0, int nch, int N) {
+// c[w][n] = t0[w][n] + t1[w][n] and g_w c[w][n].  The c_n Theta term of U_n = c_n Theta - Theta T_n goes by
+// itself into what U is used for, sum_n c_n L_n (one matrix a walker) times Theta and sum_w g_w c_n Theta_w:
+// inside the product (T_n - c_n 1) its diagonal is far above the rest of the matrix, which the digits of the
+// tensor-core form hold too few bits of (at M = 128, N = 32, 32 walkers: 0.44 ms a product of 64 vectors where
+// c_n is 30 times an entry of T, 0.17 without), and adding it to U is another read and write of all of U.
+__global__ void trace_coefficients_kernel(const cplx* t0, const cplx* t1, const cplx* g, int64_t n, int nch, cplx* c, cplx* gc) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)nc * W * N) return;
-    const int64_t cw = i / N;
-    const int a = (int)(i % N), w = (int)(cw % W);
-    const int64_t ti = (int64_t)w * nch + n0 + cw / W;
-    cplx& d = T[cw * N * N + (int64_t)a * N + a];
-    const cplx cn = t0[ti] + t1[ti];
-    d = cplx{d.re - cn.re, d.im - cn.im};
+    if (i >= n) return;
+    const cplx v = t0[i] + t1[i];
+    c[i] = v;
+    gc[i] = g[i / nch] * v;
 }
 
 // V[c][e] = sum_w g_w U[w][c][e]   (fixed walker order)
@@ -118,11 +117,32 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
         AFQMC_CUDA_TRY(call_alloc(wk->ham, reinterpret_cast<void**>(&dLd), sizeof(double) * (size_t)nch * M * M, st));
         AFQMC_CUDA_TRY(cudaMemsetAsync(dLd, 0, sizeof(double) * (size_t)nch * M * M, st));
     }
+    cplx* gc = nullptr;
+    AFQMC_CUDA_TRY(call_alloc(wk->ham, reinterpret_cast<void**>(&gc), sizeof(cplx) * (size_t)W * nch, st));
+    count_launch();
+    trace_coefficients_kernel<<<nb((int64_t)W * nch), kT, 0, st>>>(f.t[0], f.t[1], gE, (int64_t)W * nch, nch, wk->coef, gc);
+    {   // A_w = sum_n c_n L_n
+        GemmArgs g;
+        g.m = W; g.n = M * M; g.k = nch;
+        g.A.ptr = wk->coef; g.A.ld = nch;
+        g.B.ptr = wk->ham->L; g.B.real = true; g.B.ld = (int64_t)M * M;
+        g.C = f.A; g.ldc = (int64_t)M * M;
+        g.ws = &f.ws;
+        zgemm(g, st);
+    }
     cplx* outs[2] = {dPsi_up, dPsi_dn};
     for (int s = 0; s < 2; ++s) {
         const int N = wk->N[s];
         const int64_t MN = (int64_t)M * N;
-        fill_cplx(G, (int64_t)W * MN, cplx{0.0, 0.0}, st);
+        {   // G_w = A_w^T Theta_w
+            GemmArgs g;
+            g.m = M; g.n = N; g.k = M; g.nb1 = W;
+            g.A.ptr = f.A; g.A.op = OP_T; g.A.ld = M; g.A.s1 = (int64_t)M * M;
+            g.B.ptr = f.Theta[s]; g.B.ld = N; g.B.s1 = MN;
+            g.C = G; g.ldc = N; g.sc1 = MN;
+            g.ws = &f.ws;
+            zgemm(g, st);
+        }
         for (int n0 = 0; n0 < nch; n0 += nu) {
             const int nc = std::min(nu, nch - n0);
             {   // T[c][w] = Lt_{n0+c} Theta_w
@@ -138,9 +158,7 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
                 g.ws = &f.ws;
                 zgemm(g, st);
             }
-            count_launch();
-            shift_diagonal_kernel<<<nb((int64_t)nc * W * N), kT, 0, st>>>(f.T, f.t[0], f.t[1], W, nc, n0, nch, N);
-            {   // U[w][c] = -Theta_w (T[c][w] - c_n 1)
+            {   // U[w][c] = -Theta_w T[c][w]
                 GemmArgs g;
                 g.m = M; g.n = N; g.k = N; g.nb1 = W; g.nb2 = nc;
                 g.A.ptr = f.Theta[s]; g.A.ld = N; g.A.s1 = MN;
@@ -163,6 +181,14 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
             if (want_L) {
                 count_launch();
                 weighted_walker_sum_kernel<<<nb((int64_t)nc * MN), kT, 0, st>>>(U, gE, W, nc, MN, V);
+                GemmArgs v;   // V[c] += sum_w g_w c_n Theta_w
+                v.m = nc; v.n = (int)MN; v.k = W;
+                v.A.ptr = gc + n0; v.A.op = OP_T; v.A.ld = nch;
+                v.B.ptr = f.Theta[s]; v.B.ld = MN;
+                v.beta = cplx{1.0, 0.0};
+                v.C = V; v.ldc = MN;
+                v.ws = &f.ws;
+                zgemm(v, st);
                 GemmArgs g;   // F[c] = V_c Psi^+   [M][M]
                 g.m = M; g.n = M; g.k = N; g.nb1 = nc;
                 g.A.ptr = V; g.A.ld = N; g.A.s1 = MN;
@@ -209,7 +235,7 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
         if (outs[s]) AFQMC_CUDA_TRY(cudaMemcpyAsync(outs[s], gP, sizeof(cplx) * MN, cudaMemcpyDefault, st));
     }
     if (want_L) AFQMC_CUDA_TRY(cudaMemcpyAsync(dL, dLd, sizeof(double) * (size_t)nch * M * M, cudaMemcpyDefault, st));
-    void* frees[] = {U, V, F, G, Z, gP, dLd, gE, gS, dEd, dSd};
+    void* frees[] = {U, V, F, G, Z, gP, gc, dLd, gE, gS, dEd, dSd};
     for (void* p : frees)
         if (p) cudaFreeAsync(p, st);
     AFQMC_CUDA_TRY(cudaStreamSynchronize(st));

@@ -316,6 +316,7 @@ extern "C" int afqmc_debug_gemm(const long long* d, const long long* sizes, cons
     ws.buf = dw.p;
     ws.bytes = (size_t)ws_bytes;
     ws.flags = static_cast<unsigned*>(flags.p);
+    AFQMC_TRY(slice_scratch_init(&ws));
     if (chose) *chose = zgemm_form(g, &ws);
     cudaEvent_t e0, e1;
     AFQMC_CUDA_TRY(cudaEventCreate(&e0));

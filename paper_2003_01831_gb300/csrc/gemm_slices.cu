@@ -4,28 +4,33 @@
 // product of integers small enough to be summed exactly in fp32 is worth some thirty of them for
 // each FP64 one (the splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59 (2012), with
 // digits sized for fp16 operands and fp32 accumulators):
-//   * Every row of an operand (along the contracted index) gets the exponent e of its largest
-//     entry (|x| < 2^e) and each entry is rounded to a fixed-point number of 58 or 59 bits below
-//     2^e, cut into S signed digits d_p of BETA bits (|d_p| <= 2^(BETA-1)), the last with 11 bits
-//     (its fraction bits included): x = 2^(e - BETA + 1) sum_p d_p 2^(-BETA p).  Every digit is
-//     exact in fp16.
+//   * The contraction runs in pieces of at most 128 real products.  Every row of an operand (along
+//     the contracted index) gets, in each piece, the exponent e of its largest entry (|x| < 2^e), and
+//     each entry is rounded to a fixed-point number of 58 bits below 2^e, cut into 7 signed digits
+//     d_p of 8 bits (|d_p| <= 2^7), the last with 11 bits (its fraction bits included): x = 2^(e - 7)
+//     sum_p d_p 2^(-8 p).  Every digit is exact in fp16.
 //   * The products of digits p and q of equal weight p + q = d go to one tensor-memory accumulator
-//     per d < D.  With BETA = 8 for K <= 128 and BETA = 7 for K <= 512 at most 8 x 2^21 bounds
-//     every partial sum, so the accumulators are exact integers (the last one, which the
-//     fractional digits reach, is rounded 24 bits below its own small weight).  Dropped weights
-//     d >= D lie 2^-56 and less below |a||b|.
-//   * The epilogue adds the accumulators as one 64-bit integer (its unit 2^-53 of the product of the
-//     rows' largest entries, or less) and rounds it to FP64 in integer instructions (a few FP64
-//     operations per output would cost as much as the tile's MMAs).
-// The result carries the rounding of its operands to 2^-59 of their rows' largest entries, the
-// dropped weights and one rounding: against a 128-bit sum the error measured is at most that of
-// the multiply-add loop of zgemm_kernel (tests/test_gpu_gemm_slices.py).  Longer contractions run in
-// pieces of at most 512, each with its own exponents, added in FP64.
+//     per d < 8.  At most 8 x 2^21 bounds every partial sum, so the accumulators are exact integers
+//     (the last two, which the fractional digits reach, are rounded 24 bits below their own small
+//     weight).  Dropped weights d >= 8 lie 2^-64 and less below |a||b|.
+//   * The epilogue adds the accumulators as one 64-bit integer and rounds it to FP64 in integer
+//     instructions (a few FP64 operations per output would cost as much as the tile's MMAs).
+// What that loses are the operands' roundings, 2^-59 of their rows' largest entries: next to nothing
+// in a sum that contains products near 2^(ea + eb), the scale of its row and column, but everything
+// in one whose large a_k meet small b_k throughout.  So each output is certified by a lower bound
+// of sum_k |a_k b_k|, the product of the first digits' sizes less half a unit (by mma.sync, while
+// the tensor core works on the tile's digits): where that is at least 2^-4 of 2^(ea + eb), the result lies
+// within (k + 1) 2^-53 sum_k |a_k b_k|, the bound of the multiply-add loop, and the errors measured are
+// a third of that loop's and less.  All other outputs, and the rows and columns that digits cannot hold
+// (infinities, NaN, numbers near the ends of the FP64 range), are listed and formed by the multiply-add
+// loop in a second kernel, over all SMs (in the tile's epilogue they pile up on a few).
+// The rms error / (2^-53 sum |a_k b_k|) of 128 products, of the loop -> of digits (in exact arithmetic;
+// tests/test_gpu_graded_products.py holds the kernels to the loop's): normal entries 0.39 -> 0.05; one operand decaying as e^(-k / 20) 1.1 -> 0.13; entries
+// graded oppositely over 1 to 1e2 0.47 -> 0.13, over 1 to 1e4 and more 0.5 -> 0.5 (by the loop).
 //
 // Complex operands become real ones: a real operand times a complex one has the complex one's re
 // and im as separate rows; two complex operands are contracted over [re | im] rows of the one
 // against the rows [re | -im], [im | re] of the other, the "expanded" one.
-// A NaN or infinity anywhere in a row gives NaN in all of its results.
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -49,21 +54,25 @@ constexpr int kChunk = 32;      // contracted entries per stage (64-byte swizzle
 constexpr int kMaxStages = 3;
 constexpr int kEpiWarps = 16;   // four per tensor-memory lane quadrant, 16 columns each
 constexpr int kThreadsG = 64 + 32 * kEpiWarps;
-constexpr int kNanExp = 1 << 20;   // exponent of a row with a NaN or an infinity
+// A row's word: its exponent times 4 and a bit for each half of the row ([re | im], or the whole row) that
+// is zero throughout.
+constexpr int kLoopExp = 1 << 22;     // exponent of a row that digits cannot hold: its outputs by the loop
+constexpr int kZeroRow = 3;           // word of a row of zeros
+constexpr int kMaxExp = 900;          // sums of two exponents beyond this: by the loop
+constexpr float kEven = 1024.0f;      // certificate: 2^-4 in units of the first digits' products, 2^-14
 
-// K <= 128: eight-bit digits, 7 slices, 28 products; K <= 512: seven bits, 8 slices, 36 products.
-template <int S_>
-struct Digits {
-    static constexpr int S = S_;
-    static constexpr int BETA = S_ == 7 ? 8 : 7;
-    static constexpr int D = S_;                       // accumulators (weights 0 .. D - 1)
-    static constexpr int kTail = 11;                   // bits of the last digit
-    static constexpr int kFrac = kTail - BETA;         // fraction bits of the last digit
-    // fixed-point value v = x 2^(kPoint - e): BETA - 1 bits above the first digit's unit
-    static constexpr int kPoint = BETA - 1 + BETA * (S - 1) + kFrac;
-};
+constexpr int S = 7;                            // digits
+constexpr int BETA = 8;                         // bits of a digit
+constexpr int D = 8;                            // accumulators (weights 0 .. D - 1)
+constexpr int kTail = 11;                       // bits of the last digit
+constexpr int kFrac = kTail - BETA;             // fraction bits of the last digit
+// fixed-point value v = x 2^(kPoint - e): BETA - 1 bits above the first digit's unit
+constexpr int kPoint = BETA - 1 + BETA * (S - 1) + kFrac;
+constexpr int kMaxK = 128;                      // contracted real products of a piece
+constexpr int kMmas = S * (S + 1) / 2 + (S - 1);   // of 16 contracted entries
+
 // A stage of one CTA: the R rows of its tile and the Q rows, or half of them for a CTA pair.
-template <int S, bool PAIR>
+template <bool PAIR>
 struct Stage {
     static constexpr int kQRows = PAIR ? kCols / 2 : kCols;
     static constexpr int kBytes = S * (kRows + kQRows) * kChunk * 2;
@@ -133,9 +142,10 @@ struct PackArgs {
     Div dn, dbatch;            // by n, by nbatch
     int64_t own_rows;          // rows before expansion
     int64_t nbatch;
+    Div dblocks;               // by the blocks of one (piece, batch)
     __half* out;               // [S][pieces][nbatch][own_rows (x 2)][Kp]
     int64_t plane;             // elements per slice
-    int* exps;                 // [pieces][nbatch][own_rows]
+    int* exps;                 // words of the rows [pieces][nbatch][own_rows (x 2)]
     cplx alpha;
 };
 
@@ -150,20 +160,22 @@ __device__ __forceinline__ cplx pack_load(const PackArgs& a, int64_t off) {
     if (a.scale) v = a.real ? cplx{a.alpha.re * v.re, 0.0} : a.alpha * v;
     return v;
 }
+// The exponent field; 1, that of the smallest normal number, for subnormal ones, 0 for zero.
 __device__ __forceinline__ int exp_field(double x) {
-    return (int)(((uint32_t)((unsigned long long)__double_as_longlong(x) >> 32) >> 20) & 0x7ffu);
+    const uint32_t hi = (uint32_t)__double2hiint(x), e = (hi >> 20) & 0x7ffu;
+    return e != 0u ? (int)e : (((hi << 1) | (uint32_t)__double2loint(x)) != 0u ? 1 : 0);
 }
+// Row exponent from the largest field m: largest entry < 2^e.
+__device__ __forceinline__ int row_exp(int m) { return m == 0 ? 0 : (m < 64 || m == 0x7ff ? kLoopExp : m - 1022); }
 
 // The S digits of x at the row exponent e as fp16 bit patterns.
-template <int S>
 __device__ __forceinline__ void digits_of(double x, int e, unsigned short (&d)[S]) {
-    using P = Digits<S>;
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const int E = (int)((b >> 52) & 0x7ffu);
     long long v = 0;
-    if (E != 0 && e != kNanExp) {   // subnormals count as zero
+    if (E != 0 && e != kLoopExp) {   // subnormals are less than half a unit
         const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
-        const int sh = E - 1075 + P::kPoint - e;   // x = m 2^(E - 1075); at most 6
+        const int sh = E - 1075 + kPoint - e;   // x = m 2^(E - 1075); at most 5
         if (sh >= 0) v = (long long)(m << sh);
         else if (sh > -56) v = (long long)((m + (1ull << (-sh - 1))) >> -sh);
         if (b >> 63) v = -v;
@@ -171,144 +183,145 @@ __device__ __forceinline__ void digits_of(double x, int e, unsigned short (&d)[S
     {   // last digit: 11 bits, in units of 2^-kFrac
         const int t = (int)((v + 1024) & 2047) - 1024;
         v = (v - t) >> 11;
-        d[S - 1] = __half_as_ushort(__float2half_rn((float)t * (1.0f / (1 << P::kFrac))));
+        d[S - 1] = __half_as_ushort(__float2half_rn((float)t * (1.0f / (1 << kFrac))));
     }
 #pragma unroll
     for (int p = S - 2; p > 0; --p) {
-        constexpr int h = 1 << (P::BETA - 1);
+        constexpr int h = 1 << (BETA - 1);
         const int t = (int)((v + h) & (2 * h - 1)) - h;
-        v = (v - t) >> P::BETA;
+        v = (v - t) >> BETA;
         d[p] = __half_as_ushort(__float2half_rn((float)t));
     }
     d[0] = __half_as_ushort(__float2half_rn((float)(int)v));
 }
 
-// RB rows per block (8, or 32 of at most 64 entries).  Pass 1 finds each row's exponent, pass 2 takes
-// 2048 entries at a time from shared memory (filled coalesced along whichever index is contiguous,
-// by pass 1 already if the rows fit) and writes the digits, two neighbours per store.  Most calls
-// have a few hundred rows, so a block's chain of loads and digits is the time, not the bytes
-// (8 in and 2 S out per entry): 32 rows a block of any length took 83 us for 1024 complex rows of
-// 3072 (55 now), 25 for 64 x 32 rows of 128 (9), 13 for 90 real rows of 90 (4).
+// RB rows per block (8, or 32 of at most 64 entries).  The rows of one piece are read once, coalesced along
+// whichever index is contiguous, into shared memory; their exponents found; and the digits
+// written, two neighbours per store.  Most calls have a few hundred rows, so a block's chain of
+// loads and digits is the time, not the bytes (8 in, 14 out per entry): 32 rows a block of any length
+// took 83 us for 1024 complex rows of 3072 (55 with 8 rows a block), 25 for 64 x 32 rows of 128 (9), 13 for 90 real
+// rows of 90 (4).
 constexpr int kPackT = 256;
-template <int S, int RB>
+template <int RB>
 __global__ void __launch_bounds__(kPackT) pack_slices_kernel(PackArgs a) {
-    constexpr int KB = 2048 / RB, KS = kPackT / RB;
+    constexpr int KB = RB == 32 ? 64 : kMaxK, KS = kPackT / RB;
     __shared__ cplx tile[RB][KB + 1];
     __shared__ int64_t off[RB];
-    __shared__ int rowexp[RB];
+    __shared__ int rowexp[2][RB];   // of re and im (of both where they share a row)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t r0 = (int64_t)blockIdx.x * RB, bt = blockIdx.y;   // bt = (piece, shared batch)
-    uint32_t piece, sb;
-    a.dbatch.divmod(blockIdx.y, piece, sb);
+    uint32_t btu, blk, piece, sb;
+    a.dblocks.divmod(blockIdx.x, btu, blk);
+    a.dbatch.divmod(btu, piece, sb);
+    const int64_t r0 = (int64_t)blk * RB, bt = btu;   // bt = (piece, shared batch)
     const int kn = min(a.klen, a.k - (int)piece * a.klen);
     if (tid < RB) {
         const int64_t r = r0 + tid;
         uint32_t ob, i;
         a.dn.divmod((uint32_t)r, ob, i);
         off[tid] = r < a.own_rows ? a.shared.at(sb) + a.own.at(ob) + i * a.si + (int64_t)piece * a.klen * a.sk : -1;
-        rowexp[tid] = 0;
+        rowexp[0][tid] = rowexp[1][tid] = 0;
     }
     __syncthreads();
-    const bool once = a.koff <= KB;
     if (a.idx_contig) {
         const int i = tid % RB;
-        int m = 0;
+        int mr = 0, mi = 0;
         if (off[i] >= 0) {
 #pragma unroll 4
             for (int kk = tid / RB; kk < kn; kk += KS) {
                 const cplx v = pack_load(a, off[i] + kk * a.sk);
-                m = max(m, max(exp_field(v.re), exp_field(v.im)));
-                if (once) tile[i][kk] = v;
+                mr = max(mr, exp_field(v.re));
+                mi = max(mi, exp_field(v.im));
+                tile[i][kk] = v;
             }
-            atomicMax(&rowexp[i], m);
+            atomicMax(&rowexp[0][i], mr);
+            if (!a.real) atomicMax(&rowexp[1][i], mi);
         }
     } else {
         for (int i = warp; i < RB; i += kPackT / 32) {
-            int m = 0;
+            int mr = 0, mi = 0;
             if (off[i] >= 0) {
 #pragma unroll 4
                 for (int kk = lane; kk < kn; kk += 32) {
                     const cplx v = pack_load(a, off[i] + kk * a.sk);
-                    m = max(m, max(exp_field(v.re), exp_field(v.im)));
-                    if (once) tile[i][kk] = v;
+                    mr = max(mr, exp_field(v.re));
+                    mi = max(mi, exp_field(v.im));
+                    tile[i][kk] = v;
                 }
             }
-            m = __reduce_max_sync(0xffffffffu, m);
-            if (lane == 0) rowexp[i] = m;
+            mr = __reduce_max_sync(0xffffffffu, mr);
+            mi = __reduce_max_sync(0xffffffffu, mi);
+            if (lane == 0) {
+                rowexp[0][i] = mr;
+                rowexp[1][i] = mi;
+            }
         }
     }
-    if (once) {
+    {
         const int pad = a.koff - kn;   // a few entries
         for (int q = tid; q < RB * pad; q += kPackT) tile[q % RB][kn + q / RB] = cplx{0.0, 0.0};
     }
     __syncthreads();
+    const int ex = a.expand ? 2 : 1;
+    const int64_t rows = a.own_rows * ex;
     if (tid < RB) {
-        const int m = rowexp[tid];
-        const int e = m == 0x7ff ? kNanExp : (m == 0 ? 0 : m - 1022);   // largest entry < 2^e
-        rowexp[tid] = e;
-        if (off[tid] >= 0) a.exps[bt * a.own_rows + r0 + tid] = e;
-    }
-    const int64_t rows = a.own_rows * (a.expand ? 2 : 1);
-    for (int k0 = 0; k0 < a.koff; k0 += KB) {
-        const int kc = min(KB, a.koff - k0);   // even, as koff is
-        __syncthreads();
-        if (!once) {
-            if (a.idx_contig) {
-                const int i = tid % RB;
-#pragma unroll 4
-                for (int kk = tid / RB; kk < kc; kk += KS) {
-                    cplx v{0.0, 0.0};
-                    if (off[i] >= 0 && k0 + kk < kn) v = pack_load(a, off[i] + (k0 + kk) * a.sk);
-                    tile[i][kk] = v;
-                }
-            } else {
-                for (int i = warp; i < RB; i += kPackT / 32) {
-#pragma unroll 4
-                    for (int kk = lane; kk < kc; kk += 32) {
-                        cplx v{0.0, 0.0};
-                        if (off[i] >= 0 && k0 + kk < kn) v = pack_load(a, off[i] + (k0 + kk) * a.sk);
-                        tile[i][kk] = v;
-                    }
-                }
-            }
-            __syncthreads();
+        int mr = rowexp[0][tid], mi = rowexp[1][tid];
+        int zr = mr == 0 ? 3 : 0, zi = mi == 0 ? 3 : 0;   // the zero halves of the rows of re and of im
+        if (a.parts == 2) {
+            const int re = mr == 0, im = mi == 0;
+            zr = re | im << 1;
+            zi = im | re << 1;
+            mr = mi = max(mr, mi);
         }
-        const int half = kc / 2;
+        const int er = row_exp(mr), ei = row_exp(mi);
+        rowexp[0][tid] = er;
+        rowexp[1][tid] = ei;
+        if (off[tid] >= 0) {
+            int* e = a.exps + bt * rows + ex * (r0 + tid);
+            e[0] = 4 * er + zr;
+            if (a.expand) e[1] = 4 * ei + zi;
+        }
+    }
+    __syncthreads();
+    const int half = a.koff / 2;   // koff is even
 #pragma unroll 1
-        for (int q = tid; q < RB * half; q += kPackT) {
-            const int i = q / half, kk = 2 * (q - i * half);
-            if (off[i] < 0) break;
-            const int e = rowexp[i];
-            const cplx v0 = tile[i][kk], v1 = tile[i][kk + 1];
-            unsigned short x[S], y[S];
-            unsigned re[S], im[S];
-            digits_of<S>(v0.re, e, x);
-            digits_of<S>(v1.re, e, y);
+    for (int q = tid; q < RB * half; q += kPackT) {
+        const int i = q / half, kk = 2 * (q - i * half);
+        if (off[i] < 0) break;
+        const cplx v0 = tile[i][kk], v1 = tile[i][kk + 1];
+        unsigned short x[S], y[S];
+        unsigned re[S], im[S];
+        digits_of(v0.re, rowexp[0][i], x);
+        digits_of(v1.re, rowexp[0][i], y);
 #pragma unroll
-            for (int p = 0; p < S; ++p) re[p] = (unsigned)x[p] | ((unsigned)y[p] << 16);
-            if (!a.real) {
-                digits_of<S>(v0.im, e, x);
-                digits_of<S>(v1.im, e, y);
+        for (int p = 0; p < S; ++p) re[p] = (unsigned)x[p] | ((unsigned)y[p] << 16);
+        if (!a.real) {
+            digits_of(v0.im, rowexp[1][i], x);
+            digits_of(v1.im, rowexp[1][i], y);
 #pragma unroll
-                for (int p = 0; p < S; ++p) im[p] = (unsigned)x[p] | ((unsigned)y[p] << 16);
-            }
-            const int64_t r = r0 + i;
-            const int64_t row = (bt * rows + (a.expand ? 2 * r : r)) * a.Kp + k0 + kk;
+            for (int p = 0; p < S; ++p) im[p] = (unsigned)x[p] | ((unsigned)y[p] << 16);
+        }
+        const int64_t row = (bt * rows + ex * (r0 + i)) * a.Kp + kk;
 #pragma unroll
-            for (int p = 0; p < S; ++p) {
-                __half* o = a.out + p * a.plane + row;
-                *reinterpret_cast<unsigned*>(o) = re[p];
-                if (a.real) continue;
-                if (a.parts == 2) *reinterpret_cast<unsigned*>(o + a.koff) = a.expand ? im[p] ^ 0x80008000u : im[p];
-                if (a.expand) {
-                    *reinterpret_cast<unsigned*>(o + a.Kp) = im[p];
-                    if (a.parts == 2) *reinterpret_cast<unsigned*>(o + a.Kp + a.koff) = re[p];
-                }
+        for (int p = 0; p < S; ++p) {
+            __half* o = a.out + p * a.plane + row;
+            *reinterpret_cast<unsigned*>(o) = re[p];
+            if (a.real) continue;
+            if (a.parts == 2) *reinterpret_cast<unsigned*>(o + a.koff) = a.expand ? im[p] ^ 0x80008000u : im[p];
+            if (a.expand) {
+                *reinterpret_cast<unsigned*>(o + a.Kp) = im[p];
+                if (a.parts == 2) *reinterpret_cast<unsigned*>(o + a.Kp + a.koff) = re[p];
             }
         }
     }
 }
 
+// An operand as the multiply-add loop reads it.
+struct Source {
+    const void* ptr;
+    int real, conj;
+    int64_t si, sk;
+    Strides own, shared;
+};
 struct OutArgs {
     int64_t rows, cols;        // per batch, after expansion
     int rexp, cexp;            // which side is expanded (at most one)
@@ -317,7 +330,15 @@ struct OutArgs {
     Strides rown, cown, shared;    // output strides of the batch dimensions
     Strides drown, dcown, dshared;
     int64_t drs, dcs;
-    const int *er, *ec;        // exponents [pieces][nbatch][rows before expansion]
+    const int *er, *ec;        // words of the rows and columns [pieces][nbatch][rows]
+    const __half *dr, *dc;     // their first digits [pieces][nbatch][rows][Kp]
+    int Kp;
+    // for the outputs by the multiply-add loop: the operands of the rows and of the columns
+    Source srow, scol;
+    int k, klen;
+    cplx alpha;
+    uint32_t *list, *head;     // pairs of outputs for the loop (see slice_gemm_kernel), [entries listed, CTAs done]
+    uint32_t room;
     cplx *C, *D;
     double beta;
     int64_t tiles;             // row tiles x column tiles x batches
@@ -342,30 +363,21 @@ struct Ctl {
     int abort;
 };
 
-// FP64 value of I 2^x, rounded to nearest.  The common case, a result well inside the exponent range
-// with |I| >= 2^32, takes one count of leading zeros and two funnel shifts; the other (small and zero
-// I; x beyond the range: 0, infinity or, from a row marked kNanExp, NaN) is out of line.
-__device__ __noinline__ double round64_rare(unsigned hi0, unsigned lo0, unsigned sign, int x) {
-    const unsigned long long X0 = ((unsigned long long)hi0 << 32) | lo0;
-    if (x > kNanExp / 2) return __longlong_as_double(0x7ff8000000000000ll);
-    if (X0 == 0) return 0.0;
-    const int lz = __clzll((long long)X0);
-    const unsigned long long X = X0 << lz, m = (X >> 11) + ((X >> 10) & 1ull);   // 2^52 .. 2^53
-    const int eb = 1023 + 63 - lz + x;
-    const unsigned long long r = eb < 1 ? 0ull : (eb > 2046 ? 0x7ff0000000000000ull : ((unsigned long long)(eb - 1) << 52) + m);
-    return __longlong_as_double((long long)(r | ((unsigned long long)sign << 32)));
-}
+// FP64 value of I 2^x, rounded to nearest; x is such that the result is zero or well inside the exponent
+// range.
 __device__ __forceinline__ double round64(long long I, int x) {
     const int s = (int)(I >> 63);
     const unsigned long long X = (unsigned long long)((I ^ s) - s);
-    const unsigned hi0 = (unsigned)(X >> 32), lo0 = (unsigned)X, sign = (unsigned)s & 0x80000000u;
-    const int lz = __clz((int)hi0);
-    const int eb1 = 1023 + 63 - 1 + x - lz;   // biased exponent - 1
-    if (hi0 == 0u || (unsigned)eb1 > 2045u) return round64_rare(hi0, lo0, sign, x);
-    const unsigned hi = __funnelshift_l(lo0, hi0, lz), lo = lo0 << lz;
+    const unsigned sign = (unsigned)s & 0x80000000u;
+    const bool big = (X >> 32) != 0ull;
+    const unsigned h = big ? (unsigned)(X >> 32) : (unsigned)X, l = big ? (unsigned)X : 0u;
+    const int lz = __clz((int)h);
+    const int eb1 = (big ? 1023 + 63 - 1 : 1023 + 31 - 1) + x - lz;   // biased exponent - 1
+    const unsigned hi = __funnelshift_l(l, h, lz), lo = l << lz;
     // bits 63 .. 11 plus the rounding bit; the leading one carries into the exponent field
     const unsigned long long m = (((unsigned long long)(hi >> 11) << 32) | __funnelshift_r(lo, hi, 11)) + ((lo >> 10) & 1u);
-    return __hiloint2double((int)(((unsigned)(m >> 32) + ((unsigned)eb1 << 20)) | sign), (int)(unsigned)m);
+    const unsigned top = ((unsigned)(m >> 32) + ((unsigned)eb1 << 20)) | sign;
+    return __hiloint2double(h != 0u ? (int)top : 0, (int)(unsigned)m);
 }
 
 // Barrier of the epilogue warps with the conjunction of `pred`.
@@ -382,29 +394,225 @@ __device__ __forceinline__ int epi_and(int pred) {
     return r;
 }
 
-// One output's accumulators a_d 2^(-BETA d) as an integer in units of 2^-kGather of accumulator 0's:
-// 62 or 63 bits, the lowest 2^-54 (S = 7) or 2^-53 (S = 8) of the product of the rows' largest
-// entries.  Every sum below is exact but the last, of the two smallest accumulators.
-template <int S>
-struct Gather {
-    static constexpr int kPoint = S == 7 ? 40 : 41;
-    __device__ static long long of(const uint32_t (&a)[S][8], int j) {
-        auto f = [&](int d) { return __uint_as_float(a[d][j]); };
-        auto in = [&](int d) { return __float2int_rn(f(d)); };
-        if (S == 7) {   // BETA = 8: a0 2^40 + a1 2^32 + ... + a5 + a6 2^-8
-            long long I = (long long)((in(0) << 8) + in(1)) << 32;
-            I += (long long)((in(2) << 8) + in(3)) * 65536;
-            I += (long long)in(4) * 256;
-            return I + __float2int_rn(fmaf(f(6), 0x1p-8f, f(5)));
+// Eight outputs' accumulators a_d 2^(-8 d) as integers in units of 2^-kGather of accumulator 0's, 2^-55 of
+// the scale 2^(ea + eb); below 2^53 of them (a quarter of the scale) in units 2^-8 of that, whose bit in
+// `fine` is set.  Every sum is exact but that of the two smallest accumulators.  Two accumulators at a
+// time, to hold few of them in registers.  Conversion to integers by adding 1.5 2^23, which leaves the
+// integer in the low bits (the conversion instruction has an eighth of the rate and took half of the time
+// that tensor memory waits for its readers); beyond 2^22, which only accumulators 2 to 5 of all but equal
+// entries reach, by the instruction.
+constexpr int kGather = 41;
+constexpr float kMagic = 12582912.0f;
+constexpr int kMagicBits = 0x4b400000;
+template <int STEP>
+__device__ __forceinline__ void gather(long long (&I)[16], int c0, const uint32_t (&a)[2][8], unsigned& fine) {
+    auto f = [&](int d, int j) { return __uint_as_float(a[d][j]); };
+    if (STEP < 3) {   // a0 2^41 + a1 2^33, a2 2^25 + a3 2^17, a4 2^9 + a5 2
+        int top[8];
+        unsigned over = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int r0 = __float_as_int(f(0, j) + kMagic), r1 = __float_as_int(f(1, j) + kMagic);
+            over |= (unsigned)((r0 ^ kMagicBits) | (r1 ^ kMagicBits));
+            top[j] = (int)(((unsigned)(r0 - kMagicBits) << 8) + (unsigned)(r1 - kMagicBits));
         }
-        // BETA = 7: a0 2^41 + a1 2^34 + ... + a6 2^-1 + a7 2^-8
-        long long I = (long long)((in(0) << 7) + in(1)) << 34;
-        I += (long long)((in(2) << 7) + in(3)) * (1 << 20);
-        I += (long long)in(4) * (1 << 13);
-        I += (long long)in(5) * 64;
-        return I + __float2int_rn(0.5f * fmaf(f(S - 1), 0x1p-7f, f(6)));
+        if (STEP > 0 && (over >> 23) != 0u) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) top[j] = (__float2int_rn(f(0, j)) << 8) + __float2int_rn(f(1, j));
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (STEP == 0) I[c0 + j] = (long long)top[j] << 33;
+            else I[c0 + j] += (long long)top[j] * (STEP == 1 ? 1 << 17 : 2);
+        }
+    } else {          // a6 2^-7 + a7 2^-15
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float s = fmaf(f(1, j), 0x1p-15f, f(0, j) * 0x1p-7f), m = s + kMagic;
+            long long v = I[c0 + j] + (__float_as_int(m) - kMagicBits);
+            const int hi = (int)(v >> 32);
+            if ((unsigned)(hi ^ (hi >> 31)) < 1u << 21) {
+                v = v * 256 + (__float_as_int(fmaf(s - (m - kMagic), 256.0f, kMagic)) - kMagicBits);
+                fine |= 1u << (c0 + j);
+            }
+            I[c0 + j] = v;
+        }
     }
-};
+}
+
+// Bit j: the certificate of this lane's row and column 16 h + j, for the warp's 32 rows from r0 and 16 columns
+// from c0 (rows and columns past the last repeat that, unused).  A lane of a quad takes eight entries of every 32
+// of a row or column, the same ones of both.  The sums only grow: where entries are alike 32 of them are
+// enough for all outputs, and the rest is left out (mma.sync keeps the tensor core from the tile's MMAs: all 128
+// cost 20% of the kernel's time).
+__device__ __forceinline__ void mma_sync(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                         uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t digit_size(uint32_t d) {   // max(|d| - 1/2, 0) of two digits
+    const uint32_t a = d & 0x7fff7fffu;
+    uint32_t r;
+    asm("fma.rn.relu.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(0x3c003c00u), "r"(0xb800b800u));
+    return r;
+}
+__device__ __forceinline__ unsigned certificates(const OutArgs& o, int64_t z, int64_t r0, int64_t c0) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const __half *x[4], *y[2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = o.dr + (z * o.rows + min(r0 + 8 * i + g, o.rows - 1)) * o.Kp + 8 * t;
+#pragma unroll
+    for (int n = 0; n < 2; ++n) y[n] = o.dc + (z * o.cols + min(c0 + 8 * n + g, o.cols - 1)) * o.Kp + 8 * t;
+    float d[2][2][4] = {};
+    for (int k = 0; k < o.Kp; k += 32) {
+        uint4 a[4], b[2];
+        const bool in = k + 8 * t < o.Kp;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] = in ? __ldg(reinterpret_cast<const uint4*>(x[i] + k)) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int n = 0; n < 2; ++n) b[n] = in ? __ldg(reinterpret_cast<const uint4*>(y[n] + k)) : make_uint4(0u, 0u, 0u, 0u);
+        auto size = [](uint4& v) { v = make_uint4(digit_size(v.x), digit_size(v.y), digit_size(v.z), digit_size(v.w)); };
+#pragma unroll
+        for (int i = 0; i < 4; ++i) size(a[i]);
+#pragma unroll
+        for (int n = 0; n < 2; ++n) size(b[n]);
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                mma_sync(d[m][n], a[2 * m].x, a[2 * m + 1].x, a[2 * m].y, a[2 * m + 1].y, b[n].x, b[n].y);
+                mma_sync(d[m][n], a[2 * m].z, a[2 * m + 1].z, a[2 * m].w, a[2 * m + 1].w, b[n].z, b[n].w);
+            }
+        float least = d[0][0][0];
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int n = 0; n < 2; ++n)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) least = fminf(least, d[m][n][c]);
+        if (__all_sync(0xffffffffu, least >= kEven)) return 0xffffu;
+    }
+    // element c of d[m][n]: row 16 m + 8 (c / 2) + g, column 8 n + 2 t + c % 2; to row = lane
+    unsigned even = 0;
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const unsigned b0 = __ballot_sync(0xffffffffu, d[0][n][c] >= kEven), b1 = __ballot_sync(0xffffffffu, d[0][n][2 + c] >= kEven);
+            const unsigned b2 = __ballot_sync(0xffffffffu, d[1][n][c] >= kEven), b3 = __ballot_sync(0xffffffffu, d[1][n][2 + c] >= kEven);
+            const unsigned w = lane < 16 ? (lane < 8 ? b0 : b1) : (lane < 24 ? b2 : b3);
+            unsigned v = (w >> (4 * (lane & 7))) & 15u;
+            v = (v | v << 2) & 0x33u;
+            v = (v | v << 1) & 0x55u;
+            even |= v << (8 * n + c);
+        }
+    return even;
+}
+// Whether the digits' result stands, from the words of its row and column and the certificate: a sum of zeros
+// is exact, the rest needs the certificate and room around the result.
+__device__ __forceinline__ bool stands(int wr, int wc, bool even) {
+    const int x = (wr >> 2) + (wc >> 2);
+    return abs(x) <= kMaxExp ? even || ((wr | wc) & 3) == 3 : false;
+}
+
+// The outputs of row r and columns c, c + 1 (batch b) by the multiply-add loop over contracted entries k0
+// .. k1 - 1, as real sums of real products: which parts of the row's and the columns' elements meet is the
+// form's; turn: times i (of the side with separate parts).  lane < 0: by one thread; else by the warp, entries lane, lane + 32, ... in each lane, and all lanes return
+// the sums.
+enum Form { kReal, kRowParts, kColParts, kRowComplex, kColComplex };   // the side whose re and im are separate rows
+__device__ __forceinline__ double flip(double x, bool neg) {   // -x, off the FP64 pipe
+    return __hiloint2double(__double2hiint(x) ^ (neg ? 0x80000000 : 0), __double2loint(x));
+}
+template <bool REAL>
+__device__ __forceinline__ cplx source_load(const Source& s, int64_t at) {
+    if (REAL) return cplx{__ldg(static_cast<const double*>(s.ptr) + at), 0.0};
+    const double2 v = __ldg(static_cast<const double2*>(s.ptr) + at);
+    return cplx{v.x, flip(v.y, s.conj)};
+}
+template <int FORM>
+__device__ __forceinline__ double2 loop_form(const OutArgs& o, int64_t ix, int64_t iy, int64_t iy1, int kn, bool odd, int lane,
+                                             bool turn) {
+    constexpr bool ROWS = FORM == kRowParts || FORM == kRowComplex, COLS = FORM == kColParts || FORM == kColComplex;
+    constexpr bool XR = FORM == kReal || FORM == kColParts, YR = FORM == kReal || FORM == kRowParts;
+    const Source &X = o.srow, &Y = o.scol;
+    const int first = lane < 0 ? 0 : lane, step = lane < 0 ? 1 : 32;
+    const int64_t sx = step * X.sk, sy = step * Y.sk;
+    ix += first * X.sk;
+    iy += first * Y.sk;
+    iy1 += first * Y.sk;
+    auto scaled = [&](cplx v) { return turn ? cplx{flip(v.im, true), v.re} : v; };
+    auto mac = [&](double2& z, cplx x, cplx y, cplx y1) {
+        if (ROWS) x = scaled(x);
+        if (COLS) y = scaled(y);
+        double u = x.re, v = x.im;
+        if (ROWS) u = odd ? x.im : x.re;
+        if (FORM == kRowComplex) v = odd ? x.re : flip(x.im, true);
+        z.x = fma(u, y.re, z.x);
+        z.y = fma(u, COLS ? y.im : y1.re, z.y);
+        if (FORM == kRowComplex) {
+            z.x = fma(v, y.im, z.x);
+            z.y = fma(v, y1.im, z.y);
+        } else if (FORM == kColComplex) {
+            z.x = fma(-v, y.im, z.x);
+            z.y = fma(v, y.re, z.y);
+        }
+    };
+    double2 s[4] = {};   // four sums: shorter chains, and fewer roundings in each
+    int k = first;
+    for (; k + 3 * step < kn; k += 4 * step, ix += 4 * sx, iy += 4 * sy, iy1 += 4 * sy) {
+        cplx x[4], y[4], y1[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            x[u] = source_load<XR>(X, ix + u * sx);
+            y[u] = source_load<YR>(Y, iy + u * sy);
+            if (!COLS) y1[u] = source_load<YR>(Y, iy1 + u * sy);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) mac(s[u], x[u], y[u], COLS ? cplx{0.0, 0.0} : y1[u]);
+    }
+    for (; k < kn; k += step, ix += sx, iy += sy, iy1 += sy)
+        mac(s[0], source_load<XR>(X, ix), source_load<YR>(Y, iy), COLS ? cplx{0.0, 0.0} : source_load<YR>(Y, iy1));
+    double2 z = make_double2((s[0].x + s[1].x) + (s[2].x + s[3].x), (s[0].y + s[1].y) + (s[2].y + s[3].y));
+    if (lane >= 0) {
+#pragma unroll
+        for (int h = 16; h > 0; h >>= 1) {
+            z.x += __shfl_xor_sync(0xffffffffu, z.x, h);
+            z.y += __shfl_xor_sync(0xffffffffu, z.y, h);
+        }
+    }
+    return z;
+}
+__device__ __forceinline__ double2 loop_pair(const OutArgs& o, uint32_t b, int k0, int k1, uint32_t r, uint32_t c, int lane) {
+    uint32_t q, i;
+    o.rn.divmod(o.rexp ? r >> 1 : r, q, i);
+    const int64_t ix = o.srow.shared.at(b) + o.srow.own.at(q) + i * o.srow.si + k0 * o.srow.sk;
+    auto col = [&](uint32_t cc) {
+        o.cn.divmod(cc, q, i);
+        return o.scol.shared.at(b) + o.scol.own.at(q) + i * o.scol.si + k0 * o.scol.sk;
+    };
+    const int64_t iy = col(o.cexp ? c >> 1 : c), iy1 = o.cexp || c + 1 >= o.cols ? iy : col(c + 1);
+    const int kn = k1 - k0;
+    const bool odd = r & 1u;
+    auto sums = [&](bool turn) {
+        if (o.cexp)
+            return o.srow.real ? loop_form<kColParts>(o, ix, iy, iy1, kn, odd, lane, turn)
+                               : loop_form<kColComplex>(o, ix, iy, iy1, kn, odd, lane, turn);
+        if (o.rexp)
+            return o.scol.real ? loop_form<kRowParts>(o, ix, iy, iy1, kn, odd, lane, turn)
+                               : loop_form<kRowComplex>(o, ix, iy, iy1, kn, odd, lane, turn);
+        return loop_form<kReal>(o, ix, iy, iy1, kn, odd, lane, false);
+    };
+    double2 z = make_double2(0.0, 0.0);
+#pragma unroll 1
+    for (int part = 0; part < 2; ++part) {   // alpha = a + i b: most often one of them
+        const double a = part ? o.alpha.im : o.alpha.re;
+        if (a == 0.0 && !(part == 0 && o.alpha.im == 0.0)) continue;
+        const double2 v = sums(part == 1);
+        z = make_double2(fma(a, v.x, z.x), fma(a, v.y, z.y));
+    }
+    return z;
+}
 
 // Where a thread's results go: its row's offsets, the tile's column tables.
 struct RowOut {
@@ -452,8 +660,23 @@ __device__ __forceinline__ void store_pair(const OutArgs& o, const RowOut& r, co
     }
 }
 
+// z0, z1 added to what store_pair stored.
+__device__ __forceinline__ void add_pair(const OutArgs& o, const RowOut& r, const int64_t* coff, const int64_t* cdof, int c,
+                                         double z0, double z1) {
+    double* C = reinterpret_cast<double*>(o.C);
+    double* D = reinterpret_cast<double*>(o.D);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int e = o.cexp ? c : c + q, part = o.cexp ? q : r.comp;
+        if (coff[e] < 0) return;
+        const double z = q == 0 ? z0 : z1;
+        C[2 * (r.roff + coff[e]) + part] += z;
+        if (o.D) D[2 * (r.rdof + cdof[e]) + part] += z;
+    }
+}
+
 // One persistent CTA per SM: warp 0 loads stages of all slices of both operands (one TMA copy
-// each), warp 1 issues the S (S + 1) / 2 MMAs (N = 64) of every 16 contracted entries, the
+// each), warp 1 issues the 34 MMAs (N = 64) of every 16 contracted entries, the
 // other sixteen warps turn the accumulators into FP64.  An N of 64 leaves the tensor core waiting
 // for shared memory (47 cycles an MMA of 128 rows, 32 of them its products); a wider tile
 // has no room for its accumulators.  PAIR: two CTAs take two neighbouring row tiles with one MMA of
@@ -461,19 +684,22 @@ __device__ __forceinline__ void store_pair(const OutArgs& o, const RowOut& r, co
 // for both, in stages that leave room for a third.  For lack of tensor memory the accumulators
 // have one buffer: the epilogue first folds each output's accumulators into a 64-bit integer in
 // registers, releases tensor memory, and rounds and stores while the next tile's products run.
-// MULTI: the contracted index in several pieces, whose rounded results are added in registers.
-// Measured (T_n = Ltilde_n Theta of M = 128, N = 32, 64 vectors x 512 walkers): 14.3 ms by
-// the multiply-add tiles, 0.54 ms here without pairs (80 cycles an MMA before A stayed in the
-// collector and one elected lane issued from uniform registers), 0.48 ms with them; of a tile's
-// 17600 cycles without pairs 10500 issued MMAs, 2750 waited for copies and 3200 for the
-// accumulators to be read.  Copies of 128-byte rows (two slices side by side) and more, shorter stages
-// gained nothing (0.55, 0.68 ms).
-template <int S, bool MULTI, bool PAIR>
+// MULTI: the contracted index in several pieces, whose rounded results are added in registers.  While the
+// MMAs of a tile or piece run, the epilogue warps certify its outputs (see the top of the file) and list
+// those that do not stand (a pair of columns with one is left out; its other pieces are added up all the same).
+// Measured (T_n = Ltilde_n Theta of M = 128, N = 32, 64 vectors x 512 walkers): 14.3 ms by the
+// multiply-add tiles, 0.54 ms here (0.45 with 28 products of digits and no certificates, whose errors were
+// at the loop's and, in graded sums, far above); of a tile's 17900 cycles 10700 issue MMAs, 2700 wait
+// for copies and 4400 for the accumulators to be read, while the epilogue warps take 2400 for the certificates
+// and 7000 for rounding.  Contractions of several pieces are bound by these epilogues (N = 32, K = 128
+// complex, 682 vectors x 48 walkers: 1.18 ms, 0.93 when a piece held 512 entries).
+// Copies of 128-byte rows (two slices side by side) and more, shorter stages gained nothing (0.55, 0.68 ms when
+// it was 0.54 without pairs).
+template <bool MULTI, bool PAIR>
 __global__ void __launch_bounds__(kThreadsG, 1)
-    slice_gemm_kernel(const __grid_constant__ CUtensorMap tR, const __grid_constant__ CUtensorMap tQ, OutArgs o,
-                      unsigned* flags) {
-    using P = Digits<S>;
-    using St = Stage<S, PAIR>;
+    slice_gemm_kernel(const __grid_constant__ CUtensorMap tR, const __grid_constant__ CUtensorMap tQ,
+                      const __grid_constant__ OutArgs o, unsigned* flags) {
+    using St = Stage<PAIR>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sbase = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     Ctl* ctl = reinterpret_cast<Ctl*>(sbase + St::kCount * St::kBytes);
@@ -580,17 +806,20 @@ __global__ void __launch_bounds__(kThreadsG, 1)
 #pragma unroll
                         for (int kk = 0; kk < kChunk / 16; ++kk)
 #pragma unroll
-                            for (int p = 0; p < S; ++p)   // slice p of R stays in the collector
+                            for (int p = 0; p < S; ++p) {   // slice p of R stays in the collector
+                                const int last = p + S < D ? p + S - 1 : D - 1;
 #pragma unroll
-                                for (int d = p; d < P::D; ++d) {
-                                    const uint32_t D = tmem + d * kCols, a = sr + ((p * kRows * kChunk * 2 + kk * 32) >> 4),
+                                for (int d = p; d <= last; ++d) {
+                                    // accumulator d begins with slice 0, the last one with slice 1
+                                    const bool begun = kk != 0 || p != (d < S ? 0 : d - S + 1);
+                                    const uint32_t dst = tmem + d * kCols, a = sr + ((p * kRows * kChunk * 2 + kk * 32) >> 4),
                                                    b = sq + (((d - p) * St::kQRows * kChunk * 2 + kk * 32) >> 4),
-                                                   acc = (kk | p) != 0 ? 1u : (kb != 0 ? 1u : 0u);
-                                    if (p == S - 1) mma_f16_lo<kKeepNone, PAIR>(D, a, b, hi0, idesc, acc);
-                                    else if (d == p) mma_f16_lo<kKeepFirst, PAIR>(D, a, b, hi0, idesc, acc);
-                                    else if (d < P::D - 1) mma_f16_lo<kKeepMore, PAIR>(D, a, b, hi0, idesc, acc);
-                                    else mma_f16_lo<kKeepLast, PAIR>(D, a, b, hi0, idesc, acc);
+                                                   acc = begun ? 1u : (kb != 0 ? 1u : 0u);
+                                    if (d == p) mma_f16_lo<kKeepFirst, PAIR>(dst, a, b, hi0, idesc, acc);
+                                    else if (d < last) mma_f16_lo<kKeepMore, PAIR>(dst, a, b, hi0, idesc, acc);
+                                    else mma_f16_lo<kKeepLast, PAIR>(dst, a, b, hi0, idesc, acc);
                                 }
+                            }
                         if (PAIR) mma_commit_pair(&ctl->empty[st], 3);   // free in both CTAs
                         else mma_commit(&ctl->empty[st]);
                     }
@@ -616,7 +845,7 @@ __global__ void __launch_bounds__(kThreadsG, 1)
         const int et = threadIdx.x - 64;
         const uint32_t tq = ctl->tmem_base + ((uint32_t)(q * 32) << 16) + 16 * h;
         const int rx = o.rexp ? 1 : 0, cx = o.cexp ? 1 : 0;
-        constexpr int kShift = -2 * (P::BETA - 1) - Gather<S>::kPoint;
+        constexpr int kShift = -2 * (BETA - 1) - kGather;
         int it = 0;
         bool ok = true;
         for (uint32_t w = first; w < work && ok; w += stride) {
@@ -633,6 +862,7 @@ __global__ void __launch_bounds__(kThreadsG, 1)
             ro.rdof = ro.ok && o.D ? o.dshared.at(b) + o.drown.at(ob) + i * o.drs : 0;
             if (MULTI && ro.ok) ro.roff += grp * o.gstride;
             ro.comp = o.rexp ? (int)(r & 1) : 0;
+            unsigned redo = 0;   // pairs of outputs of which some piece does not stand
             double acc[MULTI ? 16 : 1];
             if (MULTI) {
 #pragma unroll
@@ -652,9 +882,11 @@ __global__ void __launch_bounds__(kThreadsG, 1)
                     o.cn.divmod(ci, cob, cj);
                     coff[et] = in ? o.cown.at(cob) + cj * o.cs : -1;
                     cdof[et] = in && o.D ? o.dcown.at(cob) + cj * o.dcs : 0;
-                    cexp[et] = in ? o.ec[z * (o.cols >> cx) + ci] : 0;
+                    cexp[et] = in ? o.ec[z * o.cols + c] : kZeroRow;
                 }
-                const int er = ro.ok ? o.er[z * (o.rows >> rx) + ri] : 0;
+                const int er = ro.ok ? o.er[z * o.rows + r] : kZeroRow;
+                __syncwarp();
+                const unsigned even = certificates(o, z, r - lane, (int64_t)ct * kCols + 16 * h);
                 int got = 1;
                 if (lane == 0) got = mbar_wait(&ctl->tfull, (uint32_t)it & 1u, &ctl->abort) ? 1 : 0;
                 got = __shfl_sync(0xffffffffu, got, 0);
@@ -663,47 +895,69 @@ __global__ void __launch_bounds__(kThreadsG, 1)
                 // so two sets suffice.)
                 if (!epi_and(got)) { ok = false; break; }
                 tc_fence_after();
-                auto value = [&](int j, long long I) { return round64(I, er + cexp[16 * h + j] + kShift); };
-                auto release = [&]() {   // every accumulator of this warp is in registers
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) {
-                        if (PAIR) mbar_arrive_cluster_relaxed(mapa_shared(&ctl->tempty, 0));
-                        else mbar_arrive(&ctl->tempty);
-                    }
-                };
-                if (MULTI) {
+                long long I[16];
+                unsigned fine = 0;
 #pragma unroll
-                    for (int c8 = 0; c8 < 2; ++c8) {
-                        uint32_t a[S][8];
-#pragma unroll
-                        for (int d = 0; d < S; ++d) tmem_ld8_nw(tq + d * kCols + 8 * c8, a[d]);
+                for (int c8 = 0; c8 < 16; c8 += 8) {
+                    uint32_t a[2][8];
+                    auto load = [&](int d) {
+                        tmem_ld8_nw(tq + d * kCols + c8, a[0]);
+                        tmem_ld8_nw(tq + (d + 1) * kCols + c8, a[1]);
                         tmem_ld_wait();
-                        if (c8 == 1) release();
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            acc[MULTI ? 8 * c8 + j : 0] += value(8 * c8 + j, Gather<S>::of(a, j));
+                    };
+                    load(0);
+                    gather<0>(I, c8, a, fine);
+                    load(2);
+                    gather<1>(I, c8, a, fine);
+                    load(4);
+                    gather<2>(I, c8, a, fine);
+                    load(6);
+                    if (c8 == 8) {   // every accumulator of this warp is in registers
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) {
+                            if (PAIR) mbar_arrive_cluster_relaxed(mapa_shared(&ctl->tempty, 0));
+                            else mbar_arrive(&ctl->tempty);
                         }
                     }
-                    if (pc + 1 < p1) continue;
+                    gather<3>(I, c8, a, fine);
+                }
+                unsigned bad = 0;   // pairs of outputs that do not stand
+                const bool plain = even == 0xffffu && max(abs(er >> 2), abs(cexp[16 * h + (lane & 15)] >> 2)) <= kMaxExp / 2;
+                if (!__all_sync(0xffffffffu, plain)) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (!stands(er, cexp[16 * h + j], (even >> j) & 1u)) bad |= 1u << (j & ~1);
+                    if (!ro.ok) bad = 0;
+                }
+                auto value = [&](int j) {
+                    return round64(I[j], (er >> 2) + (cexp[16 * h + j] >> 2) + kShift - 8 * (int)((fine >> j) & 1u));
+                };
+#pragma unroll
+                for (int j = 0; j < 16; j += 2) {
+                    const double z0 = value(j), z1 = value(j + 1);
+                    const bool skip = (bad >> j) & 1u;
+                    if (MULTI) {
+                        acc[MULTI ? j : 0] += skip ? 0.0 : z0;
+                        acc[MULTI ? j + 1 : 0] += skip ? 0.0 : z1;
+                    } else if (!skip) {
+                        store_pair(o, ro, coff, cdof, 16 * h + j, z0, z1);
+                    }
+                }
+                redo |= bad;
+                if (MULTI && pc + 1 < p1) continue;
+                if (MULTI) {
 #pragma unroll
                     for (int j = 0; j < 16; j += 2)
                         store_pair(o, ro, coff, cdof, 16 * h + j, acc[MULTI ? j : 0], acc[MULTI ? j + 1 : 0]);
-                } else {
-                    long long I[16];
-#pragma unroll
-                    for (int c8 = 0; c8 < 2; ++c8) {
-                        uint32_t a[S][8];
-#pragma unroll
-                        for (int d = 0; d < S; ++d) tmem_ld8_nw(tq + d * kCols + 8 * c8, a[d]);
-                        tmem_ld_wait();
-                        if (c8 == 1) release();
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) I[8 * c8 + j] = Gather<S>::of(a, j);
-                    }
-#pragma unroll
-                    for (int j = 0; j < 16; j += 2)
-                        store_pair(o, ro, coff, cdof, 16 * h + j, value(j, I[j]), value(j + 1, I[j + 1]));
+                }
+                const unsigned any = __reduce_or_sync(0xffffffffu, redo);
+                if (any) {   // entry: (tile, warp, pair of columns)
+                    uint32_t at = 0;
+                    if (lane == 0) at = atomicAdd(o.head, (uint32_t)__popc(any));
+                    at = __shfl_sync(0xffffffffu, at, 0) + __popc(any & ((1u << lane) - 1u));
+                    if (((any >> lane) & 1u) && at < o.room)
+                        o.list[at] = (((PAIR ? 2 * w + rank : w) * 16 + 4 * h + q) * 8) + (lane >> 1);
                 }
             }
         }
@@ -719,6 +973,85 @@ __global__ void __launch_bounds__(kThreadsG, 1)
     if (threadIdx.x == 0 && ctl->abort) atomicOr(flags, FLAG_TIMEOUT);
 }
 
+// The listed outputs by the multiply-add loop, a warp to an entry: 32 rows by two columns, of which it
+// finds again the ones that do not stand (the certificates are exact sums, so it finds the same).  One piece:
+// stores them; several: adds the loop over the pieces that do not stand to what was stored.  A lane takes an
+// output where at least twelve of the warp's need the loop (its operations take 64 cycles each for the warp
+// either way), else the warp takes them one by one.  Bound by the FP64 pipe where many are listed: a product
+// of 512 x (128 x 32) outputs and K = 128, real by complex, all of them listed, takes 1.16 ms in all, 0.94 by the
+// tiles and 0.09 where none is listed.
+template <bool MULTI, bool PAIR>
+__global__ void __launch_bounds__(256, 2) slice_loop_kernel(const __grid_constant__ OutArgs o) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t count = min(*reinterpret_cast<volatile uint32_t*>(o.head), o.room);
+    for (uint32_t e = blockIdx.x * 8 + (threadIdx.x >> 5); e < count; e += gridDim.x * 8) {
+        const uint32_t id = o.list[e];
+        const int j = 2 * (int)(id & 7), warp = (int)(id >> 3) & 15, h = warp >> 2, q = warp & 3;
+        const uint32_t tile = id >> 7, w = PAIR ? tile >> 1 : tile;
+        uint32_t grp, t, b, ct, rt, ob, i;
+        o.dtiles.divmod(w, grp, t);
+        o.tile(t, b, ct, rt);
+        const int p0 = MULTI ? (int)grp * o.pg : 0, p1 = MULTI ? min(o.pieces, p0 + o.pg) : 1;
+        const int64_t r0 = (int64_t)(PAIR ? 2 * rt + (tile & 1u) : rt) * kRows + q * 32, r = r0 + lane;
+        const int64_t c0 = (int64_t)ct * kCols + 16 * h, c = c0 + j;
+        if (c >= o.cols) continue;
+        const bool ok = r < o.rows, two = c + 1 < o.cols;
+        double2 sum = make_double2(0.0, 0.0);
+        unsigned redo = 0;
+#pragma unroll 1
+        for (int pc = p0; pc < p1; ++pc) {
+            const int64_t z = pc * o.nbatch + b;
+            __syncwarp();
+            const unsigned even = certificates(o, z, r0, c0) >> j;
+            const int er = ok ? o.er[z * o.rows + r] : kZeroRow;
+            const int ec0 = o.ec[z * o.cols + c], ec1 = two ? o.ec[z * o.cols + c + 1] : kZeroRow;
+            const bool mine = ok && !(stands(er, ec0, even & 1u) && stands(er, ec1, even & 2u));
+            const unsigned who = __ballot_sync(0xffffffffu, mine);
+            const int k0 = pc * o.klen, k1 = min(o.k, k0 + o.klen);
+            double2 y = make_double2(0.0, 0.0);
+            if (__popc(who) >= 12) {
+                if (mine) y = loop_pair(o, b, k0, k1, (uint32_t)r, (uint32_t)c, -1);
+            } else {
+#pragma unroll 1
+                for (unsigned left = who; left; left &= left - 1u) {
+                    const int l = __ffs((int)left) - 1;
+                    const double2 v = loop_pair(o, b, k0, k1, (uint32_t)(r0 + l), (uint32_t)c, lane);
+                    if (lane == l) y = v;
+                }
+            }
+            if (mine) {
+                redo = 1;
+                sum = make_double2(sum.x + y.x, sum.y + y.y);
+            }
+        }
+        if (!redo) continue;
+        // as in slice_gemm_kernel: offsets of the row and of the columns
+        RowOut ro;
+        ro.ok = true;
+        o.rn.divmod((uint32_t)r >> (o.rexp ? 1 : 0), ob, i);
+        ro.roff = o.shared.at(b) + o.rown.at(ob) + i * o.rs + (MULTI ? grp * o.gstride : 0);
+        ro.rdof = o.D ? o.dshared.at(b) + o.drown.at(ob) + i * o.drs : 0;
+        ro.comp = o.rexp ? (int)(r & 1) : 0;
+        int64_t coff[2] = {-1, -1}, cdof[2] = {0, 0};
+        for (int u = 0; u < (two ? 2 : 1); ++u) {
+            o.cn.divmod((uint32_t)(c + u) >> (o.cexp ? 1 : 0), ob, i);
+            coff[u] = o.cown.at(ob) + i * o.cs;
+            cdof[u] = o.D ? o.dcown.at(ob) + i * o.dcs : 0;
+        }
+        if (MULTI) add_pair(o, ro, coff, cdof, 0, sum.x, sum.y);
+        else store_pair(o, ro, coff, cdof, 0, sum.x, sum.y);
+    }
+    // the last CTA empties the list for the next product
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(o.head + 1, 1u) == gridDim.x - 1) {
+            o.head[0] = 0u;
+            o.head[1] = 0u;
+        }
+    }
+}
+
 // ------------------------------------------------------------------------------------ host side
 int64_t up(int64_t n, int64_t m) { return (n + m - 1) / m * m; }
 
@@ -728,17 +1061,16 @@ struct Plan {
     Dims aown{{1, 1, 1}, {0, 0, 0}}, bown = aown, shared_a = aown, shared_b = aown, shared_c = aown, shared_d = aown,
         aown_c = aown, bown_c = aown, aown_d = aown, bown_d = aown;
     int64_t na = 1, nb = 1, ns = 1;       // own batches of A and B, shared batches
-    int parts = 1, koff = 0, klen = 0, pieces = 1, S = 7;
+    int parts = 1, koff = 0, klen = 0, pieces = 1;
     bool exp_a = false, exp_b = false, swap = false;   // swap: A supplies the tile rows
     int64_t rows_a = 0, rows_b = 0;       // after expansion
     int64_t tiles = 0;                    // pairs of row tiles with `pair`
     bool pair = false;                    // a CTA pair to two neighbouring row tiles
     int groups = 1, pg = 1;               // CTAs that share a tile's pieces, pieces of each
     size_t bytes_p = 0;                   // their partial outputs
-    size_t bytes_a = 0, bytes_b = 0, bytes = 0;
+    int64_t room = 0;                     // most entries of the list of outputs for the loop
+    size_t bytes_a = 0, bytes_b = 0, bytes_l = 0, bytes = 0;
 };
-
-constexpr int kMaxK = 512;
 
 int64_t tile_count(int64_t r, int64_t c) { return (up(r, kRows) / kRows) * (up(c, kCols) / kCols); }
 
@@ -766,8 +1098,7 @@ Plan make_plan(const GemmArgs& g) {
     const int most = kMaxK / p.parts;
     p.pieces = std::max(1, (g.k + most - 1) / most);   // of equal length, at most kMaxK with both parts
     p.klen = (g.k + p.pieces - 1) / p.pieces;
-    p.koff = (int)up(p.klen, 8);
-    p.S = p.parts * p.koff <= 128 ? 7 : 8;
+    p.koff = (int)up(p.klen, 16 / p.parts);   // a row of parts x koff entries is a multiple of 16
     // orientation and expansion with the fewest tiles; ties keep B's rows on the tile rows (the
     // output's contiguous index across lanes)
     int64_t best = -1;
@@ -793,23 +1124,27 @@ Plan make_plan(const GemmArgs& g) {
     }
     const int64_t Kp = (int64_t)p.parts * p.koff;
     const int64_t nz = p.ns * p.pieces;
-    p.bytes_a = up((int64_t)p.S * nz * p.rows_a * Kp * 2, 1024) + up(4 * nz * p.na * g.m, 1024);
-    p.bytes_b = up((int64_t)p.S * nz * p.rows_b * Kp * 2, 1024) + up(4 * nz * p.nb * g.n, 1024);
+    auto bytes = [&](int64_t rows) { return up(S * nz * rows * Kp * 2, 1024) + up(4 * nz * rows, 1024); };
+    p.bytes_a = bytes(p.rows_a);
+    p.bytes_b = bytes(p.rows_b);
     p.groups = (int)std::max<int64_t>(1, std::min<int64_t>(p.pieces, tc_num_sms() / (p.pair ? 2 : 1) / std::max<int64_t>(p.tiles, 1)));
     p.pg = (p.pieces + p.groups - 1) / p.groups;
     p.groups = (p.pieces + p.pg - 1) / p.pg;
     if (p.groups > 1) p.bytes_p = up((int64_t)p.groups * p.na * p.nb * p.ns * g.m * g.n * 16, 1024);
-    p.bytes = p.bytes_a + p.bytes_b + p.bytes_p;
+    p.room = p.tiles * (p.pair ? 2 : 1) * p.groups * 128;
+    p.bytes_l = up(4 * p.room, 1024);
+    p.bytes = p.bytes_a + p.bytes_b + p.bytes_p + p.bytes_l + kSliceHead;
     return p;
 }
 
-template <int S>
-void launch_pack(const PackArgs& a, cudaStream_t st) {
+void launch_pack(PackArgs a, cudaStream_t st) {
     count_launch();
     const int rb = a.koff <= 64 ? 32 : 8;
-    const dim3 grid((unsigned)((a.own_rows + rb - 1) / rb), (unsigned)(a.nbatch * a.pieces));
-    if (rb == 32) pack_slices_kernel<S, 32><<<grid, kPackT, 0, st>>>(a);
-    else pack_slices_kernel<S, 8><<<grid, kPackT, 0, st>>>(a);
+    const int64_t blocks = (a.own_rows + rb - 1) / rb;
+    a.dblocks = Div(blocks);
+    const unsigned grid = (unsigned)(blocks * a.nbatch * a.pieces);
+    if (rb == 32) pack_slices_kernel<32><<<grid, kPackT, 0, st>>>(a);
+    else pack_slices_kernel<8><<<grid, kPackT, 0, st>>>(a);
 }
 
 PackArgs pack_args(const GemmOperand& X, bool is_a, int n, int k, const Plan& p, void* buf, cplx alpha) {
@@ -839,7 +1174,7 @@ PackArgs pack_args(const GemmOperand& X, bool is_a, int n, int k, const Plan& p,
     const int64_t rows = is_a ? p.rows_a : p.rows_b;
     a.plane = p.ns * p.pieces * rows * a.Kp;
     a.out = static_cast<__half*>(buf);
-    a.exps = reinterpret_cast<int*>(static_cast<uint8_t*>(buf) + up((int64_t)p.S * a.plane * 2, 1024));
+    a.exps = reinterpret_cast<int*>(static_cast<uint8_t*>(buf) + up(S * a.plane * 2, 1024));
     a.alpha = alpha;
     a.scale = alpha.re != 1.0 || alpha.im != 0.0;
     return a;
@@ -862,10 +1197,10 @@ __global__ void __launch_bounds__(256) sum_groups_kernel(const cplx* part, int g
     }
 }
 
-template <int S, bool PAIR>
+template <bool PAIR>
 int launch_gemm(const CUtensorMap& r, const CUtensorMap& q, const OutArgs& o, unsigned* flags, cudaStream_t st) {
-    using St = Stage<S, PAIR>;
-    auto kern = o.pieces > 1 ? slice_gemm_kernel<S, true, PAIR> : slice_gemm_kernel<S, false, PAIR>;
+    using St = Stage<PAIR>;
+    auto kern = o.pieces > 1 ? slice_gemm_kernel<true, PAIR> : slice_gemm_kernel<false, PAIR>;
     const size_t sm = 1024 + (size_t)St::kCount * St::kBytes + sizeof(Ctl) + 2 * kCols * (2 * sizeof(int64_t) + sizeof(int));
     raise_dyn_smem(kern, sm);
     constexpr int C = PAIR ? 2 : 1;
@@ -883,31 +1218,33 @@ int launch_gemm(const CUtensorMap& r, const CUtensorMap& q, const OutArgs& o, un
     cfg.numAttrs = 1;
     count_launch();
     cudaLaunchKernelEx(&cfg, kern, r, q, o, flags);
+    count_launch();
+    const unsigned grid = 2 * (unsigned)tc_num_sms();
+    if (o.pieces > 1) slice_loop_kernel<true, PAIR><<<grid, 256, 0, st>>>(o);
+    else slice_loop_kernel<false, PAIR><<<grid, 256, 0, st>>>(o);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(AFQMC_ERR_CUDA, std::string("slice_gemm launch: ") + cudaGetErrorString(e));
     return AFQMC_OK;
 }
 int launch_gemm(const Plan& p, const CUtensorMap& r, const CUtensorMap& q, const OutArgs& o, unsigned* flags, cudaStream_t st) {
-    if (p.pair) return p.S == 7 ? launch_gemm<7, true>(r, q, o, flags, st) : launch_gemm<8, true>(r, q, o, flags, st);
-    return p.S == 7 ? launch_gemm<7, false>(r, q, o, flags, st) : launch_gemm<8, false>(r, q, o, flags, st);
+    return p.pair ? launch_gemm<true>(r, q, o, flags, st) : launch_gemm<false>(r, q, o, flags, st);
 }
 
-// One product that fits the workspace: B's slices at its start, A's at its end,
-// partial outputs between them.
+// One product that fits the workspace: B's slices at its start, then partial outputs and the list, A's slices
+// before the last kSliceHead bytes, the list's counts.
 int run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st) {
     uint8_t* buf = static_cast<uint8_t*>(ws->buf);
     // alpha multiplies B, or A where alpha is complex and B real
     const bool on_a = g.B.real && g.alpha.im != 0.0;
     const cplx one{1.0, 0.0};
     const PackArgs pb = pack_args(g.B, false, g.n, g.k, p, buf, on_a ? one : g.alpha);
-    const PackArgs pa = pack_args(g.A, true, g.m, g.k, p, buf + (ws->bytes - p.bytes_a) / 1024 * 1024, on_a ? g.alpha : one);
+    const PackArgs pa = pack_args(g.A, true, g.m, g.k, p, buf + (ws->bytes - kSliceHead - p.bytes_a) / 1024 * 1024, on_a ? g.alpha : one);
     const int64_t nz = p.ns * p.pieces;
     auto kept = [&](bool keep, SliceScratch::Packed& have, const PackArgs& x, int64_t rows) {
         const bool same = keep && have.rows == rows && have.pitch == x.Kp && have.batches == nz;
         have = SliceScratch::Packed{rows, x.Kp, nz};
         if (same) return;
-        if (p.S == 7) launch_pack<7>(x, st);
-        else launch_pack<8>(x, st);
+        launch_pack(x, st);
     };
     kept(g.keep_b, ws->b, pb, p.rows_b);
     kept(g.keep_a, ws->a, pa, p.rows_a);
@@ -915,9 +1252,9 @@ int run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st
     const int64_t rr = p.swap ? p.rows_a : p.rows_b, rc = p.swap ? p.rows_b : p.rows_a;
     CUtensorMap mr, mq;
     auto encode = [&](CUtensorMap* m, const PackArgs& x, int64_t rows, int box_rows) {
-        const uint64_t dims[4] = {(uint64_t)x.Kp, (uint64_t)rows, (uint64_t)nz, (uint64_t)p.S};
+        const uint64_t dims[4] = {(uint64_t)x.Kp, (uint64_t)rows, (uint64_t)nz, (uint64_t)S};
         const uint64_t str[3] = {(uint64_t)x.Kp * 2, (uint64_t)rows * x.Kp * 2, (uint64_t)x.plane * 2};
-        const uint32_t box[4] = {kChunk, (uint32_t)box_rows, 1, (uint32_t)p.S};
+        const uint32_t box[4] = {kChunk, (uint32_t)box_rows, 1, (uint32_t)S};
         return make_map4(m, x.out, dims, str, box, 64);
     };
     AFQMC_TRY(encode(&mr, R, rr, kRows));
@@ -939,6 +1276,18 @@ int run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st
     o.dshared = Strides(p.shared_d);
     o.er = R.exps;
     o.ec = Q.exps;
+    o.dr = R.out;
+    o.dc = Q.out;
+    o.Kp = (int)R.Kp;
+    auto source = [](const PackArgs& x) { return Source{x.ptr, x.real, x.conj, x.si, x.sk, x.own, x.shared}; };
+    o.srow = source(R);
+    o.scol = source(Q);
+    o.k = g.k;
+    o.klen = p.klen;
+    o.alpha = g.alpha;
+    o.list = reinterpret_cast<uint32_t*>(buf + p.bytes_b + p.bytes_p);
+    o.head = reinterpret_cast<uint32_t*>(buf + ws->bytes / 1024 * 1024 - kSliceHead);
+    o.room = (uint32_t)p.room;
     o.C = g.C;
     o.D = g.D;
     o.beta = g.beta.re;
@@ -981,17 +1330,27 @@ int run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st
 
 size_t slice_gemm_bytes(const GemmArgs& g) { return make_plan(g).bytes + 1024; }
 
-// Expected time in microseconds: three launches with little in each, the persistent tiles at 65 (pairs: 56) cycles an MMA and 6000
-// for the epilogue, and the operands' packing.
+// Expected time in microseconds: four launches with little in each, the persistent tiles at 65 (pairs: 56) cycles an MMA and 6000
+// for the epilogue of each piece, and the operands' packing.
 double slice_gemm_us(const GemmArgs& g) {
     if (g.beta.im != 0.0 || (g.A.real && g.B.real && g.alpha.im != 0.0)) return 1e30;
     const Plan p = make_plan(g);
-    // the pack kernel's grid, 31-bit indices
-    if (p.ns * p.pieces > 65535 || std::max(p.rows_a, p.rows_b) >= 1ll << 31 || p.tiles * p.groups >= 1ll << 31) return 1e30;
-    const double cyc = p.S * (p.S + 1) / 2 * (up((int64_t)p.parts * p.koff, 16) / 16) * (p.pair ? 56.0 : 65.0) + 6000.0;
+    // 31-bit indices
+    const int64_t nz = p.ns * p.pieces, most = 1ll << 31;
+    if (std::max(p.rows_a, p.rows_b) >= most || nz * (std::max(p.rows_a, p.rows_b) / 8 + 1) >= most || p.room >= 2 * most)
+        return 1e30;
+    const double cyc = kMmas * (up((int64_t)p.parts * p.koff, kChunk) / 16) * (p.pair ? 56.0 : 65.0) + 6000.0;
     const int ctas = tc_num_sms() / (p.pair ? 2 : 1);
     const double waves = (double)((p.tiles * p.groups + ctas - 1) / ctas);
-    return 26.0 + p.pg * waves * cyc / 1.9e3 + (double)p.bytes / 2.0e6 + (p.groups > 1 ? 4.0 : 0.0);
+    return 29.0 + p.pg * waves * cyc / 1.9e3 + (double)p.bytes / 2.0e6 + (p.groups > 1 ? 4.0 : 0.0);
+}
+
+int slice_scratch_init(SliceScratch* ws) {
+    if (ws->bytes < 2 * kSliceHead) return AFQMC_OK;   // holds no product
+    if (cudaMemset(static_cast<uint8_t*>(ws->buf) + ws->bytes / 1024 * 1024 - kSliceHead, 0, kSliceHead) != cudaSuccess ||
+        cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess)   // before any stream uses it
+        return fail(AFQMC_ERR_CUDA, "slice workspace");
+    return AFQMC_OK;
 }
 
 int slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st) {
@@ -1010,7 +1369,7 @@ int slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st) {
         hi.C = g.C + dc;
         hi.D = g.D ? g.D + dd : nullptr;
     };
-    if (p.pieces >= 8) {
+    if (p.pieces >= 32) {
         const int64_t fit = (int64_t)(ws->bytes / ((p.bytes + 1024) / p.pieces + 1));
         const int64_t share = std::max<int64_t>(1, tc_num_sms() / (p.pair ? 2 : 1) / std::max<int64_t>(p.tiles, 1));
         const int64_t n = fit > share ? fit / share * share : std::max<int64_t>(1, fit);

@@ -20,7 +20,9 @@ struct GemmOperand {
 
 // Workspace of the products that run on the tensor cores (gemm_slices.cu): device memory for the
 // operands' slices and the status word their bounded waits report to; a, b: the shapes of the
-// operands whose slices it holds (of the last product).
+// operands whose slices it holds (of the last product).  The last whole kilobyte of buf holds counts that are zero between
+// products: to be cleared when it is allocated.
+constexpr size_t kSliceHead = 1024;
 struct SliceScratch {
     void* buf = nullptr;
     size_t bytes = 0;
@@ -54,6 +56,7 @@ struct GemmArgs {
 double slice_gemm_us(const GemmArgs& g);
 size_t slice_gemm_bytes(const GemmArgs& g);
 int slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st);
+int slice_scratch_init(SliceScratch* ws);   // a new workspace: clears its counts
 
 // The product in the form expected to be fastest: zgemm_form's 0 (tiles), 1 (tensor cores, where
 // there is a workspace), 2 (one output per thread), 3 or 4 (by four or eight threads).  zgemm_as: in the form given.

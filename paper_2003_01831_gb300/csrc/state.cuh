@@ -46,6 +46,7 @@ struct Fp64Buffers {
     void* LtT[2] = {nullptr, nullptr};     // transposed: [ND][Nchol][M][N_s] (force-bias-only path)
     cplx* ht[2] = {nullptr, nullptr};      // Psi_s^+ h: [ND][N_s][M]
     double* Bh = nullptr;                  // exp(-tau h'/2): [M][M], interleaved complex if cplx_L
+    double* Bo = nullptr;                  // the same without its diagonal (FP64 walker sets)
     cplx* Phi[2] = {nullptr, nullptr};     // [W][M][N_s]
     cplx* Pnew[2] = {nullptr, nullptr};    // propagated walkers / Taylor accumulator
     cplx* Pa[2] = {nullptr, nullptr};      // Taylor term ping
@@ -131,6 +132,7 @@ struct afqmc_walkers {
 namespace afqmc {
 
 // step drivers (step_fp64.cu / step_tc.cu)
+void fp64_split_propagator(afqmc_walkers* wk, cudaStream_t st);   // once Bh is there
 int fp64_alloc(afqmc_walkers* wk);
 void fp64_free(afqmc_walkers* wk);
 // Green's function, traces, local energy and force bias at the current walkers.

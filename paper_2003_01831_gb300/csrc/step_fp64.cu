@@ -30,6 +30,20 @@ void add_logdet(const cplx* a, const cplx* b, cplx* out, int n, cudaStream_t st)
     add_logdet_kernel<<<(n + 255) / 256, 256, 0, st>>>(a, b, out, n);
 }
 
+// B without its diagonal; Y = diag(B) X for blocks of M x N orbitals
+template <class T>
+__global__ void without_diagonal_kernel(const T* B, int M, T* out) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < (int64_t)M * M) out[i] = i / M == i % M ? T{} : B[i];
+}
+template <class T>
+__global__ void scale_rows_kernel(const T* B, int M, int N, const cplx* X, int64_t total, cplx* Y) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = e / N % M;
+        Y[e] = B[i * M + i] * X[e];
+    }
+}
+
 // Y[w] = op(X) Phi[w]-style helpers --------------------------------------------------------
 // S_w = Psi^+ Phi_w   (N x N)
 void overlap(const cplx* Psi, const cplx* Phi, cplx* S, int M, int N, int W, SliceScratch* ws, cudaStream_t st) {
@@ -81,6 +95,7 @@ int fp64_alloc(afqmc_walkers* wk) {
         AFQMC_TRY(dalloc(&f.X[s], nd * W * nch));
     }
     AFQMC_TRY(dalloc(&f.Bh, (size_t)M * M * (wk->ham->cplx_L ? 2 : 1)));
+    if (wk->opts.precision == AFQMC_PREC_FP64) AFQMC_TRY(dalloc(&f.Bo, (size_t)M * M * (wk->ham->cplx_L ? 2 : 1)));
     if (Nmu > 0) {   // walker chunks of the THC densities T and of X diag(U c)
         const size_t per_w = std::max((size_t)Nmu * Nmu, (size_t)M * Nmu) * sizeof(cplx);
         f.thc_wc = (int)std::max<size_t>(1, std::min<size_t>((size_t)W, budget / per_w));
@@ -121,6 +136,7 @@ int fp64_alloc(afqmc_walkers* wk) {
         f.ws.bytes = std::min(need, (size_t)768 << 20);
         AFQMC_TRY(dalloc(reinterpret_cast<char**>(&f.ws.buf), f.ws.bytes));
         f.ws.flags = wk->flags;
+        AFQMC_TRY(slice_scratch_init(&f.ws));
     }
     if (ND > 1) {
         AFQMC_TRY(dalloc(&f.msd_cc, (size_t)ND));
@@ -141,7 +157,7 @@ void fp64_free(afqmc_walkers* wk) {
         for (void* p : ps)
             if (p) cudaFree(p);
     }
-    void* more[] = {f.ws.buf, f.ex_part, f.Bh, f.T, f.A, f.msd_cc, f.msd_ls, f.msd_E, f.msd_t, f.msd_flag, f.msd_Es, f.Tthc, f.dv, f.XD};
+    void* more[] = {f.ws.buf, f.ex_part, f.Bh, f.Bo, f.T, f.A, f.msd_cc, f.msd_ls, f.msd_E, f.msd_t, f.msd_flag, f.msd_Es, f.Tthc, f.dv, f.XD};
     for (void* p : more)
         if (p) cudaFree(p);
     f = Fp64Buffers{};
@@ -371,6 +387,45 @@ int fp64_measure(afqmc_walkers* wk, bool measure, cudaStream_t st, int Wm) {
     return AFQMC_OK;
 }
 
+void fp64_split_propagator(afqmc_walkers* wk, cudaStream_t st) {
+    if (!wk->f.Bo) return;
+    const int64_t M = wk->M, n = M * M;
+    count_launch();
+    if (wk->ham->cplx_L)
+        without_diagonal_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(reinterpret_cast<const cplx*>(wk->f.Bh), (int)M,
+                                                                            reinterpret_cast<cplx*>(wk->f.Bo));
+    else without_diagonal_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(wk->f.Bh, (int)M, wk->f.Bo);
+}
+
+namespace {
+// Y_w = B X_w for the walkers' orbitals of spin s.  B = exp(-tau h' / 2) is near the identity: an output is
+// one large product and many small ones, which the digits of the tensor-core form hold too few bits of (most
+// of the outputs would go through its loop: 1.16 ms a product at M = 128, N = 32, W = 512, 0.94 by the
+// tiles), so there the diagonal's part is formed by itself and the rest, whose entries are alike, added to it
+// (0.09 ms).
+void one_body(afqmc_walkers* wk, const cplx* X, cplx* Y, int s, cudaStream_t st) {
+    Fp64Buffers& f = wk->f;
+    const int M = wk->M, W = wk->W, N = wk->N[s];
+    const int64_t mn = (int64_t)M * N;
+    GemmArgs g;
+    g.m = M; g.n = N; g.k = M; g.nb1 = W;
+    g.A.ptr = f.Bh; g.A.real = !wk->ham->cplx_L; g.A.ld = M;
+    g.B.ptr = X; g.B.ld = N; g.B.s1 = mn;
+    g.C = Y; g.ldc = N; g.sc1 = mn;
+    g.ws = &f.ws;
+    if (f.Bo && zgemm_form(g, &f.ws) == 1) {
+        const int64_t total = W * mn;
+        const unsigned blocks = (unsigned)std::min<int64_t>((total + 255) / 256, 1 << 16);
+        count_launch();
+        if (g.A.real) scale_rows_kernel<<<blocks, 256, 0, st>>>(f.Bh, M, N, X, total, Y);
+        else scale_rows_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<const cplx*>(f.Bh), M, N, X, total, Y);
+        g.A.ptr = f.Bo;
+        g.beta = cplx{1.0, 0.0};
+    }
+    zgemm(g, st);
+}
+}  // namespace
+
 int fp64_propagate_and_weight(afqmc_walkers* wk, const double* x, cudaStream_t st) {
     Fp64Buffers& f = wk->f;
     const int M = wk->M, W = wk->W, nch = wk->Nchol;
@@ -412,13 +467,7 @@ int fp64_propagate_and_weight(afqmc_walkers* wk, const double* x, cudaStream_t s
         const int64_t mn = (int64_t)M * N;
         P0[s] = f.Pa[s];
         P1[s] = f.Pb[s];
-        GemmArgs g;   // P0 = B Phi
-        g.m = M; g.n = N; g.k = M; g.nb1 = W;
-        g.A.ptr = f.Bh; g.A.real = !wk->ham->cplx_L; g.A.ld = M;
-        g.B.ptr = f.Phi[s]; g.B.ld = N; g.B.s1 = mn;
-        g.C = P0[s]; g.ldc = N; g.sc1 = mn;
-        g.ws = &f.ws;
-        zgemm(g, st);
+        one_body(wk, f.Phi[s], P0[s], s, st);
         cudaMemcpyAsync(f.Pnew[s], P0[s], sizeof(cplx) * W * mn, cudaMemcpyDeviceToDevice, st);
     }
     for (int k = 1; k <= wk->opts.k_taylor; ++k)
@@ -439,14 +488,7 @@ int fp64_propagate_and_weight(afqmc_walkers* wk, const double* x, cudaStream_t s
         }
     for (int s = 0; s < 2; ++s) {
         const int N = wk->N[s];
-        const int64_t mn = (int64_t)M * N;
-        GemmArgs b2;  // Phi' = B Pnew  -> Pa
-        b2.m = M; b2.n = N; b2.k = M; b2.nb1 = W;
-        b2.A.ptr = f.Bh; b2.A.real = !wk->ham->cplx_L; b2.A.ld = M;
-        b2.B.ptr = f.Pnew[s]; b2.B.ld = N; b2.B.s1 = mn;
-        b2.C = f.Pa[s]; b2.ldc = N; b2.sc1 = mn;
-        b2.ws = &f.ws;
-        zgemm(b2, st);
+        one_body(wk, f.Pnew[s], f.Pa[s], s, st);   // Phi' = B Pnew
         if (wk->ND == 1) {
             overlap(f.Psi[s], f.Pa[s], f.S[s], M, N, W, &f.ws, st);
             batched_inverse_logdet(f.S[s], (int64_t)N * N, N, W, f.ld[s], false, wk->flags, st);
