@@ -321,11 +321,10 @@ extern "C" int afqmc_debug_gemm(const long long* d, const long long* sizes, cons
     cudaEvent_t e0, e1;
     AFQMC_CUDA_TRY(cudaEventCreate(&e0));
     AFQMC_CUDA_TRY(cudaEventCreate(&e1));
-    int rc = AFQMC_OK;
-    for (int r = 0; r <= reps && rc == AFQMC_OK; ++r) {
+    for (int r = 0; r <= reps; ++r) {
         if (r == reps) cudaEventRecord(e0);
         if (form == 1) {
-            rc = slice_gemm(g, &ws, 0);
+            slice_gemm(g, &ws, 0);
         } else {
             if (form == 2) g.ws = &ws;
             zgemm_as(g, form == 2 ? zgemm_form(g, &ws) : form >= 3 ? form - 1 : 0, 0);
@@ -337,8 +336,8 @@ extern "C" int afqmc_debug_gemm(const long long* d, const long long* sizes, cons
     if (e == cudaSuccess) cudaEventElapsedTime(&t, e0, e1);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    AFQMC_TRY(rc);
     AFQMC_CUDA_TRY(e);
+    AFQMC_CUDA_TRY(cudaGetLastError());
     if (ms) *ms = t;
     unsigned fl = 0;
     AFQMC_CUDA_TRY(cudaMemcpy(&fl, flags.p, 4, cudaMemcpyDeviceToHost));

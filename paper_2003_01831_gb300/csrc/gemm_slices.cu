@@ -1198,7 +1198,7 @@ __global__ void __launch_bounds__(256) sum_groups_kernel(const cplx* part, int g
 }
 
 template <bool PAIR>
-int launch_gemm(const CUtensorMap& r, const CUtensorMap& q, const OutArgs& o, unsigned* flags, cudaStream_t st) {
+void launch_gemm(const CUtensorMap& r, const CUtensorMap& q, const OutArgs& o, unsigned* flags, cudaStream_t st) {
     using St = Stage<PAIR>;
     auto kern = o.pieces > 1 ? slice_gemm_kernel<true, PAIR> : slice_gemm_kernel<false, PAIR>;
     const size_t sm = 1024 + (size_t)St::kCount * St::kBytes + sizeof(Ctl) + 2 * kCols * (2 * sizeof(int64_t) + sizeof(int));
@@ -1222,17 +1222,14 @@ int launch_gemm(const CUtensorMap& r, const CUtensorMap& q, const OutArgs& o, un
     const unsigned grid = 2 * (unsigned)tc_num_sms();
     if (o.pieces > 1) slice_loop_kernel<true, PAIR><<<grid, 256, 0, st>>>(o);
     else slice_loop_kernel<false, PAIR><<<grid, 256, 0, st>>>(o);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return fail(AFQMC_ERR_CUDA, std::string("slice_gemm launch: ") + cudaGetErrorString(e));
-    return AFQMC_OK;
 }
-int launch_gemm(const Plan& p, const CUtensorMap& r, const CUtensorMap& q, const OutArgs& o, unsigned* flags, cudaStream_t st) {
-    return p.pair ? launch_gemm<true>(r, q, o, flags, st) : launch_gemm<false>(r, q, o, flags, st);
+void launch_gemm(const Plan& p, const CUtensorMap& r, const CUtensorMap& q, const OutArgs& o, unsigned* flags, cudaStream_t st) {
+    p.pair ? launch_gemm<true>(r, q, o, flags, st) : launch_gemm<false>(r, q, o, flags, st);
 }
 
 // One product that fits the workspace: B's slices at its start, then partial outputs and the list, A's slices
-// before the last kSliceHead bytes, the list's counts.
-int run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st) {
+// before the last kSliceHead bytes, the list's counts.  False, with nothing launched, where a tensor map cannot be made.
+bool run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st) {
     uint8_t* buf = static_cast<uint8_t*>(ws->buf);
     // alpha multiplies B, or A where alpha is complex and B real
     const bool on_a = g.B.real && g.alpha.im != 0.0;
@@ -1240,14 +1237,6 @@ int run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st
     const PackArgs pb = pack_args(g.B, false, g.n, g.k, p, buf, on_a ? one : g.alpha);
     const PackArgs pa = pack_args(g.A, true, g.m, g.k, p, buf + (ws->bytes - kSliceHead - p.bytes_a) / 1024 * 1024, on_a ? g.alpha : one);
     const int64_t nz = p.ns * p.pieces;
-    auto kept = [&](bool keep, SliceScratch::Packed& have, const PackArgs& x, int64_t rows) {
-        const bool same = keep && have.rows == rows && have.pitch == x.Kp && have.batches == nz;
-        have = SliceScratch::Packed{rows, x.Kp, nz};
-        if (same) return;
-        launch_pack(x, st);
-    };
-    kept(g.keep_b, ws->b, pb, p.rows_b);
-    kept(g.keep_a, ws->a, pa, p.rows_a);
     const PackArgs &R = p.swap ? pa : pb, &Q = p.swap ? pb : pa;
     const int64_t rr = p.swap ? p.rows_a : p.rows_b, rc = p.swap ? p.rows_b : p.rows_a;
     CUtensorMap mr, mq;
@@ -1257,8 +1246,15 @@ int run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st
         const uint32_t box[4] = {kChunk, (uint32_t)box_rows, 1, (uint32_t)S};
         return make_map4(m, x.out, dims, str, box, 64);
     };
-    AFQMC_TRY(encode(&mr, R, rr, kRows));
-    AFQMC_TRY(encode(&mq, Q, rc, p.pair ? kCols / 2 : kCols));
+    if (encode(&mr, R, rr, kRows) != AFQMC_OK || encode(&mq, Q, rc, p.pair ? kCols / 2 : kCols) != AFQMC_OK) return false;
+    auto kept = [&](bool keep, SliceScratch::Packed& have, const PackArgs& x, int64_t rows) {
+        const bool same = keep && have.rows == rows && have.pitch == x.Kp && have.batches == nz;
+        have = SliceScratch::Packed{rows, x.Kp, nz};
+        if (same) return;
+        launch_pack(x, st);
+    };
+    kept(g.keep_b, ws->b, pb, p.rows_b);
+    kept(g.keep_a, ws->a, pa, p.rows_a);
     OutArgs o{};
     o.rows = rr;
     o.cols = rc;
@@ -1318,12 +1314,13 @@ int run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t st
             for (Dims* d : {&rown, &cown, &shared})
                 if (d->cnt[i] > 1) d->str[i] = dense[i];
         place();
-        AFQMC_TRY(launch_gemm(p, mr, mq, o, ws->flags, st));
+        launch_gemm(p, mr, mq, o, ws->flags, st);
         count_launch();
         sum_groups_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(o.C, p.groups, total, g);
-        return AFQMC_OK;
+    } else {
+        launch_gemm(p, mr, mq, o, ws->flags, st);
     }
-    return launch_gemm(p, mr, mq, o, ws->flags, st);
+    return true;
 }
 
 }  // namespace
@@ -1353,12 +1350,17 @@ int slice_scratch_init(SliceScratch* ws) {
     return AFQMC_OK;
 }
 
-int slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st) {
+// Each part of a product that has been cut takes this form or, where it cannot, the tiles: what earlier parts have
+// added to C and D is never added again.
+void slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st) {
     const Plan p = make_plan(g);
-    if (p.bytes + 1024 <= ws->bytes) return run_plan(g, p, ws, st);
+    if (p.bytes + 1024 <= ws->bytes) {
+        if (!run_plan(g, p, ws, st)) zgemm_as(g, 0, st);
+        return;
+    }
     // too large for the workspace: cut a long contraction (the output is then added up in rounds) after
     // as many pieces as fit, in equal shares for the CTAs of a tile where that is possible; else
-    // halve the largest of the batch dimensions, n and m
+    // halve the largest of the batch dimensions, n and m, and in the end the contraction again
     GemmArgs lo = g, hi = g;
     lo.keep_a = lo.keep_b = hi.keep_a = hi.keep_b = false;
     const int64_t big = std::max<int64_t>({g.nb0, g.nb1, g.nb2});
@@ -1369,16 +1371,19 @@ int slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st) {
         hi.C = g.C + dc;
         hi.D = g.D ? g.D + dd : nullptr;
     };
+    auto cut_k = [&](int k) {
+        lo.k = k;
+        hi.k = g.k - k;
+        shift(k * (g.A.op == OP_N ? 1 : g.A.ld), k * (g.B.op == OP_N ? g.B.ld : 1), 0, 0);
+        lo.D = nullptr;
+        hi.beta = cplx{1.0, 0.0};
+    };
     if (p.pieces >= 32) {
         const int64_t fit = (int64_t)(ws->bytes / ((p.bytes + 1024) / p.pieces + 1));
         const int64_t share = std::max<int64_t>(1, tc_num_sms() / (p.pair ? 2 : 1) / std::max<int64_t>(p.tiles, 1));
         const int64_t n = fit > share ? fit / share * share : std::max<int64_t>(1, fit);
         // (at least a 64th, which may be cut again: bounds the depth of the cuts)
-        lo.k = (int)std::min<int64_t>(std::max<int64_t>(n, p.pieces / 64), p.pieces - 1) * p.klen;
-        hi.k = g.k - lo.k;
-        shift(lo.k * (g.A.op == OP_N ? 1 : g.A.ld), lo.k * (g.B.op == OP_N ? g.B.ld : 1), 0, 0);
-        lo.D = nullptr;
-        hi.beta = cplx{1.0, 0.0};
+        cut_k((int)std::min<int64_t>(std::max<int64_t>(n, p.pieces / 64), p.pieces - 1) * p.klen);
     } else if (big > 1) {
         if (big == g.nb0) {
             lo.nb0 = g.nb0 / 2; hi.nb0 = g.nb0 - lo.nb0;
@@ -1396,11 +1401,14 @@ int slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st) {
     } else if (g.m > 1) {
         lo.m = g.m / 2; hi.m = g.m - lo.m;
         shift(lo.m * (g.A.op == OP_N ? g.A.ld : 1), 0, lo.m * g.ldc, lo.m * g.ldd);
+    } else if (p.pieces > 1) {
+        cut_k(p.pieces / 2 * p.klen);
     } else {
-        return fail(AFQMC_ERR_OOM, "slice_gemm: workspace too small");
+        zgemm_as(g, 0, st);
+        return;
     }
-    AFQMC_TRY(slice_gemm(lo, ws, st));
-    return slice_gemm(hi, ws, st);
+    slice_gemm(lo, ws, st);
+    slice_gemm(hi, ws, st);
 }
 
 }  // namespace afqmc

@@ -1908,7 +1908,10 @@ int zgemm_form(const GemmArgs& g, const SliceScratch* ws) {
 
 void zgemm_as(const GemmArgs& g, int form, cudaStream_t st) {
     if (g.m <= 0 || g.n <= 0) return;
-    if (form == 1 && slice_gemm(g, g.ws, st) == AFQMC_OK) return;
+    if (form == 1) {
+        slice_gemm(g, g.ws, st);
+        return;
+    }
     if (g.ws) g.ws->a = g.ws->b = SliceScratch::Packed{};   // no slices for the next product to keep
     const int64_t nbatch = (int64_t)g.nb0 * g.nb1 * g.nb2;
     count_launch();

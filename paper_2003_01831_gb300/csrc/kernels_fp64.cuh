@@ -55,7 +55,7 @@ struct GemmArgs {
 // it does not apply), the workspace it wants (a smaller one is used in pieces) and the product.
 double slice_gemm_us(const GemmArgs& g);
 size_t slice_gemm_bytes(const GemmArgs& g);
-int slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st);
+void slice_gemm(const GemmArgs& g, SliceScratch* ws, cudaStream_t st);
 int slice_scratch_init(SliceScratch* ws);   // a new workspace: clears its counts
 
 // The product in the form expected to be fastest: zgemm_form's 0 (tiles), 1 (tensor cores, where
