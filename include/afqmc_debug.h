@@ -134,6 +134,11 @@ int afqmc_debug_mixed_terms(afqmc_wk_debug_t wk, double* ST, double* Sinv, doubl
  * contraction are this many times the algorithmic ones.  Host only. */
 int afqmc_debug_energy_products(afqmc_wk_debug_t wk, double* mean);
 
+/* Raises bits (1: not finite, 2: singular, 4: a bounded wait gave up) in the status word of a walker set,
+ * as its kernels do, or, with wk = NULL, in that of every set which the calling thread then makes, at the
+ * start of its set-up (0: no longer).  For tests of the calls that report them.  Errors: BADARG. */
+int afqmc_debug_set_status(afqmc_wk_debug_t wk, unsigned bits);
+
 /* Failure detection without a fault: one warp waits, by the library's bounded mbarrier wait
  * (try_wait polled against a clock64 budget) with a budget of limit_cycles SM clock cycles
  * (1 .. the production bound of 4e9), on a barrier phase that completes only if

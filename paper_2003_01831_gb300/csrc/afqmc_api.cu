@@ -501,6 +501,7 @@ static int init_walkers_impl(afqmc_ham_t ham, int ND, const double* Psi_up, cons
     const double* psis[2] = {Psi_up, Psi_dn};
     // flags[0]: latched status bits; flags[1]: scratch word (imaginary part of the trial)
     cudaMemsetAsync(wk->flags, 0, 2 * sizeof(unsigned), st);
+    if (launch_policy().status) raise_status(wk->flags, launch_policy().status, st);
     for (int s = 0; s < 2; ++s) {
         const int64_t n = (int64_t)ND * M * wk->N[s];
         rc = copy_in(f.Psi[s], psis[s], sizeof(cplx) * n, st);
@@ -658,6 +659,12 @@ static int init_walkers_impl(afqmc_ham_t ham, int ND, const double* Psi_up, cons
         for (int s = 0; s < 2; ++s)
             replicate(f.Phi[s], f.Psi[s] + (int64_t)ref * M * wk->N[s], (int64_t)M * wk->N[s], W,
                       (int64_t)M * wk->N[s], st);
+    }
+    {   // the set-up's products (Psi^+ L_n, E_T) have waited too; what else the trial raised is not the walkers'
+        unsigned fl = 0;
+        rc = read_flags(wk->flags, st, &fl);
+        if (!rc) rc = flags_to_error(fl & FLAG_TIMEOUT, "init_walkers");
+        if (rc) return bail(rc);
     }
     cudaMemsetAsync(wk->flags, 0, sizeof(unsigned), st);
     if (o.precision == AFQMC_PREC_BF16X3) {

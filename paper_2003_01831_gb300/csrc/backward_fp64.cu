@@ -238,12 +238,10 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
     void* frees[] = {U, V, F, G, Z, gP, gc, dLd, gE, gS, dEd, dSd};
     for (void* p : frees)
         if (p) cudaFreeAsync(p, st);
-    AFQMC_CUDA_TRY(cudaStreamSynchronize(st));
+    AFQMC_CUDA_TRY(cudaGetLastError());
     unsigned fl = 0;
-    AFQMC_CUDA_TRY(cudaMemcpy(&fl, wk->flags, sizeof(unsigned), cudaMemcpyDeviceToHost));
-    if (fl & FLAG_NONFINITE) return fail(AFQMC_ERR_NONFINITE, "energy_backward: NaN/Inf");
-    if (fl & FLAG_SINGULAR) return fail(AFQMC_ERR_SINGULAR, "energy_backward: singular overlap");
-    return AFQMC_OK;
+    AFQMC_TRY(read_flags(wk->flags, st, &fl));
+    return flags_to_error(fl, "energy_backward");
 }
 
 }  // namespace afqmc

@@ -279,6 +279,17 @@ extern "C" int afqmc_debug_wait_probe(long long limit_cycles, int release, unsig
     return AFQMC_OK;
 }
 
+extern "C" int afqmc_debug_set_status(afqmc_wk_debug_t wk, unsigned bits) {
+    if (bits & ~7u) return fail(AFQMC_ERR_BADARG, "debug_set_status: bits must be of 1, 2, 4");
+    if (!wk) {
+        launch_policy().status = bits;
+        return AFQMC_OK;
+    }
+    raise_status(wk->flags, bits, 0);
+    AFQMC_CUDA_TRY(cudaDeviceSynchronize());
+    return AFQMC_OK;
+}
+
 extern "C" int afqmc_debug_gemm(const long long* d, const long long* sizes, const double* ab, const double* A,
                                 const double* B, double* C, double* D, int form, long long ws_bytes, int reps,
                                 int* chose, float* ms) {

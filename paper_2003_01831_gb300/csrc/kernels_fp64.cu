@@ -1869,6 +1869,8 @@ __global__ void add_identity_kernel(cplx* A, int M, double s) {
     if (i < M) A[(int64_t)i * M + i].re += s;
 }
 
+__global__ void raise_status_kernel(unsigned* flags, unsigned bits) { atomicOr(flags, bits); }
+
 inline unsigned blocks_for(int64_t n, int t = kThreads) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
@@ -1938,6 +1940,11 @@ void zgemm_as(const GemmArgs& g, int form, cudaStream_t st) {
     else if (g.A.real) go(zgemm_kernel<true, false, 32>, zgemm_kernel<true, false, 64>);
     else if (g.B.real) go(zgemm_kernel<false, true, 32>, zgemm_kernel<false, true, 64>);
     else go(zgemm_kernel<false, false, 32>, zgemm_kernel<false, false, 64>);
+}
+
+void raise_status(unsigned* flags, unsigned bits, cudaStream_t st) {
+    count_launch();
+    raise_status_kernel<<<1, 1, 0, st>>>(flags, bits);
 }
 
 void zgemm(const GemmArgs& g, cudaStream_t st) {

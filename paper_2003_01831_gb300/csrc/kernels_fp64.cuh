@@ -122,6 +122,9 @@ void real_part_times(const cplx* a, const double* b, double* out, int64_t n, cud
 // out[i] = h[i] - 0.5 * Re(R[i])
 void hprime_from(const double* h, const cplx* R, double* out, int64_t n, cudaStream_t st);
 
+// *flags |= bits, as a kernel does whose wait gave up
+void raise_status(unsigned* flags, unsigned bits, cudaStream_t st);
+
 // Philox4x32-10 + Box-Muller fields x[w][n] for global step `step`.
 // x[w][n] for walkers w0 + w (w < W): counter (n/4, w0 + w, step, 0)
 void philox_fields(uint64_t seed, int64_t step, int W, int Nchol, double* x, cudaStream_t st, int w0 = 0);
