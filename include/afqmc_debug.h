@@ -139,6 +139,10 @@ int afqmc_debug_energy_products(afqmc_wk_debug_t wk, double* mean);
  * start of its set-up (0: no longer).  For tests of the calls that report them.  Errors: BADARG. */
 int afqmc_debug_set_status(afqmc_wk_debug_t wk, unsigned bits);
 
+/* The largest workspace that walker sets made by the calling thread from now on can allocate for the slices of
+ * their FP64 products, as if device memory held no more (negative: no limit). */
+int afqmc_debug_set_slice_room(long long bytes);
+
 /* Failure detection without a fault: one warp waits, by the library's bounded mbarrier wait
  * (try_wait polled against a clock64 budget) with a budget of limit_cycles SM clock cycles
  * (1 .. the production bound of 4e9), on a barrier phase that completes only if

@@ -566,8 +566,12 @@ static int init_walkers_impl(afqmc_ham_t ham, int ND, const double* Psi_up, cons
         const int N = wk->N[s];
         const int64_t mn = (int64_t)M * N, tot = (int64_t)nch * N * M;
         cplx* tmp = nullptr;
-        if (cudaMallocAsync(&tmp, sizeof(cplx) * (size_t)tot, st) != cudaSuccess)
-            return bail(fail(AFQMC_ERR_OOM, "init_walkers: workspace"));
+        if (cudaMallocAsync(&tmp, sizeof(cplx) * (size_t)tot, st) != cudaSuccess) {
+            cudaGetLastError();
+            fp64_free_optional(wk);
+            if (cudaMallocAsync(&tmp, sizeof(cplx) * (size_t)tot, st) != cudaSuccess)
+                return bail(fail(AFQMC_ERR_OOM, "init_walkers: workspace"));
+        }
         for (int I = 0; I < ND; ++I) {
             const cplx* Psi = f.Psi[s] + I * mn;
             GemmArgs g;   // tmp[n] = Psi^+ L_n   [N][M]

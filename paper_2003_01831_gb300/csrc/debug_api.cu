@@ -290,6 +290,11 @@ extern "C" int afqmc_debug_set_status(afqmc_wk_debug_t wk, unsigned bits) {
     return AFQMC_OK;
 }
 
+extern "C" int afqmc_debug_set_slice_room(long long bytes) {
+    launch_policy().slice_room = bytes < 0 ? SIZE_MAX : (size_t)bytes;
+    return AFQMC_OK;
+}
+
 extern "C" int afqmc_debug_gemm(const long long* d, const long long* sizes, const double* ab, const double* A,
                                 const double* B, double* C, double* D, int form, long long ws_bytes, int reps,
                                 int* chose, float* ms) {

@@ -132,6 +132,7 @@ struct afqmc_walkers {
 namespace afqmc {
 
 // step drivers (step_fp64.cu / step_tc.cu)
+void fp64_free_optional(afqmc_walkers* wk);   // gives back what the set can do without
 void fp64_split_propagator(afqmc_walkers* wk, cudaStream_t st);   // once Bh is there
 int fp64_alloc(afqmc_walkers* wk);
 void fp64_free(afqmc_walkers* wk);

@@ -58,6 +58,30 @@ void overlap(const cplx* Psi, const cplx* Phi, cplx* S, int M, int N, int W, Sli
 
 }  // namespace
 
+// What the products on the tensor cores use, after everything a walker set needs: the slice workspace, or a half, a
+// quarter, ... of it down to 8 MB (products then run in parts), or none (by the multiply-add pipe); and the
+// one-body propagator without its diagonal.
+static int alloc_optional(afqmc_walkers* wk, size_t slices) {
+    Fp64Buffers& f = wk->f;
+    const size_t limit = launch_policy().slice_room;
+    for (size_t bytes = slices; bytes > 0; bytes = bytes >= (size_t)16 << 20 ? bytes / 2 : 0) {
+        if (bytes <= limit && cudaMalloc(&f.ws.buf, bytes) == cudaSuccess) {
+            f.ws.bytes = bytes;
+            f.ws.flags = wk->flags;
+            AFQMC_TRY(slice_scratch_init(&f.ws));
+            break;
+        }
+        cudaGetLastError();
+        f.ws.buf = nullptr;
+    }
+    const size_t MM = (size_t)wk->M * wk->M * (wk->ham->cplx_L ? 2 : 1);
+    if (f.ws.buf && cudaMalloc(reinterpret_cast<void**>(&f.Bo), sizeof(double) * MM) != cudaSuccess) {
+        cudaGetLastError();
+        f.Bo = nullptr;
+    }
+    return AFQMC_OK;
+}
+
 int fp64_alloc(afqmc_walkers* wk) {
     Fp64Buffers& f = wk->f;
     const int M = wk->M, W = wk->W, nch = wk->Nchol, ND = wk->ND;
@@ -95,7 +119,6 @@ int fp64_alloc(afqmc_walkers* wk) {
         AFQMC_TRY(dalloc(&f.X[s], nd * W * nch));
     }
     AFQMC_TRY(dalloc(&f.Bh, (size_t)M * M * (wk->ham->cplx_L ? 2 : 1)));
-    if (wk->opts.precision == AFQMC_PREC_FP64) AFQMC_TRY(dalloc(&f.Bo, (size_t)M * M * (wk->ham->cplx_L ? 2 : 1)));
     if (Nmu > 0) {   // walker chunks of the THC densities T and of X diag(U c)
         const size_t per_w = std::max((size_t)Nmu * Nmu, (size_t)M * Nmu) * sizeof(cplx);
         f.thc_wc = (int)std::max<size_t>(1, std::min<size_t>((size_t)W, budget / per_w));
@@ -112,6 +135,7 @@ int fp64_alloc(afqmc_walkers* wk) {
         AFQMC_TRY(dalloc(&f.T, (size_t)f.nc * nd * W * Nmax * Nmax));
     }
     AFQMC_TRY(dalloc(&f.A, (size_t)W * M * M));
+    size_t slices = 0;
     if (wk->opts.precision == AFQMC_PREC_FP64) {
         // slices of the step's largest products, up to a bound beyond which they run in pieces
         auto shape = [&](int64_t m, int64_t n, int64_t k, int64_t nba, int64_t nbb, int64_t nbs, bool ar, bool br) {
@@ -133,10 +157,7 @@ int fp64_alloc(afqmc_walkers* wk) {
         }
         if (Nmu > 0) need = std::max(need, shape(M, M, Nmu, f.thc_wc, 1, 1, false, true));
         else need = std::max(need, shape(W, (int64_t)M * M, nch, 1, 1, 1, false, rl));
-        f.ws.bytes = std::min(need, (size_t)768 << 20);
-        AFQMC_TRY(dalloc(reinterpret_cast<char**>(&f.ws.buf), f.ws.bytes));
-        f.ws.flags = wk->flags;
-        AFQMC_TRY(slice_scratch_init(&f.ws));
+        slices = std::min(need, (size_t)768 << 20);
     }
     if (ND > 1) {
         AFQMC_TRY(dalloc(&f.msd_cc, (size_t)ND));
@@ -146,7 +167,16 @@ int fp64_alloc(afqmc_walkers* wk) {
         AFQMC_TRY(dalloc(&f.msd_flag, 2));
         AFQMC_TRY(dalloc(&f.msd_Es, nd * W));
     }
+    if (slices > 0) AFQMC_TRY(alloc_optional(wk, slices));
     return AFQMC_OK;
+}
+
+void fp64_free_optional(afqmc_walkers* wk) {
+    Fp64Buffers& f = wk->f;
+    if (f.ws.buf) cudaFree(f.ws.buf);
+    if (f.Bo) cudaFree(f.Bo);
+    f.ws = SliceScratch{};
+    f.Bo = nullptr;
 }
 
 void fp64_free(afqmc_walkers* wk) {
