@@ -1247,14 +1247,22 @@ bool run_plan(const GemmArgs& g, const Plan& p, SliceScratch* ws, cudaStream_t s
         return make_map4(m, x.out, dims, str, box, 64);
     };
     if (encode(&mr, R, rr, kRows) != AFQMC_OK || encode(&mq, Q, rc, p.pair ? kCols / 2 : kCols) != AFQMC_OK) return false;
-    auto kept = [&](bool keep, SliceScratch::Packed& have, const PackArgs& x, int64_t rows) {
-        const bool same = keep && have.rows == rows && have.pitch == x.Kp && have.batches == nz;
-        have = SliceScratch::Packed{rows, x.Kp, nz};
-        if (same) return;
-        launch_pack(x, st);
+    auto kept = [&](bool keep, SliceScratch::Packed& have, const PackArgs& x, int64_t rows, bool is_a) {
+        const Dims &own = is_a ? p.aown : p.bown, &shared = is_a ? p.shared_a : p.shared_b;
+        SliceScratch::Packed now{x.ptr, x.out, {rows, x.Kp, nz, x.n, x.k, x.klen, x.si, x.sk}, {}, x.scale ? x.alpha : one,
+                                 x.real | x.conj << 1 | x.expand << 2 | x.scale << 3};
+        for (int i = 0; i < 3; ++i) {
+            now.batch[i] = own.cnt[i];
+            now.batch[3 + i] = own.str[i];
+            now.batch[6 + i] = shared.cnt[i];
+            now.batch[9 + i] = shared.str[i];
+        }
+        const bool same = keep && have == now;
+        have = now;
+        if (!same) launch_pack(x, st);
     };
-    kept(g.keep_b, ws->b, pb, p.rows_b);
-    kept(g.keep_a, ws->a, pa, p.rows_a);
+    kept(g.keep_b, ws->b, pb, p.rows_b, false);
+    kept(g.keep_a, ws->a, pa, p.rows_a, true);
     OutArgs o{};
     o.rows = rr;
     o.cols = rc;

@@ -19,16 +19,26 @@ struct GemmOperand {
 };
 
 // Workspace of the products that run on the tensor cores (gemm_slices.cu): device memory for the
-// operands' slices and the status word their bounded waits report to; a, b: the shapes of the
-// operands whose slices it holds (of the last product).  The last whole kilobyte of buf holds counts that are zero between
+// operands' slices and the status word their bounded waits report to; a, b: the operands whose slices it
+// holds (of the last product).  The last whole kilobyte of buf holds counts that are zero between
 // products: to be cleared when it is allocated.
 constexpr size_t kSliceHead = 1024;
 struct SliceScratch {
     void* buf = nullptr;
     size_t bytes = 0;
     unsigned* flags = nullptr;
-    struct Packed {
-        int64_t rows = -1, pitch = 0, batches = 0;
+    struct Packed {   // all that decides the slices but the operand's contents, and where they lie
+        const void *ptr = nullptr, *out = nullptr;
+        int64_t shape[8] = {}, batch[12] = {};
+        cplx alpha{0.0, 0.0};
+        int form = -1;
+        bool operator==(const Packed& o) const {
+            for (int i = 0; i < 8; ++i)
+                if (shape[i] != o.shape[i]) return false;
+            for (int i = 0; i < 12; ++i)
+                if (batch[i] != o.batch[i]) return false;
+            return ptr == o.ptr && out == o.out && alpha.re == o.alpha.re && alpha.im == o.alpha.im && form == o.form;
+        }
     } a, b;
 };
 
