@@ -493,8 +493,19 @@ __global__ void __launch_bounds__(kT) gram_planar_kernel(const double* PhiT, int
 }
 
 // 1 / sqrt(d) for a float pair d > 0: one step y (1 + e / 2 + 3 e^2 / 8), e = 1 - d y^2, from the
-// single-precision value, e and the product as float pairs (2^-22 -> 2^-48).
+// single-precision value, e and the product as float pairs (2^-22 -> 2^-48).  d is scaled by an even power of
+// two to [1, 4) first: y^2 overflows for d below 2^-128, and its error's error is lost for d above 2^100.
 __device__ __forceinline__ void ff_rsqrt(float dh, float dl, float& rh, float& rl) {
+    int half = 0;   // d = (scaled d) 4^-half
+    if (dh < 0x1p-100f) {
+        dh *= 0x1p64f;
+        dl *= 0x1p64f;
+        half = 32;
+    }
+    const int m = (int)(__float_as_uint(dh) >> 23) - 127 >> 1;
+    const float s4 = __uint_as_float((unsigned)(127 - 2 * m) << 23), back = __uint_as_float((unsigned)(127 - m + half) << 23);
+    dh *= s4;
+    dl *= s4;
     const float y = rsqrtf(dh);
     const float p = y * y, pe = fmaf(y, y, -p);
     const float q = dh * p, qe = fmaf(dh, p, -q);
@@ -505,8 +516,9 @@ __device__ __forceinline__ void ff_rsqrt(float dh, float dl, float& rh, float& r
     float s, t;
     two_sum(y, c, s, t);
     t += ce;
-    rh = s + t;
-    rl = t - (rh - s);
+    const float h = s + t;
+    rh = h * back;
+    rl = (t - (h - s)) * back;
 }
 
 // In place on G[ws]: the inverse X of the upper Cholesky factor R (G = R^H R, real positive
