@@ -2218,10 +2218,12 @@ namespace {
 // for such L_n it equals X^+ X with X[(n, k)][i] = L[n][k][i], a contiguous [Nchol*M][M]
 // matrix.  The K = Nchol*M reduction is split into `parts` GEMMs (fixed split, reduced in a
 // fixed order by the caller's kernel) to fill the GPU.  gram_parts: two CTAs a SM over the
-// output's tiles, at least 4 vectors a part beyond 16.  Returns the workspace, or NULL.
+// output's tiles, at least 4 vectors a part beyond 16; and 16 in any case, which bounds the length of a part's
+// sum (2560 vectors of M = 512 in five parts: errors of 1.9e-14 relative on the diagonal, in sixteen
+// 0.75e-14).  Returns the workspace, or NULL.
 int gram_parts(int M, int Nchol) {
-    const int tiles = ((M + 63) / 64) * ((M + 63) / 64);
-    return std::max(1, std::min({Nchol, (304 + tiles - 1) / tiles, std::max(16, Nchol / 4)}));
+    const int tiles = ((M + 63) / 64) * ((M + 63) / 64), fill = (2 * tc_num_sms() + tiles - 1) / tiles;
+    return std::max({1, std::min(Nchol, 16), std::min({Nchol, fill, Nchol / 4})});
 }
 
 cplx* gram_of_cholesky(const void* L, bool real, int M, int Nchol, int parts, cudaStream_t st) {
