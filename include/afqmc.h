@@ -29,6 +29,8 @@
  *     (re, im) pairs of doubles, i.e. numpy complex128 / C double _Complex.
  *   - Handles own their device memory; destroy them with the matching
  *     afqmc_destroy_* call.  A handle must not be used from two threads at once.
+ *     A Hamiltonian on which gradients or back-propagation estimates have run keeps
+ *     up to 1 GB of the memory they used for the next of them until it is destroyed.
  */
 #ifndef AFQMC_GB300_H
 #define AFQMC_GB300_H

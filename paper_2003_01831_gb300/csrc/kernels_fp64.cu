@@ -1896,7 +1896,7 @@ int zgemm_form(const GemmArgs& g, const SliceScratch* ws) {
     const double per = (g.A.real ? 1.0 : 2.0) * (g.B.real ? 1.0 : 2.0) * g.k;   // multiply-adds an output
     const int ts = zgemm_tile(g);
     const double tiles = nbatch * ((g.m + ts - 1) / ts) * ((g.n + ts - 1) / ts);
-    const double tiled_us = 3.0 + ceil(tiles / 152.0) * ts * ts * per / 3.4e3;
+    const double tiled_us = 3.0 + ceil(tiles / tc_num_sms()) * ts * ts * per / 3.4e3;
     const double outputs = nbatch * g.m * g.n;
     const double thread_us = outputs < 2e9 ? 3.0 + std::max(outputs * per / 3.0e5, 0.05 * g.k) + 0.01 * g.k : 1e30;
     const double slice_us = ws && ws->buf && g.k > 0 ? slice_gemm_us(g) : 1e30;
@@ -2058,18 +2058,19 @@ void trace_terms(const cplx* T, int nc, int W, int N, int n0, cplx* t_out, cplx*
         count_launch();
         kern<<<(unsigned)grid, threads, one * groups, st>>>(T, count, W, N, n0, t_out, X_out, ldo);
     };
-    // CTAs: as many as shared memory lets an SM hold, 152 SMs, a few rounds each
+    // CTAs: as many as shared memory lets an SM hold, on every SM, a few rounds each
+    const int sms = tc_num_sms();
     if (N <= 32) {
         // one CTA of twelve matrices where two of eight do not fit an SM (N = 32: 3.9 -> 3.6 ms a step)
         if (2 * 8 * one > 220000)
-            go(trace_pairs_kernel<32, 384>, 384, 12, 152 * 4);
+            go(trace_pairs_kernel<32, 384>, 384, 12, sms * 4);
         else
             go(trace_pairs_kernel<32, kThreads>, kThreads, kThreads / 32,
-               152 * std::max(1, std::min(8, (int)(220000 / (one * (kThreads / 32))))) * 4);
+               sms * std::max(1, std::min(8, (int)(220000 / (one * (kThreads / 32))))) * 4);
         return;
     }
     if (one <= 220000) {   // N <= 117
-        go(trace_pairs_kernel<kThreads, kThreads>, kThreads, 1, 152 * std::max(1, std::min(8, (int)(220000 / one))) * 4);
+        go(trace_pairs_kernel<kThreads, kThreads>, kThreads, 1, sms * std::max(1, std::min(8, (int)(220000 / one))) * 4);
         return;
     }
     dim3 grid(W, nc);

@@ -1637,7 +1637,7 @@ __global__ void __launch_bounds__(kG3Threads, 1)
             constexpr uint32_t idesc = idesc_bf16(PAIR ? 2 * kBM : kBM, 128, true);
             constexpr uint32_t A = kG3ABytes >> 4, B = St::kBBytes >> 4;
             const uint32_t d1 = ctl->tmem_base, d2 = d1 + 128, d3 = d1 + 256, d4 = d1 + 384;
-            const uint64_t d0 = kG3BK == 64 ? desc_sw128(smem_u32(sbase)) : desc_sw64(smem_u32(sbase));
+            const uint64_t d0 = desc_sw128(smem_u32(sbase));   // rows of kG3BK x 2 = 128 bytes
             const uint32_t lo0 = (uint32_t)d0, hi = (uint32_t)(d0 >> 32);
             int64_t g = 0;
             int it = 0;

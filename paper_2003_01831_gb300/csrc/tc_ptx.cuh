@@ -203,13 +203,10 @@ __device__ __forceinline__ uint32_t mapa_shared(const void* p, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
     return r;
 }
-// Arrive on an mbarrier given by its cluster-window address (this CTA's or the peer's).
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
-}
-// The same without ordering this thread's earlier memory operations, whose way to the cluster (1400
-// cycles behind a few global stores) it would otherwise wait for: where the arrival says only that
-// tensor memory has been read (tcgen05.wait::ld).
+// Arrive on an mbarrier given by its cluster-window address (this CTA's or the peer's), without ordering
+// this thread's earlier memory operations, whose way to the cluster (1400 cycles behind a few global
+// stores) it would otherwise wait for: where the arrival says only that tensor memory has been read
+// (tcgen05.wait::ld).
 __device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t bar_cluster_addr) {
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
 }
@@ -249,17 +246,8 @@ __device__ __forceinline__ void tmem_relinquish_pair() {
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
-// D[tmem of both CTAs] (+)= A * B^T over the pair (M = 256), f16 inputs, f32 accumulate.
-__device__ __forceinline__ void mma_f16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                             uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// The same from the low words of the two descriptors and their common high word (see mma_f16_lo).
+// D[tmem of both CTAs] (+)= A * B^T over the pair (M = 256), f16 inputs, f32 accumulate, from the low words of
+// the two descriptors and their common high word (see mma_f16_lo).
 __device__ __forceinline__ void mma_f16_pair_lo(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
                                                 uint32_t accumulate) {
     asm volatile(

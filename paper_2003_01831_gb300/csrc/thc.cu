@@ -20,6 +20,7 @@
 #include <string>
 
 #include "kernels_fp64.cuh"
+#include "kernels_tc.cuh"
 
 namespace afqmc {
 
@@ -226,7 +227,7 @@ int thc_pivoted_cholesky(const double* Mk, int n, double rtol, double* work, dou
 
 int thc_exchange_shares(int wc, int Nmu) {
     const int nt = (Nmu + 31) / 32;
-    return std::max(1, std::min(nt * (nt + 1) / 2, (152 * 4 + wc - 1) / wc));   // four CTAs fit an SM
+    return std::max(1, std::min(nt * (nt + 1) / 2, (4 * tc_num_sms() + wc - 1) / wc));   // four CTAs fit an SM
 }
 
 void thc_exchange(const cplx* T, int wc, int Nmu, const double* Mk, cplx* g, cplx* ex, cplx* part, cudaStream_t st) {
