@@ -398,9 +398,9 @@ __device__ __forceinline__ int epi_and(int pred) {
 // the scale 2^(ea + eb); below 2^53 of them (a quarter of the scale) in units 2^-8 of that, whose bit in
 // `fine` is set.  Every sum is exact but that of the two smallest accumulators.  Two accumulators at a
 // time, to hold few of them in registers.  Conversion to integers by adding 1.5 2^23, which leaves the
-// integer in the low bits (the conversion instruction has an eighth of the rate and took half of the time
-// that tensor memory waits for its readers); beyond 2^22, which only accumulators 2 to 5 of all but equal
-// entries reach, by the instruction.
+// integer in the low bits (the conversion instruction has an eighth of the rate); beyond 2^22, which only
+// accumulators 2 to 5 of all but equal entries reach, by the instruction.  Bound by the reads of tensor memory:
+// 4300 cycles for its 256 KB; half of the instructions here gained nothing.
 constexpr int kGather = 41;
 constexpr float kMagic = 12582912.0f;
 constexpr int kMagicBits = 0x4b400000;
@@ -416,14 +416,13 @@ __device__ __forceinline__ void gather(long long (&I)[16], int c0, const uint32_
             over |= (unsigned)((r0 ^ kMagicBits) | (r1 ^ kMagicBits));
             top[j] = (int)(((unsigned)(r0 - kMagicBits) << 8) + (unsigned)(r1 - kMagicBits));
         }
-        if (STEP > 0 && (over >> 23) != 0u) {
+        constexpr long long unit = STEP == 0 ? 1ll << 33 : (STEP == 1 ? 1ll << 17 : 2ll);
+        if (STEP > 0 && (over >> 23) != 0u) {   // a pair may be beyond 32 bits
 #pragma unroll
-            for (int j = 0; j < 8; ++j) top[j] = (__float2int_rn(f(0, j)) << 8) + __float2int_rn(f(1, j));
-        }
+            for (int j = 0; j < 8; ++j) I[c0 + j] += (256ll * __float2int_rn(f(0, j)) + __float2int_rn(f(1, j))) * unit;
+        } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            if (STEP == 0) I[c0 + j] = (long long)top[j] << 33;
-            else I[c0 + j] += (long long)top[j] * (STEP == 1 ? 1 << 17 : 2);
+            for (int j = 0; j < 8; ++j) I[c0 + j] = (STEP == 0 ? 0ll : I[c0 + j]) + top[j] * unit;
         }
     } else {          // a6 2^-7 + a7 2^-15
 #pragma unroll
