@@ -188,7 +188,7 @@ int afqmc_destroy_hamiltonian(afqmc_ham_t ham);
  * afqmc_create_batch pads any shape exactly).
  * An FP64 set also takes device memory for its products' operands on the tensor cores, up to 768 MB, or
  * what part of it, down to none, can be allocated (the products then run in parts or on the
- * multiply-add pipe: slower, not refused).
+ * multiply-add pipe: slower, not refused).  A later call on the set that finds no memory gives it back.
  * Errors: BADARG, SHAPE, UNSUPPORTED, SINGULAR (a walker with zero overlap),
  * NONFINITE, OOM, CUDA. */
 int afqmc_init_walkers(afqmc_ham_t ham, const double* Psi_up, const double* Psi_dn, int Nup, int Ndn,

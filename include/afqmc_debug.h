@@ -143,6 +143,13 @@ int afqmc_debug_set_status(afqmc_wk_debug_t wk, unsigned bits);
  * their FP64 products, as if device memory held no more (negative: no limit). */
 int afqmc_debug_set_slice_room(long long bytes);
 
+/* The next n allocations that the calling thread's calls make for a walker set (trace and field buffers, a window's,
+ * a gradient's or an estimate's memory, parts of a set-up) find no memory at the first attempt. */
+int afqmc_debug_short_allocs(int n);
+
+/* Bytes of the slice workspace that a walker set holds now (0: none, -1: wk is NULL). */
+long long afqmc_debug_slice_bytes(afqmc_wk_debug_t wk);
+
 /* Failure detection without a fault: one warp waits, by the library's bounded mbarrier wait
  * (try_wait polled against a clock64 budget) with a budget of limit_cycles SM clock cycles
  * (1 .. the production bound of 4e9), on a barrier phase that completes only if

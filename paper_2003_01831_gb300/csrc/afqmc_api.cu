@@ -117,7 +117,8 @@ int copy_out(void* dst, const void* src, size_t bytes, cudaStream_t st, bool* ne
     return AFQMC_OK;
 }
 
-cudaError_t call_alloc(afqmc_ham* ham, void** p, size_t bytes, cudaStream_t st) {
+cudaError_t call_alloc(afqmc_walkers* wk, void** p, size_t bytes, cudaStream_t st) {
+    afqmc_ham* ham = wk->ham;
     std::call_once(ham->call_pool_once, [ham] {
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
@@ -131,7 +132,17 @@ cudaError_t call_alloc(afqmc_ham* ham, void** p, size_t bytes, cudaStream_t st) 
             ham->call_pool = nullptr;
         }
     });
-    return ham->call_pool ? cudaMallocFromPoolAsync(p, bytes, ham->call_pool, st) : cudaMallocAsync(p, bytes, st);
+    return with_room(wk, [&] {
+        return ham->call_pool ? cudaMallocFromPoolAsync(p, bytes, ham->call_pool, st) : cudaMallocAsync(p, bytes, st);
+    });
+}
+
+cudaError_t give_room(afqmc_walkers* wk) {
+    if (!wk->f.ws.buf && !wk->ham->call_pool) return cudaErrorMemoryAllocation;
+    cudaDeviceSynchronize();   // what the pool has been given back is free once its streams have come to it
+    fp64_free_optional(wk);
+    if (wk->ham->call_pool) cudaMemPoolTrimTo(wk->ham->call_pool, 0);
+    return cudaSuccess;
 }
 
 int read_flags(unsigned* dflags, cudaStream_t st, unsigned* out) {
@@ -566,12 +577,8 @@ static int init_walkers_impl(afqmc_ham_t ham, int ND, const double* Psi_up, cons
         const int N = wk->N[s];
         const int64_t mn = (int64_t)M * N, tot = (int64_t)nch * N * M;
         cplx* tmp = nullptr;
-        if (cudaMallocAsync(&tmp, sizeof(cplx) * (size_t)tot, st) != cudaSuccess) {
-            cudaGetLastError();
-            fp64_free_optional(wk);
-            if (cudaMallocAsync(&tmp, sizeof(cplx) * (size_t)tot, st) != cudaSuccess)
-                return bail(fail(AFQMC_ERR_OOM, "init_walkers: workspace"));
-        }
+        if (with_room(wk, [&] { return cudaMallocAsync(&tmp, sizeof(cplx) * (size_t)tot, st); }) != cudaSuccess)
+            return bail(fail(AFQMC_ERR_OOM, "init_walkers: workspace"));
         for (int I = 0; I < ND; ++I) {
             const cplx* Psi = f.Psi[s] + I * mn;
             GemmArgs g;   // tmp[n] = Psi^+ L_n   [N][M]
@@ -604,9 +611,16 @@ static int init_walkers_impl(afqmc_ham_t ham, int ND, const double* Psi_up, cons
         }
         cudaFreeAsync(tmp, st);
     }
-    rc = ham->cplx_L ? expm_complex(reinterpret_cast<const cplx*>(ham->hp), -0.5 * tau, M,
-                                    reinterpret_cast<cplx*>(f.Bh), st)
-                     : expm_real(ham->hp, -0.5 * tau, M, f.Bh, st);
+    auto expm = [&] {
+        return ham->cplx_L ? expm_complex(reinterpret_cast<const cplx*>(ham->hp), -0.5 * tau, M,
+                                          reinterpret_cast<cplx*>(f.Bh), st)
+                           : expm_real(ham->hp, -0.5 * tau, M, f.Bh, st);
+    };
+    rc = expm();
+    if (rc == AFQMC_ERR_OOM && give_room(wk) == cudaSuccess) {
+        cudaGetLastError();
+        rc = expm();
+    }
     if (rc) return bail(rc);
     fp64_split_propagator(wk, st);
     // trial energy E_T: the trial's energy shift (its variational energy unless two determinants
@@ -624,9 +638,10 @@ static int init_walkers_impl(afqmc_ham_t ham, int ND, const double* Psi_up, cons
         AFQMC_CUDA_TRY(cudaMemcpyAsync(&et, wk->E_L, sizeof(cplx), cudaMemcpyDeviceToHost, st));
     } else {
         cplx *EIJ = nullptr, *LIJ = nullptr, *d_et = nullptr;
-        if (cudaMallocAsync(&EIJ, sizeof(cplx) * ND * ND, st) != cudaSuccess ||
-            cudaMallocAsync(&LIJ, sizeof(cplx) * ND * ND, st) != cudaSuccess ||
-            cudaMallocAsync(&d_et, sizeof(cplx), st) != cudaSuccess)
+        auto get = [&](cplx** p, size_t n) {
+            return with_room(wk, [&] { return cudaMallocAsync(p, sizeof(cplx) * n, st); }) == cudaSuccess;
+        };
+        if (!get(&EIJ, (size_t)ND * ND) || !get(&LIJ, (size_t)ND * ND) || !get(&d_et, 1))
             return bail(fail(AFQMC_ERR_OOM, "init_walkers: workspace"));
         for (int J = 0; J < ND; ++J) {
             for (int s = 0; s < 2; ++s)
@@ -702,11 +717,24 @@ static int init_walkers_impl(afqmc_ham_t ham, int ND, const double* Psi_up, cons
     return AFQMC_OK;
 }
 
+// The set-up, once more without what the call pool keeps where memory is short.
+static int init_walkers_room(afqmc_ham_t ham, int ND, const double* Psi_up, const double* Psi_dn, const double* coef,
+                             int Nup, int Ndn, int W, const double* Phi0, double tau, const afqmc_opts* opts, void* stream,
+                             afqmc_wk_t* out) {
+    auto go = [&] { return init_walkers_impl(ham, ND, Psi_up, Psi_dn, coef, Nup, Ndn, W, Phi0, tau, opts, stream, out); };
+    const int rc = go();
+    if (rc != AFQMC_ERR_OOM || !ham->call_pool) return rc;
+    cudaDeviceSynchronize();
+    cudaMemPoolTrimTo(ham->call_pool, 0);
+    cudaGetLastError();
+    return go();
+}
+
 extern "C" {
 
 int afqmc_init_walkers(afqmc_ham_t ham, const double* Psi_up, const double* Psi_dn, int Nup, int Ndn, int W,
                        const double* Phi0, double tau, const afqmc_opts* opts, void* stream, afqmc_wk_t* out) {
-    return init_walkers_impl(ham, 1, Psi_up, Psi_dn, nullptr, Nup, Ndn, W, Phi0, tau, opts, stream, out);
+    return init_walkers_room(ham, 1, Psi_up, Psi_dn, nullptr, Nup, Ndn, W, Phi0, tau, opts, stream, out);
 }
 
 int afqmc_init_walkers_msd(afqmc_ham_t ham, int ND, const double* D_up, const double* D_dn, const double* c,
@@ -716,7 +744,7 @@ int afqmc_init_walkers_msd(afqmc_ham_t ham, int ND, const double* D_up, const do
         if (out) *out = nullptr;
         return fail(AFQMC_ERR_BADARG, "init_walkers_msd: NULL coefficients");
     }
-    return init_walkers_impl(ham, ND, D_up, D_dn, c, Nup, Ndn, W, Phi0, tau, opts, stream, out);
+    return init_walkers_room(ham, ND, D_up, D_dn, c, Nup, Ndn, W, Phi0, tau, opts, stream, out);
 }
 
 int afqmc_destroy_walkers(afqmc_wk_t wk) {
@@ -731,7 +759,7 @@ static int ensure_x(afqmc_walkers* wk, int steps) {
     if (steps <= wk->x_cap) return AFQMC_OK;
     cudaFree(wk->x);
     wk->x = nullptr;
-    if (cudaMalloc(&wk->x, sizeof(double) * (size_t)steps * wk->W * wk->Nchol) != cudaSuccess) {
+    if (set_malloc(wk, (void**)&wk->x, sizeof(double) * (size_t)steps * wk->W * wk->Nchol) != cudaSuccess) {
         cudaGetLastError();
         wk->x_cap = 0;
         return fail(AFQMC_ERR_OOM, "step: field buffer");
@@ -746,7 +774,8 @@ static int ensure_emix(afqmc_walkers* wk, int n) {
     cudaFree(wk->esum);
     wk->emix = nullptr;
     wk->esum = nullptr;
-    if (cudaMalloc(&wk->emix, sizeof(cplx) * n) != cudaSuccess || cudaMalloc(&wk->esum, sizeof(cplx) * 2 * n) != cudaSuccess) {
+    if (set_malloc(wk, (void**)&wk->emix, sizeof(cplx) * n) != cudaSuccess ||
+        set_malloc(wk, (void**)&wk->esum, sizeof(cplx) * 2 * n) != cudaSuccess) {
         cudaGetLastError();
         wk->emix_cap = 0;
         return fail(AFQMC_ERR_OOM, "step: trace buffer");
@@ -821,10 +850,10 @@ int afqmc_population_control(afqmc_wk_t wk, double xi, int* idx, void* stream) {
                 if (q) cudaFree(q);
         }
     } sc;
-    if (cudaMalloc(&sc.p[0], sizeof(int) * W) != cudaSuccess || cudaMalloc(&sc.p[1], sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&sc.p[2], sizeof(cplx) * (size_t)W * std::max<size_t>((size_t)M * std::max(wk->N[0], wk->N[1]),
-                                                                          (size_t)wk->Nchol)) != cudaSuccess ||
-        cudaMalloc(&sc.p[3], sizeof(cplx) * W) != cudaSuccess) {
+    const size_t row = std::max<size_t>((size_t)M * std::max(wk->N[0], wk->N[1]), (size_t)wk->Nchol);
+    if (set_malloc(wk, &sc.p[0], sizeof(int) * W) != cudaSuccess || set_malloc(wk, &sc.p[1], sizeof(double)) != cudaSuccess ||
+        set_malloc(wk, &sc.p[2], sizeof(cplx) * (size_t)W * row) != cudaSuccess ||
+        set_malloc(wk, &sc.p[3], sizeof(cplx) * W) != cudaSuccess) {
         cudaGetLastError();
         return fail(AFQMC_ERR_OOM, "population_control: scratch");
     }

@@ -151,13 +151,13 @@ int walker_chunks(int W, int M) {
 
 struct Scratch {
     std::vector<void*> p;
-    afqmc_ham* ham;
+    afqmc_walkers* wk;
     cudaStream_t st;
-    Scratch(afqmc_walkers* wk, cudaStream_t s) : ham(wk->ham), st(s) {}
+    Scratch(afqmc_walkers* w, cudaStream_t s) : wk(w), st(s) {}
     template <typename T>
     T* get(size_t count) {
         void* q = nullptr;
-        if (call_alloc(ham, &q, sizeof(T) * std::max<size_t>(count, 1), st) != cudaSuccess) {
+        if (call_alloc(wk, &q, sizeof(T) * std::max<size_t>(count, 1), st) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;
         }
@@ -188,8 +188,8 @@ int bp_open(afqmc_walkers* wk, int nbp, cudaStream_t st) {
     const int M = wk->M, W = wk->W;
     bool ok = true;
     for (int s = 0; s < 2; ++s)
-        ok = ok && cudaMalloc(&wk->bp_Phi[s], sizeof(cplx) * (size_t)W * M * wk->N[s]) == cudaSuccess;
-    ok = ok && cudaMalloc(&wk->bp_coef, sizeof(cplx) * (size_t)std::max(nbp, 1) * W * wk->Nchol) == cudaSuccess;
+        ok = ok && set_malloc(wk, (void**)&wk->bp_Phi[s], sizeof(cplx) * (size_t)W * M * wk->N[s]) == cudaSuccess;
+    ok = ok && set_malloc(wk, (void**)&wk->bp_coef, sizeof(cplx) * (size_t)std::max(nbp, 1) * W * wk->Nchol) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         bp_close(wk);

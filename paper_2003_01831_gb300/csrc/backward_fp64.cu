@@ -82,14 +82,14 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
     if (wk->opts.precision == AFQMC_PREC_BF16X3) AFQMC_TRY(tc_sync_walkers_to_fp64(wk, st));
     // upstream factors (conjugated), device copies
     cplx *gE = nullptr, *gS = nullptr, *dEd = nullptr, *dSd = nullptr;
-    AFQMC_CUDA_TRY(call_alloc(wk->ham, reinterpret_cast<void**>(&gE), sizeof(cplx) * W, st));
-    AFQMC_CUDA_TRY(call_alloc(wk->ham, reinterpret_cast<void**>(&gS), sizeof(cplx) * W, st));
+    AFQMC_CUDA_TRY(call_alloc(wk, reinterpret_cast<void**>(&gE), sizeof(cplx) * W, st));
+    AFQMC_CUDA_TRY(call_alloc(wk, reinterpret_cast<void**>(&gS), sizeof(cplx) * W, st));
     if (dE) {
-        AFQMC_CUDA_TRY(call_alloc(wk->ham, reinterpret_cast<void**>(&dEd), sizeof(cplx) * W, st));
+        AFQMC_CUDA_TRY(call_alloc(wk, reinterpret_cast<void**>(&dEd), sizeof(cplx) * W, st));
         AFQMC_CUDA_TRY(cudaMemcpyAsync(dEd, dE, sizeof(cplx) * W, cudaMemcpyDefault, st));
     }
     if (dlogS) {
-        AFQMC_CUDA_TRY(call_alloc(wk->ham, reinterpret_cast<void**>(&dSd), sizeof(cplx) * W, st));
+        AFQMC_CUDA_TRY(call_alloc(wk, reinterpret_cast<void**>(&dSd), sizeof(cplx) * W, st));
         AFQMC_CUDA_TRY(cudaMemcpyAsync(dSd, dlogS, sizeof(cplx) * W, cudaMemcpyDefault, st));
     }
     count_launch();
@@ -106,19 +106,19 @@ int fp64_backward(afqmc_walkers* wk, const cplx* dE, const cplx* dlogS, cplx* dP
                                                                  ((int64_t)256 << 20) / (per_u * 16)}));
     cplx *U = nullptr, *V = nullptr, *F = nullptr, *G = nullptr, *Z = nullptr, *gP = nullptr;
     double* dLd = nullptr;
-    AFQMC_CUDA_TRY(call_alloc(wk->ham, reinterpret_cast<void**>(&U), sizeof(cplx) * nu * per_u, st));
-    AFQMC_CUDA_TRY(call_alloc(wk->ham, reinterpret_cast<void**>(&V), sizeof(cplx) * (size_t)nu * M * Nmax, st));
-    AFQMC_CUDA_TRY(call_alloc(wk->ham, reinterpret_cast<void**>(&F), sizeof(cplx) * (size_t)nu * M * M, st));
-    AFQMC_CUDA_TRY(call_alloc(wk->ham, reinterpret_cast<void**>(&G), sizeof(cplx) * per_u, st));
-    AFQMC_CUDA_TRY(call_alloc(wk->ham, reinterpret_cast<void**>(&Z), sizeof(cplx) * (size_t)W * Nmax * Nmax, st));
-    AFQMC_CUDA_TRY(call_alloc(wk->ham, reinterpret_cast<void**>(&gP), sizeof(cplx) * (size_t)M * Nmax, st));
+    AFQMC_CUDA_TRY(call_alloc(wk, reinterpret_cast<void**>(&U), sizeof(cplx) * nu * per_u, st));
+    AFQMC_CUDA_TRY(call_alloc(wk, reinterpret_cast<void**>(&V), sizeof(cplx) * (size_t)nu * M * Nmax, st));
+    AFQMC_CUDA_TRY(call_alloc(wk, reinterpret_cast<void**>(&F), sizeof(cplx) * (size_t)nu * M * M, st));
+    AFQMC_CUDA_TRY(call_alloc(wk, reinterpret_cast<void**>(&G), sizeof(cplx) * per_u, st));
+    AFQMC_CUDA_TRY(call_alloc(wk, reinterpret_cast<void**>(&Z), sizeof(cplx) * (size_t)W * Nmax * Nmax, st));
+    AFQMC_CUDA_TRY(call_alloc(wk, reinterpret_cast<void**>(&gP), sizeof(cplx) * (size_t)M * Nmax, st));
     const bool want_L = dL != nullptr;
     if (want_L) {
-        AFQMC_CUDA_TRY(call_alloc(wk->ham, reinterpret_cast<void**>(&dLd), sizeof(double) * (size_t)nch * M * M, st));
+        AFQMC_CUDA_TRY(call_alloc(wk, reinterpret_cast<void**>(&dLd), sizeof(double) * (size_t)nch * M * M, st));
         AFQMC_CUDA_TRY(cudaMemsetAsync(dLd, 0, sizeof(double) * (size_t)nch * M * M, st));
     }
     cplx* gc = nullptr;
-    AFQMC_CUDA_TRY(call_alloc(wk->ham, reinterpret_cast<void**>(&gc), sizeof(cplx) * (size_t)W * nch, st));
+    AFQMC_CUDA_TRY(call_alloc(wk, reinterpret_cast<void**>(&gc), sizeof(cplx) * (size_t)W * nch, st));
     count_launch();
     trace_coefficients_kernel<<<nb((int64_t)W * nch), kT, 0, st>>>(f.t[0], f.t[1], gE, (int64_t)W * nch, nch, wk->coef, gc);
     {   // A_w = sum_n c_n L_n

@@ -65,6 +65,7 @@ struct LaunchPolicy {
     int energy_pair = 1;       // fused energy kernel: 1 CTA pairs (cta_group::2, default), 0 one CTA per tile
     unsigned status = 0;       // status bits raised in every new walker set (tests of the error paths)
     size_t slice_room = SIZE_MAX;   // largest slice workspace of new walker sets that can be allocated (tests)
+    int short_allocs = 0;      // allocations of walker sets after their set-up that find no memory at first (tests)
     int batch_n_granule = 8;   // batches pad N to a multiple of 8 (default), or 32: N' in {32, 64, 128}
 };
 LaunchPolicy& launch_policy();

@@ -295,6 +295,13 @@ extern "C" int afqmc_debug_set_slice_room(long long bytes) {
     return AFQMC_OK;
 }
 
+extern "C" int afqmc_debug_short_allocs(int n) {
+    launch_policy().short_allocs = n;
+    return AFQMC_OK;
+}
+
+extern "C" long long afqmc_debug_slice_bytes(afqmc_wk_debug_t wk) { return wk ? (long long)wk->f.ws.bytes : -1; }
+
 extern "C" int afqmc_debug_gemm(const long long* d, const long long* sizes, const double* ab, const double* A,
                                 const double* B, double* C, double* D, int form, long long ws_bytes, int reps,
                                 int* chose, float* ms) {

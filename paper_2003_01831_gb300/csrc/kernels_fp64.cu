@@ -2358,8 +2358,10 @@ int expm_real(const double* X, double s, int M, double* out, cudaStream_t st) {
     AFQMC_TRY(norm1_on_host(X, true, M, st, &nrm));
     cplx *Y = nullptr, *E = nullptr;
     const size_t bytes = sizeof(cplx) * M * M;
-    if (cudaMallocAsync(&Y, bytes, st) != cudaSuccess || cudaMallocAsync(&E, bytes, st) != cudaSuccess)
+    if (cudaMallocAsync(&Y, bytes, st) != cudaSuccess || cudaMallocAsync(&E, bytes, st) != cudaSuccess) {
+        if (Y) cudaFreeAsync(Y, st);
         return fail(AFQMC_ERR_OOM, "expm workspace");
+    }
     real_to_cplx(X, Y, (int64_t)M * M, st);
     const int rc = expm_taylor_squaring(Y, nrm, s, M, E, st);
     if (rc == AFQMC_OK) {

@@ -186,7 +186,24 @@ int bp_follow_comb(afqmc_walkers* wk, const int* idx, cplx* tmp, cudaStream_t st
 // 6.6 ms of a back-propagation estimate (M = 256, 128 walkers) and 0.7 of the 25.4 ms of a gradient
 // (M = 128, 32 walkers).  The pool goes with the Hamiltonian.
 constexpr uint64_t kCallPoolKeep = 1ull << 30;
-cudaError_t call_alloc(afqmc_ham* ham, void** p, size_t bytes, cudaStream_t st);
+cudaError_t call_alloc(afqmc_walkers* wk, void** p, size_t bytes, cudaStream_t st);
+
+// Memory of a walker set after its set-up.  Where none is left, the set's products go without their slice
+// workspace from then on, the call pool gives back what it keeps, and the allocation is tried again.
+// Not for the sets of a batch, whose captured steps hold the workspace's address (they need no such memory).
+cudaError_t give_room(afqmc_walkers* wk);   // whether there was anything to give back
+template <class F>
+cudaError_t with_room(afqmc_walkers* wk, F alloc) {
+    cudaError_t e = cudaErrorMemoryAllocation;
+    if (launch_policy().short_allocs > 0) --launch_policy().short_allocs;
+    else e = alloc();
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    return give_room(wk) == cudaSuccess ? alloc() : e;
+}
+inline cudaError_t set_malloc(afqmc_walkers* wk, void** p, size_t bytes) {
+    return with_room(wk, [&] { return cudaMalloc(p, bytes); });
+}
 
 // host helpers of the C-ABI front end (afqmc_api.cu)
 bool is_device_ptr(const void* p);

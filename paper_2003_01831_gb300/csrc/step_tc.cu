@@ -964,13 +964,13 @@ namespace {
 // stream-ordered scratch of one call, freed when it goes out of scope
 struct CallScratch {
     std::vector<void*> p;
-    afqmc_ham* ham;
+    afqmc_walkers* wk;
     cudaStream_t st;
-    CallScratch(afqmc_walkers* wk, cudaStream_t s) : ham(wk->ham), st(s) {}
+    CallScratch(afqmc_walkers* w, cudaStream_t s) : wk(w), st(s) {}
     template <typename T>
     T* get(int64_t count) {
         void* q = nullptr;
-        if (call_alloc(ham, &q, sizeof(T) * (size_t)std::max<int64_t>(count, 1), st) != cudaSuccess) {
+        if (call_alloc(wk, &q, sizeof(T) * (size_t)std::max<int64_t>(count, 1), st) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;
         }
