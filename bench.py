@@ -64,11 +64,11 @@ def l2_note(wl):
 # profiles/).  The figure holds for the kernel source it was taken on: a digest of that source
 # (the energy-kernel section of kernels_tc.cu and the PTX wrappers) gates it.
 # DRAM bytes per launch of the energy kernel at the bench workload: one-pass ncu counters on a
-# W = 16 launch of the same kernel (2,467,877,376 read + 8,650,496 written), scaled by 64 to
+# W = 16 launch of the same kernel (2,468,024,576 read + 8,796,416 written), scaled by 64 to
 # W = 1024 -- the kernel streams L~ once per window of 8 walker-spin groups, so its traffic grows
 # in proportion to W (profiles/energy_pair_kernel_traffic_m512.md).  Reported only while the
 # kernel's source matches the digest it was measured on.
-ENERGY_TRAFFIC = {"bytes": 64 * (2467877376 + 8650496), "src_digest": "c70929e6bd3dd0a8"}
+ENERGY_TRAFFIC = {"bytes": 64 * (2468024576 + 8796416), "src_digest": "29469b1bec7b8d48"}
 
 
 def energy_src_digest() -> str:
